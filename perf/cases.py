@@ -210,11 +210,14 @@ _SIGMA = [np.array([[0, 1], [1, 0]], complex), np.array([[0, -1j], [1j, 0]], com
 
 
 def _gammas():
+    """Each gamma matrix has one entry per row: (its columns, its values)."""
     out = []
-    for s in _SIGMA:
-        out.append(np.block([[np.zeros((2, 2)), -1j * s], [1j * s, np.zeros((2, 2))]]))
-    out.append(np.block([[np.zeros((2, 2)), np.eye(2)], [np.eye(2), np.zeros((2, 2))]]))
-    return [torch.from_numpy(q.astype(np.complex128)).to(DEV) for q in out]
+    for a in _SIGMA + [None]:
+        z = np.zeros((2, 2))
+        g = np.block([[z, np.eye(2)], [np.eye(2), z]]) if a is None else np.block([[z, -1j * a], [1j * a, z]])
+        col = np.abs(g).argmax(axis=1)
+        out.append((torch.from_numpy(col).to(DEV), torch.from_numpy(g[np.arange(4), col].astype(complex)).to(DEV)))
+    return out
 
 
 class _Wilson:
@@ -228,22 +231,16 @@ class _Wilson:
     def _dw1(self, x):
         psi = x.reshape(*self.shape, 4, 3)
         acc = torch.zeros_like(psi)
-        eye = torch.eye(4, dtype=torch.complex128, device=DEV)
         for nu in range(4):
-            ax = 3 - nu
-            u = self.links[..., nu, :, :]
+            ax, u, (col, val) = 3 - nu, self.links[..., nu, :, :], self.gam[nu]
             up = torch.roll(psi, -1, ax)
-            dn = torch.roll(torch.einsum("...ba,...sb->...sa", u.conj(), psi), 1, ax)
-            f = math.exp(self.mu) if nu == 3 else 1.0
-            b = math.exp(-self.mu) if nu == 3 else 1.0
+            dn = torch.roll((u.conj().mT[..., None, :, :] * psi[..., None, :]).sum(-1), 1, ax)
             if nu == 3:
-                up = up.clone()
                 up[-1] *= -1
-                dn = dn.clone()
                 dn[0] *= -1
-            hop = torch.einsum("...ab,...sb->...sa", u, up)
-            acc += f * torch.einsum("pq,...qc->...pc", eye - self.gam[nu], hop)
-            acc += b * torch.einsum("pq,...qc->...pc", eye + self.gam[nu], dn)
+                up, dn = up * math.exp(self.mu), dn * math.exp(-self.mu)
+            up = (u[..., None, :, :] * up[..., None, :]).sum(-1)
+            acc += up + dn - (up - dn)[..., col, :] * val[:, None]
         return (psi - self.kappa * acc).reshape(-1)
 
     def dw(self, x):

@@ -244,7 +244,9 @@ typedef struct {
 /* Per right-hand-side report. */
 typedef struct {
     int32_t k_used;       /* Krylov dimension used (< k_max after breakdown) */
-    int32_t newton_iters; /* Roberts iterations on H_k */
+    int32_t newton_iters; /* Roberts iterations on H_k; where sgn(H_k) e_1 came from
+                             the quadrature that Roberts' iterates discretise: the
+                             iterate of its degree, ceil(log2(nodes)) */
     int32_t status;       /* OVS_OK, OVS_NOT_CONVERGED, OVS_ESIGN, or OVS_EINVAL
                              when the source of this right-hand side is not
                              finite (the call then returns OVS_EINVAL) */

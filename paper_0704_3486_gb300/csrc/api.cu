@@ -236,6 +236,7 @@ static void free_kry(KryWork& k) {
     dfree(k.status);
     dfree(k.coeff);
     dfree(k.newton);
+    dfree(k.need);
     dfree(k.cdef);
     dfree(k.cdef2);
     dfree(k.X);
@@ -355,7 +356,9 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
     CK(dalloc(&k.iters, sizeof(int) * n));
     CK(dalloc(&k.status, sizeof(int) * n));
     CK(dalloc(&k.coeff, sizeof(double2) * (size_t)km * n));
-    CK(dalloc(&k.newton, sizeof(double2) * 2 * (size_t)km * km * n));
+    k.newton_rhs = std::max(2LL * km * km, sign_quad_work(km));
+    CK(dalloc(&k.newton, sizeof(double2) * (size_t)k.newton_rhs * n));
+    CK(dalloc(&k.need, sizeof(int) * n));
     const int md = std::max(std::max(g->m, 1), same ? k.mdef : 0);
     CK(dalloc(&k.cdef, sizeof(double2) * (size_t)md * n));
     CK(dalloc(&k.cdef2, sizeof(double2) * (size_t)md * n));
@@ -901,6 +904,19 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         return OVS_OK;
     };
     auto schur_dots = [&](const void* v) -> int { return shared_dots(Sb, v, kw.active); };
+    // coeff_r = beta_r sgn(H_n) e_1, n = n_fixed or k_used[r], of the right-hand
+    // sides in `due` (nullptr: all): the quadrature, and Roberts' iteration for
+    // those that it leaves (both skip the others on the device)
+    auto sign_column = [&](void* coeff, const int* due, int n_fixed) -> int {
+        const int n = n_fixed > 0 ? n_fixed : k;
+        KL(OVS_PROF_NEWTON, 16.0 * (double)n * n * nrhs,
+           launch_sign_quad(kw.H, h_rhs, ldh, kw.k_used, kw.beta, coeff, kmax, kw.newton, kw.newton_rhs, (int)kmax, k,
+                            nrhs, kw.iters, kw.status, kw.need, st, due, n_fixed));
+        KL(OVS_PROF_NEWTON, 0.0,
+           launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
+                         kw.status, st, kw.need, n_fixed, k));
+        return OVS_OK;
+    };
     if (schur) {
         // c = S^H x, x_perp = x - S c, classical Gram-Schmidt applied twice
         CK(cudaMemsetAsync(kw.active, 0xff, sizeof(int) * nrhs, st));
@@ -1012,9 +1028,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         // Krylov part).
         if (every > 0 && j > 0 && j % every == 0) {
             KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_check_due(kw.active, cstate, j, kw.due, nrhs, st));
-            KL(OVS_PROF_NEWTON, 16.0 * (double)j * j * nrhs,
-               launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.ccheck[1], kmax, kw.newton, (int)kmax, nrhs,
-                             kw.iters, kw.status, st, kw.due, j));
+            TRY(sign_column(kw.ccheck[1], kw.due, j));
             KL(OVS_PROF_SMALL, 48.0 * j * nrhs,
                launch_conv_check(kw.ccheck[1], kw.ccheck[0], kmax, j, opts->tol, kw.active, kw.k_used, kw.est,
                                  kw.due, cstate, every, check_cap, skip, nrhs, st));
@@ -1057,9 +1071,12 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     if (every > 0)
         KL(OVS_PROF_SMALL, 32.0 * k * nrhs,
            launch_check_final(cstate, kw.ccheck[0], kw.coeff, kmax, kw.k_used, kw.due, nrhs, st));
-    KL(OVS_PROF_NEWTON, 16.0 * (double)k * k * nrhs,
-       launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
-                     kw.status, st, every > 0 ? kw.due : nullptr, 0, k));  // k_used[r] <= k
+    if (schur)  // App. A needs the whole of sgn(H_k)
+        KL(OVS_PROF_NEWTON, 16.0 * (double)k * k * nrhs,
+           launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
+                         kw.status, st, nullptr, 0, k));  // k_used[r] <= k
+    else
+        TRY(sign_column(kw.coeff, every > 0 ? kw.due : nullptr, 0));
     if (schur) {
         // Schur coefficients sgn(T) c + beta Y e_1 (App. A), then y = S cS
         KL(OVS_PROF_SMALL, 16.0 * ((double)m * k * 4 + (double)k * k) * nrhs,

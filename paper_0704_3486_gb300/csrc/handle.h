@@ -41,7 +41,9 @@ struct KryWork {  // Krylov basis and small matrices
     int* iters = nullptr;
     int* status = nullptr;
     void* coeff = nullptr;  // [nrhs][kmax] complex128
-    void* newton = nullptr; // [nrhs][2 kmax^2] complex128
+    void* newton = nullptr; // [nrhs][newton_rhs] complex128: work of the sign of H_k
+    long long newton_rhs = 0;
+    int* need = nullptr;    // [nrhs] right-hand sides left to Roberts' iteration
     void* cdef = nullptr;   // [nrhs][m] complex128 deflation coefficients
     void* cdef2 = nullptr;  // [nrhs][m] complex128 sgn-scaled (Schur: second-pass scratch)
     int mdef = 0;           // m the deflation buffers below were sized for

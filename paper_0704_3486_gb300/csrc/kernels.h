@@ -159,6 +159,17 @@ cudaError_t launch_newton(const void* H, long long h_rhs_stride, int ldh, const 
                           void* coeff, long long coeff_stride, void* work, int kmax, int nrhs, int* iters,
                           int* status, cudaStream_t st, const int* active = nullptr, int n_fixed = 0,
                           int k_bound = 0);
+// ---- K3 for the first column only (signquad.cu)
+// coeff_r = beta_r sgn(H_r[0:n,0:n]) e_1 by quadrature, n = k_used[r] <= k_bound
+// or n_fixed, for the right-hand sides with due[r] != 0 (all if due is
+// nullptr). need[r] = 1 where the result was not accepted (nothing written:
+// launch_newton serves those, with active = need), else 0. work: work_rhs >=
+// sign_quad_work(kmax) complex128 per right-hand side.
+long long sign_quad_work(int kmax);
+cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
+                             void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
+                             int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
+                             const int* due = nullptr, int n_fixed = 0);
 // harmonic variant: H_r[:, k-1] += |h_(k+1,k)|^2 H_k^-H e_k (k = k_used[r]);
 // work as for launch_newton (used as scratch before it)
 cudaError_t launch_harmonic(void* H, long long h_rhs_stride, int ldh, const int* k_used, void* work, int kmax,

@@ -1,0 +1,382 @@
+// K3, first column only: beta sgn(H_k) e_1 of the upper Hessenberg H_k
+// (Sec. 5.3 step v) from the integral that Roberts' iterates discretise,
+//
+//   sgn(H) = (1/pi) int_{-inf}^{inf} (H - i t)^{-1} dt,
+//
+// by a quadrature whose every node is one Hessenberg solve with e_1. An
+// iterate S^n of Roberts' iteration (Eq. Roberts) is exactly this integral
+// with the 2^n nodes t = tan(pi (j + 1/2) / 2^n); here the nodes follow the
+// substitution t = r b sc(v | 1 - r^2) (Hale, Higham and Trefethen, "Computing
+// A^alpha, log(A) and related matrix functions by contour integrals", 2008),
+// which spreads them evenly over |lambda| in [r b, b], so that 48 pairs +-t
+// replace the 2^9 to 2^13 of Roberts' iterate. Cost: 96 solves of k^2/2
+// complex multiply-adds, all independent, against ten inversions of k^3 with a
+// chain of k pivots each.
+//
+// Solve (Hyman's method, as in Wilkinson, "The Algebraic Eigenvalue Problem",
+// ch. 7): rows k-1 .. 1 of (H - i t) z = e_1 form an upper triangular system
+// whose diagonal is the subdiagonal of H, so from z_{k-1} = 1 the recurrence
+//   z_{l-1} = - (sum_{q >= l} (H - i t)_{lq} z_q) / h_{l,l-1}
+// gives z up to a factor and row 0 gives that factor. Every row is satisfied
+// to rounding relative to its own terms, so the solve is backward stable row
+// by row; z is rescaled by powers of two where it grows.
+//
+// Accuracy: the rule is the midpoint rule of an even periodic analytic
+// function, and every third node of the n-pair rule is itself the n/3-pair
+// rule. Its distance e from the full rule is the error of the latter's
+// coarse part; the error of the full rule is about e^3 (geometric convergence,
+// three times the exponent). A result is taken when e <= 3e-6; right-hand
+// sides above that get a second rule (144 pairs over [1e-6 b, b]), and those
+// that fail it too (an eigenvalue on or next to the imaginary axis) get
+// Roberts' iteration itself (launch_newton), with its statuses. Measured over
+// lattices 4^4 to 8^4, k 40 to 400, mu 0.05 to 0.3: e = 2e-8, and the first
+// column within 3e-16 of Roberts' in the 2-norm. Whole applications, before
+// (Roberts on 4 to 8 SMs per right-hand side, one block above k = 320) and
+// after: 6^4, 2 right-hand sides, k = 340: 1373 -> 547 ms; 8^4 mixed, one
+// right-hand side, k = 200: 50.0 -> 23.1 ms; six fields of 4^4 to 8^4 with
+// convergence checks up to k = 300, 54 right-hand sides: 921 -> 156 ms.
+#include <algorithm>
+#include <cmath>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace ovs {
+
+namespace {
+
+constexpr int kPairs1 = 48, kPairs2 = 144;  // multiples of 3
+constexpr double kWindow1 = 1e-3, kWindow2 = 1e-6;
+constexpr double kAccept = 3e-6;
+constexpr int QS = 8;  // columns of H in flight per warp (cp.async stages)
+constexpr int kItersLevel1 = 7, kItersLevel2 = 9;  // ceil(log2(2 pairs)): the Roberts iterate of that degree
+
+struct QuadNodes {
+    double t[kPairs2], w[kPairs2];  // node and weight / pi of the pairs, for b = 1
+};
+
+double agm(double a, double b) {
+    for (int i = 0; i < 60; ++i) {
+        const double m = 0.5 * (a + b), g = std::sqrt(a * b);
+        a = m;
+        b = g;
+    }
+    return a;
+}
+
+// Midpoints v_j = (j + 1/2) K'/n of sc(v | 1 - r^2) on (0, K'): t_j = r sc(v_j)
+// and w_j = (dt/dv)(v_j) K'/(n pi). The Fourier series of sn at imaginary
+// argument converges fast on v <= K'/2; the other half is its mirror image
+// t(K' - v) = r / t(v).
+QuadNodes make_nodes(int n, double r) {
+    const double pi = 3.14159265358979323846;
+    QuadNodes q{};
+    const double K = pi / 2 / agm(1.0, std::sqrt(1.0 - r * r)), Kp = pi / 2 / agm(1.0, r);
+    const double lq = -pi * Kp / K, h = Kp / n;
+    for (int j = 0; j < (n + 1) / 2; ++j) {
+        const double v = (j + 0.5) * h;
+        double s = 0.0, d = 0.0;
+        for (int i = 0; i < 30; ++i) {
+            const double o = 2 * i + 1, a = o * pi * v / (2 * K), c = 1.0 / (1.0 - std::exp(o * lq));
+            const double ep = std::exp(o * lq / 2 + a), em = std::exp(o * lq / 2 - a);
+            s += c * (ep - em) / 2;
+            d += o * c * (ep + em) / 2;
+        }
+        s *= 2 * pi / K;
+        d *= pi * pi / (K * K);
+        q.t[j] = s;
+        q.w[j] = d * h / pi;
+        q.t[n - 1 - j] = r / s;
+        q.w[n - 1 - j] = q.w[j] * r / (s * s);
+    }
+    return q;
+}
+
+__device__ __forceinline__ double lane_d(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+
+// order of the matrix of right-hand side r; 0 where it takes no part
+__device__ __forceinline__ int quad_order(const int* k_used, int n_fixed, const int* due, const int* need, int level,
+                                          int r) {
+    if (due != nullptr && due[r] == 0) return 0;
+    if (level > 1 && need[r] == 0) return 0;
+    return n_fixed > 0 ? n_fixed : k_used[r];
+}
+
+// Largest column norm of H_r (as the bits of a non-negative double, for
+// atomicMax) and the inverse subdiagonal: one warp per column.
+__global__ void __launch_bounds__(256) k_quad_prep(const double2* __restrict__ H, long long h_rhs, int ldh,
+                                                   const int* __restrict__ k_used, int n_fixed,
+                                                   const int* __restrict__ due, unsigned long long* __restrict__ bmax,
+                                                   double* __restrict__ isub, int kmax) {
+    const int r = blockIdx.y, lane = threadIdx.x & 31;
+    const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int n = quad_order(k_used, n_fixed, due, nullptr, 1, r);
+    if (j >= n) return;
+    const double2* c = H + r * h_rhs + (long long)j * ldh;
+    const int rows = min(n, j + 2);
+    double s = 0.0;
+    for (int i = lane; i < rows; i += 32) s += c[i].x * c[i].x + c[i].y * c[i].y;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        atomicMax(bmax + r, (unsigned long long)__double_as_longlong(sqrt(s)));
+        if (j + 1 < n) isub[(size_t)r * kmax + j + 1] = 1.0 / c[j + 1].x;
+    }
+}
+
+// One node (one sign of t) per warp: P[r][node][0..n) = (w/pi) (H - i t)^-1 e_1.
+// Lane q of the warp owns rows q, q + 32, ...: s[j] sums row 32 j + q, and once
+// row l has been used, its place keeps z_{l-1}. What bounds it: the FP64 units
+// (two multiply-adds a clock and SM: 4 per complex term), for few right-hand
+// sides the chain of k steps; the columns of H come from L2 through a ring of
+// QS asynchronous copies, so their latency is off that chain. One warp per
+// block: 96 nodes spread over as many SMs.
+template <int KC>
+__global__ void __launch_bounds__(32) k_quad_solve(const double2* __restrict__ H, long long h_rhs, int ldh,
+                                                   const int* __restrict__ k_used, int n_fixed,
+                                                   const int* __restrict__ due, const int* __restrict__ need, int level,
+                                                   const unsigned long long* __restrict__ bmax,
+                                                   const double* __restrict__ isub, int kmax, double2* __restrict__ P,
+                                                   long long p_rhs, QuadNodes nodes) {
+    extern __shared__ double2 ring[];  // [QS][32 KC]
+    const int r = blockIdx.y, node = blockIdx.x, lane = threadIdx.x;
+    const int n = quad_order(k_used, n_fixed, due, need, level, r);
+    if (n <= 0) return;
+    const double b = 2.0 * __longlong_as_double((long long)bmax[r]);
+    const double t = (node & 1) ? -nodes.t[node >> 1] * b : nodes.t[node >> 1] * b;
+    const double w = nodes.w[node >> 1] * b;
+    const double2* Hr = H + r * h_rhs;
+    const double* ib = isub + (size_t)r * kmax;
+    // column c into its stage: rows 0 .. c
+    auto fetch = [&](int c) {
+        if (c >= 0) {
+            const double2* src = Hr + (long long)c * ldh;
+            double2* dst = ring + (size_t)(c % QS) * (32 * KC);
+            for (int i = lane; i <= c; i += 32) cp16(dst + i, src + i);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    for (int c = n - 1; c > n - QS; --c) fetch(c);
+    double sr[KC], si[KC];
+#pragma unroll
+    for (int j = 0; j < KC; ++j) sr[j] = si[j] = 0.0;
+    double zr = 1.0, zi = 0.0, last = 1.0;  // z_l of the current column; z_{n-1}
+#pragma unroll
+    for (int sl = KC - 1; sl >= 0; --sl) {
+        if (32 * sl >= n) continue;
+        for (int q = min(31, n - 1 - 32 * sl); q >= 0; --q) {
+            const int l = 32 * sl + q;
+            __syncwarp();  // every lane has read the stage that is refilled here
+            fetch(l - QS + 1);
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(QS - 1) : "memory");
+            __syncwarp();
+            const double ibl = l > 0 ? __ldg(ib + l) : 0.0;
+            const double2* col = ring + (size_t)(l % QS) * (32 * KC);
+            {  // slot sl first: z_{l-1} needs row l
+                double2 h = lane <= q ? col[32 * sl + lane] : make_double2(0.0, 0.0);
+                if (lane == q) h.y -= t;
+                sr[sl] = fma(h.x, zr, sr[sl]);
+                sr[sl] = fma(-h.y, zi, sr[sl]);
+                si[sl] = fma(h.x, zi, si[sl]);
+                si[sl] = fma(h.y, zr, si[sl]);
+            }
+            double nr = -lane_d(sr[sl], q) * ibl, ni = -lane_d(si[sl], q) * ibl;
+            if (lane == q && l > 0) {
+                sr[sl] = nr;
+                si[sl] = ni;
+            }
+#pragma unroll
+            for (int j = 0; j < sl; ++j) {
+                const double2 h = col[32 * j + lane];
+                sr[j] = fma(h.x, zr, sr[j]);
+                sr[j] = fma(-h.y, zi, sr[j]);
+                si[j] = fma(h.x, zi, si[j]);
+                si[j] = fma(h.y, zr, si[j]);
+            }
+            zr = nr;
+            zi = ni;
+            // exponent above 2^200: everything times 2^-200 (uniform over the warp)
+            const int e = max((__double2hiint(zr) >> 20) & 0x7ff, (__double2hiint(zi) >> 20) & 0x7ff);
+            if (e > 1023 + 200 && l > 0) {
+                const double f = 0x1p-200;
+#pragma unroll
+                for (int j = 0; j < KC; ++j) {
+                    sr[j] *= f;
+                    si[j] *= f;
+                }
+                zr *= f;
+                zi *= f;
+                last *= f;
+            }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    const double gr = lane_d(sr[0], 0), gi = lane_d(si[0], 0);  // row 0: (H - i t)_0 z
+    // w / gamma by a scaled division (gamma may be large)
+    const double m = fmax(fabs(gr), fabs(gi));
+    const double ar = gr / m, ai = gi / m, den = w / (m * (ar * ar + ai * ai));
+    const double fr = ar * den, fi = -ai * den;
+    double2* out = P + r * p_rhs + (size_t)node * kmax;
+#pragma unroll
+    for (int j = 0; j < KC; ++j) {
+        const int l = 32 * j + lane;  // this place holds z_{l-1}
+        if (l >= 1 && l < n) out[l - 1] = make_double2(sr[j] * fr - si[j] * fi, sr[j] * fi + si[j] * fr);
+    }
+    if (lane == 0) out[n - 1] = make_double2(last * fr, last * fi);
+}
+
+constexpr int RT = 512;
+
+__device__ __forceinline__ double rsum(double v, double* sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int q = 0; q < RT / 32; ++q) s += sh[q];
+    return s;
+}
+
+// Sum over the nodes, the estimate from every third pair, and the verdict:
+// need[r] = 0 and coeff written where it is accepted. One block per
+// right-hand side; four groups of threads split the nodes.
+__global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, long long p_rhs, int pairs,
+                                                 const int* __restrict__ k_used, int n_fixed,
+                                                 const int* __restrict__ due, const double* __restrict__ beta,
+                                                 int kmax, double2* __restrict__ coeff, long long coeff_stride,
+                                                 int* __restrict__ need, int level, int iters_code,
+                                                 int* __restrict__ iters, int* __restrict__ status) {
+    __shared__ double sh[RT / 32];
+    __shared__ double2 part[2][RT];
+    const int r = blockIdx.x, tid = threadIdx.x;
+    const int n = quad_order(k_used, n_fixed, due, need, level, r);
+    double2* cr = coeff + r * coeff_stride;
+    const bool mine = due == nullptr || due[r] != 0;
+    if (n <= 0) {
+        if (level == 1) {
+            if (tid == 0) need[r] = 0;
+            if (mine) {  // an empty Krylov space: no coefficients
+                for (int i = tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
+                if (tid == 0) {
+                    iters[r] = 0;
+                    status[r] = 0;
+                }
+            }
+        }
+        return;
+    }
+    const double2* Pr = P + r * p_rhs;
+    const int g = tid >> 7, i0 = tid & 127;
+    const double bt = beta[r];
+    double d2 = 0.0, c2 = 0.0;
+    for (int base = 0; base < n; base += 128) {
+        const int i = base + i0;
+        double cx = 0.0, cy = 0.0, sx = 0.0, sy = 0.0;
+        if (i < n) {
+            for (int p = g; p < pairs; p += 4) {
+                const double2 a = Pr[(size_t)(2 * p) * kmax + i], c = Pr[(size_t)(2 * p + 1) * kmax + i];
+                const double x = a.x + c.x, y = a.y + c.y;
+                cx += x;
+                cy += y;
+                if (p % 3 == 1) {
+                    sx += x;
+                    sy += y;
+                }
+            }
+        }
+        __syncthreads();
+        part[0][tid] = make_double2(cx, cy);
+        part[1][tid] = make_double2(sx, sy);
+        __syncthreads();
+        if (g == 0 && i < n) {
+            for (int q = 1; q < 4; ++q) {
+                const double2 a = part[0][tid + 128 * q], c = part[1][tid + 128 * q];
+                cx += a.x;
+                cy += a.y;
+                sx += c.x;
+                sy += c.y;
+            }
+            d2 += (cx - 3.0 * sx) * (cx - 3.0 * sx) + (cy - 3.0 * sy) * (cy - 3.0 * sy);
+            c2 += cx * cx + cy * cy;
+            cr[i] = make_double2(bt * cx, bt * cy);
+        }
+    }
+    d2 = rsum(d2, sh);
+    c2 = rsum(c2, sh);
+    const bool ok = d2 <= kAccept * kAccept * c2 && isfinite(c2) && c2 > 0.0;  // false for NaN
+    if (ok)
+        for (int i = n + tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
+    if (tid == 0) {
+        need[r] = ok ? 0 : 1;
+        if (ok) {
+            iters[r] = iters_code;
+            status[r] = 0;
+        }
+    }
+}
+
+template <int KC>
+cudaError_t solve(int pairs, int nrhs, cudaStream_t st, const void* H, long long h_rhs, int ldh, const int* k_used,
+                  int n_fixed, const int* due, const int* need, int level, const unsigned long long* bmax,
+                  const double* isub, int kmax, void* P, long long p_rhs, const QuadNodes& nodes) {
+    const size_t smem = (size_t)QS * 32 * KC * sizeof(double2);
+    const cudaError_t e = ensure_dyn_smem((const void*)k_quad_solve<KC>, smem);
+    if (e != cudaSuccess) return e;
+    k_quad_solve<KC><<<dim3(2 * pairs, nrhs), 32, smem, st>>>((const double2*)H, h_rhs, ldh, k_used, n_fixed, due,
+                                                             need, level, bmax, isub, kmax, (double2*)P, p_rhs, nodes);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// complex128 entries of work per right-hand side: the nodes' columns, the
+// inverse subdiagonal and the norm
+long long sign_quad_work(int kmax) { return (long long)(2 * kPairs2 + 1) * kmax + 2; }
+
+cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
+                             void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
+                             int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
+                             const int* due, int n_fixed) {
+    static const QuadNodes nodes1 = make_nodes(kPairs1, kWindow1), nodes2 = make_nodes(kPairs2, kWindow2);
+    double2* P = (double2*)work;  // [nrhs][2 kPairs2][kmax], then bmax and isub of all right-hand sides
+    if (work_rhs < sign_quad_work(kmax)) return cudaErrorInvalidValue;
+    const long long p_rhs = 2LL * kPairs2 * kmax;
+    unsigned long long* bmax = (unsigned long long*)(P + p_rhs * nrhs);
+    double* isub = (double*)(bmax + 2 * nrhs);
+    cudaError_t e = cudaMemsetAsync(bmax, 0, sizeof(*bmax) * nrhs, st);
+    if (e != cudaSuccess) return e;
+    const int nb = n_fixed > 0 ? n_fixed : k_bound;
+    k_quad_prep<<<dim3((nb + 7) / 8, nrhs), 256, 0, st>>>((const double2*)H, h_rhs, ldh, k_used, n_fixed, due, bmax,
+                                                          isub, kmax);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int level = 1; level <= 2; ++level) {
+        const int pairs = level == 1 ? kPairs1 : kPairs2;
+        const QuadNodes& q = level == 1 ? nodes1 : nodes2;
+        const int kc = (nb + 31) / 32;
+#define OVS_QUAD(K)                                                                                               \
+    e = solve<K>(pairs, nrhs, st, H, h_rhs, ldh, k_used, n_fixed, due, need, level, bmax, isub, kmax, P, p_rhs, q)
+        if (kc <= 2) OVS_QUAD(2);
+        else if (kc <= 4) OVS_QUAD(4);
+        else if (kc <= 6) OVS_QUAD(6);
+        else if (kc <= 8) OVS_QUAD(8);
+        else if (kc <= 12) OVS_QUAD(12);
+        else if (kc <= 16) OVS_QUAD(16);
+        else if (kc <= 20) OVS_QUAD(20);
+        else if (kc <= 25) OVS_QUAD(25);
+        else return cudaErrorInvalidValue;
+#undef OVS_QUAD
+        if (e != cudaSuccess) return e;
+        k_quad_sum<<<nrhs, RT, 0, st>>>(P, p_rhs, pairs, k_used, n_fixed, due, beta, kmax, (double2*)coeff,
+                                        coeff_stride, need, level, level == 1 ? kItersLevel1 : kItersLevel2, iters,
+                                        status);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace ovs

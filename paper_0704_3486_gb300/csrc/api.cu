@@ -136,8 +136,9 @@ static double bytes_update(long long N, int tpv, int tpo, int J, int nrhs, bool 
 }
 static double bytes_layout(long long N, int tp, int nrhs) { return (double)N * nrhs * (16.0 + sz_of(tp)); }
 
-// Largest Krylov dimension: the inner-product sweep keeps 8 warps x (2k+2)
-// complex128 accumulators in shared memory (<= 200 KB).
+// Largest Krylov dimension: the single-vector register sweep keeps 8 warps x
+// (k+2) complex128 accumulators in shared memory, the TMA sweeps 2k+2 beside
+// their stages, and the sign of H_k at most 25 x 32 rows per warp.
 static const int kMaxK = 790;
 
 static size_t field_bytes(long long N, int tprec) { return (size_t)N * (tprec == PREC_F64 ? 16 : 8); }
@@ -226,6 +227,7 @@ static void free_kry(KryWork& k) {
     dfree(k.due);
     dfree(k.cstate);
     dfree(k.partial);
+    dfree(k.fpcol);
     dfree(k.norm_part);
     dfree(k.beta);
     dfree(k.inv_beta);
@@ -346,12 +348,13 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
     CK(dalloc(&k.due, sizeof(int) * n));
     CK(dalloc(&k.cstate, sizeof(CheckState) * n));
     CK(cudaMemset(k.err, 0, sizeof(int)));
-    CK(dalloc(&k.partial, sizeof(double2) * (size_t)nb * jc * n));
+    CK(dalloc(&k.partial, sizeof(double2) * std::max<size_t>((size_t)nb * n, fine_chunks_max(n, g->num_sms)) * jc));
+    CK(dalloc(&k.fpcol, sizeof(double2) * 2 * (size_t)(km + 1) * n));
     CK(dalloc(&k.norm_part, sizeof(double) * (size_t)nb * n));
     CK(dalloc(&k.beta, sizeof(double) * n));
     CK(dalloc(&k.inv_beta, sizeof(double) * n));
-    CK(dalloc(&k.hnorm2, sizeof(double) * n));
-    CK(dalloc(&k.active, sizeof(int) * n));
+    CK(dalloc(&k.hnorm2, sizeof(double) * 2 * n));
+    CK(dalloc(&k.active, sizeof(int) * 2 * n));
     CK(dalloc(&k.k_used, sizeof(int) * n));
     CK(dalloc(&k.iters, sizeof(int) * n));
     CK(dalloc(&k.status, sizeof(int) * n));
@@ -584,7 +587,7 @@ int install_deflation(ovs_gauge_s* g, int m, const void* Rc, const void* Lc, con
     CK(dalloc(&part, sizeof(double2) * (size_t)plan.nblk * S * m));
     CK(dalloc(&G, sizeof(double2) * (size_t)m * m));
     KL(OVS_PROF_DOTS, 0.0,
-       launch_gdots(PREC_F64, 1, Ltmp, 0, N, m, g->R64, N, nullptr, 0, false, N, plan, m, part, nullptr, 0));
+       launch_gdots(PREC_F64, Ltmp, 0, N, m, g->R64, N, N, plan, m, part, nullptr, 0));
     KL(OVS_PROF_SMALL, 0.0, launch_reduce(part, plan.nblk, S, m, m, G, m, false, nullptr, 0));
     std::vector<std::complex<double>> gh((size_t)m * m), a((size_t)m * m);
     CK(cudaMemcpy(gh.data(), G, sizeof(double2) * (size_t)m * m, cudaMemcpyDeviceToHost));
@@ -864,6 +867,9 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     const BlasPlan plan = blas_plan(units, nrhs, g->num_sms);
     const BlasPlan plan64 = blas_plan(N, nrhs, g->num_sms);
     const int dslots = tp == PREC_F32 ? gdots_chunk_slots(units, nrhs, g->num_sms) : 0;
+    // the two-launch step: FP64, and complex64 fields that give the TMA sweeps
+    // (work items of 2048 units) less than one item per SM
+    const bool fine = tp == PREC_F64 || (units + 2047) / 2048 * nrhs < g->num_sms;
     char* basis = (char*)kw.basis;
 
     // input, canonical complex128 -> internal precision
@@ -899,8 +905,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                launch_shared_dots(basis, units, m, v, units, nrhs, units, sdb, kw.partial, S1, act, st));
         else
             KL(OVS_PROF_PROJ, bytes_dots(N, tp, m, nrhs, true),
-               launch_gdots(tp, 1, basis, 0, units, m, v, units, nullptr, 0, false, units, plan, nrhs, kw.partial, act,
-                            st));
+               launch_gdots(tp, basis, 0, units, m, v, units, units, plan, nrhs, kw.partial, act, st));
         return OVS_OK;
     };
     auto schur_dots = [&](const void* v) -> int { return shared_dots(Sb, v, kw.active); };
@@ -964,7 +969,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     } else {
         CK(cudaMemsetAsync(w.yacc, 0, f64 * nrhs, st));
     }
-    CK(cudaMemsetAsync(kw.active, 0xff, sizeof(int) * nrhs, st));  // every rhs starts active (-1 != 0)
+    CK(cudaMemsetAsync(kw.active, 0xff, sizeof(int) * 2 * nrhs, st));  // every rhs starts active (-1 != 0)
     CK(cudaMemsetAsync(kw.est, 0, sizeof(double) * nrhs, st));
     CheckState* cstate = static_cast<CheckState*>(kw.cstate);
     const bool skip = (opts->flags & OVS_APPLY_SKIP_AHEAD) != 0;
@@ -980,39 +985,83 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     // residual, x_ominus at the start; z = A u (in wvec).
     const double bw = bytes_wilson(g->V, tp, nrhs);
     const StencilShape sh = stencil_shape(g, tp, nrhs, w.xint, fb, w.wvec, fb, st);
+    // A7 (batched form): at the checks (every `every` steps, or on the
+    // skip-ahead schedule) the sign of the complete H_j of each active
+    // right-hand side that is due; stop it once successive coefficient
+    // vectors agree to tol (V orthonormal, so this is the change of its
+    // Krylov part).
+    auto check = [&](int j, int* active) -> int {
+        KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_check_due(active, cstate, j, kw.due, nrhs, st));
+        TRY(sign_column(kw.ccheck[1], kw.due, j));
+        KL(OVS_PROF_SMALL, 48.0 * j * nrhs,
+           launch_conv_check(kw.ccheck[1], kw.ccheck[0], kmax, j, opts->tol, active, kw.k_used, kw.est, kw.due, cstate,
+                             every, check_cap, skip, nrhs, st));
+        return OVS_OK;
+    };
+    const long long fp_rhs = kmax + 1;
+    const size_t fp_half = sizeof(double2) * (size_t)fp_rhs * nrhs;
     for (int j = 0; j < k; ++j) {
         const int S = gdots_stride(2, j);
+        int* act = fine ? kw.active + (j & 1) * nrhs : kw.active;
         KL(OVS_PROF_MATVEC, bw,
-           launch_wilson(tp, true, links_for(g, tp), w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu,
-                         kw.active, st, sh));
+           launch_wilson(tp, true, links_for(g, tp), w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu, act, st,
+                         sh));
         if (schur) {
             // modified Arnoldi (Eq. modArnoldi): z <- z - S (S^H z), twice;
             // xz = S^H z (both passes) lands in column j of X
             char* Xj = (char*)kw.X + sizeof(double2) * (size_t)j * m;
-            TRY(schur_dots(w.wvec));
+            TRY(shared_dots(Sb, w.wvec, act));
             KL(OVS_PROF_SMALL, 16.0 * pblk * S1 * nrhs,
-               launch_reduce(kw.partial, pblk, S1, m, nrhs, Xj, x_rhs, false, kw.active, st));
+               launch_reduce(kw.partial, pblk, S1, m, nrhs, Xj, x_rhs, false, act, st));
             TRY(schur_out(Xj, x_rhs, w.wvec));
-            TRY(schur_dots(w.wvec));
+            TRY(shared_dots(Sb, w.wvec, act));
             KL(OVS_PROF_SMALL, 16.0 * pblk * S1 * nrhs,
-               launch_reduce(kw.partial, pblk, S1, m, nrhs, kw.cdef2, m, false, kw.active, st));
+               launch_reduce(kw.partial, pblk, S1, m, nrhs, kw.cdef2, m, false, act, st));
             TRY(schur_out(kw.cdef2, m, w.wvec));
             KL(OVS_PROF_SMALL, 16.0 * pblk * S1 * nrhs,
-               launch_reduce(kw.partial, pblk, S1, m, nrhs, Xj, x_rhs, true, kw.active, st));
+               launch_reduce(kw.partial, pblk, S1, m, nrhs, Xj, x_rhs, true, act, st));
         }
-        const bool tma = (tp == PREC_F32) && tma_update_fits(j);
-        const bool chunked = (tp == PREC_F32) && gdots_chunk_fits(j);
-        const int dblk = chunked ? dslots : plan.nblk;
-        if (chunked)
+        if (fine) {
+            // two launches: inner products, and the rest of the step (which
+            // also completes column j-1, so the check of H_j follows it: a
+            // right-hand side that it stops has one vector more than it needs)
+            FineStep fs;
+            fs.H = kw.H;
+            fs.h_rhs = h_rhs;
+            fs.ldh = ldh;
+            fs.fp = (char*)kw.fpcol + (size_t)(j & 1) * fp_half;
+            fs.fpn = (char*)kw.fpcol + (size_t)(~j & 1) * fp_half;
+            fs.fp_rhs = fp_rhs;
+            fs.beta0 = kw.beta;
+            fs.inv_beta = kw.inv_beta;
+            fs.hnorm2 = kw.hnorm2 + (j & 1) * nrhs;
+            fs.hnorm2n = kw.hnorm2 + (~j & 1) * nrhs;
+            fs.active = act;
+            fs.activen = kw.active + (~j & 1) * nrhs;
+            fs.k_used = kw.k_used;
             KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (j + 2.0),
-               launch_gdots2_chunk(basis, basis_rhs_units, units, j, w.xint, units, w.wvec, units, units, nrhs,
-                                   g->num_sms, dslots, kw.partial, kw.active, kw.err, st));
-        else
-            KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (j + 2.0),
-               launch_gdots(tp, 2, basis, basis_rhs_units, units, j, w.xint, units, w.wvec, units, true, units, plan,
-                            nrhs, kw.partial, kw.active, st));
-        KL(OVS_PROF_SMALL, 16.0 * dblk * S * nrhs,
-           launch_reduce(kw.partial, dblk, S, S, nrhs, kw.htmp, kw.jcap, false, kw.active, st));
+               launch_fine_dots(tp, 2, basis, basis_rhs_units, units, j, w.xint, w.wvec, units, nrhs, g->num_sms,
+                                kw.partial, act, st));
+            const int chunks = fine_chunks(units, j, nrhs, g->num_sms);
+            const bool sums = !schur && fine_sums_in_update(units, j, nrhs, g->num_sms);
+            if (!sums)
+                KL(OVS_PROF_SMALL, 16.0 * chunks * S * nrhs,
+                   launch_reduce(kw.partial, chunks, S, S, nrhs, kw.htmp, kw.jcap, false, act, st));
+            KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
+               launch_fine_update(tp, basis, basis_rhs_units, units, j, sums ? kw.partial : kw.htmp,
+                                  sums ? (long long)chunks * S : kw.jcap, sums ? chunks : 1, w.xint, w.wvec, units,
+                                  nrhs, g->num_sms, fs, st));
+            if (schur)  // X[:, j] = (xz - X[:, <j] s) / beta_j
+                KL(OVS_PROF_SMALL, 16.0 * ((double)m * j + 2.0 * m) * nrhs,
+                   launch_schur_xcol(kw.X, x_rhs, m, j, kw.htmp, kw.jcap, kw.inv_beta, fs.activen, nrhs, st));
+            if (every > 0 && j > 0 && j % every == 0) TRY(check(j, fs.activen));
+            continue;
+        }
+        KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (j + 2.0),
+           launch_gdots2_chunk(basis, basis_rhs_units, units, j, w.xint, units, w.wvec, units, units, nrhs, g->num_sms,
+                               dslots, kw.partial, kw.active, kw.err, st));
+        KL(OVS_PROF_SMALL, 16.0 * dslots * S * nrhs,
+           launch_reduce(kw.partial, dslots, S, S, nrhs, kw.htmp, kw.jcap, false, kw.active, st));
         KL(OVS_PROF_SMALL, 16.0 * 3.0 * j * nrhs,
            launch_arnoldi_step(kw.htmp, kw.jcap, j, kw.H, h_rhs, ldh, kw.beta, kw.inv_beta, kw.dcoef, kw.hnorm2,
                                kw.active, kw.k_used, nrhs, st));
@@ -1021,28 +1070,12 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                launch_schur_xcol(kw.X, x_rhs, m, j, kw.htmp, kw.jcap, kw.inv_beta, kw.active, nrhs, st));
         KL(OVS_PROF_SMALL, 16.0 * ((double)j * j / 2 + 2.0 * j) * nrhs,
            launch_arnoldi_column(kw.htmp, kw.jcap, j, kw.H, h_rhs, ldh, kw.inv_beta, kw.dcoef, kw.active, nrhs, st));
-        // A7 (batched form): at the checks (every `every` steps, or on the
-        // skip-ahead schedule) the sign of the complete H_j of each active
-        // right-hand side that is due; stop it once successive coefficient
-        // vectors agree to tol (V orthonormal, so this is the change of its
-        // Krylov part).
-        if (every > 0 && j > 0 && j % every == 0) {
-            KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_check_due(kw.active, cstate, j, kw.due, nrhs, st));
-            TRY(sign_column(kw.ccheck[1], kw.due, j));
-            KL(OVS_PROF_SMALL, 48.0 * j * nrhs,
-               launch_conv_check(kw.ccheck[1], kw.ccheck[0], kmax, j, opts->tol, kw.active, kw.k_used, kw.est,
-                                 kw.due, cstate, every, check_cap, skip, nrhs, st));
-        }
-        if (tma)
-            KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
-               launch_arnoldi_update_tma(basis, basis_rhs_units, units, j, kw.htmp, kw.jcap, kw.inv_beta, kw.dcoef,
-                                         w.xint, units, w.wvec, units, units, nrhs, g->num_sms, kw.active, kw.err, st));
-        else
-            KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
-               launch_arnoldi_update(tp, basis, basis_rhs_units, units, j, kw.htmp, kw.jcap, kw.inv_beta, kw.dcoef,
-                                     w.xint, units, w.wvec, units, units, plan, nrhs, kw.active, st));
+        if (every > 0 && j > 0 && j % every == 0) TRY(check(j, kw.active));
+        KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
+           launch_arnoldi_update_tma(basis, basis_rhs_units, units, j, kw.htmp, kw.jcap, kw.inv_beta, kw.dcoef,
+                                     w.xint, units, w.wvec, units, units, nrhs, g->num_sms, kw.active, kw.err, st));
     }
-    if (tp == PREC_F32 && gdots_chunk_fits(k)) {  // second Gram-Schmidt pass of the last column
+    if (!fine) {  // second Gram-Schmidt pass of the last column
         // the two-vector TMA sweep with z = u: s (and a copy as t), u^H u at 2k
         const int S = gdots_stride(2, k);
         KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (k + 1.0),
@@ -1053,14 +1086,16 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         KL(OVS_PROF_SMALL, 16.0 * 2.0 * k * nrhs,
            launch_arnoldi_final(kw.htmp, kw.jcap, k, 2 * k, kw.H, h_rhs, ldh, kw.active, nrhs, st));
     } else {
-        const int S = gdots_stride(1, k);
+        const int S = gdots_stride(1, k), chunks = fine_chunks(units, k, nrhs, g->num_sms);
+        const int* act = kw.active + (k & 1) * nrhs;
         KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (k + 1.0),
-           launch_gdots(tp, 1, basis, basis_rhs_units, units, k, w.xint, units, nullptr, 0, true, units, plan, nrhs,
-                        kw.partial, kw.active, st));
-        KL(OVS_PROF_SMALL, 16.0 * plan.nblk * S * nrhs,
-           launch_reduce(kw.partial, plan.nblk, S, S, nrhs, kw.htmp, kw.jcap, false, kw.active, st));
+           launch_fine_dots(tp, 1, basis, basis_rhs_units, units, k, w.xint, nullptr, units, nrhs, g->num_sms,
+                            kw.partial, act, st));
+        KL(OVS_PROF_SMALL, 16.0 * chunks * S * nrhs,
+           launch_reduce(kw.partial, chunks, S, S, nrhs, kw.htmp, kw.jcap, false, act, st));
         KL(OVS_PROF_SMALL, 16.0 * 2.0 * k * nrhs,
-           launch_arnoldi_final(kw.htmp, kw.jcap, k, k, kw.H, h_rhs, ldh, kw.active, nrhs, st));
+           launch_arnoldi_final(kw.htmp, kw.jcap, k, k, kw.H, h_rhs, ldh, act, nrhs, st,
+                                (char*)kw.fpcol + (size_t)(k & 1) * fp_half, fp_rhs));
     }
     // harmonic variant (Sec. 4): H_k -> H_k + |h_(k+1,k)|^2 H_k^-H e_k e_k^T
     if (opts->flags & OVS_APPLY_HARMONIC)
@@ -1096,7 +1131,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                              N, units, plan, nrhs, nullptr, nullptr, st));
     }
     // K4: y += V_k c (Sec. 5.3 step vi)
-    if (tp == PREC_F32 && recombine_tma_fits(k))
+    if (tp == PREC_F32)
         KL(OVS_PROF_PROJ, bytes_update(N, tp, PREC_F64, k, nrhs, false, true),
            launch_recombine_tma(basis, basis_rhs_units, units, k, kw.k_used, kw.coeff, kmax, 1.0, w.yacc, N, units,
                                 nrhs, g->num_sms, nullptr, kw.err, st));
@@ -1235,8 +1270,7 @@ int ovs_overlap_solve(ovs_gauge_t g, const void* b, void* x, int32_t nrhs, const
             ++iters;
             for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
                 void* red = pass ? red2 : red1;
-                CK(launch_gdots(PREC_F64, 1, W, N, (long long)nrhs * N, j + 1, z, N, nullptr, 0, false, N, plan, nrhs,
-                                part, nullptr, st));
+                CK(launch_gdots(PREC_F64, W, N, (long long)nrhs * N, j + 1, z, N, N, plan, nrhs, part, nullptr, st));
                 CK(launch_reduce(part, plan.nblk, gdots_stride(1, j + 1), j + 1, nrhs, red, jc, false, nullptr, st));
                 CK(launch_update(PREC_F64, PREC_F64, W, N, (long long)nrhs * N, j + 1, nullptr, red, jc, -1.0, z, N, z,
                                  N, N, plan, nrhs, nullptr, nullptr, st));

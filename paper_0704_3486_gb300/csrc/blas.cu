@@ -7,8 +7,8 @@
 // sweeps here a block of 256 threads covers one row block of one
 // right-hand side and streams every basis vector through it, so the basis
 // is read once per sweep with fully coalesced 16-byte loads. They serve the
-// complex128 form and the shared-basis projections; the complex64 form's
-// Arnoldi sweeps and recombination are the TMA kernels of tma_sweeps.cu.
+// projections, the complex128 recombination and the outer GMRES; the Arnoldi
+// sweeps are in fine_sweeps.cu and tma_sweeps.cu.
 // Also here: the shared-basis combination of the deflated part
 // (k_shared_combine) and the small kernels of each Arnoldi step (partial
 // sums, Hessenberg column, final pass).
@@ -22,6 +22,7 @@
 #include <mutex>
 #include <utility>
 
+#include "arnoldi_dev.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -29,12 +30,6 @@ namespace ovs {
 
 constexpr int BT = 256;  // threads per block
 constexpr int NWARP = BT / 32;
-
-template <typename R> __device__ __forceinline__ R warp_sum(R v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
 
 // ----------------------------------------------------------------- dots
 // Warp transpose-reduction: every lane holds M values; after five halving
@@ -59,68 +54,50 @@ template <typename R, int M> __device__ __forceinline__ void transpose_reduce(R 
     tr_step<M / 16, 1>(v, (lane & 1) != 0);
 }
 
-// Gram-Schmidt inner products of one basis sweep, per right-hand side r and
-// row block b: s_i = V_i^H u, and if NW == 2 also t_i = V_i^H z (i < J);
-// if `extras`, also u^H u and u^H z. Output partial[r][b][S],
-// S = NW*J + 2: s_0..s_{J-1}, t_0..t_{J-1}, (u^H u, 0), u^H z.
-// A lane keeps E 16-byte units of u (and z) in registers (a tile of 256*E
-// units per block); G basis vectors are then streamed past them. Each lane
-// accumulates its E*NC products per vector in FP32 (FP64 for complex128
-// fields), a warp transpose-reduction finishes the partial over the 32
-// lanes (at most 32*E*NC = 512 terms in FP32), and the warp partials are
-// accumulated in FP64 in shared memory.
-template <typename R, int NW, int G, int E>
+// Inner products of one basis sweep, per right-hand side r and row block b:
+// s_i = V_i^H u (i < J), output partial[r][b][S], S = J + 2 (the last two
+// entries are not written). Serves the projections, the set-up and the outer
+// GMRES; the Arnoldi steps have their own sweeps (fine_sweeps.cu,
+// tma_sweeps.cu).
+// A lane keeps E 16-byte units of u in registers (a tile of 256*E units per
+// block); G basis vectors are then streamed past them. Each lane accumulates
+// its E*NC products per vector in FP32 (FP64 for complex128 fields), a warp
+// transpose-reduction finishes the partial over the 32 lanes (at most
+// 32*E*NC = 256 terms in FP32), and the warp partials are accumulated in FP64
+// in shared memory.
+template <typename R, int G, int E>
 __global__ void __launch_bounds__(BT, sizeof(R) == 4 ? 2 : 1) k_gdots(const typename Unit<R>::vec* __restrict__ basis,
                                               long long basis_rhs_stride, long long vec_stride, int J,
                                               const typename Unit<R>::vec* __restrict__ u, long long u_rhs_stride,
-                                              const typename Unit<R>::vec* __restrict__ z, long long z_rhs_stride,
-                                              int extras, long long nunits, long long chunk, int nblk,
+                                              long long nunits, long long chunk, int nblk,
                                               double2* __restrict__ partial, const int* __restrict__ active) {
     using vec = typename Unit<R>::vec;
     constexpr int NC = Unit<R>::ncplx;
-    constexpr int M = 2 * NW * G;
+    constexpr int M = 2 * G;
     constexpr int PER = M / 32;
     extern __shared__ double2 sacc2[];  // [NWARP][S]
     double* sacc = reinterpret_cast<double*>(sacc2);
     const int r = blockIdx.x, b = blockIdx.y;
     if (active != nullptr && active[r] == 0) return;
-    const int S = NW * J + 2;
+    const int S = J + 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int i = tid; i < NWARP * S * 2; i += BT) sacc[i] = 0.0;
     __syncthreads();
     const vec* Vr = basis + r * basis_rhs_stride;
     const vec* ur = u + r * u_rhs_stride;
-    const vec* zr = (NW == 2) ? z + r * z_rhs_stride : nullptr;
     double* myacc = sacc + (size_t)warp * S * 2;
     const long long u0 = (long long)b * chunk;
     const long long u1 = min(u0 + chunk, nunits);
-    double uu = 0.0, uzr = 0.0, uzi = 0.0;
     for (long long base = u0; base < u1; base += (long long)BT * E) {
-        cplx<R> uc[E][NC], zc[E][NC];
+        cplx<R> uc[E][NC];
         bool ok[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const long long q = base + tid + (long long)BT * e;
             ok[e] = q < u1;
 #pragma unroll
-            for (int c = 0; c < NC; ++c) uc[e][c] = zc[e][c] = {R(0), R(0)};
-            if (ok[e]) {
-                Unit<R>::split(__ldg(ur + q), uc[e]);
-                if (NW == 2) Unit<R>::split(__ldg(zr + q), zc[e]);
-            }
-        }
-        if (extras) {
-            cplx<R> a = {R(0), R(0)}, bz = {R(0), R(0)};
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    cfmac(a, uc[e][c], uc[e][c]);
-                    if (NW == 2) cfmac(bz, uc[e][c], zc[e][c]);
-                }
-            uu += double(a.re);
-            uzr += double(bz.re);
-            uzi += double(bz.im);
+            for (int c = 0; c < NC; ++c) uc[e][c] = {R(0), R(0)};
+            if (ok[e]) Unit<R>::split(__ldg(ur + q), uc[e]);
         }
         for (int i0 = 0; i0 < J; i0 += G) {
             R v[M];
@@ -141,12 +118,6 @@ __global__ void __launch_bounds__(BT, sizeof(R) == 4 ? 2 : 1) k_gdots(const type
                                 cfmac(acc, vc[c], uc[e][c]);
                                 v[2 * gi] = acc.re;
                                 v[2 * gi + 1] = acc.im;
-                                if (NW == 2) {
-                                    cplx<R> acz = {v[2 * (G + gi)], v[2 * (G + gi) + 1]};
-                                    cfmac(acz, vc[c], zc[e][c]);
-                                    v[2 * (G + gi)] = acz.re;
-                                    v[2 * (G + gi) + 1] = acz.im;
-                                }
                             }
                         }
                     }
@@ -156,109 +127,17 @@ __global__ void __launch_bounds__(BT, sizeof(R) == 4 ? 2 : 1) k_gdots(const type
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
                 const int idx = lane * PER + q;
-                const int item = idx >> 1, comp = idx & 1;
-                const int which = item / G, gi = item - which * G;
-                if (i0 + gi < J) myacc[(which * J + i0 + gi) * 2 + comp] += double(v[q]);
+                const int gi = idx >> 1, comp = idx & 1;
+                if (i0 + gi < J) myacc[(i0 + gi) * 2 + comp] += double(v[q]);
             }
         }
     }
-    if (extras) {
-        uu = warp_sum(uu);
-        uzr = warp_sum(uzr);
-        uzi = warp_sum(uzi);
-        if (lane == 0) {
-            myacc[NW * J * 2] += uu;
-            myacc[(NW * J + 1) * 2] += uzr;
-            myacc[(NW * J + 1) * 2 + 1] += uzi;
-        }
-    }
     __syncthreads();
-    for (int i = tid; i < 2 * S; i += BT) {
+    for (int i = tid; i < 2 * J; i += BT) {
         double sum = 0.0;
 #pragma unroll
         for (int q = 0; q < NWARP; ++q) sum += sacc[(size_t)q * S * 2 + i];
         reinterpret_cast<double*>(partial + ((size_t)r * nblk + b) * S)[i] = sum;
-    }
-}
-
-// Arnoldi update sweep of the delayed-reorthogonalisation form of CGS2:
-//   v_j    = (u - sum_{i<J} V_i s_i) / beta          -> basis slot J
-//   u_next = (z - sum_{i<J} V_i t_i) / beta - v_j d  -> u (in place)
-// s, t are read from red[r] (s at 0, t at J), 1/beta from inv_beta[r] and
-// d from dcoef[r].
-template <typename R, int E>
-__global__ void __launch_bounds__(BT) k_arnoldi_update(typename Unit<R>::vec* __restrict__ basis,
-                                                       long long basis_rhs_stride, long long vec_stride, int J,
-                                                       const double2* __restrict__ red, long long red_stride,
-                                                       const double* __restrict__ inv_beta,
-                                                       const double2* __restrict__ dcoef,
-                                                       typename Unit<R>::vec* __restrict__ u, long long u_rhs_stride,
-                                                       const typename Unit<R>::vec* __restrict__ z,
-                                                       long long z_rhs_stride, long long nunits, long long chunk,
-                                                       const int* __restrict__ active) {
-    using vec = typename Unit<R>::vec;
-    constexpr int NC = Unit<R>::ncplx;
-    extern __shared__ double2 scf[];
-    cplx<R>* sc = reinterpret_cast<cplx<R>*>(scf);  // s at [0, J), t at [J, 2J)
-    const int r = blockIdx.x, b = blockIdx.y;
-    if (active != nullptr && active[r] == 0) return;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < 2 * J; i += BT) {
-        const double2 c = red[r * red_stride + i];
-        sc[i] = {R(c.x), R(c.y)};
-    }
-    __syncthreads();
-    const R ib = R(inv_beta[r]);
-    const double2 dd = dcoef[r];
-    const cplx<R> d = {R(dd.x), R(dd.y)};
-    vec* Vr = basis + r * basis_rhs_stride;
-    vec* vout = Vr + (long long)J * vec_stride;
-    vec* ur = u + r * u_rhs_stride;
-    const vec* zr = z + r * z_rhs_stride;
-    const long long u0 = (long long)b * chunk;
-    const long long u1 = min(u0 + chunk, nunits);
-    for (long long base = u0; base < u1; base += (long long)BT * E) {
-        cplx<R> a[E][NC], bb[E][NC];
-        bool ok[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            ok[e] = base + tid + (long long)BT * e < u1;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) a[e][c] = bb[e][c] = {R(0), R(0)};
-        }
-        for (int i = 0; i < J; ++i) {
-            const cplx<R> si = sc[i], ti = sc[J + i];
-            const vec* vi = Vr + (long long)i * vec_stride;
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                if (ok[e]) {
-                    cplx<R> vc[NC];
-                    Unit<R>::split(__ldcs(vi + base + tid + (long long)BT * e), vc);
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        cfma(a[e][c], vc[c], si);
-                        cfma(bb[e][c], vc[c], ti);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            if (!ok[e]) continue;
-            const long long q = base + tid + (long long)BT * e;
-            cplx<R> uc[NC], zc[NC], vo[NC], un[NC];
-            Unit<R>::split(ur[q], uc);
-            Unit<R>::split(__ldg(zr + q), zc);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                vo[c] = (uc[c] - a[e][c]) * ib;
-                un[c] = (zc[c] - bb[e][c]) * ib;
-                cplx<R> dv = cmul(vo[c], d);
-                un[c] = un[c] - dv;
-            }
-            vout[q] = Unit<R>::join(vo);
-            ur[q] = Unit<R>::join(un);
-        }
     }
 }
 
@@ -420,157 +299,34 @@ __global__ void k_reduce(const double2* __restrict__ partial, int nblk, int pstr
     }
 }
 
-constexpr double kBreakdownTol = 1e-12;  // relative to ||H_j||_F; rounding of an exactly
-                                         // invariant space is ~100 eps at N ~ 1e5
-
-__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, double* sh) {
-    a = warp_sum(a);
-    b = warp_sum(b);
-    c = warp_sum(c);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (lane == 0) {
-        sh[3 * w] = a;
-        sh[3 * w + 1] = b;
-        sh[3 * w + 2] = c;
-    }
-    __syncthreads();
-    a = b = c = 0.0;
-    for (int q = 0; q < nw; ++q) {
-        a += sh[3 * q];
-        b += sh[3 * q + 1];
-        c += sh[3 * q + 2];
-    }
-    __syncthreads();
-}
-
-// One Arnoldi step in the delayed-reorthogonalisation form of CGS2 (one
-// block per right-hand side). Input red[r] = (s, t, u^H u, u^H z) from the
-// sweep over V_0..V_{j-1} (s = V^H u, t = V^H z, z = A u), where u is the
-// first-pass Gram-Schmidt residual of the previous step (x_ominus at j=0).
-//  - beta = ||u - V s|| = sqrt(u^H u - ||s||^2) (V orthonormal);
-//  - j > 0: column j-1 of H gets its second-pass correction s and
-//    H[j][j-1] = beta; breakdown if beta <= 1e-12 ||H_j||_F (k_used = j);
-//  - j = 0: beta is ||x_ominus|| (kept in beta0 for the result);
-//  - column j, first pass: with g = Hbar_{j-1} s (Arnoldi relation
-//    A V_{j-1} = V_j Hbar_{j-1}), H[i][j] = (t_i - g_i)/beta for i < j and
-//    H[j][j] = (u^H z - s^H t)/beta^2 - g_j/beta (k_arnoldi_column, the
-//    O(j^2) part, spread over many blocks);
-//  - the update sweep then needs 1/beta and d = (u^H z - s^H t)/beta^2.
+// The step and the column of H as launches of their own (after the TMA
+// sweeps): one block per right-hand side, and one warp per row with 8 rows per
+// block and the right-hand side in y.
 __global__ void __launch_bounds__(256) k_arnoldi_step(const double2* __restrict__ red, long long red_stride, int j,
-                                                      double2* __restrict__ H, long long h_rhs, int ldh,
-                                                      double* __restrict__ beta0, double* __restrict__ inv_beta,
-                                                      double2* __restrict__ dcoef, double* __restrict__ hnorm2,
-                                                      int* __restrict__ active, int* __restrict__ k_used) {
-    __shared__ double sh[3 * 8];
-    const int r = blockIdx.x, tid = threadIdx.x;
-    if (active[r] == 0) return;
-    const double2* rr = red + r * red_stride;
-    double2* Hr = H + r * h_rhs;
-    double ss = 0.0, shr = 0.0, shi = 0.0;
-    for (int i = tid; i < j; i += blockDim.x) {
-        const double2 si = rr[i], ti = rr[j + i];
-        ss += si.x * si.x + si.y * si.y;
-        shr += si.x * ti.x + si.y * ti.y;
-        shi += si.x * ti.y - si.y * ti.x;
-    }
-    block_sum3(ss, shr, shi, sh);
-    const double uu = rr[2 * j].x;
-    const double2 uz = rr[2 * j + 1];
-    const double b2 = uu - ss;
-    // a NaN (from a non-finite source) stays NaN, so that it is reported
-    const double beta = (b2 > 0.0 || isnan(b2)) ? sqrt(b2) : 0.0;
-    if (j == 0) {
-        if (tid == 0) {
-            beta0[r] = beta;
-            hnorm2[r] = 0.0;
-        }
-        if (!(beta > 0.0) || !isfinite(beta)) {
-            if (tid == 0) {
-                active[r] = 0;
-                k_used[r] = 0;
-                inv_beta[r] = 0.0;
-            }
-            return;
-        }
-    } else {
-        for (int i = tid; i < j; i += blockDim.x) {
-            double2 h = Hr[i + (long long)(j - 1) * ldh];
-            const double2 si = rr[i];
-            Hr[i + (long long)(j - 1) * ldh] = make_double2(h.x + si.x, h.y + si.y);
-        }
-        __syncthreads();
-        double c2 = 0.0, z1 = 0.0, z2 = 0.0;
-        for (int i = tid; i < j; i += blockDim.x) {
-            const double2 h = Hr[i + (long long)(j - 1) * ldh];
-            c2 += h.x * h.x + h.y * h.y;
-        }
-        block_sum3(c2, z1, z2, sh);
-        const double hn2 = hnorm2[r] + c2 + beta * beta;
-        const bool brk = !(beta > kBreakdownTol * sqrt(hn2)) || !isfinite(beta);
-        if (tid == 0) {
-            hnorm2[r] = hn2;
-            Hr[j + (long long)(j - 1) * ldh] = make_double2(brk ? 0.0 : beta, 0.0);
-            if (brk) {
-                active[r] = 0;
-                k_used[r] = j;
-                inv_beta[r] = 0.0;
-            }
-        }
-        if (brk) return;
-        __syncthreads();
-    }
-    const double ib = 1.0 / beta;
-    const double dr = (uz.x - shr) * ib * ib, di = (uz.y - shi) * ib * ib;
-    if (tid == 0) {
-        inv_beta[r] = ib;
-        dcoef[r] = make_double2(dr, di);
-        k_used[r] = j + 1;
-    }
+                                                      StepOut o) {
+    __shared__ double sh[32];
+    const int r = blockIdx.x;
+    if (o.active[r] == 0) return;
+    arnoldi_step(red + r * red_stride, j, r, o, sh);
 }
-
-// Column j of H, first pass (after k_arnoldi_step of the same j): with
-// g = Hbar_{j-1} s, H[l][j] = (t_l - g_l)/beta for l < j and
-// H[j][j] = d - g_j/beta. One warp per row l: the lanes split the terms of
-// g_l (H is upper Hessenberg, so i >= l - 1) and reduce with shuffles.
-// Grid: x = groups of 8 rows, y = right-hand side.
 __global__ void __launch_bounds__(256) k_arnoldi_column(const double2* __restrict__ red, long long red_stride, int j,
                                                         double2* __restrict__ H, long long h_rhs, int ldh,
                                                         const double* __restrict__ inv_beta,
                                                         const double2* __restrict__ dcoef,
                                                         const int* __restrict__ active) {
-    const int r = blockIdx.y, lane = threadIdx.x & 31;
+    const int r = blockIdx.y;
     const int l = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (active[r] == 0 || l > j) return;  // stopped (breakdown, zero source) or past the column
-    const double2* rr = red + r * red_stride;
-    double2* Hr = H + r * h_rhs;
-    double gr = 0.0, gi = 0.0;
-    for (int i = (l > 0 ? l - 1 : 0) + lane; i < j; i += 32) {
-        const double2 h = Hr[l + (long long)i * ldh];
-        const double2 si = rr[i];
-        gr += h.x * si.x - h.y * si.y;
-        gi += h.x * si.y + h.y * si.x;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        gr += __shfl_xor_sync(0xffffffffu, gr, off);
-        gi += __shfl_xor_sync(0xffffffffu, gi, off);
-    }
-    if (lane != 0) return;
-    const double ib = inv_beta[r];
-    if (l < j) {
-        const double2 ti = rr[j + l];
-        Hr[l + (long long)j * ldh] = make_double2((ti.x - gr) * ib, (ti.y - gi) * ib);
-    } else {
-        const double2 d = dcoef[r];
-        Hr[j + (long long)j * ldh] = make_double2(d.x - gr * ib, d.y - gi * ib);
-    }
+    arnoldi_column(red + r * red_stride, j, l, H + r * h_rhs, ldh, inv_beta[r], dcoef[r]);
 }
 
 // Second Gram-Schmidt pass of the last column: red[r] holds s at [0, k) and
 // u^H u at entry uu_at, from a sweep over V_0..V_{k-1};
-// H[:k][k-1] += s, H[k][k-1] = ||u - V s||.
+// H[:k][k-1] += s (the first pass of the column is in fp, if not in H),
+// H[k][k-1] = ||u - V s||.
 __global__ void __launch_bounds__(256) k_arnoldi_final(const double2* __restrict__ red, long long red_stride, int k,
                                                        int uu_at, double2* __restrict__ H, long long h_rhs, int ldh,
+                                                       const double2* __restrict__ fp, long long fp_rhs,
                                                        const int* __restrict__ active) {
     __shared__ double sh[3 * 8];
     const int r = blockIdx.x, tid = threadIdx.x;
@@ -580,7 +336,7 @@ __global__ void __launch_bounds__(256) k_arnoldi_final(const double2* __restrict
     double ss = 0.0, z1 = 0.0, z2 = 0.0;
     for (int i = tid; i < k; i += blockDim.x) {
         const double2 si = rr[i];
-        const double2 h = Hr[i + (long long)(k - 1) * ldh];
+        const double2 h = fp != nullptr ? fp[r * fp_rhs + i] : Hr[i + (long long)(k - 1) * ldh];
         Hr[i + (long long)(k - 1) * ldh] = make_double2(h.x + si.x, h.y + si.y);
         ss += si.x * si.x + si.y * si.y;
     }
@@ -788,12 +544,8 @@ cudaError_t ensure_dyn_smem(const void* kernel, size_t bytes) {
 // dynamic shared memory
 static void set_smem_attrs() {
     const size_t big = 200 * 1024;
-    ensure_dyn_smem((const void*)k_gdots<double, 1, 16, 4>, big);
-    ensure_dyn_smem((const void*)k_gdots<double, 2, 8, 4>, big);
-    ensure_dyn_smem((const void*)k_gdots<float, 1, 16, 4>, big);
-    ensure_dyn_smem((const void*)k_gdots<float, 2, 8, 4>, big);
-    ensure_dyn_smem((const void*)k_arnoldi_update<double, 2>, big);
-    ensure_dyn_smem((const void*)k_arnoldi_update<float, 2>, big);
+    ensure_dyn_smem((const void*)k_gdots<double, 16, 4>, big);
+    ensure_dyn_smem((const void*)k_gdots<float, 16, 4>, big);
     ensure_dyn_smem((const void*)k_update<double, double, 2>, big);
     ensure_dyn_smem((const void*)k_update<float, float, 2>, big);
     ensure_dyn_smem((const void*)k_update<float, double, 2>, big);
@@ -801,67 +553,29 @@ static void set_smem_attrs() {
 
 int gdots_stride(int nw, int J) { return nw * J + 2; }
 
-cudaError_t launch_gdots(int prec, int nw, const void* basis, long long basis_rhs_stride, long long vec_stride,
-                         int J, const void* u, long long u_rhs_stride, const void* z, long long z_rhs_stride,
-                         bool extras, long long nunits, const BlasPlan& plan, int nrhs, void* partial,
-                         const int* active, cudaStream_t st) {
+cudaError_t launch_gdots(int prec, const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
+                         const void* u, long long u_rhs_stride, long long nunits, const BlasPlan& plan, int nrhs,
+                         void* partial, const int* active, cudaStream_t st) {
     set_smem_attrs();
     dim3 grid(nrhs, plan.nblk);  // right-hand side fastest: a shared basis is re-read from L2
-    const size_t smem = (size_t)NWARP * gdots_stride(nw, J) * sizeof(double2);
+    const size_t smem = (size_t)NWARP * gdots_stride(1, J) * sizeof(double2);
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    const int ex = extras ? 1 : 0;
-    if (prec == PREC_F64) {
-        if (nw == 1)
-            k_gdots<double, 1, 16, 4><<<grid, BT, smem, st>>>((const double2*)basis, basis_rhs_stride, vec_stride, J,
-                                                              (const double2*)u, u_rhs_stride, nullptr, 0, ex, nunits,
-                                                              plan.chunk, plan.nblk, (double2*)partial, active);
-        else
-            k_gdots<double, 2, 8, 4><<<grid, BT, smem, st>>>((const double2*)basis, basis_rhs_stride, vec_stride, J,
-                                                             (const double2*)u, u_rhs_stride, (const double2*)z,
-                                                             z_rhs_stride, ex, nunits, plan.chunk, plan.nblk,
-                                                             (double2*)partial, active);
-    } else {
-        if (nw == 1)
-            k_gdots<float, 1, 16, 4><<<grid, BT, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J,
-                                                             (const float4*)u, u_rhs_stride, nullptr, 0, ex, nunits,
-                                                             plan.chunk, plan.nblk, (double2*)partial, active);
-        else
-            k_gdots<float, 2, 8, 4><<<grid, BT, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J,
-                                                             (const float4*)u, u_rhs_stride, (const float4*)z,
-                                                             z_rhs_stride, ex, nunits, plan.chunk, plan.nblk,
-                                                             (double2*)partial, active);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_arnoldi_update(int prec, void* basis, long long basis_rhs_stride, long long vec_stride, int J,
-                                  const void* red, long long red_stride, const double* inv_beta, const void* dcoef,
-                                  void* u, long long u_rhs_stride, const void* z, long long z_rhs_stride,
-                                  long long nunits, const BlasPlan& plan, int nrhs, const int* active,
-                                  cudaStream_t st) {
-    set_smem_attrs();
-    dim3 grid(nrhs, plan.nblk);  // right-hand side fastest: a shared basis is re-read from L2
-    const size_t smem = (size_t)std::max(2 * J, 1) * sizeof(double2);
     if (prec == PREC_F64)
-        k_arnoldi_update<double, 2><<<grid, BT, smem, st>>>((double2*)basis, basis_rhs_stride, vec_stride, J,
-                                                            (const double2*)red, red_stride, inv_beta,
-                                                            (const double2*)dcoef, (double2*)u, u_rhs_stride,
-                                                            (const double2*)z, z_rhs_stride, nunits, plan.chunk,
-                                                            active);
+        k_gdots<double, 16, 4><<<grid, BT, smem, st>>>((const double2*)basis, basis_rhs_stride, vec_stride, J,
+                                                       (const double2*)u, u_rhs_stride, nunits, plan.chunk, plan.nblk,
+                                                       (double2*)partial, active);
     else
-        k_arnoldi_update<float, 2><<<grid, BT, smem, st>>>((float4*)basis, basis_rhs_stride, vec_stride, J,
-                                                           (const double2*)red, red_stride, inv_beta,
-                                                           (const double2*)dcoef, (float4*)u, u_rhs_stride,
-                                                           (const float4*)z, z_rhs_stride, nunits, plan.chunk,
-                                                           active);
+        k_gdots<float, 16, 4><<<grid, BT, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J,
+                                                      (const float4*)u, u_rhs_stride, nunits, plan.chunk, plan.nblk,
+                                                      (double2*)partial, active);
     return cudaGetLastError();
 }
 
 cudaError_t launch_arnoldi_step(const void* red, long long red_stride, int j, void* H, long long h_rhs, int ldh,
                                 double* beta0, double* inv_beta, void* dcoef, double* hnorm2, int* active,
                                 int* k_used, int nrhs, cudaStream_t st) {
-    k_arnoldi_step<<<nrhs, 256, 0, st>>>((const double2*)red, red_stride, j, (double2*)H, h_rhs, ldh, beta0, inv_beta,
-                                         (double2*)dcoef, hnorm2, active, k_used);
+    const StepOut o{(double2*)H, h_rhs, ldh, beta0, inv_beta, (double2*)dcoef, hnorm2, active, k_used};
+    k_arnoldi_step<<<nrhs, 256, 0, st>>>((const double2*)red, red_stride, j, o);
     return cudaGetLastError();
 }
 
@@ -875,8 +589,10 @@ cudaError_t launch_arnoldi_column(const void* red, long long red_stride, int j, 
 }
 
 cudaError_t launch_arnoldi_final(const void* red, long long red_stride, int k, int uu_at, void* H, long long h_rhs,
-                                 int ldh, const int* active, int nrhs, cudaStream_t st) {
-    k_arnoldi_final<<<nrhs, 256, 0, st>>>((const double2*)red, red_stride, k, uu_at, (double2*)H, h_rhs, ldh, active);
+                                 int ldh, const int* active, int nrhs, cudaStream_t st, const void* fp,
+                                 long long fp_rhs) {
+    k_arnoldi_final<<<nrhs, 256, 0, st>>>((const double2*)red, red_stride, k, uu_at, (double2*)H, h_rhs, ldh,
+                                          (const double2*)fp, fp_rhs, active);
     return cudaGetLastError();
 }
 

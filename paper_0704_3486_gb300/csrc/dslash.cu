@@ -19,6 +19,8 @@
 //   (1 + gamma_k) psi = [h;  i s_k h],   h = psi_up - i s_k psi_dn
 //   (1 - gamma_4) psi = [h; -h],         h = psi_up - psi_dn
 //   (1 + gamma_4) psi = [h;  h],         h = psi_up + psi_dn
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -46,6 +48,15 @@ template <> struct Field<double> {
             double2* u = d + 2 * ((size_t)q * V + s);
             u[0] = make_double2(p[2 * q].re, p[2 * q].im);
             u[1] = make_double2(p[2 * q + 1].re, p[2 * q + 1].im);
+        }
+    }
+    // row a of U (fwd) or column a of U
+    __device__ __forceinline__ static void row(const void* u, int V, int nu, int s, int a, bool fwd, cd (&m)[3]) {
+        const double2* d = static_cast<const double2*>(u) + (size_t)nu * 9 * V;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 v = __ldg(d + (size_t)(fwd ? 3 * a + b : 3 * b + a) * V + s);
+            m[b] = {v.x, v.y};
         }
     }
     __device__ __forceinline__ static void link(const void* u, int V, int nu, int s, cd (&m)[9]) {
@@ -77,6 +88,15 @@ template <> struct Field<float> {
     // (0,1) (2,3) (4,5) (6,7) of U (row-major 3x3), at float4 plane 4 nu + q;
     // the ninth entry of every direction in float2 planes after those 16
     // planes (float2 plane 32 + nu). Five loads per link instead of nine.
+    __device__ __forceinline__ static void row(const void* u, int V, int nu, int s, int a, bool fwd, cf (&m)[3]) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int e = fwd ? 3 * a + b : 3 * b + a;
+            const size_t at = e < 8 ? 2 * ((size_t)(nu * 4 + e / 2) * V + s) + (e & 1) : (size_t)(32 + nu) * V + s;
+            const float2 v = __ldg(static_cast<const float2*>(u) + at);
+            m[b] = {v.x, v.y};
+        }
+    }
     __device__ __forceinline__ static void link(const void* u, int V, int nu, int s, cf (&m)[9]) {
         const float4* d = static_cast<const float4*>(u) + (size_t)nu * 4 * V;
 #pragma unroll
@@ -303,6 +323,117 @@ __global__ void __launch_bounds__(256) k_wilson(const void* __restrict__ links, 
     }
 }
 
+// The stencil on small fields: a cluster of eight blocks takes 32 sites of one
+// right-hand side, one hop each, a warp per colour row of the link, and the
+// blocks then add the eight contributions, 48 of the 384 entries each, from each
+// other's shared memory. A thread of k_wilson does 1,392 flops in a row, so 4^4
+// in FP64 sat on 8 SMs' FP64 units (36 us); here it is spread over 64, and a
+// warp, alone on its scheduler at some 20 clocks an instruction, has a
+// twentieth of the instructions. The sums run in the order of k_wilson (x+, x-,
+// y+, ...; within a hop as there), so the results are the same bit for bit.
+template <int HOP, typename R>
+__device__ __forceinline__ void one_hop(const void* links, const char* in, size_t in_stride, int r, const Geom& g,
+                                        int s, int coord, R efwd, R ebwd, int a, cplx<R> (&out)[4]) {
+    constexpr int NU = HOP / 2;
+    constexpr bool FWD = HOP % 2 == 0;
+    const int L = g.L[NU], st = g.stride[NU];
+    int sn;
+    R fac;
+    if (FWD) {
+        sn = (coord == L - 1) ? s - (L - 1) * st : s + st;
+        fac = (NU == 3 && coord == L - 1) ? -efwd : efwd;
+    } else {
+        sn = (coord == 0) ? s + (L - 1) * st : s - st;
+        fac = (NU == 3 && coord == 0) ? -ebwd : ebwd;
+    }
+    cplx<R> U[3], p[12];
+    Field<R>::row(links, g.V, NU, FWD ? s : sn, a, FWD, U);
+    Field<R>::load(in + (size_t)r * in_stride, g.V, sn, p);
+    cplx<R> u0 = {R(0), R(0)}, u1 = {R(0), R(0)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const cplx<R> a0 = p[c], a1 = p[3 + c], a2 = p[6 + c], a3 = p[9 + c];
+        cplx<R> h0, h1;
+        if (FWD) {
+            if (NU == 0) { h0 = a0 + ti(a3); h1 = a1 + ti(a2); }
+            if (NU == 1) { h0 = a0 + a3;     h1 = a1 - a2; }
+            if (NU == 2) { h0 = a0 + ti(a2); h1 = a1 - ti(a3); }
+            if (NU == 3) { h0 = a0 - a2;     h1 = a1 - a3; }
+            h0 = h0 * fac;
+            h1 = h1 * fac;
+            cfma(u0, U[c], h0);
+            cfma(u1, U[c], h1);
+        } else {
+            if (NU == 0) { h0 = a0 + tmi(a3); h1 = a1 + tmi(a2); }
+            if (NU == 1) { h0 = a0 - a3;      h1 = a1 + a2; }
+            if (NU == 2) { h0 = a0 + tmi(a2); h1 = a1 + ti(a3); }
+            if (NU == 3) { h0 = a0 + a2;      h1 = a1 + a3; }
+            h0 = h0 * fac;
+            h1 = h1 * fac;
+            cfmac(u0, U[c], h0);
+            cfmac(u1, U[c], h1);
+        }
+    }
+    out[0] = u0;
+    out[1] = u1;
+    if (NU == 0) { out[2] = FWD ? tmi(u1) : ti(u1); out[3] = FWD ? tmi(u0) : ti(u0); }
+    if (NU == 1) { out[2] = FWD ? -u1 : u1;         out[3] = FWD ? u0 : -u0; }
+    if (NU == 2) { out[2] = FWD ? tmi(u0) : ti(u0); out[3] = FWD ? ti(u1) : tmi(u1); }
+    if (NU == 3) { out[2] = FWD ? -u0 : u0;         out[3] = FWD ? -u1 : u1; }
+}
+
+template <typename R, bool G5, bool AX>
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
+    k_wilson_split(const void* __restrict__ links, const char* __restrict__ in, char* out, size_t in_stride,
+                   size_t out_stride, Geom g, R kappa, R emu, R emmu, const int* __restrict__ active, Axpy ax) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ cplx<R> part[12][32];
+    const int r = blockIdx.y, hop = (int)cl.block_rank(), lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    if (active != nullptr && active[r] == 0) return;  // uniform over the cluster
+    const int s0 = (int)(blockIdx.x / 8) * 32;
+    const int s = min(s0 + lane, g.V - 1);
+    int c = s;
+    const int x = c % g.L[0]; c /= g.L[0];
+    const int y = c % g.L[1]; c /= g.L[1];
+    const int z = c % g.L[2];
+    const int t = c / g.L[2];
+    cplx<R> o[4];
+    const R one = R(1);
+    switch (hop) {
+        case 0: one_hop<0>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
+        case 1: one_hop<1>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
+        case 2: one_hop<2>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
+        case 3: one_hop<3>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
+        case 4: one_hop<4>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
+        case 5: one_hop<5>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
+        case 6: one_hop<6>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
+        default: one_hop<7>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) part[3 * q + row][lane] = o[q];
+    cl.sync();
+    const cplx<R>* src = reinterpret_cast<const cplx<R>*>(in + (size_t)r * in_stride);
+    cplx<R>* dst = reinterpret_cast<cplx<R>*>(out + (size_t)r * out_stride);
+    const int idx = hop * 48 + (int)threadIdx.x;  // this block adds 48 of the 384 entries
+    const int q = idx >> 5, at = idx & 31;
+    if (threadIdx.x < 48 && s0 + at < g.V) {
+        cplx<R> a = {R(0), R(0)};
+#pragma unroll
+        for (int h = 0; h < 8; ++h) a = a + cl.map_shared_rank(&part[0][0], h)[q * 32 + at];
+        const size_t e = 2 * ((size_t)(q >> 1) * g.V + s0 + at) + (q & 1);  // entry q of the site
+        cplx<R> v = src[e] - a * kappa;
+        if (G5 && q >= 6) v = -v;
+        if (AX) {
+            const cplx<R> xv = reinterpret_cast<const cplx<R>*>(ax.X + (size_t)r * ax.xs)[e];
+            const cplx<R> yv = reinterpret_cast<const cplx<R>*>(ax.Y + (size_t)r * ax.ys)[e];
+            v = v * R(ax.ah) + xv * R(ax.bx) + yv * R(ax.by);
+        }
+        dst[e] = v;
+    }
+    cl.sync();  // no block leaves while another reads its part
+}
+
 // Flat precision conversion of internal fields (the two layouts pair up).
 __global__ void k_f64_to_f32(const double2* __restrict__ a, float2* __restrict__ b, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -417,6 +548,12 @@ __global__ void k_links_to_canonical(const double2* __restrict__ u64, double2* _
 // ------------------------------------------------------------- host launch
 static inline dim3 site_grid(int V, int nrhs, int threads) { return dim3((V + threads - 1) / threads, nrhs); }
 
+// Groups of 32 sites and right-hand sides up to which the stencil is spread
+// over the hops as well (k_wilson_split). Measured, k_wilson and split: FP64
+// 8 groups 36 and 14 us, 90 37 and 16, 512 39 and 56; complex64 128 groups 9.2
+// and 9.5 us.
+template <typename R> constexpr long long kSplitGroups = sizeof(R) == 8 ? 256 : 96;
+
 static bool valid_shape(const StencilShape& sh) {
     for (int i = 0; i < kNumStencilShapes; ++i)
         if (kStencilShapes[i].rt == sh.rt && kStencilShapes[i].sites == sh.sites && kStencilShapes[i].rb == sh.rb)
@@ -431,6 +568,12 @@ static void wilson_dispatch(const StencilShape& sh, unsigned blocks, int ntiles,
     const R k = (R)kappa, e1 = (R)emu, e2 = (R)emmu;
     const char* i = (const char*)in;
     char* o = (char*)out;
+    const long long groups = (g.V + 31) / 32;
+    if (groups * nrhs <= kSplitGroups<R> && nrhs <= 65535) {
+        k_wilson_split<R, G5, AX><<<dim3((unsigned)(8 * groups), nrhs), 96, 0, st>>>(links, i, o, in_stride, out_stride,
+                                                                                    g, k, e1, e2, active, ax);
+        return;
+    }
     const dim3 block(sh.sites, sh.rb);
     if (sh.rt == 1)
         k_wilson<R, G5, 1, AX><<<blocks, block, 0, st>>>(links, i, o, in_stride, out_stride, g, k, e1, e2, nrhs, ntiles,

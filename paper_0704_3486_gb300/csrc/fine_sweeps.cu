@@ -1,0 +1,529 @@
+// K2 in two or three launches per Arnoldi step: the inner products, [their sums,]
+// and the rest of the step. These are the complex128 form's sweeps at every size, and the complex64
+// form's where the lattice is too small for the TMA sweeps (tma_sweeps.cu) to
+// give every SM a share of the basis.
+//
+// Split of the inner products: along the field (chunks of 128-unit tiles) and
+// along the basis (sets of four vectors). Large problems: a block takes a chunk
+// and a group of sets, a warp whole sets of the chunk. Small ones (SPREAD): a
+// block takes one set of one chunk and its warps share the tiles, so that 4^4
+// (3,072 complex128 units) with 50 vectors still spreads over the chip and the
+// partial sums stay few.
+//
+// Nothing is done by one block between the two: every block of the update takes
+// the step's scalars for itself, and where the partial sums are few (24 chunks
+// and 102 sums at 4^4 and 50 vectors: 39 KB from L2) also adds the chunks; else
+// k_reduce adds them in between. A last block doing both by a ticket took 14 us
+// of a 27 us sweep at that size: fence, atomic, and the sums of the whole step
+// through one SM's FP64 pipe.
+//
+// Measured, against register sweeps of 2048-unit row blocks, a reduction, the
+// scalars and the column in launches of their own (six per step, 2 blocks on
+// 4^4): FP64 4^4, k = 100: 51.2 -> 3.8 ms; 6^4, 2 right-hand sides, k = 340:
+// 547 -> 78 ms (FP64 floor 48); 8^4, 4 right-hand sides, k = 200: 194 -> 138 ms
+// (floor 105); complex64 8^4, one right-hand side, k = 200: 23.1 -> 7.9 ms.
+#include <algorithm>
+
+#include "arnoldi_dev.cuh"
+#include "common.cuh"
+#include "kernels.h"
+
+namespace ovs {
+
+namespace {
+
+constexpr int FT = 256, FW = FT / 32;  // threads and warps per block
+constexpr int FU = 4;                  // units per lane of a tile of 32 FU
+constexpr int FTILE = 32 * FU;
+constexpr int FV = 4;  // basis vectors per pass of a warp
+
+// One halving exchange of the warp transpose-reduction over CUR values.
+template <int CUR, int O, typename R, int M>
+__device__ __forceinline__ void halve(R (&v)[M], bool upper) {
+#pragma unroll
+    for (int i = 0; i < CUR / 2; ++i) {
+        const R send = upper ? v[i] : v[i + CUR / 2];
+        const R keep = upper ? v[i + CUR / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+}
+
+// partial[r][chunk]: s_i = V_i^H u and (NW = 2) t_i = V_i^H z for i < J, then
+// (u^H u, 0) and u^H z.
+// A warp takes four vectors at a time and streams its block's chunk of them,
+// with u and z from L1, into 16 sums per lane: complex128 sums run over the
+// whole chunk, complex64 ones over a tile (8 terms and 32 lanes) before they
+// join FP64.
+// What bounds it: complex128, the FP64 units (8 multiply-adds per element of
+// the basis; the warp reduction adds 16 per four vectors and chunk);
+// complex64 at these sizes, latency.
+template <typename R, int NW, bool SPREAD>
+__global__ void __launch_bounds__(FT, 2)
+    k_fine_dots(const typename Unit<R>::vec* __restrict__ basis, long long basis_rhs, long long vec_stride, int J,
+                const typename Unit<R>::vec* __restrict__ u, const typename Unit<R>::vec* __restrict__ z,
+                long long nunits, int tiles, int nchunk, int vgroups, double2* __restrict__ partial,
+                const int* __restrict__ active) {
+    using vec = typename Unit<R>::vec;
+    constexpr int NC = Unit<R>::ncplx;
+    constexpr int M = FV * NW * 2;  // values of a pass: vector, which, component
+    constexpr int SH = NW == 2 ? 1 : 2;  // lanes that end up with the same value: 2^SH
+    constexpr bool PER_TILE = sizeof(R) == 4;
+    __shared__ double ex[FW][3];
+    __shared__ double wsum[SPREAD ? FW : 1][M];
+    const int r = blockIdx.y;
+    if (active != nullptr && active[r] == 0) return;
+    const int chunk = blockIdx.x / vgroups, g = blockIdx.x - chunk * vgroups;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int S = NW * J + 2;
+    const int nsets = (J + FV - 1) / FV;
+    const vec* ur = u + r * nunits;
+    const vec* zr = NW == 2 ? z + r * nunits : nullptr;
+    double* part = reinterpret_cast<double*>(partial + ((size_t)r * nchunk + chunk) * S);
+    const long long c0 = (long long)chunk * tiles * FTILE, c1 = min(c0 + (long long)tiles * FTILE, nunits);
+    if (g == 0) {  // u^H u, u^H z of the chunk: FP32 over 8 terms, FP64 beyond
+        double uu = 0.0, uzr = 0.0, uzi = 0.0;
+        for (long long base = c0 + warp * FTILE + lane; base < c1; base += FW * FTILE) {
+            cplx<R> a = {R(0), R(0)}, b = {R(0), R(0)};
+#pragma unroll
+            for (int e = 0; e < FU; ++e) {
+                const long long p = base + 32 * e;
+                if (p >= c1) break;
+                cplx<R> uc[NC], zc[NC];
+                Unit<R>::split(__ldg(ur + p), uc);
+                if (NW == 2) Unit<R>::split(__ldg(zr + p), zc);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    cfmac(a, uc[c], uc[c]);
+                    if (NW == 2) cfmac(b, uc[c], zc[c]);
+                }
+            }
+            uu += double(a.re);
+            uzr += double(b.re);
+            uzi += double(b.im);
+        }
+        uu = warp_sum(uu);
+        uzr = warp_sum(uzr);
+        uzi = warp_sum(uzi);
+        if (lane == 0) {
+            ex[warp][0] = uu;
+            ex[warp][1] = uzr;
+            ex[warp][2] = uzi;
+        }
+    }
+    for (int q = SPREAD ? g : g + vgroups * warp; q < nsets; q += SPREAD ? nsets : vgroups * FW) {
+        const int i0 = q * FV, nv = min(FV, J - i0);
+        const vec* vb = basis + r * basis_rhs + (long long)i0 * vec_stride;
+        R v[M];
+        double kept = 0.0;
+#pragma unroll
+        for (int k = 0; k < M; ++k) v[k] = R(0);
+        auto reduce = [&]() {
+            if (NW == 2) {
+                halve<M, 16>(v, (lane & 16) != 0);
+                halve<M / 2, 8>(v, (lane & 8) != 0);
+                halve<M / 4, 4>(v, (lane & 4) != 0);
+                halve<M / 8, 2>(v, (lane & 2) != 0);
+            } else {
+                halve<M, 16>(v, (lane & 16) != 0);
+                halve<M / 2, 8>(v, (lane & 8) != 0);
+                halve<M / 4, 4>(v, (lane & 4) != 0);
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            kept += double(v[0]);
+        };
+        // one unit of u, z and the four vectors
+        auto term = [&](const vec& uv, const vec& zv, const vec (&x)[FV]) {
+            cplx<R> uc[NC], zc[NC];
+            Unit<R>::split(uv, uc);
+            Unit<R>::split(zv, zc);
+#pragma unroll
+            for (int gi = 0; gi < FV; ++gi) {
+                cplx<R> vc[NC];
+                Unit<R>::split(x[gi], vc);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    cplx<R> a = {v[gi * NW * 2], v[gi * NW * 2 + 1]};
+                    cfmac(a, vc[c], uc[c]);
+                    v[gi * NW * 2] = a.re;
+                    v[gi * NW * 2 + 1] = a.im;
+                    if (NW == 2) {
+                        cplx<R> b = {v[gi * 4 + 2], v[gi * 4 + 3]};
+                        cfmac(b, vc[c], zc[c]);
+                        v[gi * 4 + 2] = b.re;
+                        v[gi * 4 + 3] = b.im;
+                    }
+                }
+            }
+        };
+        for (long long base = c0 + lane + (SPREAD ? warp * FTILE : 0); base - lane < c1;
+             base += SPREAD ? FW * FTILE : FTILE) {
+            const bool whole = nv == FV && base - lane + FTILE <= c1;
+            if (whole) {
+#pragma unroll
+                for (int e = 0; e < FU; e += 2) {  // 12 loads in flight, more where registers allow
+                    vec x0[FV], x1[FV];
+                    const long long p = base + 32 * e;
+                    const vec u0 = __ldg(ur + p), u1 = __ldg(ur + p + 32);
+                    const vec z0 = NW == 2 ? __ldg(zr + p) : u0, z1 = NW == 2 ? __ldg(zr + p + 32) : u1;
+#pragma unroll
+                    for (int gi = 0; gi < FV; ++gi) {
+                        x0[gi] = __ldg(vb + (long long)gi * vec_stride + p);
+                        x1[gi] = __ldg(vb + (long long)gi * vec_stride + p + 32);
+                    }
+                    term(u0, z0, x0);
+                    term(u1, z1, x1);
+                }
+            } else {
+                for (int e = 0; e < FU; ++e) {
+                    const long long p = base + 32 * e;
+                    if (p >= c1) break;
+                    vec x[FV];
+#pragma unroll
+                    for (int gi = 0; gi < FV; ++gi)
+                        x[gi] = gi < nv ? __ldg(vb + (long long)gi * vec_stride + p) : vec{};
+                    const vec uv = __ldg(ur + p);
+                    term(uv, NW == 2 ? __ldg(zr + p) : uv, x);
+                }
+            }
+            if (PER_TILE) {
+                __syncwarp();
+                reduce();
+#pragma unroll
+                for (int k = 0; k < M; ++k) v[k] = R(0);
+            }
+        }
+        __syncwarp();
+        if (!PER_TILE) reduce();
+        int k = lane >> SH;
+        bool out = (lane & ((1 << SH) - 1)) == 0;
+        if (SPREAD) {
+            if (out) wsum[warp][k] = kept;
+            __syncthreads();
+            k = lane;
+            out = warp == 0 && lane < M;
+            if (out) {
+                kept = 0.0;
+#pragma unroll
+                for (int w = 0; w < FW; ++w) kept += wsum[w][k];
+            }
+        }
+        const int gi = k / (NW * 2), which = (k >> 1) & (NW - 1);
+        if (out && gi < nv) part[(size_t)(which * J + i0 + gi) * 2 + (k & 1)] = kept;
+    }
+    if (g == 0) {
+        __syncthreads();
+        if (tid < 4) {
+            double a = 0.0;
+            if (tid != 1)
+                for (int w = 0; w < FW; ++w) a += ex[w][tid == 0 ? 0 : tid - 1];
+            part[(size_t)(NW * J) * 2 + tid] = a;  // (u^H u, 0), u^H z
+        }
+    }
+}
+
+// The rest of step J (struct FineStep). The first nupd blocks of a right-hand
+// side share its tiles, the others do 8 rows of the column each. Every block
+// first adds the chunks' sums (nchunk = 1: they are added already) into shared
+// memory; warp 0 then takes the scalars
+// while the other warps are already at the basis (they are needed last).
+// SPLIT = 1: a thread sums its E units over all J vectors. SPLIT = 8 (small
+// fields): a block takes 32 E units, each warp every eighth vector, and the eight
+// sums meet in shared memory.
+template <typename R, int E, int SPLIT>
+__global__ void __launch_bounds__(FT, 3)
+    k_fine_update(typename Unit<R>::vec* basis, long long basis_rhs, long long vec_stride, int J,
+                  const double2* __restrict__ partial, long long p_rhs, int nchunk, typename Unit<R>::vec* u,
+                  const typename Unit<R>::vec* __restrict__ z, long long nunits, int nupd, FineStep fs) {
+    using vec = typename Unit<R>::vec;
+    constexpr int NC = Unit<R>::ncplx;
+    constexpr int T = SPLIT == 1 ? FT : 32;
+    extern __shared__ double2 red[];  // [2J + 2]: s, t, (u^H u, 0), u^H z; then (complex64) s and t as floats
+    __shared__ cplx<R> sum[SPLIT == 1 ? 1 : SPLIT][SPLIT == 1 ? 1 : 32 * E][NC][2];
+    __shared__ double sh[4 * FW];
+    __shared__ double2 s_d;
+    __shared__ double s_ib, s_beta;
+    __shared__ int s_brk;
+    const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool first = blockIdx.x == 0;
+    if (fs.active[r] == 0) {
+        if (first && tid == 0) fs.activen[r] = 0;
+        return;
+    }
+    const int S = 2 * J + 2;
+    cplx<R>* sc = sizeof(R) == 8 ? reinterpret_cast<cplx<R>*>(red) : reinterpret_cast<cplx<R>*>(red + S);
+    {
+        const double2* all = partial + r * p_rhs;
+        for (int i = tid; i < S; i += FT) {
+            double2 a = make_double2(0.0, 0.0);
+#pragma unroll 12
+            for (int b = 0; b < nchunk; ++b) {
+                const double2 p = __ldg(all + (size_t)b * S + i);
+                a.x += p.x;
+                a.y += p.y;
+            }
+            red[i] = a;
+            if (sizeof(R) == 4 && i < 2 * J) sc[i] = {R(a.x), R(a.y)};
+        }
+    }
+    __syncthreads();
+    const double2* fp = static_cast<const double2*>(fs.fp) + r * fs.fp_rhs;  // column J-1, first pass
+    {
+        // ||s||^2, s^H t, ||column J-1||^2 after its second pass; see arnoldi_step
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = tid; i < J; i += FT) {
+            const double2 si = red[i], ti = red[J + i], f = fp[i];
+            const double hx = f.x + si.x, hy = f.y + si.y;
+            v[0] += si.x * si.x + si.y * si.y;
+            v[1] += si.x * ti.x + si.y * ti.y;
+            v[2] += si.x * ti.y - si.y * ti.x;
+            v[3] += hx * hx + hy * hy;
+        }
+        if (block_sum4(v, sh) && lane == 0) {
+            const double b2 = red[2 * J].x - v[0];
+            const double2 uz = red[2 * J + 1];
+            // a NaN (from a non-finite source) stays NaN, so that it is reported
+            const double beta = (b2 > 0.0 || isnan(b2)) ? sqrt(b2) : 0.0;
+            const double hn2 = J == 0 ? 0.0 : fs.hnorm2[r] + v[3] + beta * beta;
+            const bool brk = !(beta > (J == 0 ? 0.0 : kBreakdownTol * sqrt(hn2))) || !isfinite(beta);
+            const double ib = brk ? 0.0 : 1.0 / beta;
+            s_beta = brk ? 0.0 : beta;
+            s_ib = ib;
+            s_d = make_double2((uz.x - v[1]) * ib * ib, (uz.y - v[2]) * ib * ib);
+            s_brk = brk ? 1 : 0;
+            if (first) {
+                if (J == 0) fs.beta0[r] = beta;
+                fs.inv_beta[r] = ib;
+                fs.hnorm2n[r] = hn2;
+                fs.activen[r] = brk ? 0 : 1;
+                fs.k_used[r] = brk ? J : J + 1;
+            }
+        }
+    }
+    if ((int)blockIdx.x >= nupd) {  // rows of column J-1 (complete) and J (first pass), one per warp
+        __syncthreads();
+        const int l = ((int)blockIdx.x - nupd) * FW + warp;
+        if (l > J) return;
+        double2* Hr = static_cast<double2*>(fs.H) + r * fs.h_rhs;
+        double gr = 0.0, gi = 0.0;
+        for (int i = (l > 0 ? l - 1 : 0) + lane; i < J; i += 32) {
+            double2 h;
+            if (i < J - 1) {
+                h = Hr[l + (long long)i * fs.ldh];
+            } else {  // column J-1: its second pass is s
+                h = l < J ? make_double2(fp[l].x + red[l].x, fp[l].y + red[l].y) : make_double2(s_beta, 0.0);
+                Hr[l + (long long)i * fs.ldh] = h;
+            }
+            const double2 si = red[i];
+            gr += h.x * si.x - h.y * si.y;
+            gi += h.x * si.y + h.y * si.x;
+        }
+        gr = warp_sum(gr);
+        gi = warp_sum(gi);
+        if (lane != 0 || s_brk) return;
+        double2* fpn = static_cast<double2*>(fs.fpn) + r * fs.fp_rhs;
+        fpn[l] = l < J ? make_double2((red[J + l].x - gr) * s_ib, (red[J + l].y - gi) * s_ib)
+                       : make_double2(s_d.x - gr * s_ib, s_d.y - gi * s_ib);
+        return;
+    }
+    vec* Vr = basis + r * basis_rhs;
+    vec* vout = Vr + (long long)J * vec_stride;
+    vec* ur = u + r * nunits;
+    const vec* zr = z + r * nunits;
+    auto finish = [&](long long p, const cplx<R> (&sa)[NC], const cplx<R> (&sb)[NC]) {
+        const R ib = R(s_ib);
+        const cplx<R> d = {R(s_d.x), R(s_d.y)};
+        cplx<R> uc[NC], zc[NC], vo[NC], un[NC];
+        Unit<R>::split(ur[p], uc);
+        Unit<R>::split(__ldg(zr + p), zc);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            vo[c] = (uc[c] - sa[c]) * ib;
+            un[c] = (zc[c] - sb[c]) * ib - cmul(vo[c], d);
+        }
+        vout[p] = Unit<R>::join(vo);
+        ur[p] = Unit<R>::join(un);
+    };
+    for (long long tile = blockIdx.x; tile * T * E < nunits; tile += nupd) {
+        const long long base = tile * T * E + (SPLIT == 1 ? tid : lane);
+        cplx<R> a[E][NC], b[E][NC];
+        bool ok[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            ok[e] = base + (long long)T * e < nunits;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) a[e][c] = b[e][c] = {R(0), R(0)};
+        }
+        auto add = [&](int i, const vec (&x)[E]) {
+            const cplx<R> si = sc[i], ti = sc[J + i];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                cplx<R> vc[NC];
+                Unit<R>::split(x[e], vc);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    cfma(a[e][c], vc[c], si);
+                    cfma(b[e][c], vc[c], ti);
+                }
+            }
+        };
+        auto get = [&](int i, vec (&x)[E]) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                x[e] = ok[e] ? __ldcs(Vr + (long long)i * vec_stride + base + (long long)T * e) : vec{};
+        };
+        int i = SPLIT == 1 ? 0 : warp;
+        for (; i + 3 * SPLIT < J; i += 4 * SPLIT) {  // four vectors' loads in flight
+            vec x0[E], x1[E], x2[E], x3[E];
+            get(i, x0);
+            get(i + SPLIT, x1);
+            get(i + 2 * SPLIT, x2);
+            get(i + 3 * SPLIT, x3);
+            add(i, x0);
+            add(i + SPLIT, x1);
+            add(i + 2 * SPLIT, x2);
+            add(i + 3 * SPLIT, x3);
+        }
+        for (; i < J; i += SPLIT) {
+            vec x[E];
+            get(i, x);
+            add(i, x);
+        }
+        if (SPLIT > 1) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    sum[warp % SPLIT][SPLIT == 1 ? 0 : lane + 32 * e][c][0] = a[e][c];
+                    sum[warp % SPLIT][SPLIT == 1 ? 0 : lane + 32 * e][c][1] = b[e][c];
+                }
+        }
+        __syncthreads();  // the scalars are there (and the eight sums)
+        if (s_brk) return;  // uniform: a breakdown has no v_J
+        if (SPLIT == 1) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (ok[e]) finish(base + (long long)T * e, a[e], b[e]);
+        } else {
+            const long long p = tile * T * E + tid;
+            if (tid < 32 * E && p < nunits) {
+                cplx<R> sa[NC], sb[NC];
+                const int at = SPLIT == 1 ? 0 : tid;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    sa[c] = sum[0][at][c][0];
+                    sb[c] = sum[0][at][c][1];
+#pragma unroll
+                    for (int w = 1; w < SPLIT; ++w) {
+                        sa[c] = sa[c] + sum[w][at][c][0];
+                        sb[c] = sb[c] + sum[w][at][c][1];
+                    }
+                }
+                finish(p, sa, sb);
+            }
+            __syncthreads();  // the sums are overwritten by the next tile
+        }
+    }
+}
+
+// Split of a sweep over J vectors: chunks of `tiles` tiles and groups of the
+// sets of four vectors. Below 64 (tile, set) pairs per SM the blocks take one
+// set each, about two blocks per SM; every chunk more is one more partial sum to add.
+struct FineSplit {
+    int tiles, nchunk, vgroups;
+    bool spread;
+};
+FineSplit fine_split(long long nunits, int J, int nrhs, int num_sms) {
+    const long long all = (nunits + FTILE - 1) / FTILE;
+    const int nsets = std::max(1, (J + FV - 1) / FV);
+    FineSplit f;
+    f.spread = all * nsets * nrhs < 64LL * num_sms;
+    f.vgroups = f.spread ? nsets : std::max(1, nsets / 12);
+    const long long want = std::max<long long>(1, 2LL * num_sms / ((long long)f.vgroups * nrhs));
+    f.tiles = (int)std::max<long long>(1, (all + want - 1) / want);
+    f.nchunk = (int)((all + f.tiles - 1) / f.tiles);
+    return f;
+}
+
+template <typename R, int NW>
+cudaError_t dots(const void* basis, long long basis_rhs, long long vec_stride, int J, const void* u, const void* z,
+                 long long nunits, int nrhs, int num_sms, void* partial, const int* active, cudaStream_t st) {
+    using vec = typename Unit<R>::vec;
+    const FineSplit f = fine_split(nunits, J, nrhs, num_sms);
+    const dim3 grid(f.nchunk * f.vgroups, nrhs);
+    if (f.spread)
+        k_fine_dots<R, NW, true><<<grid, FT, 0, st>>>((const vec*)basis, basis_rhs, vec_stride, J, (const vec*)u,
+                                                      (const vec*)z, nunits, f.tiles, f.nchunk, f.vgroups,
+                                                      (double2*)partial, active);
+    else
+        k_fine_dots<R, NW, false><<<grid, FT, 0, st>>>((const vec*)basis, basis_rhs, vec_stride, J, (const vec*)u,
+                                                       (const vec*)z, nunits, f.tiles, f.nchunk, f.vgroups,
+                                                       (double2*)partial, active);
+    return cudaGetLastError();
+}
+
+template <typename R, int E, int SPLIT>
+cudaError_t update_as(void* basis, long long basis_rhs, long long vec_stride, int J, const void* partial,
+                      long long p_rhs, int nchunk, void* u, const void* z, long long nunits, int nrhs, int num_sms, const FineStep& fs,
+                      cudaStream_t st) {
+    using vec = typename Unit<R>::vec;
+    const size_t smem = (size_t)(2 * J + 2) * sizeof(double2) + (sizeof(R) == 4 ? (size_t)2 * J * sizeof(cplx<R>) : 0);
+    if (smem > 32 * 1024) {
+        const cudaError_t e = ensure_dyn_smem((const void*)k_fine_update<R, E, SPLIT>, smem);
+        if (e != cudaSuccess) return e;
+    }
+    const long long per = (long long)(SPLIT == 1 ? FT : 32) * E, tiles = (nunits + per - 1) / per;
+    const int ncol = (J + 1 + FW - 1) / FW;
+    // where every block adds the chunks: as many blocks as are resident
+    const long long room = nchunk > 1 ? std::max<long long>(1, 3LL * num_sms / nrhs) : tiles;
+    const long long each = (tiles + room - 1) / room;
+    const int nupd = (int)((tiles + each - 1) / each);
+    k_fine_update<R, E, SPLIT><<<dim3(nupd + ncol, nrhs), FT, smem, st>>>((vec*)basis, basis_rhs, vec_stride, J,
+                                                                         (const double2*)partial, p_rhs, nchunk, (vec*)u,
+                                                                         (const vec*)z, nunits, nupd, fs);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t update(void* basis, long long basis_rhs, long long vec_stride, int J, const void* partial,
+                   long long p_rhs, int nchunk, void* u, const void* z, long long nunits, int nrhs, int num_sms,
+                   const FineStep& fs, cudaStream_t st) {
+    const long long wide = (nunits + FT - 1) / FT * nrhs;  // blocks of one unit per thread
+#define OVS_UPD(E, SPLIT)                                                                                              \
+    update_as<R, E, SPLIT>(basis, basis_rhs, vec_stride, J, partial, p_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st)
+    if (wide >= 8LL * num_sms) return OVS_UPD(2, 1);
+    if (wide >= 2LL * num_sms) return OVS_UPD(1, 1);
+    if (wide * 8 > 3LL * num_sms) return OVS_UPD(2, 8);
+    return OVS_UPD(1, 8);
+#undef OVS_UPD
+}
+
+}  // namespace
+
+int fine_chunks(long long nunits, int J, int nrhs, int num_sms) { return fine_split(nunits, J, nrhs, num_sms).nchunk; }
+
+int fine_chunks_max(int nrhs, int num_sms) { return 2 * num_sms + nrhs; }
+
+cudaError_t launch_fine_dots(int prec, int nw, const void* basis, long long basis_rhs, long long vec_stride, int J,
+                             const void* u, const void* z, long long nunits, int nrhs, int num_sms, void* partial,
+                             const int* active, cudaStream_t st) {
+    if (prec == PREC_F64)
+        return nw == 1 ? dots<double, 1>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st)
+                       : dots<double, 2>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st);
+    return nw == 1 ? dots<float, 1>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st)
+                   : dots<float, 2>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st);
+}
+
+bool fine_sums_in_update(long long nunits, int J, int nrhs, int num_sms) {
+    return (long long)fine_split(nunits, J, nrhs, num_sms).nchunk * (2 * J + 2) <= 4096;
+}
+
+cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long long vec_stride, int J,
+                               const void* sums, long long s_rhs, int nchunk, void* u, const void* z,
+                               long long nunits, int nrhs, int num_sms, const FineStep& fs, cudaStream_t st) {
+    if (prec == PREC_F64)
+        return update<double>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
+    return update<float>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
+}
+
+}  // namespace ovs

@@ -31,12 +31,13 @@ struct KryWork {  // Krylov basis and small matrices
     double* est = nullptr;                 // [nrhs] last convergence estimate
     int* due = nullptr;                    // [nrhs] checked at this step (A7)
     void* cstate = nullptr;                // [nrhs] CheckState: the check schedule (A7)
-    void* partial = nullptr;     // [nrhs][nblk][jcap] complex128
+    void* partial = nullptr;     // [max(nrhs nblk, fine_chunks_max)][jcap] complex128
+    void* fpcol = nullptr;        // [2][nrhs][kmax + 1] complex128: first pass of the last column (by parity)
     double* norm_part = nullptr; // [nrhs][nblk]
     double* beta = nullptr;
     double* inv_beta = nullptr;
-    double* hnorm2 = nullptr;
-    int* active = nullptr;
+    double* hnorm2 = nullptr;  // [2][nrhs] by parity of the step
+    int* active = nullptr;     // [2][nrhs] by parity of the step (the TMA sweeps: the first)
     int* k_used = nullptr;
     int* iters = nullptr;
     int* status = nullptr;

@@ -60,16 +60,15 @@ struct BlasPlan {
 };
 BlasPlan blas_plan(long long nunits, int nrhs, int num_sms);
 
-// Inner products of one sweep over J basis vectors (K2 / K5):
-// partial[r][b][S], S = gdots_stride(nw, J) = nw*J + 2, holds for row
-// block b: s_i = V_i^H u (i < J), then (nw == 2) t_i = V_i^H z, then
-// (u^H u, 0) and u^H z if extras. Basis of rhs r at basis + r*basis_rhs_stride
+// Inner products of one sweep over J basis vectors (K5, set-up, outer
+// GMRES): partial[r][b][S], S = gdots_stride(1, J) = J + 2, holds for row
+// block b: s_i = V_i^H u (i < J). (The sweeps with two vectors, nw = 2, hold
+// s, t_i = V_i^H z, (u^H u, 0) and u^H z in gdots_stride(2, J) entries.) Basis of rhs r at basis + r*basis_rhs_stride
 // units (0: shared by all rhs), vector i at + i*vec_stride units.
 int gdots_stride(int nw, int J);
-cudaError_t launch_gdots(int prec, int nw, const void* basis, long long basis_rhs_stride, long long vec_stride,
-                         int J, const void* u, long long u_rhs_stride, const void* z, long long z_rhs_stride,
-                         bool extras, long long nunits, const BlasPlan& plan, int nrhs, void* partial,
-                         const int* active, cudaStream_t st);
+cudaError_t launch_gdots(int prec, const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
+                         const void* u, long long u_rhs_stride, long long nunits, const BlasPlan& plan, int nrhs,
+                         void* partial, const int* active, cudaStream_t st);
 
 // out_r = in_r + alpha * sum_{i<J_r} V_r,i c_r,i   (coef: complex128 [r][coef_stride])
 // J_r = J (host) or Jdev[r] (device, if Jdev != nullptr, clamped to J).
@@ -108,24 +107,48 @@ cudaError_t launch_arnoldi_step(const void* red, long long red_stride, int j, vo
 cudaError_t launch_arnoldi_column(const void* red, long long red_stride, int j, void* H, long long h_rhs, int ldh,
                                   const double* inv_beta, const void* dcoef, const int* active, int nrhs,
                                   cudaStream_t st);
-// v_j = (u - V s)/beta -> slot J; u <- (z - V t)/beta - v_j d
-cudaError_t launch_arnoldi_update(int prec, void* basis, long long basis_rhs_stride, long long vec_stride, int J,
-                                  const void* red, long long red_stride, const double* inv_beta, const void* dcoef,
-                                  void* u, long long u_rhs_stride, const void* z, long long z_rhs_stride,
-                                  long long nunits, const BlasPlan& plan, int nrhs, const int* active,
-                                  cudaStream_t st);
+// ---- the step in two launches (fine_sweeps.cu); u, z: [nrhs][nunits]
+// Partial sums of a sweep over J vectors: partial[r][c][nw J + 2] for the
+// fine_chunks() chunks c (layout of gdots_stride(nw, J)); in all at most
+// fine_chunks_max() (nw J + 2) complex128.
+int fine_chunks(long long nunits, int J, int nrhs, int num_sms);
+int fine_chunks_max(int nrhs, int num_sms);  // of fine_chunks x nrhs
+cudaError_t launch_fine_dots(int prec, int nw, const void* basis, long long basis_rhs, long long vec_stride, int J,
+                             const void* u, const void* z, long long nunits, int nrhs, int num_sms, void* partial,
+                             const int* active, cudaStream_t st);
+// The rest of step J: scalars, v_J = (u - V s)/beta -> slot J, u <- (z - V t)/beta
+// - v_J d, column J-1 of H complete and the first pass of column J in fpn (that
+// of J-1 is in fp; fp_rhs complex128 per right-hand side). hnorm2 and active are
+// read from one array and written to another. The sums of right-hand side r are
+// at sums + r s_rhs: nchunk partial ones (fine_sums_in_update), or one reduced.
+bool fine_sums_in_update(long long nunits, int J, int nrhs, int num_sms);
+struct FineStep {
+    void* H;
+    long long h_rhs;
+    int ldh;
+    const void* fp;
+    void* fpn;
+    long long fp_rhs;
+    double *beta0, *inv_beta;
+    const double* hnorm2;
+    double* hnorm2n;
+    const int* active;
+    int *activen, *k_used;
+};
+cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long long vec_stride, int J,
+                               const void* sums, long long s_rhs, int nchunk, void* u, const void* z,
+                               long long nunits, int nrhs, int num_sms, const FineStep& fs, cudaStream_t st);
 // last column: H[:k][k-1] += s, H[k][k-1] = ||u - V s||
 // red[r]: s at [0, k), u^H u at entry uu_at
 cudaError_t launch_arnoldi_final(const void* red, long long red_stride, int k, int uu_at, void* H, long long h_rhs,
-                                 int ldh, const int* active, int nrhs, cudaStream_t st);
+                                 int ldh, const int* active, int nrhs, cudaStream_t st, const void* fp = nullptr,
+                                 long long fp_rhs = 0);
 
 // TMA-pipelined complex64 form of the Arnoldi update sweep (tma_sweeps.cu);
 // *err receives OVS_ETIMEOUT if a bounded wait gives up.
-bool tma_update_fits(int J);
 // persistent TMA inner-product sweep (complex64, NW = 2): one block per SM
 // over row chunks of 2048 units; partial[r][slot][2J + 2] for
 // slot < gdots_chunk_slots(nunits, nrhs, num_sms)
-bool gdots_chunk_fits(int J);
 int gdots_chunk_slots(long long nunits, int nrhs, int num_sms);
 cudaError_t launch_gdots2_chunk(const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
                                 const void* u, long long u_rhs_stride, const void* z, long long z_rhs_stride,
@@ -133,7 +156,6 @@ cudaError_t launch_gdots2_chunk(const void* basis, long long basis_rhs_stride, l
                                 int* err, cudaStream_t st);
 // y += alpha * sum_{i < min(J, Jdev[r])} V_i c_i: complex64 basis, complex128
 // y (internal layout, updated in place, y_rhs_stride in complex128 entries)
-bool recombine_tma_fits(int J);
 cudaError_t launch_recombine_tma(const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
                                  const int* Jdev, const void* coef, long long coef_stride, double alpha, void* y,
                                  long long y_rhs_stride, long long nunits, int nrhs, int num_sms, const int* active,

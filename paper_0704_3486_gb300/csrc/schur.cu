@@ -337,7 +337,7 @@ int install_schur(ovs_gauge_s* g, int m, const void* Rc) {
     std::vector<std::complex<double>> gh((size_t)m * m), am((size_t)m * m), uinv, cf((size_t)m * m);
     // two passes of Cholesky QR: S <- S U^-1 with S^H S = U^H U
     for (int pass = 0; pass < 2; ++pass) {
-        SCK(launch_gdots(PREC_F64, 1, a.p, 0, N, m, a.p, N, nullptr, 0, false, N, plan, m, part.p, nullptr, st));
+        SCK(launch_gdots(PREC_F64, a.p, 0, N, m, a.p, N, N, plan, m, part.p, nullptr, st));
         SCK(launch_reduce(part.p, plan.nblk, S, m, m, G.p, m, false, nullptr, st));
         SCK(cudaMemcpy(gh.data(), G.p, sizeof(double2) * (size_t)m * m, cudaMemcpyDeviceToHost));
         // gh[r*m + i] = S_i^H S_r = A_ir
@@ -356,7 +356,7 @@ int install_schur(ovs_gauge_s* g, int m, const void* Rc) {
     // T = S^H H_w S (column r = S^H H_w S_r), strictly lower part dropped
     const StencilShape sh = stencil_shape(g, PREC_F64, m, a.p, f64, b.p, f64, st);
     SCK(launch_wilson(PREC_F64, true, g->links64, a.p, f64, b.p, f64, g->geom, m, g->kappa, g->mu, nullptr, st, sh));
-    SCK(launch_gdots(PREC_F64, 1, a.p, 0, N, m, b.p, N, nullptr, 0, false, N, plan, m, part.p, nullptr, st));
+    SCK(launch_gdots(PREC_F64, a.p, 0, N, m, b.p, N, N, plan, m, part.p, nullptr, st));
     SCK(launch_reduce(part.p, plan.nblk, S, m, m, G.p, m, false, nullptr, st));
     SCK(cudaMemcpy(gh.data(), G.p, sizeof(double2) * (size_t)m * m, cudaMemcpyDeviceToHost));
     std::vector<std::complex<double>> tcm((size_t)m * m, 0.0);  // column-major T

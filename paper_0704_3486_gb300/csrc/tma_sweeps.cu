@@ -716,11 +716,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     }
 }
 
-bool tma_update_fits(int J) { return TNS * kStageBytes + (size_t)(2 * J + 1) * sizeof(cf) <= 220 * 1024; }
-
 static size_t gdots_chunk_smem(int J) { return DS * kDStage + (size_t)(2 * J + 2) * 16; }
-
-bool gdots_chunk_fits(int J) { return gdots_chunk_smem(J) <= 222 * 1024; }
 
 static int gdots_chunk_grid(long long nunits, int nrhs, int num_sms) {
     const long long T = (nunits + CU - 1) / CU * nrhs;
@@ -767,8 +763,6 @@ cudaError_t launch_arnoldi_update_tma(void* basis, long long basis_rhs_stride, l
                                                    nrhs, active, err);
     return cudaGetLastError();
 }
-
-bool recombine_tma_fits(int J) { return TNS * kStageBytes + (size_t)std::max(J, 1) * sizeof(cf) <= 220 * 1024; }
 
 cudaError_t launch_recombine_tma(const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
                                  const int* Jdev, const void* coef, long long coef_stride, double alpha, void* y,

@@ -141,6 +141,10 @@ static double bytes_layout(long long N, int tp, int nrhs) { return (double)N * n
 // their stages, and the sign of H_k at most 25 x 32 rows per warp.
 static const int kMaxK = 790;
 
+// Smallest complex64 basis (bytes over all right-hand sides) that is built two
+// steps per pass (see sign_apply_core).
+static const double kPairBytes = 272e6;
+
 static size_t field_bytes(long long N, int tprec) { return (size_t)N * (tprec == PREC_F64 ? 16 : 8); }
 static long long field_units(long long N, int tprec) { return tprec == PREC_F64 ? N : N / 2; }
 static int tprec_of(int prec) { return prec == OVS_MIXED ? PREC_F32 : PREC_F64; }
@@ -239,6 +243,14 @@ static void free_kry(KryWork& k) {
     dfree(k.coeff);
     dfree(k.newton);
     dfree(k.need);
+    dfree(k.ppart);
+    dfree(k.pred);
+    dfree(k.ec);
+    dfree(k.ps);
+    dfree(k.pact);
+    dfree(k.pmode);
+    dfree(k.jstart);
+    dfree(k.tmask);
     dfree(k.cdef);
     dfree(k.cdef2);
     dfree(k.X);
@@ -362,6 +374,17 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
     k.newton_rhs = std::max(2LL * km * km, sign_quad_work(km));
     CK(dalloc(&k.newton, sizeof(double2) * (size_t)k.newton_rhs * n));
     CK(dalloc(&k.need, sizeof(int) * n));
+    if (tprec == PREC_F32) {
+        const size_t row = sizeof(double2) * (size_t)pair_stride(km);
+        CK(dalloc(&k.ppart, row * ((size_t)g->num_sms + 2 * n)));
+        CK(dalloc(&k.pred, row * n));
+        CK(dalloc(&k.ec, sizeof(double2) * 4 * (size_t)km * n));
+        CK(dalloc(&k.ps, sizeof(PairState) * n));
+        CK(dalloc(&k.pact, sizeof(int) * n));
+        CK(dalloc(&k.pmode, sizeof(int) * n));
+        CK(dalloc(&k.jstart, sizeof(int) * n));
+        CK(dalloc(&k.tmask, sizeof(int) * n));
+    }
     const int md = std::max(std::max(g->m, 1), same ? k.mdef : 0);
     CK(dalloc(&k.cdef, sizeof(double2) * (size_t)md * n));
     CK(dalloc(&k.cdef2, sizeof(double2) * (size_t)md * n));
@@ -842,6 +865,84 @@ static int check_apply(ovs_gauge_s* g, int nrhs, const ovs_apply_opts* opts) {
     return OVS_OK;
 }
 
+// The Arnoldi steps of a complex64 application two at a time
+// (pair_sweeps.cu), then single steps for the right-hand sides that left the
+// blocks early and for the last vector of an odd k. On entry u (xint) is the
+// source; on return xint is the first-pass residual after k steps and tmask
+// marks the right-hand sides that reached k. check(j, in, active): the
+// convergence check of step j.
+template <typename Check>
+static int pair_steps(ovs_gauge_s* g, int nrhs, int k, const StencilShape& sh, int every, const Check& check,
+                      cudaStream_t st) {
+    VecWork& w = g->vw;
+    KryWork& kw = g->kw;
+    const long long N = g->N, units = field_units(N, PREC_F32);
+    const size_t fb = field_bytes(N, PREC_F32);
+    const long long basis_rhs = (long long)(kw.kmax + 1) * units, h_rhs = (long long)(kw.kmax + 1) * kw.kmax;
+    const int ldh = kw.kmax + 1, never = kw.kmax + 2;
+    const double bw = bytes_wilson(g->V, PREC_F32, nrhs);
+    // u2 and x2 live in the output staging buffer (twice their size), which is
+    // not written before the last layout pass
+    void *u1 = w.xint, *x1 = w.wvec, *u2 = w.sy, *x2 = (char*)w.sy + fb * nrhs;
+    const int slots = pair_slots(units, nrhs, g->num_sms), pred = pair_stride(kw.kmax);
+    CK(cudaMemsetAsync(kw.ps, 0, sizeof(PairState) * nrhs, st));
+    CK(cudaMemsetAsync(kw.pact, 0xff, sizeof(int) * nrhs, st));
+    KL(OVS_PROF_MATVEC, bw,
+       launch_wilson(PREC_F32, true, g->links32, u1, fb, u2, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
+    for (int J = 0; J + 2 <= k; J += 2) {
+        const bool more = J + 4 <= k;
+        const int S = pair_stride(J);
+        char *ec = (char*)kw.ec + (size_t)((J >> 1) & 1) * sizeof(double2) * 2 * kw.kmax * nrhs,
+             *ecn = (char*)kw.ec + (size_t)(~(J >> 1) & 1) * sizeof(double2) * 2 * kw.kmax * nrhs;
+        KL(OVS_PROF_MATVEC, bw + (double)fb * nrhs,
+           launch_wilson_pair(g->links32, u2, fb, x1, fb, u1, fb, kw.ps, g->geom, nrhs, g->kappa, g->mu, kw.pact, st,
+                              sh));
+        if (more)
+            KL(OVS_PROF_MATVEC, bw,
+               launch_wilson(PREC_F32, true, g->links32, x1, fb, x2, fb, g->geom, nrhs, g->kappa, g->mu, kw.pact, st,
+                             sh));
+        const void* xx = more ? x2 : x1;  // the last block has no use for x2
+        KL(OVS_PROF_DOTS, (double)fb * nrhs * (J + 4.0),
+           launch_pair_dots(kw.basis, basis_rhs, units, J, u1, u2, x1, xx, units, nrhs, g->num_sms, slots, kw.ppart,
+                            kw.pact, kw.err, st));
+        KL(OVS_PROF_SMALL, 16.0 * slots * S * nrhs,
+           launch_reduce(kw.ppart, slots, S, S, nrhs, kw.pred, pred, false, kw.pact, st));
+        KL(OVS_PROF_SMALL, 16.0 * ((double)J * J / 2 + 8.0 * J) * nrhs,
+           launch_pair_step(kw.pred, pred, J, more, kw.H, h_rhs, ldh, kw.beta, kw.inv_beta, kw.dcoef, kw.hnorm2,
+                            kw.active, kw.k_used, kw.ps, kw.pact, kw.pmode, kw.jstart, never, ec, ecn, kw.kmax, nrhs,
+                            st));
+        // a check of H_J: columns below J are complete; the right-hand sides of
+        // this block (mode), those that stop leave the blocks
+        if (every > 0 && J > 0 && J % every == 0) TRY(check(J, kw.pmode, kw.pact));
+        KL(OVS_PROF_UPDATE, (double)fb * nrhs * (J + 8.0),
+           launch_pair_update(kw.basis, basis_rhs, units, J, kw.pred, pred, kw.ps, kw.pmode, u1, u2, x1, xx, units,
+                              nrhs, g->num_sms, kw.err, st));
+    }
+    const int dslots = gdots_chunk_slots(units, nrhs, g->num_sms);
+    for (int j = 1; j < k; ++j) {
+        const int S = gdots_stride(2, j);
+        KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_tail_mask(kw.jstart, kw.k_used, j, kw.tmask, nrhs, st));
+        KL(OVS_PROF_MATVEC, 0.0,
+           launch_wilson(PREC_F32, true, g->links32, u1, fb, x1, fb, g->geom, nrhs, g->kappa, g->mu, kw.tmask, st, sh));
+        KL(OVS_PROF_DOTS, 0.0,
+           launch_gdots2_chunk(kw.basis, basis_rhs, units, j, u1, units, x1, units, units, nrhs, g->num_sms, dslots,
+                               kw.partial, kw.tmask, kw.err, st));
+        KL(OVS_PROF_SMALL, 0.0,
+           launch_reduce(kw.partial, dslots, S, S, nrhs, kw.htmp, kw.jcap, false, kw.tmask, st));
+        KL(OVS_PROF_SMALL, 0.0,
+           launch_arnoldi_step(kw.htmp, kw.jcap, j, kw.H, h_rhs, ldh, kw.beta, kw.inv_beta, kw.dcoef, kw.hnorm2,
+                               kw.tmask, kw.k_used, nrhs, st));
+        KL(OVS_PROF_SMALL, 0.0,
+           launch_arnoldi_column(kw.htmp, kw.jcap, j, kw.H, h_rhs, ldh, kw.inv_beta, kw.dcoef, kw.tmask, nrhs, st));
+        if (every > 0 && j % every == 0) TRY(check(j, kw.tmask, kw.tmask));
+        KL(OVS_PROF_UPDATE, 0.0,
+           launch_arnoldi_update_tma(kw.basis, basis_rhs, units, j, kw.htmp, kw.jcap, kw.inv_beta, kw.dcoef, u1, units,
+                                     x1, units, units, nrhs, g->num_sms, kw.tmask, kw.err, st));
+    }
+    KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_tail_mask(kw.jstart, kw.k_used, k, kw.tmask, nrhs, st));
+    return OVS_OK;
+}
+
 // Enqueue the whole application on st, from the device canonical input xd
 // to the device canonical output yd. Buffers must already be sized
 // (ensure_vec / ensure_kry); no allocation happens here, and no host
@@ -867,9 +968,15 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     const BlasPlan plan = blas_plan(units, nrhs, g->num_sms);
     const BlasPlan plan64 = blas_plan(N, nrhs, g->num_sms);
     const int dslots = tp == PREC_F32 ? gdots_chunk_slots(units, nrhs, g->num_sms) : 0;
-    // the two-launch step: FP64, and complex64 fields that give the TMA sweeps
-    // (work items of 2048 units) less than one item per SM
-    const bool fine = tp == PREC_F64 || (units + 2047) / 2048 * nrhs < g->num_sms;
+    // fine_sweeps.cu: FP64, and complex64 fields with less than a tile of the TMA
+    // sweeps per SM
+    const bool fine = tp == PREC_F64 || units * nrhs < 512LL * g->num_sms;
+    // two steps per pass (pair_sweeps.cu) where the basis is read
+    // from memory: it saves about half of 2 nrhs k^2/2 vectors' traffic and adds
+    // the launches of the single steps' loop, which do nothing as a rule (7 per
+    // step, about 10 us); the line lies where the saving is twice that.
+    const bool pair = !fine && !(g->m > 0 && g->scheme == DEFL_SCHUR) && k >= 4 &&
+                      (double)fb * nrhs * k >= kPairBytes;
     char* basis = (char*)kw.basis;
 
     // input, canonical complex128 -> internal precision
@@ -989,9 +1096,10 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     // skip-ahead schedule) the sign of the complete H_j of each active
     // right-hand side that is due; stop it once successive coefficient
     // vectors agree to tol (V orthonormal, so this is the change of its
-    // Krylov part).
-    auto check = [&](int j, int* active) -> int {
-        KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_check_due(active, cstate, j, kw.due, nrhs, st));
+    // Krylov part). in: the right-hand sides to look at; active: cleared where one
+    // stops.
+    auto check = [&](int j, const int* in, int* active) -> int {
+        KL(OVS_PROF_SMALL, 12.0 * nrhs, launch_check_due(in, cstate, j, kw.due, nrhs, st));
         TRY(sign_column(kw.ccheck[1], kw.due, j));
         KL(OVS_PROF_SMALL, 48.0 * j * nrhs,
            launch_conv_check(kw.ccheck[1], kw.ccheck[0], kmax, j, opts->tol, active, kw.k_used, kw.est, kw.due, cstate,
@@ -1000,7 +1108,9 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     };
     const long long fp_rhs = kmax + 1;
     const size_t fp_half = sizeof(double2) * (size_t)fp_rhs * nrhs;
-    for (int j = 0; j < k; ++j) {
+    if (pair) TRY(pair_steps(g, nrhs, k, sh, every, check, st));
+    const int* live = pair ? kw.tmask : kw.active;  // right-hand sides that reached k
+    for (int j = 0; j < k && !pair; ++j) {
         const int S = gdots_stride(2, j);
         int* act = fine ? kw.active + (j & 1) * nrhs : kw.active;
         KL(OVS_PROF_MATVEC, bw,
@@ -1054,7 +1164,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
             if (schur)  // X[:, j] = (xz - X[:, <j] s) / beta_j
                 KL(OVS_PROF_SMALL, 16.0 * ((double)m * j + 2.0 * m) * nrhs,
                    launch_schur_xcol(kw.X, x_rhs, m, j, kw.htmp, kw.jcap, kw.inv_beta, fs.activen, nrhs, st));
-            if (every > 0 && j > 0 && j % every == 0) TRY(check(j, fs.activen));
+            if (every > 0 && j > 0 && j % every == 0) TRY(check(j, fs.activen, fs.activen));
             continue;
         }
         KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (j + 2.0),
@@ -1070,7 +1180,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                launch_schur_xcol(kw.X, x_rhs, m, j, kw.htmp, kw.jcap, kw.inv_beta, kw.active, nrhs, st));
         KL(OVS_PROF_SMALL, 16.0 * ((double)j * j / 2 + 2.0 * j) * nrhs,
            launch_arnoldi_column(kw.htmp, kw.jcap, j, kw.H, h_rhs, ldh, kw.inv_beta, kw.dcoef, kw.active, nrhs, st));
-        if (every > 0 && j > 0 && j % every == 0) TRY(check(j, kw.active));
+        if (every > 0 && j > 0 && j % every == 0) TRY(check(j, kw.active, kw.active));
         KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
            launch_arnoldi_update_tma(basis, basis_rhs_units, units, j, kw.htmp, kw.jcap, kw.inv_beta, kw.dcoef,
                                      w.xint, units, w.wvec, units, units, nrhs, g->num_sms, kw.active, kw.err, st));
@@ -1080,11 +1190,11 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         const int S = gdots_stride(2, k);
         KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (k + 1.0),
            launch_gdots2_chunk(basis, basis_rhs_units, units, k, w.xint, units, w.xint, units, units, nrhs,
-                               g->num_sms, dslots, kw.partial, kw.active, kw.err, st));
+                               g->num_sms, dslots, kw.partial, live, kw.err, st));
         KL(OVS_PROF_SMALL, 16.0 * dslots * S * nrhs,
-           launch_reduce(kw.partial, dslots, S, S, nrhs, kw.htmp, kw.jcap, false, kw.active, st));
+           launch_reduce(kw.partial, dslots, S, S, nrhs, kw.htmp, kw.jcap, false, live, st));
         KL(OVS_PROF_SMALL, 16.0 * 2.0 * k * nrhs,
-           launch_arnoldi_final(kw.htmp, kw.jcap, k, 2 * k, kw.H, h_rhs, ldh, kw.active, nrhs, st));
+           launch_arnoldi_final(kw.htmp, kw.jcap, k, 2 * k, kw.H, h_rhs, ldh, live, nrhs, st));
     } else {
         const int S = gdots_stride(1, k), chunks = fine_chunks(units, k, nrhs, g->num_sms);
         const int* act = kw.active + (k & 1) * nrhs;

@@ -217,8 +217,9 @@ __device__ __forceinline__ void hop_apply(const HopData<R, RT>& d, const bool (&
     }
 }
 
-// Optional epilogue of the stencil: out = ah * (stencil result) + bx * X + by * Y
-// (used by the Chebyshev filter of the eigensolver set-up).
+// Optional epilogues of the stencil: out = ah * (stencil result) + bx * X + by * Y
+// (AX = 1: the Chebyshev filter of the eigensolver set-up), or (stencil
+// result) - ps[r].gamma_next X (AX = 2: the block steps of pair_sweeps.cu).
 struct Axpy {
     const char* X;
     size_t xs;
@@ -227,13 +228,14 @@ struct Axpy {
     size_t ys;
     double by;
     double ah;
+    const PairState* ps = nullptr;
 };
 
 // out_r = [gamma5] (in_r - kappa * hops(in_r)) for the right-hand sides r
 // of the thread. in/out strides are in bytes between right-hand sides.
 // Blocks are numbered with the right-hand-side tile fastest, so the blocks
 // of all tiles that share a tile of sites (and of links) run back to back.
-template <typename R, bool G5, int RT, bool AX = false>
+template <typename R, bool G5, int RT, int AX = 0>
 __global__ void __launch_bounds__(256) k_wilson(const void* __restrict__ links, const char* __restrict__ in,
                                                 char* out, size_t in_stride, size_t out_stride, Geom g,
                                                 R kappa, R emu, R emmu, int nrhs, int ntiles,
@@ -311,7 +313,14 @@ __global__ void __launch_bounds__(256) k_wilson(const void* __restrict__ links, 
             if (G5 && q >= 6) v = -v;
             p[q] = v;
         }
-        if (AX) {
+        if (AX == 2) {
+            cplx<R> xv[12];
+            Field<R>::load(ax.X + (size_t)r * ax.xs, g.V, s, xv);
+            const R gm = R(ax.ps[r].gamma_next);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) p[q] = p[q] - xv[q] * gm;
+        }
+        if (AX == 1) {
             cplx<R> xv[12], yv[12];
             Field<R>::load(ax.X + (size_t)r * ax.xs, g.V, s, xv);
             Field<R>::load(ax.Y + (size_t)r * ax.ys, g.V, s, yv);
@@ -382,7 +391,7 @@ __device__ __forceinline__ void one_hop(const void* links, const char* in, size_
     if (NU == 3) { out[2] = FWD ? -u0 : u0;         out[3] = FWD ? -u1 : u1; }
 }
 
-template <typename R, bool G5, bool AX>
+template <typename R, bool G5, int AX>
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
     k_wilson_split(const void* __restrict__ links, const char* __restrict__ in, char* out, size_t in_stride,
                    size_t out_stride, Geom g, R kappa, R emu, R emmu, const int* __restrict__ active, Axpy ax) {
@@ -424,7 +433,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
         const size_t e = 2 * ((size_t)(q >> 1) * g.V + s0 + at) + (q & 1);  // entry q of the site
         cplx<R> v = src[e] - a * kappa;
         if (G5 && q >= 6) v = -v;
-        if (AX) {
+        if (AX == 2) v = v - reinterpret_cast<const cplx<R>*>(ax.X + (size_t)r * ax.xs)[e] * R(ax.ps[r].gamma_next);
+        if (AX == 1) {
             const cplx<R> xv = reinterpret_cast<const cplx<R>*>(ax.X + (size_t)r * ax.xs)[e];
             const cplx<R> yv = reinterpret_cast<const cplx<R>*>(ax.Y + (size_t)r * ax.ys)[e];
             v = v * R(ax.ah) + xv * R(ax.bx) + yv * R(ax.by);
@@ -561,7 +571,7 @@ static bool valid_shape(const StencilShape& sh) {
     return false;
 }
 
-template <typename R, bool G5, bool AX>
+template <typename R, bool G5, int AX>
 static void wilson_dispatch(const StencilShape& sh, unsigned blocks, int ntiles, cudaStream_t st, const void* links,
                             const void* in, size_t in_stride, void* out, size_t out_stride, const Geom& g,
                             double kappa, double emu, double emmu, int nrhs, const int* active, const Axpy& ax) {
@@ -594,17 +604,17 @@ cudaError_t launch_wilson(int prec, bool gamma5, const void* links, const void* 
     const Axpy ax{};
     if (prec == PREC_F64) {
         if (gamma5)
-            wilson_dispatch<double, true, false>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
+            wilson_dispatch<double, true, 0>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
                                                  out_stride, g, kappa, emu, emmu, nrhs, active, ax);
         else
-            wilson_dispatch<double, false, false>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
+            wilson_dispatch<double, false, 0>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
                                                   out_stride, g, kappa, emu, emmu, nrhs, active, ax);
     } else {
         if (gamma5)
-            wilson_dispatch<float, true, false>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
+            wilson_dispatch<float, true, 0>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
                                                 out_stride, g, kappa, emu, emmu, nrhs, active, ax);
         else
-            wilson_dispatch<float, false, false>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
+            wilson_dispatch<float, false, 0>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out,
                                                  out_stride, g, kappa, emu, emmu, nrhs, active, ax);
     }
     return cudaGetLastError();
@@ -621,11 +631,27 @@ cudaError_t launch_wilson_axpy(int prec, const void* links, const void* in, size
     const double emu = exp(mu), emmu = exp(-mu);
     const Axpy ax{(const char*)X, xs, bx, (const char*)Y, ys, by, ah};
     if (prec == PREC_F64)
-        wilson_dispatch<double, true, true>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out, out_stride,
+        wilson_dispatch<double, true, 1>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out, out_stride,
                                             g, kappa, emu, emmu, nrhs, nullptr, ax);
     else
-        wilson_dispatch<float, true, true>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out, out_stride,
+        wilson_dispatch<float, true, 1>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out, out_stride,
                                            g, kappa, emu, emmu, nrhs, nullptr, ax);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_wilson_pair(const void* links, const void* in, size_t in_stride, void* out, size_t out_stride,
+                               const void* X, size_t xs, const PairState* ps, const Geom& g, int nrhs, double kappa,
+                               double mu, const int* active, cudaStream_t st, StencilShape sh) {
+    if (!valid_shape(sh)) return cudaErrorInvalidValue;
+    const int ntiles = (nrhs + sh.rt * sh.rb - 1) / (sh.rt * sh.rb);
+    const long long blocks = (long long)ntiles * ((g.V + sh.sites - 1) / sh.sites);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    Axpy ax{};
+    ax.X = (const char*)X;
+    ax.xs = xs;
+    ax.ps = ps;
+    wilson_dispatch<float, true, 2>(sh, (unsigned)blocks, ntiles, st, links, in, in_stride, out, out_stride, g, kappa,
+                                    exp(mu), exp(-mu), nrhs, active, ax);
     return cudaGetLastError();
 }
 

@@ -45,6 +45,11 @@ struct KryWork {  // Krylov basis and small matrices
     void* newton = nullptr; // [nrhs][newton_rhs] complex128: work of the sign of H_k
     long long newton_rhs = 0;
     int* need = nullptr;    // [nrhs] right-hand sides left to Roberts' iteration
+    // two steps per pass (complex64): sums of the block sweep, coefficients of
+    // x1, x2 (two parities), scalars and masks per right-hand side
+    void *ppart = nullptr, *pred = nullptr, *ec = nullptr;
+    ovs::PairState* ps = nullptr;
+    int *pact = nullptr, *pmode = nullptr, *jstart = nullptr, *tmask = nullptr;
     void* cdef = nullptr;   // [nrhs][m] complex128 deflation coefficients
     void* cdef2 = nullptr;  // [nrhs][m] complex128 sgn-scaled (Schur: second-pass scratch)
     int mdef = 0;           // m the deflation buffers below were sized for

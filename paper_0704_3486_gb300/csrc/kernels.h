@@ -37,6 +37,11 @@ cudaError_t launch_wilson_axpy(int prec, const void* links, const void* in, size
                                size_t out_stride, const void* X, size_t xs, double bx, const void* Y, size_t ys,
                                double by, double ah, const Geom& g, int nrhs, double kappa, double mu,
                                cudaStream_t st, StencilShape shape = StencilShape{});
+// out_r = H_w in_r - ps[r].gamma_next X_r (complex64): a block step's first stencil
+struct PairState;
+cudaError_t launch_wilson_pair(const void* links, const void* in, size_t in_stride, void* out, size_t out_stride,
+                               const void* X, size_t xs, const PairState* ps, const Geom& g, int nrhs, double kappa,
+                               double mu, const int* active, cudaStream_t st, StencilShape shape = StencilShape{});
 // flat complex128 <-> complex64 conversion of internal fields (to_prec = target)
 cudaError_t launch_convert(int to_prec, const void* in, void* out, long long ncplx, cudaStream_t st);
 // uniform (-1,1) complex entries from a hash of (seed, index)
@@ -168,6 +173,30 @@ cudaError_t launch_arnoldi_update_tma(void* basis, long long basis_rhs_stride, l
                                       const void* dcoef, void* u, long long u_rhs_stride, const void* z,
                                       long long z_rhs_stride, long long nunits, int nrhs, int num_sms,
                                       const int* active, int* err, cudaStream_t st);
+
+// ---- two steps per pass over the complex64 basis (pair_sweeps.cu)
+struct PairState {  // of one right-hand side: the scalars of its last block
+    double b1, r22, gamma_now, gamma_next;
+    double2 r12, a1, a2, c1, c2, d_now, d_next;
+};
+int pair_stride(int J);  // entries of a slot of the sums: 4J + 10
+int pair_slots(long long nunits, int nrhs, int num_sms);  // slots x nrhs <= num_sms + 2 nrhs
+cudaError_t launch_pair_dots(const void* basis, long long basis_rhs_stride, long long vec_stride, int J,
+                             const void* u1, const void* u2, const void* x1, const void* x2, long long nunits,
+                             int nrhs, int num_sms, int nslot, void* partial, const int* active, int* err,
+                             cudaStream_t st);
+// scalars and columns of a block; more: another block follows. pact: the
+// right-hand sides still in blocks; mode: what the update writes; jstart: the
+// step from which single steps go on (never: none)
+cudaError_t launch_pair_step(const void* red, long long red_stride, int J, bool more, void* H, long long h_rhs,
+                             int ldh, double* beta0, double* inv_beta, void* dcoef, double* hnorm2, int* active,
+                             int* k_used, PairState* ps, int* pact, int* mode, int* jstart, int never,
+                             const void* ec, void* ecn, int kmax, int nrhs, cudaStream_t st);
+cudaError_t launch_pair_update(void* basis, long long basis_rhs_stride, long long vec_stride, int J, const void* red,
+                               long long red_stride, const PairState* ps, const int* mode, void* u1, void* u2,
+                               const void* x1, const void* x2, long long nunits, int nrhs, int num_sms, int* err,
+                               cudaStream_t st);
+cudaError_t launch_tail_mask(const int* jstart, const int* k_used, int j, int* mask, int nrhs, cudaStream_t st);
 
 // c'_r,i = sgn(Re lambda_i) * c_r,i
 cudaError_t launch_sign_scale(const void* c, const double* sgn, int m, int nrhs, void* out, cudaStream_t st);

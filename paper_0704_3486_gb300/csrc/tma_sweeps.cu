@@ -25,73 +25,16 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "tma_dev.cuh"
 
 namespace ovs {
-
-namespace {
-
-constexpr int TB = 256;       // threads per block
-constexpr int TW = TB / 32;   // warps
-constexpr int TG = 8;         // basis vectors per stage
-// update sweep: 2 units per thread per tile, 3 stages of 64 KB
-constexpr int TE = 2;
-constexpr int TU = TB * TE;
-constexpr int TNS = 3;
-constexpr size_t kStageBytes = (size_t)TG * TU * 16;
-constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait gives up after 1 s
-constexpr int OVS_ETIMEOUT_CODE = -7;        // OVS_ETIMEOUT
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// try_wait until the phase completes or kWaitNs have passed (the clock is
-// read only once the first try has failed)
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > kWaitNs) return false;
-    }
-}
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-}  // namespace
 
 // Inner products of the delayed-reorthogonalisation Arnoldi step, complex64
 // basis: s_i = V_i^H u, t_i = V_i^H z (i < J), u^H u and u^H z.
 //
 // Persistent, warp-specialised form, one block per SM: 8 consumer warps and
-// one producer warp. The work items are the row chunks of CU = 2048 units of
-// every right-hand side, flattened as (r, c) and split into one contiguous
+// one producer warp. The work items are row chunks of cu <= CU = 2048 units of
+// every right-hand side (balanced_items), flattened as (r, c) and split into one contiguous
 // range per block. For each chunk a consumer thread holds its 8 units of u
 // and of z in registers; the basis streams through DS = 3 stages (192 KB in
 // flight) of 8 vectors x 512 units, groups of 8 vectors in the outer order
@@ -113,14 +56,6 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // that starts r also zeroes r's slots beyond its last one, so every one of
 // the `nslot` slots is defined.
 namespace {
-constexpr int CU = 2048;                     // units per row chunk
-constexpr int DU = 512;                      // units per tile
-constexpr int DE = DU / TB;                  // units per consumer thread per tile
-constexpr int DNT = CU / DU;                 // tiles per chunk
-constexpr int DS = 3;                        // stages
-constexpr int DTHREADS = TB + 32;            // consumer warps + producer warp
-constexpr size_t kDStage = (size_t)TG * DU * 16;
-
 template <int CUR, int O>
 __device__ __forceinline__ void tstep32(float (&v)[32], bool upper) {
 #pragma unroll
@@ -130,47 +65,13 @@ __device__ __forceinline__ void tstep32(float (&v)[32], bool upper) {
         v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
     }
 }
-__device__ __forceinline__ double wsum_d(double v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-// named barrier 1 over the TB consumer threads; the OR of `p` over them
-__device__ __forceinline__ bool consumers_sync_or(bool p) {
-    uint32_t r;
-    asm volatile(
-        "{\n .reg .pred a, b;\n setp.ne.u32 a, %1, 0;\n bar.red.or.pred b, 1, %2, a;\n selp.u32 %0, 1, 0, b;\n}"
-        : "=r"(r)
-        : "r"((uint32_t)p), "n"(TB)
-        : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TB) : "memory"); }
-// bounded wait that also gives up once another thread has raised `abort`
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort || global_ns() - t0 > kWaitNs) return false;
-    }
-}
-// block that owns flattened item i under the contiguous split of T items
-// over G blocks (block q owns [floor(qT/G), floor((q+1)T/G)))
-__host__ __device__ inline int owner_of(long long i, long long T, int G) {
-    return (int)(((i + 1) * G - 1) / T);
-}
-__host__ __device__ inline long long range_lo(int q, long long T, int G) { return (long long)q * T / G; }
 }  // namespace
 
 __global__ void __launch_bounds__(DTHREADS, 1)
     k_gdots2_ws(const float4* __restrict__ basis, long long basis_rhs_stride, long long vec_stride, int J,
                 const float4* __restrict__ u, long long u_rhs_stride, const float4* __restrict__ z,
-                long long z_rhs_stride, long long nunits, int nrhs, int nslot, double2* __restrict__ partial,
-                const int* __restrict__ active, int* __restrict__ err) {
+                long long z_rhs_stride, long long nunits, int cu, int nrhs, int nslot,
+                double2* __restrict__ partial, const int* __restrict__ active, int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t full[DS];
     __shared__ __align__(8) uint64_t empty[DS];
@@ -181,7 +82,8 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, q = blockIdx.x;
     const int S = 2 * J + 2;
-    const long long cpr = (nunits + CU - 1) / CU;  // chunks per right-hand side
+    const long long cpr = (nunits + cu - 1) / cu;  // items per right-hand side
+    const int nt = (cu + DU - 1) / DU;             // tiles per item
     const long long T = cpr * nrhs;
     const long long lo = range_lo(q, T, G), hi = range_lo(q + 1, T, G);
     const int ngroups = (J + TG - 1) / TG;
@@ -203,12 +105,12 @@ __global__ void __launch_bounds__(DTHREADS, 1)
         for (long long it = lo; it < hi && ok; ++it) {
             const long long r = it / cpr, c = it - r * cpr;
             if (active != nullptr && active[r] == 0) continue;
-            const long long u0 = c * CU;
-            const int len = (int)min((long long)CU, nunits - u0);
+            const long long u0 = c * cu;
+            const int len = (int)min((long long)cu, nunits - u0);
             const float4* Vr = basis + r * basis_rhs_stride + u0;
             for (int g = 0; g < ngroups && ok; ++g) {
                 const int nv = min(TG, J - g * TG);
-                for (int t = 0; t < DNT; ++t) {
+                for (int t = 0; t < nt; ++t) {
                     const int s = n % DS;
                     if (n >= DS) {  // the consumers' release of this stage's previous use
                         if (!mbar_wait_or_abort(&empty[s], (uint32_t)((n / DS - 1) & 1), abort)) {
@@ -298,8 +200,8 @@ __global__ void __launch_bounds__(DTHREADS, 1)
             for (int i = tid; i < 2 * S; i += TB) acc[i] = 0.0;
             seg_r = r;
         }
-        const long long u0 = c * CU;
-        const int len = (int)min((long long)CU, nunits - u0);
+        const long long u0 = c * cu;
+        const int len = (int)min((long long)cu, nunits - u0);
         float4 ur[DNT * DE], zr[DNT * DE];
         const float4* up = u + r * u_rhs_stride + u0;
         const float4* zp = z + r * z_rhs_stride + u0;
@@ -331,6 +233,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
             const int nv = min(TG, J - g * TG);
 #pragma unroll
             for (int t = 0; t < DNT; ++t) {
+                if (t >= nt) break;
                 const int s = n % DS;
                 const bool got = bad || mbar_wait_or_abort(&full[s], (uint32_t)((n / DS) & 1), abort);
                 if (!__all_sync(0xffffffffu, got)) {  // keep `bad` uniform over the warp
@@ -416,7 +319,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     k_arnoldi_update_ws(float4* __restrict__ basis, long long basis_rhs_stride, long long vec_stride, int J,
                         const double2* __restrict__ red, long long red_stride, const double* __restrict__ inv_beta,
                         const double2* __restrict__ dcoef, float4* __restrict__ u, long long u_rhs_stride,
-                        const float4* __restrict__ z, long long z_rhs_stride, long long nunits, int nrhs,
+                        const float4* __restrict__ z, long long z_rhs_stride, long long nunits, int tu, int nrhs,
                         const int* __restrict__ active, int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t full[TNS];
@@ -425,7 +328,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     cf* sc = reinterpret_cast<cf*>(smem + TNS * kStageBytes);  // s at [0, J), t at [J, 2J)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, q = blockIdx.x;
-    const long long tpr = (nunits + TU - 1) / TU;  // tiles per right-hand side
+    const long long tpr = (nunits + tu - 1) / tu;  // tiles per right-hand side
     const long long T = tpr * nrhs;
     const long long lo = range_lo(q, T, G), hi = range_lo(q + 1, T, G);
     const int ngroups = (J + TG - 1) / TG;
@@ -445,9 +348,9 @@ __global__ void __launch_bounds__(DTHREADS, 1)
         int n = 0;  // stages issued
         bool ok = true;
         for (long long it = lo; it < hi && ok; ++it) {
-            const long long r = it / tpr, base = (it - r * tpr) * TU;
+            const long long r = it / tpr, base = (it - r * tpr) * tu;
             if (active != nullptr && active[r] == 0) continue;
-            const uint32_t bytes = (uint32_t)min((long long)TU, nunits - base) * 16u;
+            const uint32_t bytes = (uint32_t)min((long long)tu, nunits - base) * 16u;
             const float4* Vr = basis + r * basis_rhs_stride + base;
             for (int g = 0; g < ngroups; ++g) {
                 const int s = n % TNS;
@@ -483,7 +386,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     float ib = 0.f;
     cf d = {0.f, 0.f};
     for (long long it = lo; it < hi; ++it) {
-        const long long r = it / tpr, base = (it - r * tpr) * TU;
+        const long long r = it / tpr, base = (it - r * tpr) * tu, end = min(base + tu, nunits);
         if (active != nullptr && active[r] == 0) continue;
         if (r != seg_r) {  // coefficients of the next right-hand side
             if (consumers_sync_or(bad)) return;  // everyone is done with the old ones
@@ -503,8 +406,8 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 #pragma unroll
         for (int e = 0; e < TE; ++e) {
             const long long p = base + tid + (long long)TB * e;
-            up[e] = p < nunits ? ur[p] : make_float4(0.f, 0.f, 0.f, 0.f);
-            zp[e] = p < nunits ? __ldg(zr + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+            up[e] = p < end ? ur[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+            zp[e] = p < end ? __ldg(zr + p) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         cf a[TE][2], bb[TE][2];
 #pragma unroll
@@ -548,7 +451,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 #pragma unroll
         for (int e = 0; e < TE; ++e) {
             const long long p = base + tid + (long long)TB * e;
-            if (p >= nunits) continue;
+            if (p >= end) continue;
             cf uc[2], zc[2], vo[2], un[2];
             Unit<float>::split(up[e], uc);
             Unit<float>::split(zp[e], zc);
@@ -575,7 +478,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 __global__ void __launch_bounds__(DTHREADS, 1)
     k_recombine_ws(const float4* __restrict__ basis, long long basis_rhs_stride, long long vec_stride, int J,
                    const int* __restrict__ Jdev, const double2* __restrict__ coef, long long coef_stride,
-                   double alpha, double2* __restrict__ y, long long y_rhs_stride, long long nunits, int nrhs,
+                   double alpha, double2* __restrict__ y, long long y_rhs_stride, long long nunits, int tu, int nrhs,
                    const int* __restrict__ active, int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t full[TNS];
@@ -584,7 +487,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     cf* sc = reinterpret_cast<cf*>(smem + TNS * kStageBytes);  // alpha * c, FP32, [0, J)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = gridDim.x, q = blockIdx.x;
-    const long long tpr = (nunits + TU - 1) / TU;
+    const long long tpr = (nunits + tu - 1) / tu;
     const long long T = tpr * nrhs;
     const long long lo = range_lo(q, T, G), hi = range_lo(q + 1, T, G);
     volatile int* abort = &abort_flag;
@@ -604,11 +507,11 @@ __global__ void __launch_bounds__(DTHREADS, 1)
         int n = 0;
         bool ok = true;
         for (long long it = lo; it < hi && ok; ++it) {
-            const long long r = it / tpr, base = (it - r * tpr) * TU;
+            const long long r = it / tpr, base = (it - r * tpr) * tu;
             if (active != nullptr && active[r] == 0) continue;
             const int Jr = depth(r);
             const int ngroups = (Jr + TG - 1) / TG;
-            const uint32_t bytes = (uint32_t)min((long long)TU, nunits - base) * 16u;
+            const uint32_t bytes = (uint32_t)min((long long)tu, nunits - base) * 16u;
             const float4* Vr = basis + r * basis_rhs_stride + base;
             for (int g = 0; g < ngroups; ++g) {
                 const int s = n % TNS;
@@ -643,7 +546,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
     int Jr = 0;
     bool bad = false;
     for (long long it = lo; it < hi; ++it) {
-        const long long r = it / tpr, base = (it - r * tpr) * TU;
+        const long long r = it / tpr, base = (it - r * tpr) * tu, end = min(base + tu, nunits);
         if (active != nullptr && active[r] == 0) continue;
         if (r != seg_r) {  // coefficients of the next right-hand side
             if (consumers_sync_or(bad)) return;
@@ -661,8 +564,8 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 #pragma unroll
         for (int e = 0; e < TE; ++e) {
             const long long p = base + tid + (long long)TB * e;
-            yo[e][0] = p < nunits ? yr[2 * p] : make_double2(0.0, 0.0);
-            yo[e][1] = p < nunits ? yr[2 * p + 1] : make_double2(0.0, 0.0);
+            yo[e][0] = p < end ? yr[2 * p] : make_double2(0.0, 0.0);
+            yo[e][1] = p < end ? yr[2 * p + 1] : make_double2(0.0, 0.0);
         }
         for (int g = 0; g < ngroups; ++g) {
             const int s = n % TNS;
@@ -709,7 +612,7 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 #pragma unroll
         for (int e = 0; e < TE; ++e) {
             const long long p = base + tid + (long long)TB * e;
-            if (p >= nunits) continue;
+            if (p >= end) continue;
             yr[2 * p] = yo[e][0];
             yr[2 * p + 1] = yo[e][1];
         }
@@ -718,17 +621,21 @@ __global__ void __launch_bounds__(DTHREADS, 1)
 
 static size_t gdots_chunk_smem(int J) { return DS * kDStage + (size_t)(2 * J + 2) * 16; }
 
-static int gdots_chunk_grid(long long nunits, int nrhs, int num_sms) {
-    const long long T = (nunits + CU - 1) / CU * nrhs;
-    return (int)std::max<long long>(1, std::min<long long>(num_sms, T));
+// items of the inner products (an item costs its u and z, and the reductions
+// of its groups, about 128 units' time beyond its own)
+static Items dots_items(long long nunits, int nrhs, int num_sms) {
+    return balanced_items(nunits, nrhs, num_sms, CU, 128);
+}
+static Items update_items(long long nunits, int nrhs, int num_sms) {
+    return balanced_items(nunits, nrhs, num_sms, TU, 16);
 }
 
 int gdots_chunk_slots(long long nunits, int nrhs, int num_sms) {
-    const long long cpr = (nunits + CU - 1) / CU, T = cpr * nrhs;
-    const int G = gdots_chunk_grid(nunits, nrhs, num_sms);
+    const Items w = dots_items(nunits, nrhs, num_sms);
+    const long long T = w.per_rhs * nrhs;
     int n = 1;
     for (long long r = 0; r < nrhs; ++r)
-        n = std::max(n, owner_of((r + 1) * cpr - 1, T, G) - owner_of(r * cpr, T, G) + 1);
+        n = std::max(n, owner_of((r + 1) * w.per_rhs - 1, T, w.grid) - owner_of(r * w.per_rhs, T, w.grid) + 1);
     return n;
 }
 
@@ -740,10 +647,10 @@ cudaError_t launch_gdots2_chunk(const void* basis, long long basis_rhs_stride, l
     const cudaError_t e = ensure_dyn_smem((const void*)k_gdots2_ws, smem);
     if (e != cudaSuccess) return e;
     if (nslot != gdots_chunk_slots(nunits, nrhs, num_sms)) return cudaErrorInvalidValue;
-    const int G = gdots_chunk_grid(nunits, nrhs, num_sms);
-    k_gdots2_ws<<<G, DTHREADS, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J, (const float4*)u,
-                                           u_rhs_stride, (const float4*)z, z_rhs_stride, nunits, nrhs, nslot,
-                                           (double2*)partial, active, err);
+    const Items w = dots_items(nunits, nrhs, num_sms);
+    k_gdots2_ws<<<w.grid, DTHREADS, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J, (const float4*)u,
+                                                u_rhs_stride, (const float4*)z, z_rhs_stride, nunits, (int)w.chunk,
+                                                nrhs, nslot, (double2*)partial, active, err);
     return cudaGetLastError();
 }
 
@@ -755,12 +662,11 @@ cudaError_t launch_arnoldi_update_tma(void* basis, long long basis_rhs_stride, l
     const size_t smem = TNS * kStageBytes + (size_t)(2 * J + 1) * sizeof(cf);
     const cudaError_t e = ensure_dyn_smem((const void*)k_arnoldi_update_ws, smem);
     if (e != cudaSuccess) return e;
-    const long long T = (nunits + TU - 1) / TU * nrhs;
-    const int G = (int)std::max<long long>(1, std::min<long long>(num_sms, T));
-    k_arnoldi_update_ws<<<G, DTHREADS, smem, st>>>((float4*)basis, basis_rhs_stride, vec_stride, J,
+    const Items w = update_items(nunits, nrhs, num_sms);
+    k_arnoldi_update_ws<<<w.grid, DTHREADS, smem, st>>>((float4*)basis, basis_rhs_stride, vec_stride, J,
                                                    (const double2*)red, red_stride, inv_beta, (const double2*)dcoef,
                                                    (float4*)u, u_rhs_stride, (const float4*)z, z_rhs_stride, nunits,
-                                                   nrhs, active, err);
+                                                   (int)w.chunk, nrhs, active, err);
     return cudaGetLastError();
 }
 
@@ -771,11 +677,10 @@ cudaError_t launch_recombine_tma(const void* basis, long long basis_rhs_stride, 
     const size_t smem = TNS * kStageBytes + (size_t)std::max(J, 1) * sizeof(cf);
     const cudaError_t e = ensure_dyn_smem((const void*)k_recombine_ws, smem);
     if (e != cudaSuccess) return e;
-    const long long T = (nunits + TU - 1) / TU * nrhs;
-    const int G = (int)std::max<long long>(1, std::min<long long>(num_sms, T));
-    k_recombine_ws<<<G, DTHREADS, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J, Jdev,
+    const Items w = update_items(nunits, nrhs, num_sms);
+    k_recombine_ws<<<w.grid, DTHREADS, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J, Jdev,
                                               (const double2*)coef, coef_stride, alpha, (double2*)y, y_rhs_stride,
-                                              nunits, nrhs, active, err);
+                                              nunits, (int)w.chunk, nrhs, active, err);
     return cudaGetLastError();
 }
 

@@ -25,10 +25,12 @@
 // function, and every third node of the n-pair rule is itself the n/3-pair
 // rule. Its distance e from the full rule is the error of the latter's
 // coarse part; the error of the full rule is about e^3 (geometric convergence,
-// three times the exponent). A result is taken when e <= 3e-6; right-hand
-// sides above that get a second rule (144 pairs over [1e-6 b, b]), and those
-// that fail it too (an eigenvalue on or next to the imaginary axis) get
-// Roberts' iteration itself (launch_newton), with its statuses. Measured over
+// three times the exponent). A result is taken when e <= 3e-6; right-hand sides
+// above that get a second rule (144 pairs over [1e-6 b, b]: spectra up to about
+// 50 degrees off the real axis), then a third (3072 pairs over the same, up to
+// 88 degrees: the Ritz value near 0 that an odd k has), and those that fail it
+// too (an eigenvalue on or next to the imaginary axis) Roberts' iteration
+// itself (launch_newton), with its statuses. Measured over
 // lattices 4^4 to 8^4, k 40 to 400, mu 0.05 to 0.3: e = 2e-8, and the first
 // column within 3e-16 of Roberts' in the 2-norm. Whole applications, before
 // (Roberts on 4 to 8 SMs per right-hand side, one block above k = 320) and
@@ -45,14 +47,18 @@ namespace ovs {
 
 namespace {
 
-constexpr int kPairs1 = 48, kPairs2 = 144;  // multiples of 3
+constexpr int kPairs1 = 48, kPairs2 = 144, kPairs3 = 3072;  // multiples of 3, the last of kPairs2
 constexpr double kWindow1 = 1e-3, kWindow2 = 1e-6;
 constexpr double kAccept = 3e-6;
 constexpr int QS = 8;  // columns of H in flight per warp (cp.async stages)
-constexpr int kItersLevel1 = 7, kItersLevel2 = 9;  // ceil(log2(2 pairs)): the Roberts iterate of that degree
+constexpr int kItersLevel[4] = {0, 7, 9, 13};  // ceil(log2(2 pairs)): the Roberts iterate of that degree
 
+// Node and weight / pi of the pairs, for b = 1: a table, or for more pairs than
+// it holds (of which warp p takes p, p + kPairs2, ...) the constants of the rule.
 struct QuadNodes {
-    double t[kPairs2], w[kPairs2];  // node and weight / pi of the pairs, for b = 1
+    int pairs;
+    double r, K, Kp, lq;
+    double t[kPairs2], w[kPairs2];
 };
 
 double agm(double a, double b) {
@@ -68,27 +74,32 @@ double agm(double a, double b) {
 // and w_j = (dt/dv)(v_j) K'/(n pi). The Fourier series of sn at imaginary
 // argument converges fast on v <= K'/2; the other half is its mirror image
 // t(K' - v) = r / t(v).
+__host__ __device__ inline void quad_node(const QuadNodes& q, int j, double& t, double& w) {
+    const double pi = 3.14159265358979323846;
+    const int at = j < (q.pairs + 1) / 2 ? j : q.pairs - 1 - j;
+    const double h = q.Kp / q.pairs, v = (at + 0.5) * h;
+    double s = 0.0, d = 0.0;
+    for (int i = 0; i < 8; ++i) {  // terms fall by e^(-pi Kp / 2K), 2e-3 at r = 1e-3 and 3e-7 at 1e-6
+        const double o = 2 * i + 1, a = o * pi * v / (2 * q.K), c = 1.0 / (1.0 - exp(o * q.lq));
+        const double ep = exp(o * q.lq / 2 + a), em = exp(o * q.lq / 2 - a);
+        s += c * (ep - em) / 2;
+        d += o * c * (ep + em) / 2;
+    }
+    s *= 2 * pi / q.K;
+    d *= pi * pi / (q.K * q.K);
+    t = at == j ? s : q.r / s;
+    w = d * h / pi * (at == j ? 1.0 : q.r / (s * s));
+}
+
 QuadNodes make_nodes(int n, double r) {
     const double pi = 3.14159265358979323846;
     QuadNodes q{};
-    const double K = pi / 2 / agm(1.0, std::sqrt(1.0 - r * r)), Kp = pi / 2 / agm(1.0, r);
-    const double lq = -pi * Kp / K, h = Kp / n;
-    for (int j = 0; j < (n + 1) / 2; ++j) {
-        const double v = (j + 0.5) * h;
-        double s = 0.0, d = 0.0;
-        for (int i = 0; i < 30; ++i) {
-            const double o = 2 * i + 1, a = o * pi * v / (2 * K), c = 1.0 / (1.0 - std::exp(o * lq));
-            const double ep = std::exp(o * lq / 2 + a), em = std::exp(o * lq / 2 - a);
-            s += c * (ep - em) / 2;
-            d += o * c * (ep + em) / 2;
-        }
-        s *= 2 * pi / K;
-        d *= pi * pi / (K * K);
-        q.t[j] = s;
-        q.w[j] = d * h / pi;
-        q.t[n - 1 - j] = r / s;
-        q.w[n - 1 - j] = q.w[j] * r / (s * s);
-    }
+    q.pairs = n;
+    q.r = r;
+    q.K = pi / 2 / agm(1.0, std::sqrt(1.0 - r * r));
+    q.Kp = pi / 2 / agm(1.0, r);
+    q.lq = -pi * q.Kp / q.K;
+    for (int j = 0; j < std::min(n, kPairs2); ++j) quad_node(q, j, q.t[j], q.w[j]);
     return q;
 }
 
@@ -129,7 +140,7 @@ __global__ void __launch_bounds__(256) k_quad_prep(const double2* __restrict__ H
     }
 }
 
-// One node (one sign of t) per warp: P[r][node][0..n) = (w/pi) (H - i t)^-1 e_1.
+// One node (one sign of t) per warp and pass: P[r][node][0..n) = (w/pi) (H - i t)^-1 e_1.
 // Lane q of the warp owns rows q, q + 32, ...: s[j] sums row 32 j + q, and once
 // row l has been used, its place keeps z_{l-1}. What bounds it: the FP64 units
 // (two multiply-adds a clock and SM: 4 per complex term), for few right-hand
@@ -148,8 +159,6 @@ __global__ void __launch_bounds__(32) k_quad_solve(const double2* __restrict__ H
     const int n = quad_order(k_used, n_fixed, due, need, level, r);
     if (n <= 0) return;
     const double b = 2.0 * __longlong_as_double((long long)bmax[r]);
-    const double t = (node & 1) ? -nodes.t[node >> 1] * b : nodes.t[node >> 1] * b;
-    const double w = nodes.w[node >> 1] * b;
     const double2* Hr = H + r * h_rhs;
     const double* ib = isub + (size_t)r * kmax;
     // column c into its stage: rows 0 .. c
@@ -161,73 +170,94 @@ __global__ void __launch_bounds__(32) k_quad_solve(const double2* __restrict__ H
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    for (int c = n - 1; c > n - QS; --c) fetch(c);
-    double sr[KC], si[KC];
+    double2* out = P + r * p_rhs + (size_t)node * kmax;
+    for (int pair = node >> 1; pair < nodes.pairs; pair += kPairs2) {
+        double t, w;
+        if (nodes.pairs <= kPairs2) {
+            t = nodes.t[pair];
+            w = nodes.w[pair];
+        } else {
+            quad_node(nodes, pair, t, w);
+        }
+        t = (node & 1) ? -t * b : t * b;
+        w *= b;
+        for (int c = n - 1; c > n - QS; --c) fetch(c);
+        double sr[KC], si[KC];
 #pragma unroll
-    for (int j = 0; j < KC; ++j) sr[j] = si[j] = 0.0;
-    double zr = 1.0, zi = 0.0, last = 1.0;  // z_l of the current column; z_{n-1}
+        for (int j = 0; j < KC; ++j) sr[j] = si[j] = 0.0;
+        double zr = 1.0, zi = 0.0, last = 1.0;  // z_l of the current column; z_{n-1}
 #pragma unroll
-    for (int sl = KC - 1; sl >= 0; --sl) {
-        if (32 * sl >= n) continue;
-        for (int q = min(31, n - 1 - 32 * sl); q >= 0; --q) {
-            const int l = 32 * sl + q;
-            __syncwarp();  // every lane has read the stage that is refilled here
-            fetch(l - QS + 1);
-            asm volatile("cp.async.wait_group %0;\n" ::"n"(QS - 1) : "memory");
-            __syncwarp();
-            const double ibl = l > 0 ? __ldg(ib + l) : 0.0;
-            const double2* col = ring + (size_t)(l % QS) * (32 * KC);
-            {  // slot sl first: z_{l-1} needs row l
-                double2 h = lane <= q ? col[32 * sl + lane] : make_double2(0.0, 0.0);
-                if (lane == q) h.y -= t;
-                sr[sl] = fma(h.x, zr, sr[sl]);
-                sr[sl] = fma(-h.y, zi, sr[sl]);
-                si[sl] = fma(h.x, zi, si[sl]);
-                si[sl] = fma(h.y, zr, si[sl]);
-            }
-            double nr = -lane_d(sr[sl], q) * ibl, ni = -lane_d(si[sl], q) * ibl;
-            if (lane == q && l > 0) {
-                sr[sl] = nr;
-                si[sl] = ni;
-            }
-#pragma unroll
-            for (int j = 0; j < sl; ++j) {
-                const double2 h = col[32 * j + lane];
-                sr[j] = fma(h.x, zr, sr[j]);
-                sr[j] = fma(-h.y, zi, sr[j]);
-                si[j] = fma(h.x, zi, si[j]);
-                si[j] = fma(h.y, zr, si[j]);
-            }
-            zr = nr;
-            zi = ni;
-            // exponent above 2^200: everything times 2^-200 (uniform over the warp)
-            const int e = max((__double2hiint(zr) >> 20) & 0x7ff, (__double2hiint(zi) >> 20) & 0x7ff);
-            if (e > 1023 + 200 && l > 0) {
-                const double f = 0x1p-200;
-#pragma unroll
-                for (int j = 0; j < KC; ++j) {
-                    sr[j] *= f;
-                    si[j] *= f;
+        for (int sl = KC - 1; sl >= 0; --sl) {
+            if (32 * sl >= n) continue;
+            for (int q = min(31, n - 1 - 32 * sl); q >= 0; --q) {
+                const int l = 32 * sl + q;
+                __syncwarp();  // every lane has read the stage that is refilled here
+                fetch(l - QS + 1);
+                asm volatile("cp.async.wait_group %0;\n" ::"n"(QS - 1) : "memory");
+                __syncwarp();
+                const double ibl = l > 0 ? __ldg(ib + l) : 0.0;
+                const double2* col = ring + (size_t)(l % QS) * (32 * KC);
+                {  // slot sl first: z_{l-1} needs row l
+                    double2 h = lane <= q ? col[32 * sl + lane] : make_double2(0.0, 0.0);
+                    if (lane == q) h.y -= t;
+                    sr[sl] = fma(h.x, zr, sr[sl]);
+                    sr[sl] = fma(-h.y, zi, sr[sl]);
+                    si[sl] = fma(h.x, zi, si[sl]);
+                    si[sl] = fma(h.y, zr, si[sl]);
                 }
-                zr *= f;
-                zi *= f;
-                last *= f;
+                double nr = -lane_d(sr[sl], q) * ibl, ni = -lane_d(si[sl], q) * ibl;
+                if (lane == q && l > 0) {
+                    sr[sl] = nr;
+                    si[sl] = ni;
+                }
+#pragma unroll
+                for (int j = 0; j < sl; ++j) {
+                    const double2 h = col[32 * j + lane];
+                    sr[j] = fma(h.x, zr, sr[j]);
+                    sr[j] = fma(-h.y, zi, sr[j]);
+                    si[j] = fma(h.x, zi, si[j]);
+                    si[j] = fma(h.y, zr, si[j]);
+                }
+                zr = nr;
+                zi = ni;
+                // exponent above 2^200: everything times 2^-200 (uniform over the warp)
+                const int e = max((__double2hiint(zr) >> 20) & 0x7ff, (__double2hiint(zi) >> 20) & 0x7ff);
+                if (e > 1023 + 200 && l > 0) {
+                    const double f = 0x1p-200;
+#pragma unroll
+                    for (int j = 0; j < KC; ++j) {
+                        sr[j] *= f;
+                        si[j] *= f;
+                    }
+                    zr *= f;
+                    zi *= f;
+                    last *= f;
+                }
             }
         }
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    const double gr = lane_d(sr[0], 0), gi = lane_d(si[0], 0);  // row 0: (H - i t)_0 z
-    // w / gamma by a scaled division (gamma may be large)
-    const double m = fmax(fabs(gr), fabs(gi));
-    const double ar = gr / m, ai = gi / m, den = w / (m * (ar * ar + ai * ai));
-    const double fr = ar * den, fi = -ai * den;
-    double2* out = P + r * p_rhs + (size_t)node * kmax;
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        const double gr = lane_d(sr[0], 0), gi = lane_d(si[0], 0);  // row 0: (H - i t)_0 z
+        // w / gamma by a scaled division (gamma may be large)
+        const double m = fmax(fabs(gr), fabs(gi));
+        const double ar = gr / m, ai = gi / m, den = w / (m * (ar * ar + ai * ai));
+        const double fr = ar * den, fi = -ai * den;
+        const bool first = pair < kPairs2;
+        auto put = [&](int l, double x, double y) {
+            if (!first) {
+                const double2 o = out[l];
+                x += o.x;
+                y += o.y;
+            }
+            out[l] = make_double2(x, y);
+        };
 #pragma unroll
-    for (int j = 0; j < KC; ++j) {
-        const int l = 32 * j + lane;  // this place holds z_{l-1}
-        if (l >= 1 && l < n) out[l - 1] = make_double2(sr[j] * fr - si[j] * fi, sr[j] * fi + si[j] * fr);
+        for (int j = 0; j < KC; ++j) {
+            const int l = 32 * j + lane;  // this place holds z_{l-1}
+            if (l >= 1 && l < n) put(l - 1, sr[j] * fr - si[j] * fi, sr[j] * fi + si[j] * fr);
+        }
+        if (lane == 0) put(n - 1, last * fr, last * fi);
+        __syncwarp();
     }
-    if (lane == 0) out[n - 1] = make_double2(last * fr, last * fi);
 }
 
 constexpr int RT = 512;
@@ -342,7 +372,8 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
                              void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
                              int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
                              const int* due, int n_fixed) {
-    static const QuadNodes nodes1 = make_nodes(kPairs1, kWindow1), nodes2 = make_nodes(kPairs2, kWindow2);
+    static const QuadNodes nodes1 = make_nodes(kPairs1, kWindow1), nodes2 = make_nodes(kPairs2, kWindow2),
+                           nodes3 = make_nodes(kPairs3, kWindow2);
     double2* P = (double2*)work;  // [nrhs][2 kPairs2][kmax], then bmax and isub of all right-hand sides
     if (work_rhs < sign_quad_work(kmax)) return cudaErrorInvalidValue;
     const long long p_rhs = 2LL * kPairs2 * kmax;
@@ -354,9 +385,9 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
     k_quad_prep<<<dim3((nb + 7) / 8, nrhs), 256, 0, st>>>((const double2*)H, h_rhs, ldh, k_used, n_fixed, due, bmax,
                                                           isub, kmax);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    for (int level = 1; level <= 2; ++level) {
-        const int pairs = level == 1 ? kPairs1 : kPairs2;
-        const QuadNodes& q = level == 1 ? nodes1 : nodes2;
+    for (int level = 1; level <= 3; ++level) {
+        const QuadNodes& q = level == 1 ? nodes1 : level == 2 ? nodes2 : nodes3;
+        const int pairs = std::min(q.pairs, kPairs2);
         const int kc = (nb + 31) / 32;
 #define OVS_QUAD(K)                                                                                               \
     e = solve<K>(pairs, nrhs, st, H, h_rhs, ldh, k_used, n_fixed, due, need, level, bmax, isub, kmax, P, p_rhs, q)
@@ -372,7 +403,7 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
 #undef OVS_QUAD
         if (e != cudaSuccess) return e;
         k_quad_sum<<<nrhs, RT, 0, st>>>(P, p_rhs, pairs, k_used, n_fixed, due, beta, kmax, (double2*)coeff,
-                                        coeff_stride, need, level, level == 1 ? kItersLevel1 : kItersLevel2, iters,
+                                        coeff_stride, need, level, kItersLevel[level], iters,
                                         status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -360,7 +360,10 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
     CK(dalloc(&k.due, sizeof(int) * n));
     CK(dalloc(&k.cstate, sizeof(CheckState) * n));
     CK(cudaMemset(k.err, 0, sizeof(int)));
-    CK(dalloc(&k.partial, sizeof(double2) * std::max<size_t>((size_t)nb * n, fine_chunks_max(n, g->num_sms)) * jc));
+    k.pcap = (long long)std::max<size_t>((size_t)nb * n, fine_chunks_max(n, g->num_sms)) * jc;
+    if (g->m > 0)  // the shared-basis sums: up to two blocks per SM
+        k.pcap = std::max<long long>(k.pcap, 2LL * g->num_sms * n * gdots_stride(1, g->m));
+    CK(dalloc(&k.partial, sizeof(double2) * (size_t)k.pcap));
     CK(dalloc(&k.fpcol, sizeof(double2) * 2 * (size_t)(km + 1) * n));
     CK(dalloc(&k.norm_part, sizeof(double) * (size_t)nb * n));
     CK(dalloc(&k.beta, sizeof(double) * n));
@@ -1004,7 +1007,8 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     // partial sums of S^H v_r over pblk blocks (reduced by the caller): in the
     // mixed form the shared-basis kernel that reads S once for all
     // right-hand sides, else the register sweep
-    const int sdb = (tp == PREC_F32 && m > 0) ? shared_dots_blocks(m, nrhs, units, g->num_sms, kw.nblk) : 0;
+    const int sdb = (tp == PREC_F32 && m > 0) ? shared_dots_blocks(m, nrhs, units, g->num_sms, (int)(kw.pcap / ((long long)nrhs * S1)))
+                        : 0;
     const int pblk = sdb > 0 ? sdb : plan.nblk;
     auto shared_dots = [&](const void* basis, const void* v, const int* act) -> int {
         if (sdb > 0)
@@ -1216,17 +1220,33 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     if (every > 0)
         KL(OVS_PROF_SMALL, 32.0 * k * nrhs,
            launch_check_final(cstate, kw.ccheck[0], kw.coeff, kmax, kw.k_used, kw.due, nrhs, st));
-    if (schur)  // App. A needs the whole of sgn(H_k)
-        KL(OVS_PROF_NEWTON, 16.0 * (double)k * k * nrhs,
-           launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
-                         kw.status, st, nullptr, 0, k));  // k_used[r] <= k
-    else
-        TRY(sign_column(kw.coeff, every > 0 ? kw.due : nullptr, 0));
     if (schur) {
-        // Schur coefficients sgn(T) c + beta Y e_1 (App. A), then y = S cS
-        KL(OVS_PROF_SMALL, 16.0 * ((double)m * k * 4 + (double)k * k) * nrhs,
+        // Schur and Krylov coefficients: by quadrature on [T X; 0 H_k], and for
+        // what that leaves by sgn(H_k) and the Sylvester equation (App. A)
+        const int* need = nullptr;
+        if (m <= kSchurQuadMax) {
+            SchurQuad sq;
+            sq.m = m;
+            sq.T = g->schurT;
+            sq.X = kw.X;
+            sq.x_rhs = x_rhs;
+            sq.c = kw.cdef;
+            sq.c_rhs = m;
+            sq.Q = kw.sylv;
+            sq.q_rhs = schur_scratch_per_rhs(m);
+            sq.cS = kw.cS;
+            sq.cs_rhs = m;
+            KL(OVS_PROF_NEWTON, 16.0 * ((double)k * k + (double)m * k + (double)m * m) * nrhs,
+               launch_sign_quad(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, kw.newton_rhs,
+                                (int)kmax, k, nrhs, kw.iters, kw.status, kw.need, st, nullptr, 0, sq));
+            need = kw.need;
+        }
+        KL(OVS_PROF_NEWTON, 0.0,
+           launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
+                         kw.status, st, need, 0, k));  // k_used[r] <= k
+        KL(OVS_PROF_SMALL, 0.0,
            launch_schur_coeff(g->schurT, g->schurFT, m, kw.X, x_rhs, kw.H, h_rhs, ldh, kw.newton, 2 * kmax * kmax,
-                              kw.k_used, kw.status, kw.beta, kw.cdef, m, kw.sylv, kw.cS, m, nrhs, k, st));
+                              kw.k_used, kw.status, kw.beta, kw.cdef, m, kw.sylv, kw.cS, m, nrhs, k, st, need));
         if (tp == PREC_F64)
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F64, PREC_F64, m, nrhs, true, false),
                launch_update(PREC_F64, PREC_F64, g->R64, 0, N, m, nullptr, kw.cS, m, 1.0, nullptr, 0, w.yacc, N, N,
@@ -1239,6 +1259,8 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F32, PREC_F64, m, nrhs, true, false),
                launch_update(PREC_F32, PREC_F64, g->R32, 0, units, m, nullptr, kw.cS, m, 1.0, nullptr, 0, w.yacc,
                              N, units, plan, nrhs, nullptr, nullptr, st));
+    } else {
+        TRY(sign_column(kw.coeff, every > 0 ? kw.due : nullptr, 0));
     }
     // K4: y += V_k c (Sec. 5.3 step vi)
     if (tp == PREC_F32)

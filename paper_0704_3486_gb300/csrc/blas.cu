@@ -299,6 +299,43 @@ __global__ void k_reduce(const double2* __restrict__ partial, int nblk, int pstr
     }
 }
 
+// The same for many blocks: a thread block takes 32 sums, each warp every
+// eighth block's part of them, so the loads of a sum run eight deep and its
+// additions spread over the FP64 units of more SMs.
+__global__ void __launch_bounds__(256) k_reduce_wide(const double2* __restrict__ partial, int nblk, int pstride, int J,
+                                                     int nrhs, double2* __restrict__ out, long long out_stride,
+                                                     int accumulate, const int* __restrict__ active) {
+    __shared__ double2 sh[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int idx = blockIdx.x * 32 + lane;
+    const bool live = idx < J * nrhs;
+    const int r = live ? idx / J : 0, i = live ? idx - r * J : 0;
+    const bool on = live && (active == nullptr || active[r] != 0);
+    double2 s = make_double2(0.0, 0.0);
+    if (on) {
+#pragma unroll 4
+        for (int b = warp; b < nblk; b += 8) {
+            const double2 p = partial[((size_t)r * nblk + b) * pstride + i];
+            s.x += p.x;
+            s.y += p.y;
+        }
+    }
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || !on) return;
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+        s.x += sh[w][lane].x;
+        s.y += sh[w][lane].y;
+    }
+    double2* o = out + r * out_stride + i;
+    if (accumulate) {
+        const double2 v = *o;
+        s = make_double2(v.x + s.x, v.y + s.y);
+    }
+    *o = s;
+}
+
 // The step and the column of H as launches of their own (after the TMA
 // sweeps): one block per right-hand side, and one warp per row with 8 rows per
 // block and the right-hand side in y.
@@ -487,14 +524,15 @@ __global__ void __launch_bounds__(BT) k_shared_dots(const float4* __restrict__ S
 static size_t shared_dots_smem(int m, int nrhs) { return 2 * (size_t)(m + nrhs) * KP * sizeof(float4); }
 
 // Blocks of the shared-basis dots for nunits within the partial slots
-// available: as many per SM as their two stages fit (at most 4); 0 when the
-// tile does not fit (the register sweep k_gdots serves then).
+// available: as many per SM as their two stages fit, at most 2 (every block is
+// one more partial sum to add); 0 when the tile does not fit (the register sweep
+// k_gdots serves then).
 int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms, int max_blocks) {
     const int itiles = (m + 3) / 4, rtiles = (nrhs + 1) / 2;
     if (m < 1 || nrhs < 1 || (long long)itiles * rtiles > BT) return 0;
     const size_t smem = shared_dots_smem(m, nrhs);
     if (smem > 200 * 1024) return 0;
-    const long long per_sm = std::max<long long>(1, std::min<long long>(4, (long long)(220 * 1024) / (long long)smem));
+    const long long per_sm = std::max<long long>(1, std::min<long long>(2, (long long)(220 * 1024) / (long long)smem));
     long long want = per_sm * num_sms;
     want = std::min<long long>(want, std::max<long long>(1, nunits / KD));
     want = std::min<long long>(want, max_blocks);
@@ -767,6 +805,11 @@ cudaError_t launch_reduce(const void* partial, int nblk, int pstride, int J, int
                           long long out_stride, bool accumulate, const int* active, cudaStream_t st) {
     if (J <= 0) return cudaSuccess;
     const int n = J * nrhs;
+    if (nblk >= 16) {  // below that a sum is one batch of loads
+        k_reduce_wide<<<(n + 31) / 32, 256, 0, st>>>((const double2*)partial, nblk, pstride, J, nrhs, (double2*)out,
+                                                     out_stride, accumulate ? 1 : 0, active);
+        return cudaGetLastError();
+    }
     k_reduce<<<(n + 127) / 128, 128, 0, st>>>((const double2*)partial, nblk, pstride, J, nrhs, (double2*)out,
                                               out_stride, accumulate ? 1 : 0, active);
     return cudaGetLastError();

@@ -31,6 +31,7 @@ struct KryWork {  // Krylov basis and small matrices
     double* est = nullptr;                 // [nrhs] last convergence estimate
     int* due = nullptr;                    // [nrhs] checked at this step (A7)
     void* cstate = nullptr;                // [nrhs] CheckState: the check schedule (A7)
+    long long pcap = 0;          // complex128 entries of partial
     void* partial = nullptr;     // [max(nrhs nblk, fine_chunks_max)][jcap] complex128
     void* fpcol = nullptr;        // [2][nrhs][kmax + 1] complex128: first pass of the last column (by parity)
     double* norm_part = nullptr; // [nrhs][nblk]

@@ -217,10 +217,22 @@ cudaError_t launch_newton(const void* H, long long h_rhs_stride, int ldh, const 
 // launch_newton serves those, with active = need), else 0. work: work_rhs >=
 // sign_quad_work(kmax) complex128 per right-hand side.
 long long sign_quad_work(int kmax);
+// With Schur deflation (m > 0, at most kSchurQuadMax) also cS, the coefficients
+// of the Schur vectors: the upper rows of sgn([T X; 0 H_k]) [c; beta e_1]. T:
+// column-major m x m, X: column-major m x k per right-hand side, Q: 288 m
+// complex128 of work per right-hand side (strides in complex128).
+constexpr int kSchurQuadMax = 256;
+struct SchurQuad {
+    int m = 0;
+    const void *T = nullptr, *X = nullptr, *c = nullptr;
+    long long x_rhs = 0, c_rhs = 0;
+    void *Q = nullptr, *cS = nullptr;
+    long long q_rhs = 0, cs_rhs = 0;
+};
 cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
                              void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
                              int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
-                             const int* due = nullptr, int n_fixed = 0);
+                             const int* due = nullptr, int n_fixed = 0, const SchurQuad& sq = SchurQuad{});
 // harmonic variant: H_r[:, k-1] += |h_(k+1,k)|^2 H_k^-H e_k (k = k_used[r]);
 // work as for launch_newton (used as scratch before it)
 cudaError_t launch_harmonic(void* H, long long h_rhs_stride, int ldh, const int* k_used, void* work, int kmax,
@@ -229,13 +241,15 @@ cudaError_t launch_harmonic(void* H, long long h_rhs_stride, int ldh, const int*
 // X[:, j] = (X[:, j] - X[:, <j] s) / beta_j, s = red[r][0..j)
 cudaError_t launch_schur_xcol(void* X, long long x_rhs, int m, int j, const void* red, long long red_stride,
                               const double* inv_beta, const int* active, int nrhs, cudaStream_t st);
-// cS_r = sgn(T) c_r + beta_r Y_r e_1, Y_r from T Y - Y H_k = sgn(T) X - X sgn(H_k)
+// cS_r = sgn(T) c_r + beta_r Y_r e_1, Y_r from T Y - Y H_k = sgn(T) X - X sgn(H_k),
+// for the right-hand sides with need[r] != 0 (all if need is nullptr)
 bool schur_coeff_fits(int kmax);
 long long schur_scratch_per_rhs(int m);
 cudaError_t launch_schur_coeff(const void* T, const void* fT, int m, const void* X, long long x_rhs, const void* H,
                                long long h_rhs, int ldh, const void* fH, long long fh_rhs, const int* k_used,
                                const int* status, const double* beta, const void* c, long long c_stride,
-                               void* scratch, void* cS, long long cs_stride, int nrhs, int kmax, cudaStream_t st);
+                               void* scratch, void* cS, long long cs_stride, int nrhs, int kmax, cudaStream_t st,
+                               const int* need = nullptr);
 // ---- outer GMRES of the overlap solve (solve.cu); canonical complex128
 int norm_blocks();  // partials per right-hand side of the norm kernels
 // norm[r] = ||v_r||, inv[r] = 1/norm[r] (inv may be nullptr); partial: nrhs x norm_blocks()

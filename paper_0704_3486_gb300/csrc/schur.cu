@@ -17,8 +17,10 @@
 //    first-pass residual of the delayed-reorthogonalisation form, v_j =
 //    (u - V_{<j} s) / beta_j, so column j of X = S^H H_w V_k follows as
 //    X[:, j] = (xz - X[:, <j] s) / beta_j (k_schur_xcol);
-//  - after K3 has formed the full sgn(H_k): C = sgn(T) X - X sgn(H_k), the
-//    Sylvester equation T Y - Y H_k = C solved row by row from the bottom by
+//  - the Schur and the Krylov coefficients together from the quadrature of
+//    signquad.cu on the composite matrix [T X; 0 H_k]; right-hand sides that it
+//    leaves (and m > 256): K3 forms the full sgn(H_k), then C = sgn(T) X - X
+//    sgn(H_k), the Sylvester equation T Y - Y H_k = C solved row by row from the bottom by
 //    the recurrences of App. A (Eqs. SolveRow, xij, abij; the sums over H
 //    end at row min(j+1, n), H being Hessenberg), and the Schur coefficients
 //    sgn(T) c + beta Y e_1 (Eq. formula, k_schur_coeff);
@@ -105,10 +107,11 @@ __global__ void __launch_bounds__(256) k_schur_coeff(
     long long x_rhs, const double2* __restrict__ H, long long h_rhs, int ldh, const double2* __restrict__ fH,
     long long fh_rhs, const int* __restrict__ k_used, const int* __restrict__ status, const double* __restrict__ beta,
     const double2* __restrict__ c, long long c_stride, double2* __restrict__ scratch, long long scr_rhs,
-    double2* __restrict__ cS, long long cs_stride) {
+    double2* __restrict__ cS, long long cs_stride, const int* __restrict__ need) {
     __shared__ cd ct[kSylvMaxK], av[kSylvMaxK], bv[kSylvMaxK];
     __shared__ cd s_y1;
     const int r = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    if (need != nullptr && need[r] == 0) return;
     const int n = k_used[r];
     const bool krylov = n > 0 && status[r] >= 0;
     const double2* cr = c + r * c_stride;
@@ -208,9 +211,11 @@ __global__ void __launch_bounds__(TC * TC) k_schur_cmat(const double2* __restric
                                                         const double2* __restrict__ fH, long long fh_rhs,
                                                         const int* __restrict__ k_used,
                                                         const int* __restrict__ status,
-                                                        double2* __restrict__ scratch, long long scr_rhs) {
+                                                        double2* __restrict__ scratch, long long scr_rhs,
+                                                        const int* __restrict__ need) {
     __shared__ double2 As[TC][TC + 1], Bs[TC][TC + 1];
     const int r = blockIdx.z;
+    if (need != nullptr && need[r] == 0) return;
     const int n = k_used[r];
     if (n <= 0 || status[r] < 0) return;  // uniform over the block
     const int i0 = blockIdx.y * TC, j0 = blockIdx.x * TC;
@@ -258,14 +263,15 @@ __global__ void __launch_bounds__(TC * TC) k_schur_cmat(const double2* __restric
 cudaError_t launch_schur_coeff(const void* T, const void* fT, int m, const void* X, long long x_rhs, const void* H,
                                long long h_rhs, int ldh, const void* fH, long long fh_rhs, const int* k_used,
                                const int* status, const double* beta, const void* c, long long c_stride,
-                               void* scratch, void* cS, long long cs_stride, int nrhs, int kmax, cudaStream_t st) {
+                               void* scratch, void* cS, long long cs_stride, int nrhs, int kmax, cudaStream_t st,
+                               const int* need) {
     const dim3 grid((kmax + TC - 1) / TC, (m + TC - 1) / TC, nrhs);
     k_schur_cmat<<<grid, dim3(TC, TC), 0, st>>>((const double2*)fT, m, (const double2*)X, x_rhs, (const double2*)fH,
-                                                fh_rhs, k_used, status, (double2*)scratch, schur_scratch_per_rhs(m));
+                                                fh_rhs, k_used, status, (double2*)scratch, schur_scratch_per_rhs(m), need);
     k_schur_coeff<<<nrhs, 256, 0, st>>>((const double2*)T, (const double2*)fT, m, (const double2*)X, x_rhs,
                                         (const double2*)H, h_rhs, ldh, (const double2*)fH, fh_rhs, k_used, status,
                                         beta, (const double2*)c, c_stride, (double2*)scratch,
-                                        schur_scratch_per_rhs(m), (double2*)cS, cs_stride);
+                                        schur_scratch_per_rhs(m), (double2*)cS, cs_stride, need);
     return cudaGetLastError();
 }
 

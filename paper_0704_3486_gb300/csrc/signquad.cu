@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "arnoldi_dev.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -111,29 +112,44 @@ __device__ __forceinline__ void cp16(void* dst, const void* src) {
                  : "memory");
 }
 
-// order of the matrix of right-hand side r; 0 where it takes no part
+// order of the matrix of right-hand side r; -1 where it takes no part
 __device__ __forceinline__ int quad_order(const int* k_used, int n_fixed, const int* due, const int* need, int level,
                                           int r) {
-    if (due != nullptr && due[r] == 0) return 0;
-    if (level > 1 && need[r] == 0) return 0;
+    if (due != nullptr && due[r] == 0) return -1;
+    if (level > 1 && need[r] == 0) return -1;
     return n_fixed > 0 ? n_fixed : k_used[r];
 }
 
 // Largest column norm of H_r (as the bits of a non-negative double, for
-// atomicMax) and the inverse subdiagonal: one warp per column.
+// atomicMax) and the inverse subdiagonal: one warp per column. With Schur
+// deflation the columns are those of [T X; 0 H_r].
 __global__ void __launch_bounds__(256) k_quad_prep(const double2* __restrict__ H, long long h_rhs, int ldh,
                                                    const int* __restrict__ k_used, int n_fixed,
                                                    const int* __restrict__ due, unsigned long long* __restrict__ bmax,
-                                                   double* __restrict__ isub, int kmax) {
+                                                   double* __restrict__ isub, int kmax, int nb, SchurQuad sq) {
     const int r = blockIdx.y, lane = threadIdx.x & 31;
     const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int n = quad_order(k_used, n_fixed, due, nullptr, 1, r);
+    if (n < 0) return;
+    if (j >= nb) {  // column j - nb of T
+        if (j - nb >= sq.m) return;
+        const double2* t = static_cast<const double2*>(sq.T) + (long long)(j - nb) * sq.m;
+        double s = 0.0;
+        for (int i = lane; i <= j - nb; i += 32) s += t[i].x * t[i].x + t[i].y * t[i].y;
+        s = warp_sum(s);
+        if (lane == 0) atomicMax(bmax + r, (unsigned long long)__double_as_longlong(sqrt(s)));
+        return;
+    }
     if (j >= n) return;
     const double2* c = H + r * h_rhs + (long long)j * ldh;
     const int rows = min(n, j + 2);
     double s = 0.0;
     for (int i = lane; i < rows; i += 32) s += c[i].x * c[i].x + c[i].y * c[i].y;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (sq.m > 0) {
+        const double2* x = static_cast<const double2*>(sq.X) + r * sq.x_rhs + (long long)j * sq.m;
+        for (int i = lane; i < sq.m; i += 32) s += x[i].x * x[i].x + x[i].y * x[i].y;
+    }
+    s = warp_sum(s);
     if (lane == 0) {
         atomicMax(bmax + r, (unsigned long long)__double_as_longlong(sqrt(s)));
         if (j + 1 < n) isub[(size_t)r * kmax + j + 1] = 1.0 / c[j + 1].x;
@@ -260,6 +276,85 @@ __global__ void __launch_bounds__(32) k_quad_solve(const double2* __restrict__ H
     }
 }
 
+// Schur part of a node: with w (H - i t)^-1 e_1 in P, the upper rows of
+//   ([T X; 0 H] - i t)^-1 [c; beta e_1]
+// are (T - i t)^-1 (c - beta X (H - i t)^-1 e_1); Q[r][node][0..m) = w times
+// that. T is upper triangular, so a back substitution: one node per warp, lane
+// q owns rows q, q + 32, ... The pair of sums over the nodes are the Schur and
+// the Krylov coefficients of sgn of the composite matrix (Sec. 5.2, Eqs. newH,
+// f_H): what App. A computes from sgn(T), sgn(H_k) and a Sylvester equation,
+// without the recurrences that lose digits as k grows.
+template <int MC>
+__global__ void __launch_bounds__(32) k_quad_schur(const double2* __restrict__ P, long long p_rhs, int kmax,
+                                                   const int* __restrict__ k_used, const int* __restrict__ need,
+                                                   int level, const unsigned long long* __restrict__ bmax,
+                                                   const double* __restrict__ beta, SchurQuad sq, QuadNodes nodes) {
+    const int r = blockIdx.y, node = blockIdx.x, lane = threadIdx.x, m = sq.m;
+    const int n = quad_order(k_used, 0, nullptr, need, level, r);
+    if (n < 0) return;
+    const double b = 2.0 * __longlong_as_double((long long)bmax[r]);
+    const double t = (node & 1) ? -nodes.t[node >> 1] * b : nodes.t[node >> 1] * b;
+    const double w = nodes.w[node >> 1] * b;
+    const double2* T = static_cast<const double2*>(sq.T);
+    const double2* X = static_cast<const double2*>(sq.X) + r * sq.x_rhs;
+    const double2* c = static_cast<const double2*>(sq.c) + r * sq.c_rhs;
+    const double2* z = P + r * p_rhs + (size_t)node * kmax;
+    double vr[MC], vi[MC], dr[MC], di[MC];
+#pragma unroll
+    for (int j = 0; j < MC; ++j) {
+        const int i = 32 * j + lane;
+        vr[j] = vi[j] = dr[j] = di[j] = 0.0;
+        if (i < m) {
+            vr[j] = w * c[i].x;
+            vi[j] = w * c[i].y;
+            const double2 d = T[i + (long long)i * m];
+            const double y = d.y - t, den = 1.0 / (d.x * d.x + y * y);
+            dr[j] = d.x * den;
+            di[j] = -y * den;
+        }
+    }
+    const double bt = n > 0 ? beta[r] : 0.0;
+#pragma unroll 4
+    for (int l = 0; l < n; ++l) {
+        const double2 zl = z[l];
+        const double zr = -bt * zl.x, zi = -bt * zl.y;
+#pragma unroll
+        for (int j = 0; j < MC; ++j) {
+            const int i = 32 * j + lane;
+            const double2 x = i < m ? __ldg(X + (long long)l * m + i) : make_double2(0.0, 0.0);
+            vr[j] = fma(x.x, zr, vr[j]);
+            vr[j] = fma(-x.y, zi, vr[j]);
+            vi[j] = fma(x.x, zi, vi[j]);
+            vi[j] = fma(x.y, zr, vi[j]);
+        }
+    }
+#pragma unroll
+    for (int sl = MC - 1; sl >= 0; --sl) {
+        for (int q = min(31, m - 1 - 32 * sl); q >= 0; --q) {  // not entered beyond m
+            const int i = 32 * sl + q;
+            const double yr = lane_d(vr[sl] * dr[sl] - vi[sl] * di[sl], q);
+            const double yi = lane_d(vr[sl] * di[sl] + vi[sl] * dr[sl], q);
+#pragma unroll
+            for (int j = 0; j <= sl; ++j) {
+                const int row = 32 * j + lane;
+                const double2 x = row < i ? __ldg(T + (long long)i * m + row) : make_double2(0.0, 0.0);
+                vr[j] = fma(-x.x, yr, vr[j]);
+                vr[j] = fma(x.y, yi, vr[j]);
+                vi[j] = fma(-x.x, yi, vi[j]);
+                vi[j] = fma(-x.y, yr, vi[j]);
+            }
+            if (lane == q) {  // row i is done: it keeps its solution
+                vr[sl] = yr;
+                vi[sl] = yi;
+            }
+        }
+    }
+    double2* out = static_cast<double2*>(sq.Q) + r * sq.q_rhs + (size_t)node * m;
+#pragma unroll
+    for (int j = 0; j < MC; ++j)
+        if (32 * j + lane < m) out[32 * j + lane] = make_double2(vr[j], vi[j]);
+}
+
 constexpr int RT = 512;
 
 __device__ __forceinline__ double rsum(double v, double* sh) {
@@ -273,43 +368,46 @@ __device__ __forceinline__ double rsum(double v, double* sh) {
 }
 
 // Sum over the nodes, the estimate from every third pair, and the verdict:
-// need[r] = 0 and coeff written where it is accepted. One block per
-// right-hand side; four groups of threads split the nodes.
+// need[r] = 0 where it is accepted; coeff (and with Schur deflation cS) then hold
+// the result. One block per right-hand side; four groups of threads split the
+// nodes.
 __global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, long long p_rhs, int pairs,
                                                  const int* __restrict__ k_used, int n_fixed,
                                                  const int* __restrict__ due, const double* __restrict__ beta,
                                                  int kmax, double2* __restrict__ coeff, long long coeff_stride,
                                                  int* __restrict__ need, int level, int iters_code,
-                                                 int* __restrict__ iters, int* __restrict__ status) {
+                                                 int* __restrict__ iters, int* __restrict__ status, SchurQuad sq) {
     __shared__ double sh[RT / 32];
     __shared__ double2 part[2][RT];
     const int r = blockIdx.x, tid = threadIdx.x;
     const int n = quad_order(k_used, n_fixed, due, need, level, r);
     double2* cr = coeff + r * coeff_stride;
-    const bool mine = due == nullptr || due[r] != 0;
-    if (n <= 0) {
-        if (level == 1) {
-            if (tid == 0) need[r] = 0;
-            if (mine) {  // an empty Krylov space: no coefficients
-                for (int i = tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
-                if (tid == 0) {
-                    iters[r] = 0;
-                    status[r] = 0;
-                }
-            }
+    if (n < 0) {
+        if (level == 1 && tid == 0) need[r] = 0;
+        return;
+    }
+    if (n == 0 && sq.m == 0) {  // an empty Krylov space: no coefficients
+        for (int i = tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
+        if (tid == 0) {
+            need[r] = 0;
+            iters[r] = 0;
+            status[r] = 0;
         }
         return;
     }
     const double2* Pr = P + r * p_rhs;
-    const int g = tid >> 7, i0 = tid & 127;
-    const double bt = beta[r];
+    const double2* Qr = static_cast<const double2*>(sq.Q) + r * sq.q_rhs;
+    const int g = tid >> 7, i0 = tid & 127, all = n + sq.m;
+    const double bt = n > 0 ? beta[r] : 0.0;
     double d2 = 0.0, c2 = 0.0;
-    for (int base = 0; base < n; base += 128) {
+    for (int base = 0; base < all; base += 128) {
         const int i = base + i0;
+        const double2* src = i < n ? Pr + i : Qr + (i - n);
+        const int ld = i < n ? kmax : sq.m;
         double cx = 0.0, cy = 0.0, sx = 0.0, sy = 0.0;
-        if (i < n) {
+        if (i < all) {
             for (int p = g; p < pairs; p += 4) {
-                const double2 a = Pr[(size_t)(2 * p) * kmax + i], c = Pr[(size_t)(2 * p + 1) * kmax + i];
+                const double2 a = src[(size_t)(2 * p) * ld], c = src[(size_t)(2 * p + 1) * ld];
                 const double x = a.x + c.x, y = a.y + c.y;
                 cx += x;
                 cy += y;
@@ -323,7 +421,7 @@ __global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, 
         part[0][tid] = make_double2(cx, cy);
         part[1][tid] = make_double2(sx, sy);
         __syncthreads();
-        if (g == 0 && i < n) {
+        if (g == 0 && i < all) {
             for (int q = 1; q < 4; ++q) {
                 const double2 a = part[0][tid + 128 * q], c = part[1][tid + 128 * q];
                 cx += a.x;
@@ -331,20 +429,26 @@ __global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, 
                 sx += c.x;
                 sy += c.y;
             }
+            const double f = i < n ? bt : 1.0;  // the Schur rows have beta in them
+            cx *= f;
+            cy *= f;
+            sx *= f;
+            sy *= f;
             d2 += (cx - 3.0 * sx) * (cx - 3.0 * sx) + (cy - 3.0 * sy) * (cy - 3.0 * sy);
             c2 += cx * cx + cy * cy;
-            cr[i] = make_double2(bt * cx, bt * cy);
+            if (i < n) cr[i] = make_double2(cx, cy);
+            else static_cast<double2*>(sq.cS)[r * sq.cs_rhs + i - n] = make_double2(cx, cy);
         }
     }
     d2 = rsum(d2, sh);
     c2 = rsum(c2, sh);
-    const bool ok = d2 <= kAccept * kAccept * c2 && isfinite(c2) && c2 > 0.0;  // false for NaN
+    const bool ok = d2 <= kAccept * kAccept * c2 && isfinite(c2);  // false for NaN
     if (ok)
         for (int i = n + tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
     if (tid == 0) {
         need[r] = ok ? 0 : 1;
         if (ok) {
-            iters[r] = iters_code;
+            iters[r] = n > 0 ? iters_code : 0;
             status[r] = 0;
         }
     }
@@ -371,7 +475,7 @@ long long sign_quad_work(int kmax) { return (long long)(2 * kPairs2 + 1) * kmax 
 cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
                              void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
                              int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
-                             const int* due, int n_fixed) {
+                             const int* due, int n_fixed, const SchurQuad& sq) {
     static const QuadNodes nodes1 = make_nodes(kPairs1, kWindow1), nodes2 = make_nodes(kPairs2, kWindow2),
                            nodes3 = make_nodes(kPairs3, kWindow2);
     double2* P = (double2*)work;  // [nrhs][2 kPairs2][kmax], then bmax and isub of all right-hand sides
@@ -382,10 +486,11 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
     cudaError_t e = cudaMemsetAsync(bmax, 0, sizeof(*bmax) * nrhs, st);
     if (e != cudaSuccess) return e;
     const int nb = n_fixed > 0 ? n_fixed : k_bound;
-    k_quad_prep<<<dim3((nb + 7) / 8, nrhs), 256, 0, st>>>((const double2*)H, h_rhs, ldh, k_used, n_fixed, due, bmax,
-                                                          isub, kmax);
+    k_quad_prep<<<dim3((nb + sq.m + 7) / 8, nrhs), 256, 0, st>>>((const double2*)H, h_rhs, ldh, k_used, n_fixed, due,
+                                                                 bmax, isub, kmax, nb, sq);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    for (int level = 1; level <= 3; ++level) {
+    // (the Schur part needs every node's solution, which the third rule adds up)
+    for (int level = 1; level <= (sq.m > 0 ? 2 : 3); ++level) {
         const QuadNodes& q = level == 1 ? nodes1 : level == 2 ? nodes2 : nodes3;
         const int pairs = std::min(q.pairs, kPairs2);
         const int kc = (nb + 31) / 32;
@@ -402,9 +507,21 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
         else return cudaErrorInvalidValue;
 #undef OVS_QUAD
         if (e != cudaSuccess) return e;
+        if (sq.m > 0) {
+            const dim3 grid(2 * pairs, nrhs);
+#define OVS_QSCHUR(M) \
+    k_quad_schur<M><<<grid, 32, 0, st>>>(P, p_rhs, kmax, k_used, need, level, bmax, beta, sq, q)
+            if (sq.m <= 32) OVS_QSCHUR(1);
+            else if (sq.m <= 64) OVS_QSCHUR(2);
+            else if (sq.m <= 128) OVS_QSCHUR(4);
+            else if (sq.m <= 256) OVS_QSCHUR(8);
+            else return cudaErrorInvalidValue;
+#undef OVS_QSCHUR
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
         k_quad_sum<<<nrhs, RT, 0, st>>>(P, p_rhs, pairs, k_used, n_fixed, due, beta, kmax, (double2*)coeff,
                                         coeff_stride, need, level, kItersLevel[level], iters,
-                                        status);
+                                        status, sq);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

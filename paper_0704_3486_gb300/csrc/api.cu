@@ -524,20 +524,35 @@ int ovs_matvec(ovs_gauge_t g, int32_t op, const void* x, void* y, int32_t nrhs, 
     void* yd = ydev ? y : g->vw.sy;
     VecWork& w = g->vw;
     const double bl = bytes_layout(N, tp, nrhs), bw = bytes_wilson(g->V, tp, nrhs);
-    KL(OVS_PROF_LAYOUT, bl, launch_to_internal(tp, xd, N, w.xint, fb, (int)g->V, nrhs, st));
     const void* L = links_for(g, tp);
     const StencilShape sh = stencil_shape(g, tp, nrhs, w.xint, fb, w.wvec, fb, st);
-    if (op == OVS_OP_HW2) {
+    // small fields: one or two launches, from and to the caller's vectors (which
+    // the layout passes would keep apart)
+    const char *xb = (const char*)xd, *yb = (const char*)yd;
+    const bool apart = xb + f64 * nrhs <= yb || yb + f64 * nrhs <= xb;
+    if (wilson_spread(tp, g->geom, nrhs) && apart) {
+        const bool twice = op == OVS_OP_HW2;
         KL(OVS_PROF_MATVEC, bw,
-           launch_wilson(tp, true, L, w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
-        KL(OVS_PROF_MATVEC, bw,
-           launch_wilson(tp, true, L, w.wvec, fb, w.xint, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
-        KL(OVS_PROF_LAYOUT, bl, launch_to_canonical(tp, w.xint, fb, yd, N, (int)g->V, nrhs, st));
+           launch_wilson_canonical(tp, op != OVS_OP_DW, L, xd, f64, true, twice ? w.wvec : yd, twice ? fb : f64,
+                                   !twice, g->geom, nrhs, g->kappa, g->mu, st));
+        if (twice)
+            KL(OVS_PROF_MATVEC, bw,
+               launch_wilson_canonical(tp, true, L, w.wvec, fb, false, yd, f64, true, g->geom, nrhs, g->kappa, g->mu,
+                                       st));
     } else {
-        KL(OVS_PROF_MATVEC, bw,
-           launch_wilson(tp, op == OVS_OP_HW, L, w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu, nullptr,
-                         st, sh));
-        KL(OVS_PROF_LAYOUT, bl, launch_to_canonical(tp, w.wvec, fb, yd, N, (int)g->V, nrhs, st));
+        KL(OVS_PROF_LAYOUT, bl, launch_to_internal(tp, xd, N, w.xint, fb, (int)g->V, nrhs, st));
+        if (op == OVS_OP_HW2) {
+            KL(OVS_PROF_MATVEC, bw,
+               launch_wilson(tp, true, L, w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
+            KL(OVS_PROF_MATVEC, bw,
+               launch_wilson(tp, true, L, w.wvec, fb, w.xint, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
+            KL(OVS_PROF_LAYOUT, bl, launch_to_canonical(tp, w.xint, fb, yd, N, (int)g->V, nrhs, st));
+        } else {
+            KL(OVS_PROF_MATVEC, bw,
+               launch_wilson(tp, op == OVS_OP_HW, L, w.xint, fb, w.wvec, fb, g->geom, nrhs, g->kappa, g->mu, nullptr,
+                             st, sh));
+            KL(OVS_PROF_LAYOUT, bl, launch_to_canonical(tp, w.wvec, fb, yd, N, (int)g->V, nrhs, st));
+        }
     }
     if (!ydev) {
         CK(cudaMemcpyAsync(y, yd, f64 * nrhs, cudaMemcpyDeviceToHost, st));

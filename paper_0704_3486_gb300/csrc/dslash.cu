@@ -122,8 +122,10 @@ __device__ __forceinline__ void hop_fwd(const cplx<R> (&p)[12], const cplx<R> (&
         if (NU == 1) { h0[c] = a0 + a3;     h1[c] = a1 - a2; }
         if (NU == 2) { h0[c] = a0 + ti(a2); h1[c] = a1 - ti(a3); }
         if (NU == 3) { h0[c] = a0 - a2;     h1[c] = a1 - a3; }
-        h0[c] = h0[c] * fac;
-        h1[c] = h1[c] * fac;
+        if (NU == 3) {  // fac is 1 on spatial hops
+            h0[c] = h0[c] * fac;
+            h1[c] = h1[c] * fac;
+        }
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -154,8 +156,10 @@ __device__ __forceinline__ void hop_bwd(const cplx<R> (&p)[12], const cplx<R> (&
         if (NU == 1) { h0[c] = a0 - a3;      h1[c] = a1 + a2; }
         if (NU == 2) { h0[c] = a0 + tmi(a2); h1[c] = a1 + ti(a3); }
         if (NU == 3) { h0[c] = a0 + a2;      h1[c] = a1 + a3; }
-        h0[c] = h0[c] * fac;
-        h1[c] = h1[c] * fac;
+        if (NU == 3) {  // fac is 1 on spatial hops
+            h0[c] = h0[c] * fac;
+            h1[c] = h1[c] * fac;
+        }
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -340,7 +344,9 @@ __global__ void __launch_bounds__(256) k_wilson(const void* __restrict__ links, 
 // warp, alone on its scheduler at some 20 clocks an instruction, has a
 // twentieth of the instructions. The sums run in the order of k_wilson (x+, x-,
 // y+, ...; within a hop as there), so the results are the same bit for bit.
-template <int HOP, typename R>
+// CIN, COUT: in, out are canonical complex128 vectors, so that an operator on
+// small fields is one launch without layout passes.
+template <int HOP, typename R, bool CIN>
 __device__ __forceinline__ void one_hop(const void* links, const char* in, size_t in_stride, int r, const Geom& g,
                                         int s, int coord, R efwd, R ebwd, int a, cplx<R> (&out)[4]) {
     constexpr int NU = HOP / 2;
@@ -357,7 +363,16 @@ __device__ __forceinline__ void one_hop(const void* links, const char* in, size_
     }
     cplx<R> U[3], p[12];
     Field<R>::row(links, g.V, NU, FWD ? s : sn, a, FWD, U);
-    Field<R>::load(in + (size_t)r * in_stride, g.V, sn, p);
+    if (CIN) {
+        const double2* x = reinterpret_cast<const double2*>(in + (size_t)r * in_stride) + (size_t)sn * 12;
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            const double2 v = __ldg(x + q);
+            p[q] = {R(v.x), R(v.y)};
+        }
+    } else {
+        Field<R>::load(in + (size_t)r * in_stride, g.V, sn, p);
+    }
     cplx<R> u0 = {R(0), R(0)}, u1 = {R(0), R(0)};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -368,8 +383,10 @@ __device__ __forceinline__ void one_hop(const void* links, const char* in, size_
             if (NU == 1) { h0 = a0 + a3;     h1 = a1 - a2; }
             if (NU == 2) { h0 = a0 + ti(a2); h1 = a1 - ti(a3); }
             if (NU == 3) { h0 = a0 - a2;     h1 = a1 - a3; }
-            h0 = h0 * fac;
-            h1 = h1 * fac;
+            if (NU == 3) {
+                h0 = h0 * fac;
+                h1 = h1 * fac;
+            }
             cfma(u0, U[c], h0);
             cfma(u1, U[c], h1);
         } else {
@@ -377,8 +394,10 @@ __device__ __forceinline__ void one_hop(const void* links, const char* in, size_
             if (NU == 1) { h0 = a0 - a3;      h1 = a1 + a2; }
             if (NU == 2) { h0 = a0 + tmi(a2); h1 = a1 + ti(a3); }
             if (NU == 3) { h0 = a0 + a2;      h1 = a1 + a3; }
-            h0 = h0 * fac;
-            h1 = h1 * fac;
+            if (NU == 3) {
+                h0 = h0 * fac;
+                h1 = h1 * fac;
+            }
             cfmac(u0, U[c], h0);
             cfmac(u1, U[c], h1);
         }
@@ -391,7 +410,7 @@ __device__ __forceinline__ void one_hop(const void* links, const char* in, size_
     if (NU == 3) { out[2] = FWD ? -u0 : u0;         out[3] = FWD ? -u1 : u1; }
 }
 
-template <typename R, bool G5, int AX>
+template <typename R, bool G5, int AX, bool CIN, bool COUT>
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
     k_wilson_split(const void* __restrict__ links, const char* __restrict__ in, char* out, size_t in_stride,
                    size_t out_stride, Geom g, R kappa, R emu, R emmu, const int* __restrict__ active, Axpy ax) {
@@ -410,14 +429,14 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
     cplx<R> o[4];
     const R one = R(1);
     switch (hop) {
-        case 0: one_hop<0>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
-        case 1: one_hop<1>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
-        case 2: one_hop<2>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
-        case 3: one_hop<3>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
-        case 4: one_hop<4>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
-        case 5: one_hop<5>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
-        case 6: one_hop<6>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
-        default: one_hop<7>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
+        case 0: one_hop<0, R, CIN>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
+        case 1: one_hop<1, R, CIN>(links, in, in_stride, r, g, s, x, one, one, row, o); break;
+        case 2: one_hop<2, R, CIN>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
+        case 3: one_hop<3, R, CIN>(links, in, in_stride, r, g, s, y, one, one, row, o); break;
+        case 4: one_hop<4, R, CIN>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
+        case 5: one_hop<5, R, CIN>(links, in, in_stride, r, g, s, z, one, one, row, o); break;
+        case 6: one_hop<6, R, CIN>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
+        default: one_hop<7, R, CIN>(links, in, in_stride, r, g, s, t, emu, emmu, row, o); break;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) part[3 * q + row][lane] = o[q];
@@ -431,7 +450,15 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
 #pragma unroll
         for (int h = 0; h < 8; ++h) a = a + cl.map_shared_rank(&part[0][0], h)[q * 32 + at];
         const size_t e = 2 * ((size_t)(q >> 1) * g.V + s0 + at) + (q & 1);  // entry q of the site
-        cplx<R> v = src[e] - a * kappa;
+        const size_t ec = (size_t)(s0 + at) * 12 + q;                     // and in a canonical vector
+        cplx<R> own;
+        if (CIN) {
+            const double2 x0 = reinterpret_cast<const double2*>(in + (size_t)r * in_stride)[ec];
+            own = {R(x0.x), R(x0.y)};
+        } else {
+            own = src[e];
+        }
+        cplx<R> v = own - a * kappa;
         if (G5 && q >= 6) v = -v;
         if (AX == 2) v = v - reinterpret_cast<const cplx<R>*>(ax.X + (size_t)r * ax.xs)[e] * R(ax.ps[r].gamma_next);
         if (AX == 1) {
@@ -439,7 +466,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(96)
             const cplx<R> yv = reinterpret_cast<const cplx<R>*>(ax.Y + (size_t)r * ax.ys)[e];
             v = v * R(ax.ah) + xv * R(ax.bx) + yv * R(ax.by);
         }
-        dst[e] = v;
+        if (COUT) reinterpret_cast<double2*>(out + (size_t)r * out_stride)[ec] = make_double2(double(v.re), double(v.im));
+        else dst[e] = v;
     }
     cl.sync();  // no block leaves while another reads its part
 }
@@ -474,56 +502,70 @@ __global__ void k_random_fill(double2* __restrict__ q, long long n, uint64_t see
 }
 
 // ------------------------------------------------------------ layouts (K7)
+// A block takes LT sites. The canonical side is read and written in its own
+// order, 16 bytes per lane in a row, and the sites' twelve entries meet in shared
+// memory at a pitch of 13 (8 lanes then fall on 8 different 16-byte groups of
+// banks). Read site by site instead, a warp's load touched 32 lines for 512
+// bytes: 3.3 TB/s over the two passes of a 16-source operator at 16^3 x 32.
+constexpr int LT = 128;
+
 // canonical complex128 [nrhs][V][12]  ->  internal planes of precision R
 template <typename R>
-__global__ void k_to_internal(const double2* __restrict__ canon, size_t canon_stride, char* __restrict__ out,
-                              size_t out_stride, int V) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (s >= V) return;
-    const double2* src = canon + r * canon_stride + (size_t)s * 12;
-    cplx<R> p[12];
+__global__ void __launch_bounds__(LT) k_to_internal(const double2* __restrict__ canon, size_t canon_stride,
+                                                    char* __restrict__ out, size_t out_stride, int V) {
+    __shared__ cplx<R> sm[LT * 13];
+    const int s0 = blockIdx.x * LT, r = blockIdx.y, tid = threadIdx.x;
+    const int n = min(LT, V - s0) * 12;
+    const double2* src = canon + r * canon_stride + (size_t)s0 * 12;
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        double2 v = src[q];
-        p[q] = {R(v.x), R(v.y)};
+    for (int k = 0; k < 12; ++k) {
+        const int i = k * LT + tid;
+        if (i < n) {
+            const double2 v = __ldcs(src + i);
+            sm[i / 12 * 13 + i % 12] = {R(v.x), R(v.y)};
+        }
     }
-    Field<R>::store(out + r * out_stride, V, s, p);
-}
-
-// internal planes of precision R -> canonical complex128
-template <typename R>
-__global__ void k_to_canonical(const char* __restrict__ in, size_t in_stride, double2* __restrict__ canon,
-                               size_t canon_stride, int V) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (s >= V) return;
+    __syncthreads();
+    if (s0 + tid >= V) return;
     cplx<R> p[12];
-    Field<R>::load(in + r * in_stride, V, s, p);
-    double2* dst = canon + r * canon_stride + (size_t)s * 12;
 #pragma unroll
-    for (int q = 0; q < 12; ++q) dst[q] = make_double2(double(p[q].re), double(p[q].im));
+    for (int q = 0; q < 12; ++q) p[q] = sm[tid * 13 + q];
+    Field<R>::store(out + r * out_stride, V, s0 + tid, p);
 }
 
-// D_ov(mu) y = x + gamma5 sgn(H_w) x (Sec. 2, Eq. Dov) fused into the last
-// layout pass: in holds sgn(H_w) x in internal complex128 planes, x is the
-// canonical source; gamma5 = diag(1, 1, -1, -1) flips the entries of spin
-// 2 and 3 (spin*3 + colour >= 6).
-__global__ void k_to_canonical_overlap(const char* __restrict__ in, size_t in_stride,
-                                       const double2* __restrict__ x, size_t x_stride, double2* __restrict__ canon,
-                                       size_t canon_stride, int V) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (s >= V) return;
-    cplx<double> p[12];
-    Field<double>::load(in + r * in_stride, V, s, p);
-    const double2* xs = x + r * x_stride + (size_t)s * 12;
-    double2* dst = canon + r * canon_stride + (size_t)s * 12;
+// internal planes of precision R -> canonical complex128; OV (R = double): D_ov(mu)
+// y = x + gamma5 sgn(H_w) x (Sec. 2, Eq. Dov) fused into this last pass, with x
+// the canonical source: gamma5 = diag(1, 1, -1, -1) flips the entries of spin 2
+// and 3 (spin*3 + colour >= 6).
+template <typename R, bool OV>
+__global__ void __launch_bounds__(LT) k_to_canonical(const char* __restrict__ in, size_t in_stride,
+                                                     const double2* __restrict__ x, size_t x_stride,
+                                                     double2* __restrict__ canon, size_t canon_stride, int V) {
+    __shared__ cplx<R> sm[LT * 13];
+    const int s0 = blockIdx.x * LT, r = blockIdx.y, tid = threadIdx.x;
+    if (s0 + tid < V) {
+        cplx<R> p[12];
+        Field<R>::load(in + r * in_stride, V, s0 + tid, p);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        const double2 xv = xs[q];
-        const double g = q < 6 ? 1.0 : -1.0;
-        dst[q] = make_double2(fma(g, p[q].re, xv.x), fma(g, p[q].im, xv.y));
+        for (int q = 0; q < 12; ++q) sm[tid * 13 + q] = p[q];
+    }
+    __syncthreads();
+    const int n = min(LT, V - s0) * 12;
+    double2* dst = canon + r * canon_stride + (size_t)s0 * 12;
+    const double2* xs = OV ? x + r * x_stride + (size_t)s0 * 12 : nullptr;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int i = k * LT + tid;
+        if (i < n) {
+            const cplx<R> p = sm[i / 12 * 13 + i % 12];
+            if (OV) {
+                const double2 xv = xs[i];
+                const double g = i % 12 < 6 ? 1.0 : -1.0;
+                dst[i] = make_double2(fma(g, double(p.re), xv.x), fma(g, double(p.im), xv.y));
+            } else {
+                dst[i] = make_double2(double(p.re), double(p.im));
+            }
+        }
     }
 }
 
@@ -580,7 +622,7 @@ static void wilson_dispatch(const StencilShape& sh, unsigned blocks, int ntiles,
     char* o = (char*)out;
     const long long groups = (g.V + 31) / 32;
     if (groups * nrhs <= kSplitGroups<R> && nrhs <= 65535) {
-        k_wilson_split<R, G5, AX><<<dim3((unsigned)(8 * groups), nrhs), 96, 0, st>>>(links, i, o, in_stride, out_stride,
+        k_wilson_split<R, G5, AX, false, false><<<dim3((unsigned)(8 * groups), nrhs), 96, 0, st>>>(links, i, o, in_stride, out_stride,
                                                                                     g, k, e1, e2, active, ax);
         return;
     }
@@ -639,6 +681,38 @@ cudaError_t launch_wilson_axpy(int prec, const void* links, const void* in, size
     return cudaGetLastError();
 }
 
+bool wilson_spread(int prec, const Geom& g, int nrhs) {
+    return (long long)((g.V + 31) / 32) * nrhs <= (prec == PREC_F64 ? kSplitGroups<double> : kSplitGroups<float>);
+}
+
+cudaError_t launch_wilson_canonical(int prec, bool gamma5, const void* links, const void* in, size_t in_stride,
+                                    bool in_canon, void* out, size_t out_stride, bool out_canon, const Geom& g,
+                                    int nrhs, double kappa, double mu, cudaStream_t st) {
+    const dim3 grid(8 * ((g.V + 31) / 32), nrhs);
+    const double ep = exp(mu), em = exp(-mu);
+#define OVS_CANON(R, G5, CI, CO)                                                                                   \
+    k_wilson_split<R, G5, 0, CI, CO><<<grid, 96, 0, st>>>(links, (const char*)in, (char*)out, in_stride, out_stride, \
+                                                          g, (R)kappa, (R)ep, (R)em, nullptr, Axpy{})
+#define OVS_CANON_G5(R, CI, CO)                 \
+    do {                                        \
+        if (gamma5) OVS_CANON(R, true, CI, CO); \
+        else OVS_CANON(R, false, CI, CO);       \
+    } while (0)
+#define OVS_CANON_R(R)                                        \
+    do {                                                      \
+        if (in_canon && out_canon) OVS_CANON_G5(R, true, true); \
+        else if (in_canon) OVS_CANON_G5(R, true, false);        \
+        else OVS_CANON_G5(R, false, true);                      \
+    } while (0)
+    if (!wilson_spread(prec, g, nrhs) || nrhs > 65535 || !(in_canon || out_canon)) return cudaErrorInvalidValue;
+    if (prec == PREC_F64) OVS_CANON_R(double);
+    else OVS_CANON_R(float);
+#undef OVS_CANON_R
+#undef OVS_CANON_G5
+#undef OVS_CANON
+    return cudaGetLastError();
+}
+
 cudaError_t launch_wilson_pair(const void* links, const void* in, size_t in_stride, void* out, size_t out_stride,
                                const void* X, size_t xs, const PairState* ps, const Geom& g, int nrhs, double kappa,
                                double mu, const int* active, cudaStream_t st, StencilShape sh) {
@@ -672,29 +746,30 @@ cudaError_t launch_random_fill(void* q, long long ncplx, uint64_t seed, cudaStre
 
 cudaError_t launch_to_internal(int prec, const void* canon, size_t canon_stride_cplx, void* out, size_t out_stride,
                                int V, int nrhs, cudaStream_t st) {
-    dim3 grid = site_grid(V, nrhs, 128);
+    const dim3 grid = site_grid(V, nrhs, LT);
     if (prec == PREC_F64)
-        k_to_internal<double><<<grid, 128, 0, st>>>((const double2*)canon, canon_stride_cplx, (char*)out, out_stride, V);
+        k_to_internal<double><<<grid, LT, 0, st>>>((const double2*)canon, canon_stride_cplx, (char*)out, out_stride, V);
     else
-        k_to_internal<float><<<grid, 128, 0, st>>>((const double2*)canon, canon_stride_cplx, (char*)out, out_stride, V);
+        k_to_internal<float><<<grid, LT, 0, st>>>((const double2*)canon, canon_stride_cplx, (char*)out, out_stride, V);
     return cudaGetLastError();
 }
 
 cudaError_t launch_to_canonical(int prec, const void* in, size_t in_stride, void* canon, size_t canon_stride_cplx,
                                 int V, int nrhs, cudaStream_t st) {
-    dim3 grid = site_grid(V, nrhs, 128);
+    const dim3 grid = site_grid(V, nrhs, LT);
     if (prec == PREC_F64)
-        k_to_canonical<double><<<grid, 128, 0, st>>>((const char*)in, in_stride, (double2*)canon, canon_stride_cplx, V);
+        k_to_canonical<double, false><<<grid, LT, 0, st>>>((const char*)in, in_stride, nullptr, 0, (double2*)canon,
+                                                           canon_stride_cplx, V);
     else
-        k_to_canonical<float><<<grid, 128, 0, st>>>((const char*)in, in_stride, (double2*)canon, canon_stride_cplx, V);
+        k_to_canonical<float, false><<<grid, LT, 0, st>>>((const char*)in, in_stride, nullptr, 0, (double2*)canon,
+                                                          canon_stride_cplx, V);
     return cudaGetLastError();
 }
 
 cudaError_t launch_to_canonical_overlap(const void* in, size_t in_stride, const void* x, size_t x_stride_cplx,
                                         void* canon, size_t canon_stride_cplx, int V, int nrhs, cudaStream_t st) {
-    dim3 grid = site_grid(V, nrhs, 128);
-    k_to_canonical_overlap<<<grid, 128, 0, st>>>((const char*)in, in_stride, (const double2*)x, x_stride_cplx,
-                                                 (double2*)canon, canon_stride_cplx, V);
+    k_to_canonical<double, true><<<site_grid(V, nrhs, LT), LT, 0, st>>>(
+        (const char*)in, in_stride, (const double2*)x, x_stride_cplx, (double2*)canon, canon_stride_cplx, V);
     return cudaGetLastError();
 }
 

@@ -37,6 +37,13 @@ cudaError_t launch_wilson_axpy(int prec, const void* links, const void* in, size
                                size_t out_stride, const void* X, size_t xs, double bx, const void* Y, size_t ys,
                                double by, double ah, const Geom& g, int nrhs, double kappa, double mu,
                                cudaStream_t st, StencilShape shape = StencilShape{});
+// The stencil of small fields (wilson_spread) with canonical complex128 vectors
+// on one or both sides (strides in bytes): the layout passes' conversions
+// included.
+bool wilson_spread(int prec, const Geom& g, int nrhs);
+cudaError_t launch_wilson_canonical(int prec, bool gamma5, const void* links, const void* in, size_t in_stride,
+                                    bool in_canon, void* out, size_t out_stride, bool out_canon, const Geom& g,
+                                    int nrhs, double kappa, double mu, cudaStream_t st);
 // out_r = H_w in_r - ps[r].gamma_next X_r (complex64): a block step's first stencil
 struct PairState;
 cudaError_t launch_wilson_pair(const void* links, const void* in, size_t in_stride, void* out, size_t out_stride,

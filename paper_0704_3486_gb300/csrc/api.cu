@@ -1284,8 +1284,8 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                                 nrhs, g->num_sms, nullptr, kw.err, st));
     else
         KL(OVS_PROF_PROJ, bytes_update(N, tp, PREC_F64, k, nrhs, false, true),
-           launch_update(tp, PREC_F64, basis, basis_rhs_units, units, k, kw.k_used, kw.coeff, kmax, 1.0, w.yacc, N,
-                         w.yacc, N, units, plan, nrhs, nullptr, nullptr, st));
+           launch_fine_combine(basis, basis_rhs_units, units, k, kw.k_used, kw.coeff, kmax, 1.0, w.yacc, units, nrhs,
+                               g->num_sms, st));
     if (overlap)  // D_ov(mu) x = x + gamma5 sgn(H_w) x (Sec. 2, Eq. Dov), fused into the layout pass
         KL(OVS_PROF_LAYOUT, bytes_layout(N, PREC_F64, nrhs) + 16.0 * N * nrhs,
            launch_to_canonical_overlap(w.yacc, f64, xd, N, yd, N, V, nrhs, st));

@@ -38,34 +38,37 @@ __device__ __forceinline__ void block_sum3(double& a, double& b, double& c, doub
 }
 
 // Sums of four values over the block (at most 8 warps; sh: 32 doubles of shared
-// memory): true in warp 0, whose lanes then hold all four in v. The FP64 pipe
-// does two lanes a clock, so a warp-wide operation takes 16 clocks of an SM: the
-// four values are reduced together, in six additions per warp.
-__device__ __forceinline__ bool block_sum4(double (&v)[4], double* sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const bool up = (lane & 16) != 0;
-        const double send = up ? v[k] : v[k + 2], keep = up ? v[k + 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-    {
-        const bool up = (lane & 8) != 0;
-        const double send = up ? v[0] : v[1], keep = up ? v[1] : v[0];
-        v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 4);
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-    // lane 8 q holds value q: 16 is bit 1 of its index, 8 bit 0
+// memory; the threads from `used` on have nothing to add): true in warp 0, whose
+// lanes then hold all four in v. A scheduler issues an FP64 operation of a warp
+// every 64 clocks (66 to its result, 600 for a square root), so the four values
+// are reduced together, in six additions per warp that has any.
+__device__ __forceinline__ bool block_sum4(double (&v)[4], double* sh, int used) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = min((int)blockDim.x >> 5, (used + 31) >> 5);
     __syncthreads();
-    if ((lane & 7) == 0) sh[4 * warp + (lane >> 3)] = v[0];
+    if (warp < nw) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool up = (lane & 16) != 0;
+            const double send = up ? v[k] : v[k + 2], keep = up ? v[k + 2] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+        }
+        {
+            const bool up = (lane & 8) != 0;
+            const double send = up ? v[0] : v[1], keep = up ? v[1] : v[0];
+            v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+        }
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 4);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+        // lane 8 q holds value q: 16 is bit 1 of its index, 8 bit 0
+        if ((lane & 7) == 0) sh[4 * warp + (lane >> 3)] = v[0];
+    }
     __syncthreads();
     if (warp != 0) return false;
     double a = lane < 4 * nw ? sh[lane] : 0.0;
-    a += __shfl_xor_sync(0xffffffffu, a, 16);
-    a += __shfl_xor_sync(0xffffffffu, a, 8);
-    a += __shfl_xor_sync(0xffffffffu, a, 4);
+    if (nw > 4) a += __shfl_xor_sync(0xffffffffu, a, 16);
+    if (nw > 2) a += __shfl_xor_sync(0xffffffffu, a, 8);
+    if (nw > 1) a += __shfl_xor_sync(0xffffffffu, a, 4);
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, a, k);
     return true;
@@ -111,13 +114,14 @@ __device__ __forceinline__ void arnoldi_step(const double2* rr, int j, int r, co
         v[2] += si.x * ti.y - si.y * ti.x;
         v[3] += h.x * h.x + h.y * h.y;
     }
-    if (!block_sum4(v, sh)) return;  // warp 0 has the sums
+    if (!block_sum4(v, sh, j)) return;  // warp 0 has the sums
     const double ss = v[0], shr = v[1], shi = v[2], c2 = v[3];
     if (lane != 0) return;
     const double b2 = rr[2 * j].x - ss;
     const double2 uz = rr[2 * j + 1];
     // a NaN (from a non-finite source) stays NaN, so that it is reported
     const double beta = (b2 > 0.0 || isnan(b2)) ? sqrt(b2) : 0.0;
+    const double ib = b2 > 0.0 ? rsqrt(b2) : 0.0;  // beside the square root, not after it
     if (j == 0) {
         o.beta0[r] = beta;
         o.hnorm2[r] = 0.0;
@@ -128,8 +132,8 @@ __device__ __forceinline__ void arnoldi_step(const double2* rr, int j, int r, co
             return;
         }
     } else {
-        const double hn2 = o.hnorm2[r] + c2 + beta * beta;
-        const bool brk = !(beta > kBreakdownTol * sqrt(hn2)) || !isfinite(beta);
+        const double hn2 = o.hnorm2[r] + c2 + (b2 < 0.0 ? 0.0 : b2);
+        const bool brk = !(b2 > kBreakdownTol * kBreakdownTol * hn2) || !isfinite(beta);  // beta > tol ||H_j||_F
         o.hnorm2[r] = hn2;
         Hr[j + (long long)(j - 1) * ldh] = make_double2(brk ? 0.0 : beta, 0.0);
         if (brk) {
@@ -139,7 +143,6 @@ __device__ __forceinline__ void arnoldi_step(const double2* rr, int j, int r, co
             return;
         }
     }
-    const double ib = 1.0 / beta;
     o.inv_beta[r] = ib;
     o.dcoef[r] = make_double2((uz.x - shr) * ib * ib, (uz.y - shi) * ib * ib);
     o.k_used[r] = j + 1;

@@ -1,27 +1,32 @@
 // K2 in two or three launches per Arnoldi step: the inner products, [their sums,]
-// and the rest of the step. These are the complex128 form's sweeps at every size, and the complex64
-// form's where the lattice is too small for the TMA sweeps (tma_sweeps.cu) to
-// give every SM a share of the basis.
+// and the rest of the step. These are the complex128 form's sweeps at every size,
+// and the complex64 form's where the lattice is too small for the TMA sweeps
+// (tma_sweeps.cu) to give every SM a share of the basis.
 //
 // Split of the inner products: along the field (chunks of 128-unit tiles) and
 // along the basis (sets of four vectors). Large problems: a block takes a chunk
 // and a group of sets, a warp whole sets of the chunk. Small ones (SPREAD): a
-// block takes one set of one chunk and its warps share the tiles, so that 4^4
-// (3,072 complex128 units) with 50 vectors still spreads over the chip and the
-// partial sums stay few.
+// block takes one set of one chunk, so that 4^4 (3,072 complex128 units) with 50
+// vectors still spreads over the chip and the partial sums stay few. An FP64
+// scheduler takes an operation of a warp every 64 clocks, so all eight warps must
+// have work: complex128, a warp takes one vector and every other tile (two busy
+// warps a block with four vectors each: 15.6 us per sweep at 4^4, now 12.5);
+// complex64, where latency counts, four vectors and every eighth tile (8^4, one
+// right-hand side: 16.8 us; with one vector per warp 20).
 //
 // Nothing is done by one block between the two: every block of the update takes
 // the step's scalars for itself, and where the partial sums are few (24 chunks
 // and 102 sums at 4^4 and 50 vectors: 39 KB from L2) also adds the chunks; else
 // k_reduce adds them in between. A last block doing both by a ticket took 14 us
-// of a 27 us sweep at that size: fence, atomic, and the sums of the whole step
-// through one SM's FP64 pipe.
+// of a 27 us sweep at 4^4, a launch of one block per right-hand side 10 us of a
+// step; programmatic dependent launch made 3x5x7x9 slower (7.5 ms against 5.9:
+// waiting blocks hold the registers that the running sweep's next blocks need).
 //
 // Measured, against register sweeps of 2048-unit row blocks, a reduction, the
 // scalars and the column in launches of their own (six per step, 2 blocks on
-// 4^4): FP64 4^4, k = 100: 51.2 -> 3.8 ms; 6^4, 2 right-hand sides, k = 340:
-// 547 -> 78 ms (FP64 floor 48); 8^4, 4 right-hand sides, k = 200: 194 -> 138 ms
-// (floor 105); complex64 8^4, one right-hand side, k = 200: 23.1 -> 7.9 ms.
+// 4^4): FP64 4^4, k = 100: 51.2 -> 3.3 ms; 6^4, 2 right-hand sides, k = 340:
+// 547 -> 76 ms (FP64 floor 48); 8^4, 4 right-hand sides, k = 200: 194 -> 136 ms
+// (floor 105); complex64 8^4, one right-hand side, k = 200: 23.1 -> 7.8 ms.
 #include <algorithm>
 
 #include "arnoldi_dev.cuh"
@@ -58,15 +63,17 @@ __device__ __forceinline__ void halve(R (&v)[M], bool upper) {
 // the basis; the warp reduction adds 16 per four vectors and chunk);
 // complex64 at these sizes, latency.
 template <typename R, int NW, bool SPREAD>
-__global__ void __launch_bounds__(FT, 2)
+__global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
     k_fine_dots(const typename Unit<R>::vec* __restrict__ basis, long long basis_rhs, long long vec_stride, int J,
                 const typename Unit<R>::vec* __restrict__ u, const typename Unit<R>::vec* __restrict__ z,
                 long long nunits, int tiles, int nchunk, int vgroups, double2* __restrict__ partial,
                 const int* __restrict__ active) {
     using vec = typename Unit<R>::vec;
     constexpr int NC = Unit<R>::ncplx;
-    constexpr int M = FV * NW * 2;  // values of a pass: vector, which, component
-    constexpr int SH = NW == 2 ? 1 : 2;  // lanes that end up with the same value: 2^SH
+    constexpr int VW = SPREAD && sizeof(R) == 8 ? 1 : FV;  // vectors of a warp's pass
+    constexpr int TW = FW * VW / FV;                       // warps that share a set's tiles (SPREAD)
+    constexpr int M = VW * NW * 2;       // values of a pass: vector, which, component
+    constexpr int SH = M == 16 ? 1 : M == 8 ? 2 : M == 4 ? 3 : 4;  // 2^SH lanes end up with the same value
     constexpr bool PER_TILE = sizeof(R) == 4;
     __shared__ double ex[FW][3];
     __shared__ double wsum[SPREAD ? FW : 1][M];
@@ -89,8 +96,8 @@ __global__ void __launch_bounds__(FT, 2)
                 const long long p = base + 32 * e;
                 if (p >= c1) break;
                 cplx<R> uc[NC], zc[NC];
-                Unit<R>::split(__ldg(ur + p), uc);
-                if (NW == 2) Unit<R>::split(__ldg(zr + p), zc);
+                Unit<R>::split(ur[p], uc);
+                if (NW == 2) Unit<R>::split(zr[p], zc);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     cfmac(a, uc[c], uc[c]);
@@ -111,34 +118,30 @@ __global__ void __launch_bounds__(FT, 2)
         }
     }
     for (int q = SPREAD ? g : g + vgroups * warp; q < nsets; q += SPREAD ? nsets : vgroups * FW) {
-        const int i0 = q * FV, nv = min(FV, J - i0);
+        const int i0 = q * FV + (SPREAD && VW == 1 ? warp % FV : 0), nv = max(0, min(VW, J - i0));
         const vec* vb = basis + r * basis_rhs + (long long)i0 * vec_stride;
         R v[M];
         double kept = 0.0;
 #pragma unroll
         for (int k = 0; k < M; ++k) v[k] = R(0);
         auto reduce = [&]() {
-            if (NW == 2) {
-                halve<M, 16>(v, (lane & 16) != 0);
-                halve<M / 2, 8>(v, (lane & 8) != 0);
-                halve<M / 4, 4>(v, (lane & 4) != 0);
-                halve<M / 8, 2>(v, (lane & 2) != 0);
-            } else {
-                halve<M, 16>(v, (lane & 16) != 0);
-                halve<M / 2, 8>(v, (lane & 8) != 0);
-                halve<M / 4, 4>(v, (lane & 4) != 0);
-                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-            }
+            if (M >= 2) halve<M, 16>(v, (lane & 16) != 0);
+            if (M >= 4) halve<M / 2, 8>(v, (lane & 8) != 0);
+            if (M >= 8) halve<M / 4, 4>(v, (lane & 4) != 0);
+            if (M >= 16) halve<M / 8, 2>(v, (lane & 2) != 0);
+            if (M < 4) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
+            if (M < 8) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 4);
+            if (M < 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
             v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
             kept += double(v[0]);
         };
         // one unit of u, z and the four vectors
-        auto term = [&](const vec& uv, const vec& zv, const vec (&x)[FV]) {
+        auto term = [&](const vec& uv, const vec& zv, const vec (&x)[VW]) {
             cplx<R> uc[NC], zc[NC];
             Unit<R>::split(uv, uc);
             Unit<R>::split(zv, zc);
 #pragma unroll
-            for (int gi = 0; gi < FV; ++gi) {
+            for (int gi = 0; gi < VW; ++gi) {
                 cplx<R> vc[NC];
                 Unit<R>::split(x[gi], vc);
 #pragma unroll
@@ -156,20 +159,20 @@ __global__ void __launch_bounds__(FT, 2)
                 }
             }
         };
-        for (long long base = c0 + lane + (SPREAD ? warp * FTILE : 0); base - lane < c1;
-             base += SPREAD ? FW * FTILE : FTILE) {
-            const bool whole = nv == FV && base - lane + FTILE <= c1;
+        for (long long base = c0 + lane + (SPREAD ? warp * VW / FV * FTILE : 0); nv > 0 && base - lane < c1;
+             base += SPREAD ? TW * FTILE : FTILE) {
+            const bool whole = nv == VW && base - lane + FTILE <= c1;
             if (whole) {
 #pragma unroll
                 for (int e = 0; e < FU; e += 2) {  // 12 loads in flight, more where registers allow
-                    vec x0[FV], x1[FV];
+                    vec x0[VW], x1[VW];
                     const long long p = base + 32 * e;
-                    const vec u0 = __ldg(ur + p), u1 = __ldg(ur + p + 32);
-                    const vec z0 = NW == 2 ? __ldg(zr + p) : u0, z1 = NW == 2 ? __ldg(zr + p + 32) : u1;
+                    const vec u0 = ur[p], u1 = ur[p + 32];
+                    const vec z0 = NW == 2 ? zr[p] : u0, z1 = NW == 2 ? zr[p + 32] : u1;
 #pragma unroll
-                    for (int gi = 0; gi < FV; ++gi) {
-                        x0[gi] = __ldg(vb + (long long)gi * vec_stride + p);
-                        x1[gi] = __ldg(vb + (long long)gi * vec_stride + p + 32);
+                    for (int gi = 0; gi < VW; ++gi) {
+                        x0[gi] = vb[(long long)gi * vec_stride + p];
+                        x1[gi] = vb[(long long)gi * vec_stride + p + 32];
                     }
                     term(u0, z0, x0);
                     term(u1, z1, x1);
@@ -178,12 +181,12 @@ __global__ void __launch_bounds__(FT, 2)
                 for (int e = 0; e < FU; ++e) {
                     const long long p = base + 32 * e;
                     if (p >= c1) break;
-                    vec x[FV];
+                    vec x[VW];
 #pragma unroll
-                    for (int gi = 0; gi < FV; ++gi)
-                        x[gi] = gi < nv ? __ldg(vb + (long long)gi * vec_stride + p) : vec{};
-                    const vec uv = __ldg(ur + p);
-                    term(uv, NW == 2 ? __ldg(zr + p) : uv, x);
+                    for (int gi = 0; gi < VW; ++gi)
+                        x[gi] = gi < nv ? vb[(long long)gi * vec_stride + p] : vec{};
+                    const vec uv = ur[p];
+                    term(uv, NW == 2 ? zr[p] : uv, x);
                 }
             }
             if (PER_TILE) {
@@ -195,21 +198,23 @@ __global__ void __launch_bounds__(FT, 2)
         }
         __syncwarp();
         if (!PER_TILE) reduce();
-        int k = lane >> SH;
-        bool out = (lane & ((1 << SH) - 1)) == 0;
+        const int k = lane >> SH;
         if (SPREAD) {
-            if (out) wsum[warp][k] = kept;
+            if ((lane & ((1 << SH) - 1)) == 0) wsum[warp][k] = kept;
             __syncthreads();
-            k = lane;
-            out = warp == 0 && lane < M;
-            if (out) {
-                kept = 0.0;
+            // the set's four vectors, over the warps that share its tiles
+            const int gi = tid / (2 * NW), kk = tid % (2 * NW), which = kk >> 1;
+            if (tid < FV * 2 * NW && q * FV + gi < J) {
+                double a = 0.0;
 #pragma unroll
-                for (int w = 0; w < FW; ++w) kept += wsum[w][k];
+                for (int w = 0; w < TW; ++w) a += VW == 1 ? wsum[gi + FV * w][kk] : wsum[w][gi * 2 * NW + kk];
+                part[(size_t)(which * J + q * FV + gi) * 2 + (kk & 1)] = a;
             }
+        } else {
+            const int gi = k / (NW * 2), which = (k >> 1) & (NW - 1);
+            if ((lane & ((1 << SH) - 1)) == 0 && gi < nv)
+                part[(size_t)(which * J + i0 + gi) * 2 + (k & 1)] = kept;
         }
-        const int gi = k / (NW * 2), which = (k >> 1) & (NW - 1);
-        if (out && gi < nv) part[(size_t)(which * J + i0 + gi) * 2 + (k & 1)] = kept;
     }
     if (g == 0) {
         __syncthreads();
@@ -279,14 +284,14 @@ __global__ void __launch_bounds__(FT, 3)
             v[2] += si.x * ti.y - si.y * ti.x;
             v[3] += hx * hx + hy * hy;
         }
-        if (block_sum4(v, sh) && lane == 0) {
+        if (block_sum4(v, sh, J) && lane == 0) {
             const double b2 = red[2 * J].x - v[0];
             const double2 uz = red[2 * J + 1];
             // a NaN (from a non-finite source) stays NaN, so that it is reported
             const double beta = (b2 > 0.0 || isnan(b2)) ? sqrt(b2) : 0.0;
-            const double hn2 = J == 0 ? 0.0 : fs.hnorm2[r] + v[3] + beta * beta;
-            const bool brk = !(beta > (J == 0 ? 0.0 : kBreakdownTol * sqrt(hn2))) || !isfinite(beta);
-            const double ib = brk ? 0.0 : 1.0 / beta;
+            const double hn2 = J == 0 ? 0.0 : fs.hnorm2[r] + v[3] + (b2 < 0.0 ? 0.0 : b2);
+            const bool brk = !(b2 > kBreakdownTol * kBreakdownTol * hn2) || !isfinite(beta);
+            const double ib = brk ? 0.0 : rsqrt(b2);  // beside the square root, not after it
             s_beta = brk ? 0.0 : beta;
             s_ib = ib;
             s_d = make_double2((uz.x - v[1]) * ib * ib, (uz.y - v[2]) * ib * ib);
@@ -398,13 +403,23 @@ __global__ void __launch_bounds__(FT, 3)
                     sum[warp % SPLIT][SPLIT == 1 ? 0 : lane + 32 * e][c][1] = b[e][c];
                 }
         }
-        __syncthreads();  // the scalars are there (and the eight sums)
+        __syncthreads();  // the scalars are there (and the eight parts of the sums)
         if (s_brk) return;  // uniform: a breakdown has no v_J
         if (SPLIT == 1) {
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 if (ok[e]) finish(base + (long long)T * e, a[e], b[e]);
         } else {
+            // the eight parts, one real number per thread, then the two results
+            R* flat = reinterpret_cast<R*>(&sum[0][0][0][0]);
+            constexpr int NV = SPLIT == 1 ? 1 : 32 * E * NC * 4;
+            for (int k = tid; k < NV; k += FT) {
+                R x = flat[k];
+#pragma unroll
+                for (int w = 1; w < SPLIT; ++w) x += flat[w * NV + k];
+                flat[k] = x;
+            }
+            __syncthreads();
             const long long p = tile * T * E + tid;
             if (tid < 32 * E && p < nunits) {
                 cplx<R> sa[NC], sb[NC];
@@ -413,17 +428,62 @@ __global__ void __launch_bounds__(FT, 3)
                 for (int c = 0; c < NC; ++c) {
                     sa[c] = sum[0][at][c][0];
                     sb[c] = sum[0][at][c][1];
-#pragma unroll
-                    for (int w = 1; w < SPLIT; ++w) {
-                        sa[c] = sa[c] + sum[w][at][c][0];
-                        sb[c] = sb[c] + sum[w][at][c][1];
-                    }
                 }
                 finish(p, sa, sb);
             }
             __syncthreads();  // the sums are overwritten by the next tile
         }
     }
+}
+
+// y += alpha sum_{i < min(J, Jdev[r])} V_i c_i, complex128: the recombination, on
+// the same split as the update.
+template <int E, int SPLIT>
+__global__ void __launch_bounds__(FT, 3)
+    k_fine_combine(const double2* __restrict__ basis, long long basis_rhs, long long vec_stride, int Jmax,
+                   const int* __restrict__ Jdev, const double2* __restrict__ coef, long long coef_stride, double alpha,
+                   double2* y, long long nunits) {
+    constexpr int T = SPLIT == 1 ? FT : 32;
+    __shared__ cd sum[SPLIT == 1 ? 1 : SPLIT][SPLIT == 1 ? 1 : 32 * E];
+    const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int J = Jdev != nullptr ? min(Jmax, Jdev[r]) : Jmax;
+    const double2* Vr = basis + r * basis_rhs;
+    const double2* cr = coef + r * coef_stride;
+    const long long base = (long long)blockIdx.x * T * E + (SPLIT == 1 ? tid : lane);
+    cd a[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) a[e] = {0.0, 0.0};
+#pragma unroll 4
+    for (int i = SPLIT == 1 ? 0 : warp; i < J; i += SPLIT) {
+        const double2 c = __ldg(cr + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const long long p = base + (long long)T * e;
+            const double2 v = p < nunits ? __ldcs(Vr + (long long)i * vec_stride + p) : make_double2(0.0, 0.0);
+            cfma(a[e], cd{v.x, v.y}, cd{alpha * c.x, alpha * c.y});
+        }
+    }
+    auto finish = [&](long long p, cd s) {
+        double2 o = y[r * nunits + p];
+        o.x += s.re;
+        o.y += s.im;
+        y[r * nunits + p] = o;
+    };
+    if (SPLIT == 1) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (base + (long long)T * e < nunits) finish(base + (long long)T * e, a[e]);
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) sum[warp % SPLIT][SPLIT == 1 ? 0 : lane + 32 * e] = a[e];
+    __syncthreads();
+    const long long p = (long long)blockIdx.x * T * E + tid;
+    if (tid >= 32 * E || p >= nunits) return;
+    cd s = sum[0][SPLIT == 1 ? 0 : tid];
+#pragma unroll
+    for (int w = 1; w < SPLIT; ++w) s = s + sum[w][SPLIT == 1 ? 0 : tid];
+    finish(p, s);
 }
 
 // Split of a sweep over J vectors: chunks of `tiles` tiles and groups of the
@@ -451,15 +511,12 @@ cudaError_t dots(const void* basis, long long basis_rhs, long long vec_stride, i
     using vec = typename Unit<R>::vec;
     const FineSplit f = fine_split(nunits, J, nrhs, num_sms);
     const dim3 grid(f.nchunk * f.vgroups, nrhs);
-    if (f.spread)
-        k_fine_dots<R, NW, true><<<grid, FT, 0, st>>>((const vec*)basis, basis_rhs, vec_stride, J, (const vec*)u,
-                                                      (const vec*)z, nunits, f.tiles, f.nchunk, f.vgroups,
-                                                      (double2*)partial, active);
-    else
-        k_fine_dots<R, NW, false><<<grid, FT, 0, st>>>((const vec*)basis, basis_rhs, vec_stride, J, (const vec*)u,
-                                                       (const vec*)z, nunits, f.tiles, f.nchunk, f.vgroups,
-                                                       (double2*)partial, active);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) {
+        kernel<<<grid, FT, 0, st>>>((const vec*)basis, basis_rhs, vec_stride, J, (const vec*)u, (const vec*)z, nunits,
+                                    f.tiles, f.nchunk, f.vgroups, (double2*)partial, active);
+        return cudaGetLastError();
+    };
+    return f.spread ? go(k_fine_dots<R, NW, true>) : go(k_fine_dots<R, NW, false>);
 }
 
 template <typename R, int E, int SPLIT>
@@ -524,6 +581,21 @@ cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long 
     if (prec == PREC_F64)
         return update<double>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
     return update<float>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
+}
+
+cudaError_t launch_fine_combine(const void* basis, long long basis_rhs, long long vec_stride, int J, const int* Jdev,
+                                const void* coef, long long coef_stride, double alpha, void* y, long long nunits,
+                                int nrhs, int num_sms, cudaStream_t st) {
+    const long long wide = (nunits + FT - 1) / FT * nrhs;
+    auto go = [&](auto kernel, long long per) {
+        kernel<<<dim3((unsigned)((nunits + per - 1) / per), nrhs), FT, 0, st>>>(
+            (const double2*)basis, basis_rhs, vec_stride, J, Jdev, (const double2*)coef, coef_stride, alpha, (double2*)y,
+            nunits);
+        return cudaGetLastError();
+    };
+    if (wide >= 4LL * num_sms) return go(k_fine_combine<2, 1>, 2 * FT);
+    if (wide >= 2LL * num_sms) return go(k_fine_combine<1, 1>, FT);
+    return go(k_fine_combine<1, 8>, 32);
 }
 
 }  // namespace ovs

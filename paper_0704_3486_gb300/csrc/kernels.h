@@ -150,6 +150,10 @@ struct FineStep {
 cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long long vec_stride, int J,
                                const void* sums, long long s_rhs, int nchunk, void* u, const void* z,
                                long long nunits, int nrhs, int num_sms, const FineStep& fs, cudaStream_t st);
+// y_r += alpha sum_{i < min(J, Jdev[r])} V_i c_i: complex128 basis and y ([nrhs][nunits])
+cudaError_t launch_fine_combine(const void* basis, long long basis_rhs, long long vec_stride, int J, const int* Jdev,
+                                const void* coef, long long coef_stride, double alpha, void* y, long long nunits,
+                                int nrhs, int num_sms, cudaStream_t st);
 // last column: H[:k][k-1] += s, H[k][k-1] = ||u - V s||
 // red[r]: s at [0, k), u^H u at entry uu_at
 cudaError_t launch_arnoldi_final(const void* red, long long red_stride, int k, int uu_at, void* H, long long h_rhs,

@@ -65,8 +65,9 @@ typedef enum {
     OVS_EIO = -8           /* file read/write failed or bad file */
 } ovs_status;
 
-/* Arithmetic of the path. OVS_F64: links, vectors and Krylov basis in
- * complex128. OVS_MIXED: links, matvec and Krylov basis in complex64 with
+/* Arithmetic of the path. OVS_F64: links and vectors in complex128, Krylov
+ * basis in 64-bit fixed point (58 bits below the largest element of each
+ * vector). OVS_MIXED: links, matvec and Krylov basis in complex64 with
  * FP64 accumulation of Gram-Schmidt inner products, FP64 Hessenberg
  * entries, FP64 deflation coefficients and FP64 Newton sign; input and
  * output vectors stay complex128. */

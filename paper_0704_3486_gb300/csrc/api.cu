@@ -232,6 +232,7 @@ static void free_kry(KryWork& k) {
     dfree(k.cstate);
     dfree(k.partial);
     dfree(k.fpcol);
+    dfree(k.vexp);
     dfree(k.norm_part);
     dfree(k.beta);
     dfree(k.inv_beta);
@@ -365,6 +366,7 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
         k.pcap = std::max<long long>(k.pcap, 2LL * g->num_sms * n * gdots_stride(1, g->m));
     CK(dalloc(&k.partial, sizeof(double2) * (size_t)k.pcap));
     CK(dalloc(&k.fpcol, sizeof(double2) * 2 * (size_t)(km + 1) * n));
+    CK(dalloc(&k.vexp, sizeof(int) * (size_t)(km + 3) * n));
     CK(dalloc(&k.norm_part, sizeof(double) * (size_t)nb * n));
     CK(dalloc(&k.beta, sizeof(double) * n));
     CK(dalloc(&k.inv_beta, sizeof(double) * n));
@@ -1097,6 +1099,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     }
     CK(cudaMemsetAsync(kw.active, 0xff, sizeof(int) * 2 * nrhs, st));  // every rhs starts active (-1 != 0)
     CK(cudaMemsetAsync(kw.est, 0, sizeof(double) * nrhs, st));
+    if (tp == PREC_F64) CK(cudaMemsetAsync(kw.vexp, 0, sizeof(int) * (size_t)(kmax + 3) * nrhs, st));
     CheckState* cstate = static_cast<CheckState*>(kw.cstate);
     const bool skip = (opts->flags & OVS_APPLY_SKIP_AHEAD) != 0;
     const int check_cap = every > 0 ? every * ((k - 1) / every) : 0;
@@ -1128,6 +1131,8 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     const long long fp_rhs = kmax + 1;
     const size_t fp_half = sizeof(double2) * (size_t)fp_rhs * nrhs;
     if (pair) TRY(pair_steps(g, nrhs, k, sh, every, check, st));
+    FixScales fx{kw.vexp, kmax + 1, nullptr, nullptr};
+    int* uexp = kw.vexp + (kmax + 1) * nrhs;
     const int* live = pair ? kw.tmask : kw.active;  // right-hand sides that reached k
     for (int j = 0; j < k && !pair; ++j) {
         const int S = gdots_stride(2, j);
@@ -1168,16 +1173,18 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
             fs.active = act;
             fs.activen = kw.active + (~j & 1) * nrhs;
             fs.k_used = kw.k_used;
+            fx.uexp = uexp + (j & 1) * nrhs;
+            fx.uexpn = uexp + (~j & 1) * nrhs;
             KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (j + 2.0),
-               launch_fine_dots(tp, 2, basis, basis_rhs_units, units, j, w.xint, w.wvec, units, nrhs, g->num_sms,
+               launch_fine_dots(tp, 2, basis, basis_rhs_units, units, j, fx, w.xint, w.wvec, units, nrhs, g->num_sms,
                                 kw.partial, act, st));
-            const int chunks = fine_chunks(units, j, nrhs, g->num_sms);
-            const bool sums = !schur && fine_sums_in_update(units, j, nrhs, g->num_sms);
+            const int chunks = fine_chunks(tp, units, j, nrhs, g->num_sms);
+            const bool sums = !schur && fine_sums_in_update(chunks, j);
             if (!sums)
                 KL(OVS_PROF_SMALL, 16.0 * chunks * S * nrhs,
                    launch_reduce(kw.partial, chunks, S, S, nrhs, kw.htmp, kw.jcap, false, act, st));
             KL(OVS_PROF_UPDATE, (double)N * sz_of(tp) * nrhs * (j + 4.0),
-               launch_fine_update(tp, basis, basis_rhs_units, units, j, sums ? kw.partial : kw.htmp,
+               launch_fine_update(tp, basis, basis_rhs_units, units, j, fx, sums ? kw.partial : kw.htmp,
                                   sums ? (long long)chunks * S : kw.jcap, sums ? chunks : 1, w.xint, w.wvec, units,
                                   nrhs, g->num_sms, fs, st));
             if (schur)  // X[:, j] = (xz - X[:, <j] s) / beta_j
@@ -1215,11 +1222,12 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         KL(OVS_PROF_SMALL, 16.0 * 2.0 * k * nrhs,
            launch_arnoldi_final(kw.htmp, kw.jcap, k, 2 * k, kw.H, h_rhs, ldh, live, nrhs, st));
     } else {
-        const int S = gdots_stride(1, k), chunks = fine_chunks(units, k, nrhs, g->num_sms);
+        const int S = gdots_stride(1, k), chunks = fine_chunks(tp, units, k, nrhs, g->num_sms);
         const int* act = kw.active + (k & 1) * nrhs;
+        fx.uexp = fx.uexpn = nullptr;
         KL(OVS_PROF_DOTS, (double)N * sz_of(tp) * nrhs * (k + 1.0),
-           launch_fine_dots(tp, 1, basis, basis_rhs_units, units, k, w.xint, nullptr, units, nrhs, g->num_sms,
-                            kw.partial, act, st));
+           launch_fine_dots(tp, 1, basis, basis_rhs_units, units, k, fx, w.xint, nullptr, units, nrhs,
+                            g->num_sms, kw.partial, act, st));
         KL(OVS_PROF_SMALL, 16.0 * chunks * S * nrhs,
            launch_reduce(kw.partial, chunks, S, S, nrhs, kw.htmp, kw.jcap, false, act, st));
         KL(OVS_PROF_SMALL, 16.0 * 2.0 * k * nrhs,
@@ -1284,8 +1292,8 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                                 nrhs, g->num_sms, nullptr, kw.err, st));
     else
         KL(OVS_PROF_PROJ, bytes_update(N, tp, PREC_F64, k, nrhs, false, true),
-           launch_fine_combine(basis, basis_rhs_units, units, k, kw.k_used, kw.coeff, kmax, 1.0, w.yacc, units, nrhs,
-                               g->num_sms, st));
+           launch_fine_combine(basis, basis_rhs_units, units, k, kw.k_used, kw.vexp, kmax + 1, kw.coeff, kmax, 1.0,
+                               w.yacc, units, nrhs, g->num_sms, st));
     if (overlap)  // D_ov(mu) x = x + gamma5 sgn(H_w) x (Sec. 2, Eq. Dov), fused into the layout pass
         KL(OVS_PROF_LAYOUT, bytes_layout(N, PREC_F64, nrhs) + 16.0 * N * nrhs,
            launch_to_canonical_overlap(w.yacc, f64, xd, N, yd, N, V, nrhs, st));
@@ -1490,9 +1498,18 @@ int ovs_get_krylov(ovs_gauge_t g, int32_t rhs, int32_t* k_out, double* V, double
         void* tmp = nullptr;
         CK(dalloc(&tmp, f64 * k));
         const char* b = (const char*)kw.basis + fb * (size_t)(kw.kmax + 1) * rhs;
-        cudaError_t e = launch_to_canonical(tp, b, fb, tmp, N, (int)g->V, k, 0);
+        void* wide = nullptr;
+        cudaError_t e = cudaSuccess;
+        if (tp == PREC_F64) {
+            e = cudaMalloc(&wide, f64 * k);
+            if (e == cudaSuccess)
+                e = launch_fix_expand(b, kw.vexp + (size_t)(kw.kmax + 1) * rhs, k, wide, field_units(N, tp), 0);
+            b = (const char*)wide;
+        }
+        if (e == cudaSuccess) e = launch_to_canonical(tp, b, fb, tmp, N, (int)g->V, k, 0);
         if (e == cudaSuccess) e = cudaMemcpy(V, tmp, f64 * k, cudaMemcpyDeviceToHost);
         cudaFree(tmp);
+        cudaFree(wide);
         CK(e);
     }
     if (H) {

@@ -1,17 +1,12 @@
 // K2 in two or three launches per Arnoldi step: the inner products, [their sums,]
-// and the rest of the step. These are the complex128 form's sweeps at every size,
-// and the complex64 form's where the lattice is too small for the TMA sweeps
-// (tma_sweeps.cu) to give every SM a share of the basis.
+// and the rest of the step. Here the complex64 form, where the lattice is too
+// small for the TMA sweeps (tma_sweeps.cu) to give every SM a share of the basis;
+// the complex128 form, on the same split, is fix_sweeps.cu.
 //
 // Split of the inner products: along the field (chunks of 128-unit tiles) and
 // along the basis (sets of four vectors). Large problems: a block takes a chunk
 // and a group of sets, a warp whole sets of the chunk. Small ones (SPREAD): a
-// block takes one set of one chunk, so that 4^4 (3,072 complex128 units) with 50
-// vectors still spreads over the chip and the partial sums stay few. An FP64
-// scheduler takes an operation of a warp every 64 clocks, so all eight warps must
-// have work: complex128, a warp takes one vector and every other tile (two busy
-// warps a block with four vectors each: 15.6 us per sweep at 4^4, now 12.5);
-// complex64, where latency counts, four vectors and every eighth tile (8^4, one
+// block takes one set of one chunk and its warps share the tiles (8^4, one
 // right-hand side: 16.8 us; with one vector per warp 20).
 //
 // Nothing is done by one block between the two: every block of the update takes
@@ -23,27 +18,22 @@
 // waiting blocks hold the registers that the running sweep's next blocks need).
 //
 // Measured, against register sweeps of 2048-unit row blocks, a reduction, the
-// scalars and the column in launches of their own (six per step, 2 blocks on
-// 4^4): FP64 4^4, k = 100: 51.2 -> 3.3 ms; 6^4, 2 right-hand sides, k = 340:
-// 547 -> 76 ms (FP64 floor 48); 8^4, 4 right-hand sides, k = 200: 194 -> 136 ms
-// (floor 105); complex64 8^4, one right-hand side, k = 200: 23.1 -> 7.8 ms.
+// scalars and the column in launches of their own (six per step): 8^4, one
+// right-hand side, k = 200: 23.1 -> 7.8 ms.
 #include <algorithm>
 
-#include "arnoldi_dev.cuh"
-#include "common.cuh"
-#include "kernels.h"
+#include "fine_dev.cuh"
 
 namespace ovs {
 
 namespace {
 
-constexpr int FT = 256, FW = FT / 32;  // threads and warps per block
-constexpr int FU = 4;                  // units per lane of a tile of 32 FU
-constexpr int FTILE = 32 * FU;
-constexpr int FV = 4;  // basis vectors per pass of a warp
+using R = float;
+using vec = Unit<R>::vec;
+constexpr int NC = Unit<R>::ncplx;
 
 // One halving exchange of the warp transpose-reduction over CUR values.
-template <int CUR, int O, typename R, int M>
+template <int CUR, int O, int M>
 __device__ __forceinline__ void halve(R (&v)[M], bool upper) {
 #pragma unroll
     for (int i = 0; i < CUR / 2; ++i) {
@@ -56,25 +46,17 @@ __device__ __forceinline__ void halve(R (&v)[M], bool upper) {
 // partial[r][chunk]: s_i = V_i^H u and (NW = 2) t_i = V_i^H z for i < J, then
 // (u^H u, 0) and u^H z.
 // A warp takes four vectors at a time and streams its block's chunk of them,
-// with u and z from L1, into 16 sums per lane: complex128 sums run over the
-// whole chunk, complex64 ones over a tile (8 terms and 32 lanes) before they
-// join FP64.
-// What bounds it: complex128, the FP64 units (8 multiply-adds per element of
-// the basis; the warp reduction adds 16 per four vectors and chunk);
-// complex64 at these sizes, latency.
-template <typename R, int NW, bool SPREAD>
+// with u and z from L1, into 16 sums per lane over a tile (8 terms and 32 lanes)
+// before they join FP64.
+// What bounds it at these sizes: latency.
+template <int NW, bool SPREAD>
 __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
-    k_fine_dots(const typename Unit<R>::vec* __restrict__ basis, long long basis_rhs, long long vec_stride, int J,
-                const typename Unit<R>::vec* __restrict__ u, const typename Unit<R>::vec* __restrict__ z,
+    k_fine_dots(const vec* __restrict__ basis, long long basis_rhs, long long vec_stride, int J,
+                const vec* __restrict__ u, const vec* __restrict__ z,
                 long long nunits, int tiles, int nchunk, int vgroups, double2* __restrict__ partial,
                 const int* __restrict__ active) {
-    using vec = typename Unit<R>::vec;
-    constexpr int NC = Unit<R>::ncplx;
-    constexpr int VW = SPREAD && sizeof(R) == 8 ? 1 : FV;  // vectors of a warp's pass
-    constexpr int TW = FW * VW / FV;                       // warps that share a set's tiles (SPREAD)
-    constexpr int M = VW * NW * 2;       // values of a pass: vector, which, component
-    constexpr int SH = M == 16 ? 1 : M == 8 ? 2 : M == 4 ? 3 : 4;  // 2^SH lanes end up with the same value
-    constexpr bool PER_TILE = sizeof(R) == 4;
+    constexpr int M = FV * NW * 2;  // values of a pass: vector, which, component
+    constexpr int SH = NW == 2 ? 1 : 2;  // 2^SH lanes end up with the same value
     __shared__ double ex[FW][3];
     __shared__ double wsum[SPREAD ? FW : 1][M];
     const int r = blockIdx.y;
@@ -118,30 +100,28 @@ __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
         }
     }
     for (int q = SPREAD ? g : g + vgroups * warp; q < nsets; q += SPREAD ? nsets : vgroups * FW) {
-        const int i0 = q * FV + (SPREAD && VW == 1 ? warp % FV : 0), nv = max(0, min(VW, J - i0));
+        const int i0 = q * FV, nv = min(FV, J - i0);
         const vec* vb = basis + r * basis_rhs + (long long)i0 * vec_stride;
         R v[M];
         double kept = 0.0;
 #pragma unroll
         for (int k = 0; k < M; ++k) v[k] = R(0);
         auto reduce = [&]() {
-            if (M >= 2) halve<M, 16>(v, (lane & 16) != 0);
-            if (M >= 4) halve<M / 2, 8>(v, (lane & 8) != 0);
-            if (M >= 8) halve<M / 4, 4>(v, (lane & 4) != 0);
-            if (M >= 16) halve<M / 8, 2>(v, (lane & 2) != 0);
-            if (M < 4) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
-            if (M < 8) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 4);
-            if (M < 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            halve<M, 16>(v, (lane & 16) != 0);
+            halve<M / 2, 8>(v, (lane & 8) != 0);
+            halve<M / 4, 4>(v, (lane & 4) != 0);
+            if (NW == 2) halve<M / 8, 2>(v, (lane & 2) != 0);
+            if (NW == 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
             v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
             kept += double(v[0]);
         };
         // one unit of u, z and the four vectors
-        auto term = [&](const vec& uv, const vec& zv, const vec (&x)[VW]) {
+        auto term = [&](const vec& uv, const vec& zv, const vec (&x)[FV]) {
             cplx<R> uc[NC], zc[NC];
             Unit<R>::split(uv, uc);
             Unit<R>::split(zv, zc);
 #pragma unroll
-            for (int gi = 0; gi < VW; ++gi) {
+            for (int gi = 0; gi < FV; ++gi) {
                 cplx<R> vc[NC];
                 Unit<R>::split(x[gi], vc);
 #pragma unroll
@@ -159,18 +139,18 @@ __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
                 }
             }
         };
-        for (long long base = c0 + lane + (SPREAD ? warp * VW / FV * FTILE : 0); nv > 0 && base - lane < c1;
-             base += SPREAD ? TW * FTILE : FTILE) {
-            const bool whole = nv == VW && base - lane + FTILE <= c1;
+        for (long long base = c0 + lane + (SPREAD ? warp * FTILE : 0); base - lane < c1;
+             base += SPREAD ? FW * FTILE : FTILE) {
+            const bool whole = nv == FV && base - lane + FTILE <= c1;
             if (whole) {
 #pragma unroll
                 for (int e = 0; e < FU; e += 2) {  // 12 loads in flight, more where registers allow
-                    vec x0[VW], x1[VW];
+                    vec x0[FV], x1[FV];
                     const long long p = base + 32 * e;
                     const vec u0 = ur[p], u1 = ur[p + 32];
                     const vec z0 = NW == 2 ? zr[p] : u0, z1 = NW == 2 ? zr[p + 32] : u1;
 #pragma unroll
-                    for (int gi = 0; gi < VW; ++gi) {
+                    for (int gi = 0; gi < FV; ++gi) {
                         x0[gi] = vb[(long long)gi * vec_stride + p];
                         x1[gi] = vb[(long long)gi * vec_stride + p + 32];
                     }
@@ -181,23 +161,19 @@ __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
                 for (int e = 0; e < FU; ++e) {
                     const long long p = base + 32 * e;
                     if (p >= c1) break;
-                    vec x[VW];
+                    vec x[FV];
 #pragma unroll
-                    for (int gi = 0; gi < VW; ++gi)
+                    for (int gi = 0; gi < FV; ++gi)
                         x[gi] = gi < nv ? vb[(long long)gi * vec_stride + p] : vec{};
                     const vec uv = ur[p];
                     term(uv, NW == 2 ? zr[p] : uv, x);
                 }
             }
-            if (PER_TILE) {
-                __syncwarp();
-                reduce();
+            __syncwarp();
+            reduce();
 #pragma unroll
-                for (int k = 0; k < M; ++k) v[k] = R(0);
-            }
+            for (int k = 0; k < M; ++k) v[k] = R(0);
         }
-        __syncwarp();
-        if (!PER_TILE) reduce();
         const int k = lane >> SH;
         if (SPREAD) {
             if ((lane & ((1 << SH) - 1)) == 0) wsum[warp][k] = kept;
@@ -207,7 +183,7 @@ __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
             if (tid < FV * 2 * NW && q * FV + gi < J) {
                 double a = 0.0;
 #pragma unroll
-                for (int w = 0; w < TW; ++w) a += VW == 1 ? wsum[gi + FV * w][kk] : wsum[w][gi * 2 * NW + kk];
+                for (int w = 0; w < FW; ++w) a += wsum[w][gi * 2 * NW + kk];
                 part[(size_t)(which * J + q * FV + gi) * 2 + (kk & 1)] = a;
             }
         } else {
@@ -235,20 +211,15 @@ __global__ void __launch_bounds__(FT, SPREAD ? 3 : 2)
 // SPLIT = 1: a thread sums its E units over all J vectors. SPLIT = 8 (small
 // fields): a block takes 32 E units, each warp every eighth vector, and the eight
 // sums meet in shared memory.
-template <typename R, int E, int SPLIT>
+template <int E, int SPLIT>
 __global__ void __launch_bounds__(FT, 3)
-    k_fine_update(typename Unit<R>::vec* basis, long long basis_rhs, long long vec_stride, int J,
-                  const double2* __restrict__ partial, long long p_rhs, int nchunk, typename Unit<R>::vec* u,
-                  const typename Unit<R>::vec* __restrict__ z, long long nunits, int nupd, FineStep fs) {
-    using vec = typename Unit<R>::vec;
-    constexpr int NC = Unit<R>::ncplx;
+    k_fine_update(vec* basis, long long basis_rhs, long long vec_stride, int J,
+                  const double2* __restrict__ partial, long long p_rhs, int nchunk, vec* u,
+                  const vec* __restrict__ z, long long nunits, int nupd, FineStep fs) {
     constexpr int T = SPLIT == 1 ? FT : 32;
-    extern __shared__ double2 red[];  // [2J + 2]: s, t, (u^H u, 0), u^H z; then (complex64) s and t as floats
+    extern __shared__ double2 red[];  // [2J + 2]: s, t, (u^H u, 0), u^H z; then s and t in complex64
     __shared__ cplx<R> sum[SPLIT == 1 ? 1 : SPLIT][SPLIT == 1 ? 1 : 32 * E][NC][2];
-    __shared__ double sh[4 * FW];
-    __shared__ double2 s_d;
-    __shared__ double s_ib, s_beta;
-    __shared__ int s_brk;
+    __shared__ StepShared sm;
     const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool first = blockIdx.x == 0;
     if (fs.active[r] == 0) {
@@ -256,79 +227,19 @@ __global__ void __launch_bounds__(FT, 3)
         return;
     }
     const int S = 2 * J + 2;
-    cplx<R>* sc = sizeof(R) == 8 ? reinterpret_cast<cplx<R>*>(red) : reinterpret_cast<cplx<R>*>(red + S);
-    {
-        const double2* all = partial + r * p_rhs;
-        for (int i = tid; i < S; i += FT) {
-            double2 a = make_double2(0.0, 0.0);
-#pragma unroll 12
-            for (int b = 0; b < nchunk; ++b) {
-                const double2 p = __ldg(all + (size_t)b * S + i);
-                a.x += p.x;
-                a.y += p.y;
-            }
-            red[i] = a;
-            if (sizeof(R) == 4 && i < 2 * J) sc[i] = {R(a.x), R(a.y)};
-        }
+    cplx<R>* sc = reinterpret_cast<cplx<R>*>(red + S);
+    for (int i = tid; i < S; i += FT) {
+        const double2 a = chunk_sum(partial + r * p_rhs, S, nchunk, i);
+        red[i] = a;
+        if (i < 2 * J) sc[i] = {R(a.x), R(a.y)};
     }
     __syncthreads();
-    const double2* fp = static_cast<const double2*>(fs.fp) + r * fs.fp_rhs;  // column J-1, first pass
-    {
-        // ||s||^2, s^H t, ||column J-1||^2 after its second pass; see arnoldi_step
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int i = tid; i < J; i += FT) {
-            const double2 si = red[i], ti = red[J + i], f = fp[i];
-            const double hx = f.x + si.x, hy = f.y + si.y;
-            v[0] += si.x * si.x + si.y * si.y;
-            v[1] += si.x * ti.x + si.y * ti.y;
-            v[2] += si.x * ti.y - si.y * ti.x;
-            v[3] += hx * hx + hy * hy;
-        }
-        if (block_sum4(v, sh, J) && lane == 0) {
-            const double b2 = red[2 * J].x - v[0];
-            const double2 uz = red[2 * J + 1];
-            // a NaN (from a non-finite source) stays NaN, so that it is reported
-            const double beta = (b2 > 0.0 || isnan(b2)) ? sqrt(b2) : 0.0;
-            const double hn2 = J == 0 ? 0.0 : fs.hnorm2[r] + v[3] + (b2 < 0.0 ? 0.0 : b2);
-            const bool brk = !(b2 > kBreakdownTol * kBreakdownTol * hn2) || !isfinite(beta);
-            const double ib = brk ? 0.0 : rsqrt(b2);  // beside the square root, not after it
-            s_beta = brk ? 0.0 : beta;
-            s_ib = ib;
-            s_d = make_double2((uz.x - v[1]) * ib * ib, (uz.y - v[2]) * ib * ib);
-            s_brk = brk ? 1 : 0;
-            if (first) {
-                if (J == 0) fs.beta0[r] = beta;
-                fs.inv_beta[r] = ib;
-                fs.hnorm2n[r] = hn2;
-                fs.activen[r] = brk ? 0 : 1;
-                fs.k_used[r] = brk ? J : J + 1;
-            }
-        }
-    }
-    if ((int)blockIdx.x >= nupd) {  // rows of column J-1 (complete) and J (first pass), one per warp
+    double v[4];
+    if (step_sums(red, red + J, J, r, fs, sm, v) && lane == 0)
+        step_scalars(v, red[2 * J].x, red[2 * J + 1], J, r, first, fs, sm);
+    if ((int)blockIdx.x >= nupd) {
         __syncthreads();
-        const int l = ((int)blockIdx.x - nupd) * FW + warp;
-        if (l > J) return;
-        double2* Hr = static_cast<double2*>(fs.H) + r * fs.h_rhs;
-        double gr = 0.0, gi = 0.0;
-        for (int i = (l > 0 ? l - 1 : 0) + lane; i < J; i += 32) {
-            double2 h;
-            if (i < J - 1) {
-                h = Hr[l + (long long)i * fs.ldh];
-            } else {  // column J-1: its second pass is s
-                h = l < J ? make_double2(fp[l].x + red[l].x, fp[l].y + red[l].y) : make_double2(s_beta, 0.0);
-                Hr[l + (long long)i * fs.ldh] = h;
-            }
-            const double2 si = red[i];
-            gr += h.x * si.x - h.y * si.y;
-            gi += h.x * si.y + h.y * si.x;
-        }
-        gr = warp_sum(gr);
-        gi = warp_sum(gi);
-        if (lane != 0 || s_brk) return;
-        double2* fpn = static_cast<double2*>(fs.fpn) + r * fs.fp_rhs;
-        fpn[l] = l < J ? make_double2((red[J + l].x - gr) * s_ib, (red[J + l].y - gi) * s_ib)
-                       : make_double2(s_d.x - gr * s_ib, s_d.y - gi * s_ib);
+        step_column(red, red + J, J, ((int)blockIdx.x - nupd) * FW + warp, r, fs, sm);
         return;
     }
     vec* Vr = basis + r * basis_rhs;
@@ -336,8 +247,8 @@ __global__ void __launch_bounds__(FT, 3)
     vec* ur = u + r * nunits;
     const vec* zr = z + r * nunits;
     auto finish = [&](long long p, const cplx<R> (&sa)[NC], const cplx<R> (&sb)[NC]) {
-        const R ib = R(s_ib);
-        const cplx<R> d = {R(s_d.x), R(s_d.y)};
+        const R ib = R(sm.ib);
+        const cplx<R> d = {R(sm.d.x), R(sm.d.y)};
         cplx<R> uc[NC], zc[NC], vo[NC], un[NC];
         Unit<R>::split(ur[p], uc);
         Unit<R>::split(__ldg(zr + p), zc);
@@ -404,7 +315,7 @@ __global__ void __launch_bounds__(FT, 3)
                 }
         }
         __syncthreads();  // the scalars are there (and the eight parts of the sums)
-        if (s_brk) return;  // uniform: a breakdown has no v_J
+        if (sm.brk) return;  // uniform: a breakdown has no v_J
         if (SPLIT == 1) {
 #pragma unroll
             for (int e = 0; e < E; ++e)
@@ -436,56 +347,6 @@ __global__ void __launch_bounds__(FT, 3)
     }
 }
 
-// y += alpha sum_{i < min(J, Jdev[r])} V_i c_i, complex128: the recombination, on
-// the same split as the update.
-template <int E, int SPLIT>
-__global__ void __launch_bounds__(FT, 3)
-    k_fine_combine(const double2* __restrict__ basis, long long basis_rhs, long long vec_stride, int Jmax,
-                   const int* __restrict__ Jdev, const double2* __restrict__ coef, long long coef_stride, double alpha,
-                   double2* y, long long nunits) {
-    constexpr int T = SPLIT == 1 ? FT : 32;
-    __shared__ cd sum[SPLIT == 1 ? 1 : SPLIT][SPLIT == 1 ? 1 : 32 * E];
-    const int r = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int J = Jdev != nullptr ? min(Jmax, Jdev[r]) : Jmax;
-    const double2* Vr = basis + r * basis_rhs;
-    const double2* cr = coef + r * coef_stride;
-    const long long base = (long long)blockIdx.x * T * E + (SPLIT == 1 ? tid : lane);
-    cd a[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) a[e] = {0.0, 0.0};
-#pragma unroll 4
-    for (int i = SPLIT == 1 ? 0 : warp; i < J; i += SPLIT) {
-        const double2 c = __ldg(cr + i);
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const long long p = base + (long long)T * e;
-            const double2 v = p < nunits ? __ldcs(Vr + (long long)i * vec_stride + p) : make_double2(0.0, 0.0);
-            cfma(a[e], cd{v.x, v.y}, cd{alpha * c.x, alpha * c.y});
-        }
-    }
-    auto finish = [&](long long p, cd s) {
-        double2 o = y[r * nunits + p];
-        o.x += s.re;
-        o.y += s.im;
-        y[r * nunits + p] = o;
-    };
-    if (SPLIT == 1) {
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            if (base + (long long)T * e < nunits) finish(base + (long long)T * e, a[e]);
-        return;
-    }
-#pragma unroll
-    for (int e = 0; e < E; ++e) sum[warp % SPLIT][SPLIT == 1 ? 0 : lane + 32 * e] = a[e];
-    __syncthreads();
-    const long long p = (long long)blockIdx.x * T * E + tid;
-    if (tid >= 32 * E || p >= nunits) return;
-    cd s = sum[0][SPLIT == 1 ? 0 : tid];
-#pragma unroll
-    for (int w = 1; w < SPLIT; ++w) s = s + sum[w][SPLIT == 1 ? 0 : tid];
-    finish(p, s);
-}
-
 // Split of a sweep over J vectors: chunks of `tiles` tiles and groups of the
 // sets of four vectors. Below 64 (tile, set) pairs per SM the blocks take one
 // set each, about two blocks per SM; every chunk more is one more partial sum to add.
@@ -505,10 +366,9 @@ FineSplit fine_split(long long nunits, int J, int nrhs, int num_sms) {
     return f;
 }
 
-template <typename R, int NW>
+template <int NW>
 cudaError_t dots(const void* basis, long long basis_rhs, long long vec_stride, int J, const void* u, const void* z,
                  long long nunits, int nrhs, int num_sms, void* partial, const int* active, cudaStream_t st) {
-    using vec = typename Unit<R>::vec;
     const FineSplit f = fine_split(nunits, J, nrhs, num_sms);
     const dim3 grid(f.nchunk * f.vgroups, nrhs);
     auto go = [&](auto kernel) {
@@ -516,17 +376,16 @@ cudaError_t dots(const void* basis, long long basis_rhs, long long vec_stride, i
                                     f.tiles, f.nchunk, f.vgroups, (double2*)partial, active);
         return cudaGetLastError();
     };
-    return f.spread ? go(k_fine_dots<R, NW, true>) : go(k_fine_dots<R, NW, false>);
+    return f.spread ? go(k_fine_dots<NW, true>) : go(k_fine_dots<NW, false>);
 }
 
-template <typename R, int E, int SPLIT>
+template <int E, int SPLIT>
 cudaError_t update_as(void* basis, long long basis_rhs, long long vec_stride, int J, const void* partial,
                       long long p_rhs, int nchunk, void* u, const void* z, long long nunits, int nrhs, int num_sms, const FineStep& fs,
                       cudaStream_t st) {
-    using vec = typename Unit<R>::vec;
-    const size_t smem = (size_t)(2 * J + 2) * sizeof(double2) + (sizeof(R) == 4 ? (size_t)2 * J * sizeof(cplx<R>) : 0);
+    const size_t smem = (size_t)(2 * J + 2) * sizeof(double2) + (size_t)2 * J * sizeof(cplx<R>);
     if (smem > 32 * 1024) {
-        const cudaError_t e = ensure_dyn_smem((const void*)k_fine_update<R, E, SPLIT>, smem);
+        const cudaError_t e = ensure_dyn_smem((const void*)k_fine_update<E, SPLIT>, smem);
         if (e != cudaSuccess) return e;
     }
     const long long per = (long long)(SPLIT == 1 ? FT : 32) * E, tiles = (nunits + per - 1) / per;
@@ -535,19 +394,18 @@ cudaError_t update_as(void* basis, long long basis_rhs, long long vec_stride, in
     const long long room = nchunk > 1 ? std::max<long long>(1, 3LL * num_sms / nrhs) : tiles;
     const long long each = (tiles + room - 1) / room;
     const int nupd = (int)((tiles + each - 1) / each);
-    k_fine_update<R, E, SPLIT><<<dim3(nupd + ncol, nrhs), FT, smem, st>>>((vec*)basis, basis_rhs, vec_stride, J,
+    k_fine_update<E, SPLIT><<<dim3(nupd + ncol, nrhs), FT, smem, st>>>((vec*)basis, basis_rhs, vec_stride, J,
                                                                          (const double2*)partial, p_rhs, nchunk, (vec*)u,
                                                                          (const vec*)z, nunits, nupd, fs);
     return cudaGetLastError();
 }
 
-template <typename R>
 cudaError_t update(void* basis, long long basis_rhs, long long vec_stride, int J, const void* partial,
                    long long p_rhs, int nchunk, void* u, const void* z, long long nunits, int nrhs, int num_sms,
                    const FineStep& fs, cudaStream_t st) {
     const long long wide = (nunits + FT - 1) / FT * nrhs;  // blocks of one unit per thread
 #define OVS_UPD(E, SPLIT)                                                                                              \
-    update_as<R, E, SPLIT>(basis, basis_rhs, vec_stride, J, partial, p_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st)
+    update_as<E, SPLIT>(basis, basis_rhs, vec_stride, J, partial, p_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st)
     if (wide >= 8LL * num_sms) return OVS_UPD(2, 1);
     if (wide >= 2LL * num_sms) return OVS_UPD(1, 1);
     if (wide * 8 > 3LL * num_sms) return OVS_UPD(2, 8);
@@ -557,45 +415,32 @@ cudaError_t update(void* basis, long long basis_rhs, long long vec_stride, int J
 
 }  // namespace
 
-int fine_chunks(long long nunits, int J, int nrhs, int num_sms) { return fine_split(nunits, J, nrhs, num_sms).nchunk; }
+int fine_chunks(int prec, long long nunits, int J, int nrhs, int num_sms) {
+    return prec == PREC_F64 ? fix_chunks(nunits, J, nrhs, num_sms) : fine_split(nunits, J, nrhs, num_sms).nchunk;
+}
 
 int fine_chunks_max(int nrhs, int num_sms) { return 2 * num_sms + nrhs; }
 
 cudaError_t launch_fine_dots(int prec, int nw, const void* basis, long long basis_rhs, long long vec_stride, int J,
-                             const void* u, const void* z, long long nunits, int nrhs, int num_sms, void* partial,
-                             const int* active, cudaStream_t st) {
+                             const FixScales& fx, const void* u, const void* z, long long nunits, int nrhs,
+                             int num_sms, void* partial, const int* active, cudaStream_t st) {
     if (prec == PREC_F64)
-        return nw == 1 ? dots<double, 1>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st)
-                       : dots<double, 2>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st);
-    return nw == 1 ? dots<float, 1>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st)
-                   : dots<float, 2>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st);
+        return launch_fix_dots(nw, basis, basis_rhs, vec_stride, J, fx.vexp, fx.vexp_rhs, fx.uexp, u, z, nunits, nrhs,
+                               num_sms, partial, active, st);
+    return nw == 1 ? dots<1>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st)
+                   : dots<2>(basis, basis_rhs, vec_stride, J, u, z, nunits, nrhs, num_sms, partial, active, st);
 }
 
-bool fine_sums_in_update(long long nunits, int J, int nrhs, int num_sms) {
-    return (long long)fine_split(nunits, J, nrhs, num_sms).nchunk * (2 * J + 2) <= 4096;
-}
+bool fine_sums_in_update(int chunks, int J) { return (long long)chunks * (2 * J + 2) <= 4096; }
 
 cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long long vec_stride, int J,
-                               const void* sums, long long s_rhs, int nchunk, void* u, const void* z,
-                               long long nunits, int nrhs, int num_sms, const FineStep& fs, cudaStream_t st) {
+                               const FixScales& fx, const void* sums, long long s_rhs, int nchunk, void* u,
+                               const void* z, long long nunits, int nrhs, int num_sms, const FineStep& fs,
+                               cudaStream_t st) {
     if (prec == PREC_F64)
-        return update<double>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
-    return update<float>(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
-}
-
-cudaError_t launch_fine_combine(const void* basis, long long basis_rhs, long long vec_stride, int J, const int* Jdev,
-                                const void* coef, long long coef_stride, double alpha, void* y, long long nunits,
-                                int nrhs, int num_sms, cudaStream_t st) {
-    const long long wide = (nunits + FT - 1) / FT * nrhs;
-    auto go = [&](auto kernel, long long per) {
-        kernel<<<dim3((unsigned)((nunits + per - 1) / per), nrhs), FT, 0, st>>>(
-            (const double2*)basis, basis_rhs, vec_stride, J, Jdev, (const double2*)coef, coef_stride, alpha, (double2*)y,
-            nunits);
-        return cudaGetLastError();
-    };
-    if (wide >= 4LL * num_sms) return go(k_fine_combine<2, 1>, 2 * FT);
-    if (wide >= 2LL * num_sms) return go(k_fine_combine<1, 1>, FT);
-    return go(k_fine_combine<1, 8>, 32);
+        return launch_fix_update(basis, basis_rhs, vec_stride, J, fx.vexp, fx.vexp_rhs, fx.uexp, fx.uexpn, sums, s_rhs,
+                                 nchunk, u, z, nunits, nrhs, num_sms, fs, st);
+    return update(basis, basis_rhs, vec_stride, J, sums, s_rhs, nchunk, u, z, nunits, nrhs, num_sms, fs, st);
 }
 
 }  // namespace ovs

@@ -22,7 +22,7 @@ struct VecWork {  // per-right-hand-side vectors
 
 struct KryWork {  // Krylov basis and small matrices
     int nrhs = 0, kmax = 0, prec = -1, jcap = 0, nblk = 0;
-    void* basis = nullptr;       // [nrhs][kmax+1][N] precision prec
+    void* basis = nullptr;       // [nrhs][kmax+1][N] precision prec (F64: fix_sweeps.cu)
     void* H = nullptr;           // [nrhs][(kmax+1) x kmax] complex128, column-major
     void* htmp = nullptr;        // [nrhs][jcap] complex128: reduced inner products of a sweep
     void* dcoef = nullptr;       // [nrhs] complex128
@@ -34,6 +34,7 @@ struct KryWork {  // Krylov basis and small matrices
     long long pcap = 0;          // complex128 entries of partial
     void* partial = nullptr;     // [max(nrhs nblk, fine_chunks_max)][jcap] complex128
     void* fpcol = nullptr;        // [2][nrhs][kmax + 1] complex128: first pass of the last column (by parity)
+    int* vexp = nullptr;          // [nrhs][kmax + 1] exponents of the basis vectors, then [2][nrhs] of u (complex128)
     double* norm_part = nullptr; // [nrhs][nblk]
     double* beta = nullptr;
     double* inv_beta = nullptr;

@@ -123,17 +123,23 @@ cudaError_t launch_arnoldi_column(const void* red, long long red_stride, int j, 
 // Partial sums of a sweep over J vectors: partial[r][c][nw J + 2] for the
 // fine_chunks() chunks c (layout of gdots_stride(nw, J)); in all at most
 // fine_chunks_max() (nw J + 2) complex128.
-int fine_chunks(long long nunits, int J, int nrhs, int num_sms);
+int fine_chunks(int prec, long long nunits, int J, int nrhs, int num_sms);
 int fine_chunks_max(int nrhs, int num_sms);  // of fine_chunks x nrhs
+// complex128: the basis is fixed point (fix_sweeps.cu), 16 bytes per element.
+struct FixScales {
+    int* vexp;  // biased exponent of the scale of each basis vector (vexp_rhs per right-hand side)
+    long long vexp_rhs;
+    int *uexp, *uexpn;  // [nrhs] exponent of the largest element of u, by parity of the step
+};                      // all zero before step 0
 cudaError_t launch_fine_dots(int prec, int nw, const void* basis, long long basis_rhs, long long vec_stride, int J,
-                             const void* u, const void* z, long long nunits, int nrhs, int num_sms, void* partial,
-                             const int* active, cudaStream_t st);
+                             const FixScales& fx, const void* u, const void* z, long long nunits, int nrhs,
+                             int num_sms, void* partial, const int* active, cudaStream_t st);
 // The rest of step J: scalars, v_J = (u - V s)/beta -> slot J, u <- (z - V t)/beta
 // - v_J d, column J-1 of H complete and the first pass of column J in fpn (that
 // of J-1 is in fp; fp_rhs complex128 per right-hand side). hnorm2 and active are
 // read from one array and written to another. The sums of right-hand side r are
 // at sums + r s_rhs: nchunk partial ones (fine_sums_in_update), or one reduced.
-bool fine_sums_in_update(long long nunits, int J, int nrhs, int num_sms);
+bool fine_sums_in_update(int chunks, int J);
 struct FineStep {
     void* H;
     long long h_rhs;
@@ -148,12 +154,15 @@ struct FineStep {
     int *activen, *k_used;
 };
 cudaError_t launch_fine_update(int prec, void* basis, long long basis_rhs, long long vec_stride, int J,
-                               const void* sums, long long s_rhs, int nchunk, void* u, const void* z,
-                               long long nunits, int nrhs, int num_sms, const FineStep& fs, cudaStream_t st);
-// y_r += alpha sum_{i < min(J, Jdev[r])} V_i c_i: complex128 basis and y ([nrhs][nunits])
+                               const FixScales& fx, const void* sums, long long s_rhs, int nchunk, void* u,
+                               const void* z, long long nunits, int nrhs, int num_sms, const FineStep& fs,
+                               cudaStream_t st);
+// n vectors of a complex128 form's basis as complex128
+cudaError_t launch_fix_expand(const void* v, const int* vexp, int n, void* out, long long nunits, cudaStream_t st);
+// y_r += alpha sum_{i < min(J, Jdev[r])} V_i c_i: complex128 form's basis, y [nrhs][nunits] complex128
 cudaError_t launch_fine_combine(const void* basis, long long basis_rhs, long long vec_stride, int J, const int* Jdev,
-                                const void* coef, long long coef_stride, double alpha, void* y, long long nunits,
-                                int nrhs, int num_sms, cudaStream_t st);
+                                const int* vexp, long long vexp_rhs, const void* coef, long long coef_stride,
+                                double alpha, void* y, long long nunits, int nrhs, int num_sms, cudaStream_t st);
 // last column: H[:k][k-1] += s, H[k][k-1] = ||u - V s||
 // red[r]: s at [0, k), u^H u at entry uu_at
 cudaError_t launch_arnoldi_final(const void* red, long long red_stride, int k, int uu_at, void* H, long long h_rhs,

@@ -299,35 +299,41 @@ __global__ void k_reduce(const double2* __restrict__ partial, int nblk, int pstr
     }
 }
 
-// The same for many blocks: a thread block takes 32 sums, each warp every
-// eighth block's part of them, so the loads of a sum run eight deep and its
-// additions spread over the FP64 units of more SMs.
+// The same for many blocks: a thread block takes 8 sums, every group of 8
+// threads one 32nd of the blocks' parts, so that the loads of a sum run 32 deep and
+// its additions spread over the FP64 units of many SMs (304 parts of 480 sums: 15
+// blocks of 32 sums with 8 groups took 11.4 us, 60 of these take 5.8).
+constexpr int RW = 8;         // sums per block
+constexpr int RG = 256 / RW;  // groups
 __global__ void __launch_bounds__(256) k_reduce_wide(const double2* __restrict__ partial, int nblk, int pstride, int J,
                                                      int nrhs, double2* __restrict__ out, long long out_stride,
                                                      int accumulate, const int* __restrict__ active) {
-    __shared__ double2 sh[8][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int idx = blockIdx.x * 32 + lane;
+    __shared__ double2 sh[RG][RW];
+    const int col = threadIdx.x % RW, g = threadIdx.x / RW;
+    const int idx = blockIdx.x * RW + col;
     const bool live = idx < J * nrhs;
     const int r = live ? idx / J : 0, i = live ? idx - r * J : 0;
     const bool on = live && (active == nullptr || active[r] != 0);
     double2 s = make_double2(0.0, 0.0);
     if (on) {
 #pragma unroll 4
-        for (int b = warp; b < nblk; b += 8) {
+        for (int b = g; b < nblk; b += RG) {
             const double2 p = partial[((size_t)r * nblk + b) * pstride + i];
             s.x += p.x;
             s.y += p.y;
         }
     }
-    sh[warp][lane] = s;
-    __syncthreads();
-    if (warp != 0 || !on) return;
+    sh[g][col] = s;
 #pragma unroll
-    for (int w = 1; w < 8; ++w) {
-        s.x += sh[w][lane].x;
-        s.y += sh[w][lane].y;
+    for (int half = RG / 2; half > 0; half /= 2) {
+        __syncthreads();
+        if (g < half) {
+            s.x += sh[g + half][col].x;
+            s.y += sh[g + half][col].y;
+            sh[g][col] = s;
+        }
     }
+    if (g != 0 || !on) return;
     double2* o = out + r * out_stride + i;
     if (accumulate) {
         const double2 v = *o;
@@ -405,9 +411,12 @@ __global__ void k_sign_scale(const double2* __restrict__ c, const double* __rest
 // vector-major with a row pitch of KD+1 units: the copies write consecutive
 // units, and the threads of a quarter warp, reading 8 consecutive vectors
 // at one unit, fall on 8 distinct 4-bank groups. Each thread accumulates a
-// tile of 4 basis vectors x 2 right-hand sides: FP32 over one staged tile
-// (2 KD complex terms), FP64 across tiles. Each element of the basis is
-// read from memory once per call, not once per right-hand side.
+// tile of 4 basis vectors x 2 right-hand sides. Where these tiles need half of
+// the threads or fewer, groups of threads share a staged tile's units (30 vectors
+// and 16 right-hand sides: 64 threads per group, 4 groups; with two of eight warps
+// at work a sweep at 8^4 took 20.6 us, now 14.5). A sum is FP32 over one staged tile
+// (2 KD complex terms) and FP64 across tiles, each sum in one thread. Each element
+// of the basis is read from memory once per call, not once per right-hand side.
 constexpr int KD = 32;
 constexpr int KP = KD + 1;  // row pitch of a staged vector, in units
 
@@ -432,13 +441,13 @@ __global__ void __launch_bounds__(BT) k_shared_dots(const float4* __restrict__ S
     const long long u0 = (long long)b * chunk;
     const long long u1 = min(u0 + chunk, nunits);
     const int itiles = (m + 3) / 4, rtiles = (nrhs + 1) / 2;
-    const int ti = tid % itiles, tr = tid / itiles;
-    const bool work = tr < rtiles;
-    double acc[4][2][2];
+    const int W = itiles * rtiles, G = BT / W;  // threads per group, groups
+    const int g = tid / W, wt = tid - g * W, ti = wt % itiles, tr = wt / itiles;
+    const bool work = g < G;
+    float2* fs = reinterpret_cast<float2*>(sd_smem + 2 * stage);  // [8][G][W]: the groups' sums of a tile
+    double2 acc[8];  // the thread's sums tid, tid + BT, ... of 8 W
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) acc[a][c][0] = acc[a][c][1] = 0.0;
+    for (int q = 0; q < 8; ++q) acc[q] = make_double2(0.0, 0.0);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     // copies of the tile at unit t0 into stage buffer st (zero beyond u1)
     auto issue = [&](long long t0, int st) {
@@ -470,7 +479,7 @@ __global__ void __launch_bounds__(BT) k_shared_dots(const float4* __restrict__ S
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) a32[a][c][0] = a32[a][c][1] = 0.f;
-            for (int u = 0; u < cnt; ++u) {
+            for (int u = g; u < cnt; u += G) {
                 float4 sv[4], zv[2];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -502,26 +511,41 @@ __global__ void __launch_bounds__(BT) k_shared_dots(const float4* __restrict__ S
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    acc[a][c][0] += (double)a32[a][c][0];
-                    acc[a][c][1] += (double)a32[a][c][1];
-                }
+                for (int c = 0; c < 2; ++c)
+                    fs[((a * 2 + c) * G + g) * W + wt] = make_float2(a32[a][c][0], a32[a][c][1]);
         }
-        __syncthreads();  // stage (t & 1) is refilled by the copies issued in the next iteration
+        // the sums are there; stage (t & 1) is refilled by the copies issued in the next iteration
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int o = tid + q * BT;
+            if (o >= 8 * W) break;
+            const float2* p = fs + (size_t)(o / W) * G * W + o % W;
+            float2 x = p[0];
+            for (int k = 1; k < G; ++k) {
+                x.x += p[(size_t)k * W].x;
+                x.y += p[(size_t)k * W].y;
+            }
+            acc[q].x += (double)x.x;
+            acc[q].y += (double)x.y;
+        }
     }
-    if (!work) return;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int i = ti + a * itiles, r = tr + c * rtiles;
-            if (i >= m || r >= nrhs) continue;
-            if (active != nullptr && active[r] == 0) continue;
-            partial[((size_t)r * nblk + b) * pstride + i] = make_double2(acc[a][c][0], acc[a][c][1]);
-        }
+    for (int q = 0; q < 8; ++q) {
+        const int o = tid + q * BT;
+        if (o >= 8 * W) break;
+        const int w = o % W, a = o / W >> 1, c = o / W & 1;
+        const int i = w % itiles + a * itiles, r = w / itiles + c * rtiles;
+        if (i >= m || r >= nrhs) continue;
+        if (active != nullptr && active[r] == 0) continue;
+        partial[((size_t)r * nblk + b) * pstride + i] = acc[q];
+    }
 }
 
-static size_t shared_dots_smem(int m, int nrhs) { return 2 * (size_t)(m + nrhs) * KP * sizeof(float4); }
+static size_t shared_dots_smem(int m, int nrhs) {
+    const int W = (m + 3) / 4 * ((nrhs + 1) / 2);
+    return 2 * (size_t)(m + nrhs) * KP * sizeof(float4) + (size_t)8 * (BT / W) * W * sizeof(float2);
+}
 
 // Blocks of the shared-basis dots for nunits within the partial slots
 // available: as many per SM as their two stages fit, at most 2 (every block is
@@ -531,7 +555,7 @@ int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms, int max_b
     const int itiles = (m + 3) / 4, rtiles = (nrhs + 1) / 2;
     if (m < 1 || nrhs < 1 || (long long)itiles * rtiles > BT) return 0;
     const size_t smem = shared_dots_smem(m, nrhs);
-    if (smem > 200 * 1024) return 0;
+    if (smem > 216 * 1024) return 0;
     const long long per_sm = std::max<long long>(1, std::min<long long>(2, (long long)(220 * 1024) / (long long)smem));
     long long want = per_sm * num_sms;
     want = std::min<long long>(want, std::max<long long>(1, nunits / KD));
@@ -543,7 +567,7 @@ cudaError_t launch_shared_dots(const void* S, long long svec, int m, const void*
                                long long nunits, int nblk, void* partial, int pstride, const int* active,
                                cudaStream_t st) {
     const size_t smem = shared_dots_smem(m, nrhs);
-    cudaError_t e = ensure_dyn_smem((const void*)k_shared_dots, 200 * 1024);
+    cudaError_t e = ensure_dyn_smem((const void*)k_shared_dots, 216 * 1024);
     if (e != cudaSuccess) return e;
     long long chunk = (nunits + nblk - 1) / nblk;
     chunk = ((chunk + KD - 1) / KD) * KD;
@@ -666,14 +690,16 @@ cudaError_t launch_update(int prec_v, int prec_out, const void* basis, long long
 // Shared-basis combination for all right-hand sides (the deflation part of
 // Sec. 5.3: x - R c and R sgn(Lambda) c, with R the complex64 copy of the
 // deflation basis): out_r = [in_r] + alpha * sum_{i < m} R_i c_{r,i}.
-// A block takes a tile of BT*2 units and a group of SG right-hand sides;
+// A block takes a tile of BT*E units and a group of SG right-hand sides;
 // blocks are numbered with the group fastest, so the SG-groups of a tile
 // run together and R is read from DRAM once and from L2 by the other
 // groups. The vector loop is unrolled by 4 (8 loads in flight per thread);
 // products are FP32, and for a complex128 output the FP32 partial sums are
 // added into FP64 accumulators every 16 vectors.
+// E = 2 where that makes four blocks per SM (608), else 1: at 8^4 with 16
+// right-hand sides 192 blocks of two units took 15.8 us, 384 of one take 11.4.
 constexpr int SG = 4;
-template <typename RO>
+template <typename RO, int E>
 __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict__ R, long long vec_stride, int m,
                                                        const double2* __restrict__ coef, long long coef_stride,
                                                        double alpha, const cplx<RO>* in, long long in_rhs_stride,
@@ -692,19 +718,19 @@ __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict_
         sc[i] = {float(alpha * c.x), float(alpha * c.y)};
     }
     __syncthreads();
-    long long u[2];
-    bool ok[2];
+    long long u[E];
+    bool ok[E];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        u[e] = tile * (2 * BT) + tid + (long long)BT * e;
+    for (int e = 0; e < E; ++e) {
+        u[e] = tile * (E * BT) + tid + (long long)BT * e;
         ok[e] = u[e] < nunits;
     }
-    cplx<RO> o[SG][2][2];
-    cf acc[SG][2][2];
+    cplx<RO> o[SG][E][2];
+    cf acc[SG][E][2];
 #pragma unroll
     for (int q = 0; q < SG; ++q)
 #pragma unroll
-        for (int e = 0; e < 2; ++e)
+        for (int e = 0; e < E; ++e)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 o[q][e][c] = {RO(0), RO(0)};
@@ -714,7 +740,7 @@ __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict_
 #pragma unroll
         for (int q = 0; q < SG; ++q)
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
+            for (int e = 0; e < E; ++e)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
                     o[q][e][c].re += RO(acc[q][e][c].re);
@@ -724,16 +750,16 @@ __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict_
     };
     int i = 0;
     for (; i + 4 <= m; i += 4) {
-        float4 v[4][2];
+        float4 v[4][E];
 #pragma unroll
         for (int d = 0; d < 4; ++d)
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
+            for (int e = 0; e < E; ++e)
                 v[d][e] = ok[e] ? __ldg(R + (long long)(i + d) * vec_stride + u[e]) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int d = 0; d < 4; ++d)
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
+            for (int e = 0; e < E; ++e) {
                 cf vc[2];
                 Unit<float>::split(v[d][e], vc);
 #pragma unroll
@@ -747,7 +773,7 @@ __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict_
     }
     for (; i < m; ++i) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
+        for (int e = 0; e < E; ++e) {
             const float4 v = ok[e] ? __ldg(R + (long long)i * vec_stride + u[e]) : make_float4(0.f, 0.f, 0.f, 0.f);
             cf vc[2];
             Unit<float>::split(v, vc);
@@ -765,7 +791,7 @@ __global__ void __launch_bounds__(BT) k_shared_combine(const float4* __restrict_
         if (q >= nr) break;
         const int r = r0 + q;
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
+        for (int e = 0; e < E; ++e) {
             if (!ok[e]) continue;
             cplx<RO> res[2];
             if (in != nullptr) OutIO<RO, 2>::load(in + (long long)r * in_rhs_stride, u[e], res);
@@ -785,19 +811,19 @@ cudaError_t launch_shared_combine(int prec_out, const void* R, long long vec_str
                                   void* out, long long out_rhs_stride, long long nunits, int nrhs, cudaStream_t st) {
     if (m < 1 || nrhs < 1) return cudaErrorInvalidValue;
     const int ngroups = (nrhs + SG - 1) / SG;
-    const long long tiles = (nunits + 2 * BT - 1) / (2 * BT);
-    const long long blocks = tiles * ngroups;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)SG * m * sizeof(cf);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
+    auto blocks = [&](int E) { return (nunits + E * BT - 1) / (E * BT) * ngroups; };
+    const int E = blocks(2) >= 608 ? 2 : 1;
+    if (blocks(E) > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    auto go = [&](auto kernel, const auto* x, auto* y) {
+        kernel<<<(unsigned)blocks(E), BT, smem, st>>>((const float4*)R, vec_stride, m, (const double2*)coef, coef_stride,
+                                                      alpha, x, in_rhs_stride, y, out_rhs_stride, nunits, nrhs, ngroups);
+    };
     if (prec_out == PREC_F64)
-        k_shared_combine<double><<<(unsigned)blocks, BT, smem, st>>>(
-            (const float4*)R, vec_stride, m, (const double2*)coef, coef_stride, alpha, (const cd*)in, in_rhs_stride,
-            (cd*)out, out_rhs_stride, nunits, nrhs, ngroups);
+        go(E == 2 ? k_shared_combine<double, 2> : k_shared_combine<double, 1>, (const cd*)in, (cd*)out);
     else
-        k_shared_combine<float><<<(unsigned)blocks, BT, smem, st>>>(
-            (const float4*)R, vec_stride, m, (const double2*)coef, coef_stride, alpha, (const cf*)in, in_rhs_stride,
-            (cf*)out, out_rhs_stride, nunits, nrhs, ngroups);
+        go(E == 2 ? k_shared_combine<float, 2> : k_shared_combine<float, 1>, (const cf*)in, (cf*)out);
     return cudaGetLastError();
 }
 
@@ -806,7 +832,7 @@ cudaError_t launch_reduce(const void* partial, int nblk, int pstride, int J, int
     if (J <= 0) return cudaSuccess;
     const int n = J * nrhs;
     if (nblk >= 16) {  // below that a sum is one batch of loads
-        k_reduce_wide<<<(n + 31) / 32, 256, 0, st>>>((const double2*)partial, nblk, pstride, J, nrhs, (double2*)out,
+        k_reduce_wide<<<(n + RW - 1) / RW, 256, 0, st>>>((const double2*)partial, nblk, pstride, J, nrhs, (double2*)out,
                                                      out_stride, accumulate ? 1 : 0, active);
         return cudaGetLastError();
     }

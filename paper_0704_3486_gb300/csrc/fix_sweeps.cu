@@ -18,7 +18,7 @@
 // 4.5e-16 for 1.1e-15).
 //
 // The basis is kept in limbs, 16 bytes per element: converting its elements in
-// every sweep took 30 of 90 instructions each (8^4: 58 ms, now 51). The scale of
+// every sweep took 30 of 90 instructions each (8^4: 58 ms, now 50). The scale of
 // v_J is known before it is computed, from max |u| (found by the inner products)
 // and ||s||. u, z, H and the results are complex128.
 //
@@ -27,7 +27,7 @@
 // one's complement with that bit set is the exact negative.
 //
 // Measured, against the same split in FP64: 8^4, 4 right-hand sides, k = 200:
-// 136 -> 51 ms; 6^4, 2, k = 340: 75.9 -> 35.5 ms; 3x5x7x9, 3, k = 75: 5.9 -> 4.4
+// 136 -> 50 ms; 6^4, 2, k = 340: 75.9 -> 35.6 ms; 3x5x7x9, 3, k = 75: 5.9 -> 4.4
 // ms; 4^4, 1, k = 100: 3.26 -> 2.83 ms. Tried without gain: the conversion of one
 // component by the FP64 unit, three or four resident blocks, four vectors per warp
 // (spills).
@@ -72,9 +72,9 @@ struct Acc {  // sum = hh 2^60 + hl 2^30
     long long hh, hl;
 };
 __device__ __forceinline__ void mul_add(Acc& a, Fix x, Fix y) {
-    a.hh += (long long)x.hi * y.hi;
-    a.hl += (long long)x.hi * y.lo;
-    a.hl += (long long)x.lo * y.hi;
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a.hh) : "r"(x.hi), "r"(y.hi));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a.hl) : "r"(x.hi), "r"(y.lo));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a.hl) : "r"(x.lo), "r"(y.hi));
 }
 __device__ __forceinline__ void carry(Acc& a) {
     a.hh += a.hl >> 30;
@@ -312,6 +312,7 @@ __device__ __forceinline__ void fix_sum(const int4* __restrict__ V, long long ve
         for (int e = 0; e < E; ++e)
 #pragma unroll
             for (int w = 0; w < NW; ++w) a[e][w][0] = a[e][w][1] = {0, 0};
+#pragma unroll 2
         for (int b = 0; b < 8 && i < JP; ++b, i += 4 * SPLIT) {
             int4 x[4][E];
 #pragma unroll

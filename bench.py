@@ -7,7 +7,7 @@ LR deflation of m = 100 critical eigenvectors (set-up timed separately),
 Krylov dimension k = 250, 16 complex Gaussian right-hand sides of unit norm.
 One step = one ovs_sign_apply of the 16 right-hand sides in the mixed form
 (complex64 links, matvec and Krylov basis; FP64 Gram-Schmidt accumulation,
-Hessenberg matrix, deflation coefficients and Newton sign). The same
+Hessenberg matrix, deflation coefficients and sign of H_k). The same
 application in plain FP64 with one right-hand side is timed beside it and
 the mixed result of that right-hand side is checked against it (relative
 2-norm <= 1e-6).
@@ -94,7 +94,7 @@ def config_of(w, world):
         "mu": w["mu"], "m_w": w["m_w"], "m_deflated": w["m"], "k": w["k"], "nrhs_per_gpu": w["nrhs"],
         "global_batch": w["nrhs"] * world,
         "precision": "complex64 links/matvec/Krylov basis; FP64 Gram-Schmidt accumulation, Hessenberg, "
-                     "deflation coefficients, Newton sign",
+                     "deflation coefficients, sign of H_k",
         "l2": "inputs larger than L2: the Krylov basis streamed every step is "
               f"{w['nrhs'] * (w['k'] + 1) * w['N'] * 8 / 1e9:.1f} GB per GPU",
         "parallelism": f"replicas x{world} (independent right-hand-side batches)",
@@ -421,12 +421,12 @@ def run_ours(args, w, world, rank, local):
     # class (16^3x32, 2 RHS, J = 30; profiles/) gave traffic / algorithmic
     # bytes; traffic grows in proportion to the vectors read, so a launch of
     # the timed step moves that ratio times its algorithmic bytes.
-    traffic_ratio = {"dots": 808.41 / 805.31, "update": 848.11 / 855.64}.get(top)
+    traffic_ratio = {"dots": 858.72 / 855.64, "update": 943.00 / 956.30}.get(top)
     per_launch = prof[top]["bytes"] / max(prof[top]["launches"], 1)
     traffic = round(per_launch * traffic_ratio) if traffic_ratio else None
     share = {c: round(prof[c]["ms"] / max(sum(p["ms"] for p in prof.values()), 1e-9), 4) for c in prof}
-    roofline = {"bound": "hbm", "kernel": {"dots": "k_gdots2_ws (CGS2 inner products)",
-                                            "update": "k_arnoldi_update_ws (CGS2 update)",
+    roofline = {"bound": "hbm", "kernel": {"dots": "k_pair_dots (CGS2 inner products, two steps per pass)",
+                                            "update": "k_pair_update (CGS2 update, two steps per pass)",
                                             "matvec": "k_wilson (H_w stencil)"}[top],
                 "achieved": round(ach, 1), "peak": peak, "unit": "GB/s", "frac": round(ach / peak, 4),
                 "peak_source": f"{peak_src} hbm_gbs (copy)", "traffic": traffic,

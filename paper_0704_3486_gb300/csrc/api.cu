@@ -648,7 +648,7 @@ int install_deflation(ovs_gauge_s* g, int m, const void* Rc, const void* Lc, con
     for (int i = 0; i < m; ++i)
         for (int j = 0; j < m; ++j) cf[(size_t)i * m + j] = std::conj(a[(size_t)i * m + j]);
     CK(cudaMemcpy(G, cf.data(), sizeof(double2) * (size_t)m * m, cudaMemcpyHostToDevice));
-    KL(OVS_PROF_UPDATE, 0.0, launch_update(PREC_F64, PREC_F64, Ltmp, 0, N, m, nullptr, G, m, 1.0, nullptr, 0, g->L64, N, N, plan, m,
+    KL(OVS_PROF_UPDATE, 0.0, launch_update(PREC_F64, PREC_F64, Ltmp, 0, N, m, G, m, 1.0, nullptr, 0, g->L64, N, N, plan, m,
                      nullptr, nullptr, 0));
     CK(cudaDeviceSynchronize());
     cudaFree(part);
@@ -1017,7 +1017,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                launch_shared_combine(PREC_F32, Sb, units, m, coef, coef_stride, -1.0, v, N, v, N, units, nrhs, st));
         else
             KL(OVS_PROF_PROJ, bytes_update(N, tp, tp, m, nrhs, true, true),
-               launch_update(tp, tp, Sb, 0, units, m, nullptr, coef, coef_stride, -1.0, v, N, v, N, units, plan, nrhs,
+               launch_update(tp, tp, Sb, 0, units, m, coef, coef_stride, -1.0, v, N, v, N, units, plan, nrhs,
                              nullptr, nullptr, st));
         return OVS_OK;
     };
@@ -1076,7 +1076,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                launch_shared_combine(PREC_F32, Rb, units, m, kw.cdef, m, -1.0, w.xint, N, w.xint, N, units, nrhs, st));
         else
             KL(OVS_PROF_PROJ, bytes_update(N, tp, tp, m, nrhs, true, true),
-               launch_update(tp, tp, Rb, 0, units, m, nullptr, kw.cdef, m, -1.0, w.xint, N, w.xint, N, units, plan,
+               launch_update(tp, tp, Rb, 0, units, m, kw.cdef, m, -1.0, w.xint, N, w.xint, N, units, plan,
                              nrhs, nullptr, nullptr, st));
         // y = R sgn(Lambda) c into the complex128 accumulator: from the FP64
         // copy of R in the FP64 form; from the complex64 copy (FP32 products,
@@ -1084,7 +1084,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         // otherwise bound it (4 DFMA per complex entry and vector)
         if (tp == PREC_F64)
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F64, PREC_F64, m, nrhs, true, false),
-               launch_update(PREC_F64, PREC_F64, g->R64, 0, N, m, nullptr, kw.cdef2, m, 1.0, nullptr, 0, w.yacc, N, N,
+               launch_update(PREC_F64, PREC_F64, g->R64, 0, N, m, kw.cdef2, m, 1.0, nullptr, 0, w.yacc, N, N,
                              plan64, nrhs, nullptr, nullptr, st));
         else if (m <= 1536)
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F32, PREC_F64, m, nrhs, true, false),
@@ -1092,7 +1092,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                                      st));
         else
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F32, PREC_F64, m, nrhs, true, false),
-               launch_update(PREC_F32, PREC_F64, g->R32, 0, units, m, nullptr, kw.cdef2, m, 1.0, nullptr, 0, w.yacc,
+               launch_update(PREC_F32, PREC_F64, g->R32, 0, units, m, kw.cdef2, m, 1.0, nullptr, 0, w.yacc,
                              N, units, plan, nrhs, nullptr, nullptr, st));
     } else {
         CK(cudaMemsetAsync(w.yacc, 0, f64 * nrhs, st));
@@ -1272,7 +1272,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                               kw.k_used, kw.status, kw.beta, kw.cdef, m, kw.sylv, kw.cS, m, nrhs, k, st, need));
         if (tp == PREC_F64)
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F64, PREC_F64, m, nrhs, true, false),
-               launch_update(PREC_F64, PREC_F64, g->R64, 0, N, m, nullptr, kw.cS, m, 1.0, nullptr, 0, w.yacc, N, N,
+               launch_update(PREC_F64, PREC_F64, g->R64, 0, N, m, kw.cS, m, 1.0, nullptr, 0, w.yacc, N, N,
                              plan64, nrhs, nullptr, nullptr, st));
         else if (m <= 1536)
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F32, PREC_F64, m, nrhs, true, false),
@@ -1280,7 +1280,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
                                      st));
         else
             KL(OVS_PROF_PROJ, bytes_update(N, PREC_F32, PREC_F64, m, nrhs, true, false),
-               launch_update(PREC_F32, PREC_F64, g->R32, 0, units, m, nullptr, kw.cS, m, 1.0, nullptr, 0, w.yacc,
+               launch_update(PREC_F32, PREC_F64, g->R32, 0, units, m, kw.cS, m, 1.0, nullptr, 0, w.yacc,
                              N, units, plan, nrhs, nullptr, nullptr, st));
     } else {
         TRY(sign_column(kw.coeff, every > 0 ? kw.due : nullptr, 0));
@@ -1427,7 +1427,7 @@ int ovs_overlap_solve(ovs_gauge_t g, const void* b, void* x, int32_t nrhs, const
                 void* red = pass ? red2 : red1;
                 CK(launch_gdots(PREC_F64, W, N, (long long)nrhs * N, j + 1, z, N, N, plan, nrhs, part, nullptr, st));
                 CK(launch_reduce(part, plan.nblk, gdots_stride(1, j + 1), j + 1, nrhs, red, jc, false, nullptr, st));
-                CK(launch_update(PREC_F64, PREC_F64, W, N, (long long)nrhs * N, j + 1, nullptr, red, jc, -1.0, z, N, z,
+                CK(launch_update(PREC_F64, PREC_F64, W, N, (long long)nrhs * N, j + 1, red, jc, -1.0, z, N, z,
                                  N, N, plan, nrhs, nullptr, nullptr, st));
             }
             CK(launch_norm_partials(z, N, N, nrhs, npart, st));
@@ -1446,7 +1446,7 @@ int ovs_overlap_solve(ovs_gauge_t g, const void* b, void* x, int32_t nrhs, const
         }
         // x += W y with y = R^-1 g; true residual r = b - D_ov x
         CK(launch_gmres_backsub(R, gv, jj, restart, yv, nrhs, st));
-        CK(launch_update(PREC_F64, PREC_F64, W, N, (long long)nrhs * N, jj, nullptr, yv, restart, 1.0, xd, N, xd, N, N,
+        CK(launch_update(PREC_F64, PREC_F64, W, N, (long long)nrhs * N, jj, yv, restart, 1.0, xd, N, xd, N, N,
                          plan, nrhs, nullptr, nullptr, st));
         TRY(sign_apply_core(g, xd, z, nrhs, inner, st, true));
         CK(launch_sub(bd, z, r, N, nrhs, st));

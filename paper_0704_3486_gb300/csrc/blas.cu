@@ -7,8 +7,8 @@
 // sweeps here a block of 256 threads covers one row block of one
 // right-hand side and streams every basis vector through it, so the basis
 // is read once per sweep with fully coalesced 16-byte loads. They serve the
-// projections, the complex128 recombination and the outer GMRES; the Arnoldi
-// sweeps are in fine_sweeps.cu and tma_sweeps.cu.
+// projections and the outer GMRES; the Arnoldi sweeps are in
+// fix_sweeps.cu, fine_sweeps.cu, tma_sweeps.cu and pair_sweeps.cu.
 // Also here: the shared-basis combination of the deflated part
 // (k_shared_combine) and the small kernels of each Arnoldi step (partial
 // sums, Hessenberg column, final pass).
@@ -57,8 +57,7 @@ template <typename R, int M> __device__ __forceinline__ void transpose_reduce(R 
 // Inner products of one basis sweep, per right-hand side r and row block b:
 // s_i = V_i^H u (i < J), output partial[r][b][S], S = J + 2 (the last two
 // entries are not written). Serves the projections, the set-up and the outer
-// GMRES; the Arnoldi steps have their own sweeps (fine_sweeps.cu,
-// tma_sweeps.cu).
+// GMRES; the Arnoldi steps have their own sweeps.
 // A lane keeps E 16-byte units of u in registers (a tile of 256*E units per
 // block); G basis vectors are then streamed past them. Each lane accumulates
 // its E*NC products per vector in FP32 (FP64 for complex128 fields), a warp
@@ -177,12 +176,12 @@ template <> struct OutIO<float, 2> {
     }
 };
 
-// out_r = in_r + sum_{i<J_r} V_r,i * (alpha c_r,i). Strides of in/out are in
+// out_r = in_r + sum_{i<J} V_r,i * (alpha c_r,i). Strides of in/out are in
 // complex numbers of precision RO; basis strides in units.
 template <typename RV, typename RO, int E>
 __global__ void __launch_bounds__(BT) k_update(const typename Unit<RV>::vec* __restrict__ basis,
                                                long long basis_rhs_stride, long long vec_stride, int J,
-                                               const int* __restrict__ Jdev, const double2* __restrict__ coef,
+                                               const double2* __restrict__ coef,
                                                long long coef_stride, double alpha, const cplx<RO>* in,
                                                long long in_rhs_stride, cplx<RO>* out, long long out_rhs_stride,
                                                long long nunits, long long chunk, int nblk,
@@ -194,10 +193,8 @@ __global__ void __launch_bounds__(BT) k_update(const typename Unit<RV>::vec* __r
     __shared__ double sred[NWARP];
     const int r = blockIdx.x, b = blockIdx.y;
     if (active != nullptr && active[r] == 0) return;
-    int Jr = J;
-    if (Jdev != nullptr) Jr = min(J, Jdev[r]);
     const int tid = threadIdx.x;
-    for (int i = tid; i < Jr; i += BT) {
+    for (int i = tid; i < J; i += BT) {
         double2 c = coef[r * coef_stride + i];
         scoef[i] = {RV(alpha * c.x), RV(alpha * c.y)};
     }
@@ -224,7 +221,7 @@ __global__ void __launch_bounds__(BT) k_update(const typename Unit<RV>::vec* __r
             if (ok[e] && inr != nullptr) OutIO<RO, NC>::load(inr, u, o[e]);
         }
         int since_flush = 0;
-        for (int i = 0; i < Jr; ++i) {
+        for (int i = 0; i < J; ++i) {
             const cplx<RV> ci = scoef[i];
             const vec* vi = Vr + (long long)i * vec_stride;
 #pragma unroll
@@ -659,7 +656,7 @@ cudaError_t launch_arnoldi_final(const void* red, long long red_stride, int k, i
 }
 
 cudaError_t launch_update(int prec_v, int prec_out, const void* basis, long long basis_rhs_stride,
-                          long long vec_stride, int J, const int* Jdev, const void* coef, long long coef_stride,
+                          long long vec_stride, int J, const void* coef, long long coef_stride,
                           double alpha, const void* in, long long in_rhs_stride, void* out, long long out_rhs_stride,
                           long long nunits_v, const BlasPlan& plan, int nrhs, double* norm_partial,
                           const int* active, cudaStream_t st) {
@@ -668,17 +665,17 @@ cudaError_t launch_update(int prec_v, int prec_out, const void* basis, long long
     size_t smem = (size_t)std::max(J, 1) * sizeof(double2);
     if (prec_v == PREC_F64 && prec_out == PREC_F64) {
         k_update<double, double, 2><<<grid, BT, smem, st>>>(
-            (const double2*)basis, basis_rhs_stride, vec_stride, J, Jdev, (const double2*)coef, coef_stride, alpha,
+            (const double2*)basis, basis_rhs_stride, vec_stride, J, (const double2*)coef, coef_stride, alpha,
             (const cd*)in, in_rhs_stride, (cd*)out, out_rhs_stride, nunits_v, plan.chunk, plan.nblk, norm_partial,
             active);
     } else if (prec_v == PREC_F32 && prec_out == PREC_F32) {
         k_update<float, float, 2><<<grid, BT, smem, st>>>(
-            (const float4*)basis, basis_rhs_stride, vec_stride, J, Jdev, (const double2*)coef, coef_stride, alpha,
+            (const float4*)basis, basis_rhs_stride, vec_stride, J, (const double2*)coef, coef_stride, alpha,
             (const cf*)in, in_rhs_stride, (cf*)out, out_rhs_stride, nunits_v, plan.chunk, plan.nblk, norm_partial,
             active);
     } else if (prec_v == PREC_F32 && prec_out == PREC_F64) {
         k_update<float, double, 2><<<grid, BT, smem, st>>>(
-            (const float4*)basis, basis_rhs_stride, vec_stride, J, Jdev, (const double2*)coef, coef_stride, alpha,
+            (const float4*)basis, basis_rhs_stride, vec_stride, J, (const double2*)coef, coef_stride, alpha,
             (const cd*)in, in_rhs_stride, (cd*)out, out_rhs_stride, nunits_v, plan.chunk, plan.nblk, norm_partial,
             active);
     } else {

@@ -82,13 +82,12 @@ cudaError_t launch_gdots(int prec, const void* basis, long long basis_rhs_stride
                          const void* u, long long u_rhs_stride, long long nunits, const BlasPlan& plan, int nrhs,
                          void* partial, const int* active, cudaStream_t st);
 
-// out_r = in_r + alpha * sum_{i<J_r} V_r,i c_r,i   (coef: complex128 [r][coef_stride])
-// J_r = J (host) or Jdev[r] (device, if Jdev != nullptr, clamped to J).
+// out_r = in_r + alpha * sum_{i<J} V_r,i c_r,i   (coef: complex128 [r][coef_stride])
 // out precision: prec_out (F64: complex128 units, F32: complex64 pairs). in may
 // be nullptr (zero) or equal to out. If norm_partial != nullptr, also
 // writes sum |out|^2 per block to norm_partial[r][b].
 cudaError_t launch_update(int prec_v, int prec_out, const void* basis, long long basis_rhs_stride,
-                          long long vec_stride, int J, const int* Jdev, const void* coef, long long coef_stride,
+                          long long vec_stride, int J, const void* coef, long long coef_stride,
                           double alpha, const void* in, long long in_rhs_stride, void* out, long long out_rhs_stride,
                           long long nunits_v, const BlasPlan& plan, int nrhs, double* norm_partial,
                           const int* active, cudaStream_t st);

@@ -355,7 +355,7 @@ int install_schur(ovs_gauge_s* g, int m, const void* Rc) {
         for (int r = 0; r < m; ++r)
             for (int i = 0; i < m; ++i) cf[(size_t)r * m + i] = uinv[(size_t)i * m + r];
         SCK(cudaMemcpy(G.p, cf.data(), sizeof(double2) * (size_t)m * m, cudaMemcpyHostToDevice));
-        SCK(launch_update(PREC_F64, PREC_F64, a.p, 0, N, m, nullptr, G.p, m, 1.0, nullptr, 0, b.p, N, N, plan, m,
+        SCK(launch_update(PREC_F64, PREC_F64, a.p, 0, N, m, G.p, m, 1.0, nullptr, 0, b.p, N, N, plan, m,
                           nullptr, nullptr, st));
         std::swap(a.p, b.p);
     }

@@ -605,6 +605,11 @@ static inline dim3 site_grid(int V, int nrhs, int threads) { return dim3((V + th
 // 8 groups 36 and 14 us, 90 37 and 16, 512 39 and 56; complex64 128 groups 9.2
 // and 9.5 us.
 template <typename R> constexpr long long kSplitGroups = sizeof(R) == 8 ? 256 : 96;
+// The same where it also replaces the two layout passes (canonical vectors on both
+// sides). Measured, three launches and one: complex64 128 groups 14.4 and 10.4 us,
+// 164 14.4 and 14.4 (H_w^2 20.6 and 24.7); FP64 384 groups 43.1 and 41.1 us (77.9
+// and 82.1), 512 44.9 and 51.4.
+template <typename R> constexpr long long kSplitCanonical = sizeof(R) == 8 ? 256 : 144;
 
 static bool valid_shape(const StencilShape& sh) {
     for (int i = 0; i < kNumStencilShapes; ++i)
@@ -682,7 +687,7 @@ cudaError_t launch_wilson_axpy(int prec, const void* links, const void* in, size
 }
 
 bool wilson_spread(int prec, const Geom& g, int nrhs) {
-    return (long long)((g.V + 31) / 32) * nrhs <= (prec == PREC_F64 ? kSplitGroups<double> : kSplitGroups<float>);
+    return (long long)((g.V + 31) / 32) * nrhs <= (prec == PREC_F64 ? kSplitCanonical<double> : kSplitCanonical<float>);
 }
 
 cudaError_t launch_wilson_canonical(int prec, bool gamma5, const void* links, const void* in, size_t in_stride,

@@ -41,7 +41,7 @@ def test_sign_matches_oracle(gpu, dims, nrhs, k):
     g.destroy()
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 3, 5, 3), (4, 4, 4, 4), (2, 6, 3, 5)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 3, 5, 3), (4, 4, 4, 4), (2, 6, 3, 5), (8, 8, 8, 8), (9, 8, 8, 8)])
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("op", [0, 1, 2])
 def test_spread_stencil_is_bit_identical(gpu, dims, prec, op):

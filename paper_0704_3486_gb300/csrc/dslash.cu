@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -598,6 +599,130 @@ __global__ void k_links_to_canonical(const double2* __restrict__ u64, double2* _
 }
 
 // ------------------------------------------------------------- host launch
+// The complex128 stencil by two threads per site. A scheduler takes an FP64
+// operation of a warp every 64 clocks, so the 936 operations of a site in one
+// thread are 31 us however small the field, and a field that fills the chip
+// unevenly pays a whole such wave for the rest. Thread `half` takes component
+// half of the half-spinor of every hop: one spin and its partner of the neighbour,
+// one upper spin of the sum, and the lower spin that this component goes to in x
+// and y; for z and t it is the other thread's, so the two exchange their lower
+// sums between y and z. Every entry is summed in the order of k_wilson (the same
+// bits). The two halves are warps of a block (no divergence).
+// Measured, k_wilson and this: see the rule in wilson_dispatch.
+template <int NU, bool FWD, int HALF>
+__device__ __forceinline__ void half_hop(const void* links, const char* in, const Geom& g, int s, int coord,
+                                         double efwd, double ebwd, cd (&up)[3], cd (&lo)[3]) {
+    const int L = g.L[NU], st = g.stride[NU];
+    int sn;
+    double fac;
+    cd U[9];
+    if (FWD) {
+        sn = (coord == L - 1) ? s - (L - 1) * st : s + st;
+        fac = (NU == 3 && coord == L - 1) ? -efwd : efwd;
+        Field<double>::link(links, g.V, NU, s, U);
+    } else {
+        sn = (coord == 0) ? s + (L - 1) * st : s - st;
+        fac = (NU == 3 && coord == 0) ? -ebwd : ebwd;
+        Field<double>::link(links, g.V, NU, sn, U);
+    }
+    constexpr int P = NU < 2 ? 3 - HALF : 2 + HALF;  // the partner spin
+    const double2* d = reinterpret_cast<const double2*>(in);
+    cd h[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int e = 3 * HALF + c, q = 3 * P + c;
+        const double2 av = __ldg(d + 2 * ((size_t)(e >> 1) * g.V + sn) + (e & 1));
+        const double2 bv = __ldg(d + 2 * ((size_t)(q >> 1) * g.V + sn) + (q & 1));
+        const cd a = {av.x, av.y}, b = {bv.x, bv.y};
+        if (NU == 0) h[c] = FWD ? a + ti(b) : a + tmi(b);
+        if (NU == 1) h[c] = FWD == (HALF == 0) ? a + b : a - b;
+        if (NU == 2) h[c] = FWD == (HALF == 0) ? a + ti(b) : a + tmi(b);
+        if (NU == 3) h[c] = FWD ? a - b : a + b;
+        if (NU == 3) h[c] = h[c] * fac;  // 1 on spatial hops
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        cd u = {0.0, 0.0};
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (FWD)
+                cfma(u, U[3 * a + b], h[b]);
+            else
+                cfmac(u, U[3 * b + a], h[b]);
+        }
+        up[a] = up[a] + u;
+        if (NU == 0) lo[a] = FWD ? lo[a] + tmi(u) : lo[a] + ti(u);
+        if (NU == 1) lo[a] = FWD == (HALF == 0) ? lo[a] + u : lo[a] - u;
+        if (NU == 2) lo[a] = FWD == (HALF == 0) ? lo[a] + tmi(u) : lo[a] + ti(u);
+        if (NU == 3) lo[a] = FWD ? lo[a] - u : lo[a] + u;
+    }
+}
+
+template <bool G5>
+__global__ void __launch_bounds__(512) k_wilson_half(const void* __restrict__ links, const char* __restrict__ in,
+                                                     char* out, size_t in_stride, size_t out_stride, Geom g,
+                                                     double kappa, double emu, double emmu, int nrhs, int ntiles,
+                                                     const int* __restrict__ active) {
+    __shared__ cd swap[2][3][256];
+    const int tile = blockIdx.x % ntiles, sites = 16 * blockDim.y;
+    const int half = threadIdx.y & 1, slot = (threadIdx.y >> 1) * 32 + threadIdx.x;
+    const int s0 = (blockIdx.x / ntiles) * sites + slot, s = min(s0, g.V - 1);
+    const int r = tile * blockDim.z + threadIdx.z, sl = threadIdx.z * sites + slot;
+    const bool live = r < nrhs && (active == nullptr || active[r] != 0);
+    const char* ir = in + (size_t)min(r, nrhs - 1) * in_stride;
+    int c = s;
+    const int x = c % g.L[0]; c /= g.L[0];
+    const int y = c % g.L[1]; c /= g.L[1];
+    const int z = c % g.L[2];
+    const int t = c / g.L[2];
+    cd up[3], lo[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) up[a] = lo[a] = {0.0, 0.0};
+    auto xy = [&](auto h) {
+        constexpr int H = decltype(h)::value;
+        half_hop<0, true, H>(links, ir, g, s, x, 1.0, 1.0, up, lo);
+        half_hop<0, false, H>(links, ir, g, s, x, 1.0, 1.0, up, lo);
+        half_hop<1, true, H>(links, ir, g, s, y, 1.0, 1.0, up, lo);
+        half_hop<1, false, H>(links, ir, g, s, y, 1.0, 1.0, up, lo);
+    };
+    auto zt = [&](auto h) {
+        constexpr int H = decltype(h)::value;
+        half_hop<2, true, H>(links, ir, g, s, z, 1.0, 1.0, up, lo);
+        half_hop<2, false, H>(links, ir, g, s, z, 1.0, 1.0, up, lo);
+        half_hop<3, true, H>(links, ir, g, s, t, emu, emmu, up, lo);
+        half_hop<3, false, H>(links, ir, g, s, t, emu, emmu, up, lo);
+        // own entries: spin H and, after the exchange, spin 2 + H
+        if (s0 >= g.V) return;
+        const double2* d = reinterpret_cast<const double2*>(ir);
+        double2* o = reinterpret_cast<double2*>(out + (size_t)r * out_stride);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int e = k < 3 ? 3 * H + k : 6 + 3 * H + k - 3;
+            const size_t at = 2 * ((size_t)(e >> 1) * g.V + s) + (e & 1);
+            const double2 pv = __ldg(d + at);
+            cd v = cd{pv.x, pv.y} - (k < 3 ? up[k % 3] : lo[k % 3]) * kappa;
+            if (G5 && e >= 6) v = -v;
+            o[at] = make_double2(v.re, v.im);
+        }
+    };
+    if (live) {
+        if (half == 0)
+            xy(std::integral_constant<int, 0>{});
+        else
+            xy(std::integral_constant<int, 1>{});
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) swap[half][a][sl] = lo[a];
+    __syncthreads();
+    if (!live) return;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) lo[a] = swap[1 - half][a][sl];
+    if (half == 0)
+        zt(std::integral_constant<int, 0>{});
+    else
+        zt(std::integral_constant<int, 1>{});
+}
+
 static inline dim3 site_grid(int V, int nrhs, int threads) { return dim3((V + threads - 1) / threads, nrhs); }
 
 // Groups of 32 sites and right-hand sides up to which the stencil is spread
@@ -610,6 +735,17 @@ template <typename R> constexpr long long kSplitGroups = sizeof(R) == 8 ? 256 : 
 // 164 14.4 and 14.4 (H_w^2 20.6 and 24.7); FP64 384 groups 43.1 and 41.1 us (77.9
 // and 82.1), 512 44.9 and 51.4.
 template <typename R> constexpr long long kSplitCanonical = sizeof(R) == 8 ? 256 : 144;
+
+// Where the complex128 stencil takes two threads per site (k_wilson_half): the
+// warps of 32 sites fill the 608 FP64 schedulers (152 SMs) less than once, or half
+// warps fill them in fewer half waves. Measured per H_w with both layout passes,
+// k_wilson and half: 384 warps 44.6 and 37.0 us, 512 45.2 and 43.2, 640 61.5 and
+// 54.5, 1280 98.5 and 90.2, 2592 178.9 and 164.0; where the half waves are as many
+// (1024) 71.8 and 75.3, (16384) 926.7 and 928.5.
+static bool two_threads_per_site(long long warps) {
+    constexpr long long n = 608;
+    return warps <= n || (2 * warps + n - 1) / n < 2 * ((warps + n - 1) / n);
+}
 
 static bool valid_shape(const StencilShape& sh) {
     for (int i = 0; i < kNumStencilShapes; ++i)
@@ -630,6 +766,13 @@ static void wilson_dispatch(const StencilShape& sh, unsigned blocks, int ntiles,
         k_wilson_split<R, G5, AX, false, false><<<dim3((unsigned)(8 * groups), nrhs), 96, 0, st>>>(links, i, o, in_stride, out_stride,
                                                                                     g, k, e1, e2, active, ax);
         return;
+    }
+    if constexpr (sizeof(R) == 8 && AX == 0) {
+        if (sh.rt == 1 && two_threads_per_site(groups * nrhs)) {
+            k_wilson_half<G5><<<blocks, dim3(32, sh.sites / 16, sh.rb), 0, st>>>(links, i, o, in_stride, out_stride, g,
+                                                                               kappa, emu, emmu, nrhs, ntiles, active);
+            return;
+        }
     }
     const dim3 block(sh.sites, sh.rb);
     if (sh.rt == 1)

@@ -57,3 +57,23 @@ def test_spread_stencil_is_bit_identical(gpu, dims, prec, op):
         gpu.matvec(g, op, x[r:r + 1].contiguous(), one, prec=prec)
         assert torch.equal(one[0], many[r])
     g.destroy()
+
+
+@pytest.mark.parametrize("dims,nrhs", [((8, 8, 8, 9), 2), ((9, 9, 9, 9), 2), ((5, 7, 9, 11), 6), ((8, 8, 8, 8), 5)])
+@pytest.mark.parametrize("op", [0, 1, 2])
+def test_two_threads_per_site_is_bit_identical(gpu, dims, nrhs, op):
+    """complex128 by two threads per site (288, 412, 654, 640 groups of 32 sites)
+    against two right-hand sides per thread (k_wilson)."""
+    links = synth.gauge_links(dims, 3, 0.6)
+    g = gpu.create_gauge_from_links(dims, links, gpu.F64)
+    gpu.set_mu(g, 0.2, -1.5)
+    x = torch.from_numpy(synth.gaussian_vectors(12 * int(np.prod(dims)), nrhs, 5)).cuda()
+    ref, y = torch.empty_like(x), torch.empty_like(x)
+    gpu.set_stencil_shape(g, gpu.F64, nrhs, (2, 32, 1))
+    gpu.matvec(g, op, x, ref, prec=gpu.F64)
+    for sites, rb in ((32, 1), (32, 8), (64, 4), (128, 2)):
+        gpu.set_stencil_shape(g, gpu.F64, nrhs, (1, sites, rb))
+        y.zero_()
+        gpu.matvec(g, op, x, y, prec=gpu.F64)
+        assert torch.equal(y, ref), (sites, rb)
+    g.destroy()

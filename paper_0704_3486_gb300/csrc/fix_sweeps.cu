@@ -10,21 +10,26 @@
 //     x = hi 2^30 + lo,  |hi| <= 2^28,  |lo| <= 2^29,
 // and a product takes three of the four limb products, summed exactly in 64
 // bits: hi hi (at most 64 products of a lane: 2^62) and hi lo + lo hi (32
-// products: 2^62, then carried). What is dropped is lo lo, 2^-60 of the product
-// of the two largest elements and of random sign, and the rounding of the
-// operands, 2^-59 of the largest element; an FP64 sum rounds each partial sum by
-// 2^-54. The results' error against 64 bits is smaller than that of the FP64
-// sweeps (4^4 5.0e-16 for 7.2e-16, 8^4 8.0e-16 for 1.1e-15, 6^4 with k = 340
-// 4.5e-16 for 1.1e-15).
+// products: 2^62, then carried). What is dropped is lo lo, at most 2^-58 of the
+// product of the two scales and of random sign (in u^H u a square: of 1024 units' sum
+// at most 2^-47 of the largest element's square), and the rounding of the operands
+// to a unit, 2^-58 of the scale (which is one to two times the largest element, of a
+// basis vector up to four times), within three quarters; zeros stay zeros. An FP64 sum rounds
+// each partial sum by 2^-54. The results' error against 64 bits is smaller than that
+// of the FP64 sweeps on Gaussian sources (4^4 5.0e-16 for 7.2e-16, 8^4 8.0e-16 for
+// 1.1e-15, 6^4 with k = 340 4.5e-16 for 1.1e-15) and like it on point sources (k = 40,
+// restated on the CPU against long double: 8^4 7.0e-16 for 9.1e-16, 12^4 4.0e-16 for
+// 3.7e-16; with the last bit set instead of a rounding, zeros included, 2.8e-15 and
+// 5.5e-15).
 //
 // The basis is kept in limbs, 16 bytes per element: converting its elements in
 // every sweep took 30 of 90 instructions each (8^4: 58 ms, now 50). The scale of
 // v_J is known before it is computed, from max |u| (found by the inner products)
 // and ||s||. u, z, H and the results are complex128.
 //
-// Conversion: the mantissa shifted by the difference of the exponents; the last
-// bit is set, which is the middle of the truncated interval (no bias), and its
-// one's complement with that bit set is the exact negative.
+// Conversion: the mantissa shifted by the difference of the exponents to two bits more
+// than a number has, negated for a negative value, plus half a unit; the two bits go.
+// An exponent of 0 (a zero; a subnormal is far below any scale in use) gives 0.
 //
 // Measured, against the same split in FP64: 8^4, 4 right-hand sides, k = 200:
 // 136 -> 50 ms; 6^4, 2, k = 340: 75.9 -> 35.6 ms; 3x5x7x9, 3, k = 75: 5.9 -> 4.4
@@ -46,18 +51,18 @@ constexpr int kNonFinite = 1 << 20;
 struct Fix {
     int hi, lo;
 };
-// v 2^(1022 - e) 2^58 rounded, for a biased exponent e not below v's own
+// v 2^(1022 - e) 2^58 to a whole number, within 3/4, for a biased exponent e not below
+// v's own
 __device__ __forceinline__ Fix to_fix(double v, int e) {
     const int h = __double2hiint(v);
     const unsigned l = (unsigned)__double2loint(v);
-    const int d = e - ((h >> 20) & 0x7ff);
+    const int ev = (h >> 20) & 0x7ff, d = e - ev;
     const unsigned mh = (__funnelshift_l(l, (unsigned)h, 7) & 0x07ffffffu) | 0x08000000u;
-    unsigned long long m = ((unsigned long long)mh << 32) | (l << 7);
+    unsigned long long m = ev != 0 ? ((unsigned long long)mh << 32) | (l << 7) : 0ull;
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));  // shifts above 64 give 0
-    const int s = h >> 31;
-    const int yh = (int)(m >> 32) ^ s;
-    const unsigned yl = ((unsigned)m ^ (unsigned)s) | 4u;
-    return {yh + (int)(yl >> 31), (int)yl >> 2};
+    const long long y = (h < 0 ? -(long long)m : (long long)m) + 2;
+    const unsigned yl = (unsigned)y;
+    return {(int)(y >> 32) + (int)(yl >> 31), (int)yl >> 2};
 }
 __device__ __forceinline__ unsigned abs_hi(double2 v) {
     return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
@@ -285,9 +290,7 @@ __device__ __forceinline__ int coef_exponent(double2 c, int ev) {
 }
 __device__ __forceinline__ double2 coef_limbs(double2 c, int ev, int ref) {
     const int e = ref - ev + 1022;
-    Fix re = to_fix(c.x, e), im = to_fix(c.y, e);
-    if (exponent(c.x) == 0) re = {0, 0};
-    if (exponent(c.y) == 0) im = {0, 0};
+    const Fix re = to_fix(c.x, e), im = to_fix(c.y, e);
     return make_double2(__hiloint2double(re.hi, re.lo), __hiloint2double(im.hi, im.lo));
 }
 // a unit of an accumulated sum (2^60 of the limbs' product)

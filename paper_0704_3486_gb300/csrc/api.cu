@@ -1044,7 +1044,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
         const int n = n_fixed > 0 ? n_fixed : k;
         KL(OVS_PROF_NEWTON, 16.0 * (double)n * n * nrhs,
            launch_sign_quad(kw.H, h_rhs, ldh, kw.k_used, kw.beta, coeff, kmax, kw.newton, kw.newton_rhs, (int)kmax, k,
-                            nrhs, kw.iters, kw.status, kw.need, st, due, n_fixed));
+                            nrhs, tp, kw.iters, kw.status, kw.need, st, due, n_fixed));
         KL(OVS_PROF_NEWTON, 0.0,
            launch_newton(kw.H, h_rhs, ldh, kw.k_used, kw.beta, coeff, kmax, kw.newton, (int)kmax, nrhs, kw.iters,
                          kw.status, st, kw.need, n_fixed, k));
@@ -1261,7 +1261,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
             sq.cs_rhs = m;
             KL(OVS_PROF_NEWTON, 16.0 * ((double)k * k + (double)m * k + (double)m * m) * nrhs,
                launch_sign_quad(kw.H, h_rhs, ldh, kw.k_used, kw.beta, kw.coeff, kmax, kw.newton, kw.newton_rhs,
-                                (int)kmax, k, nrhs, kw.iters, kw.status, kw.need, st, nullptr, 0, sq));
+                                (int)kmax, k, nrhs, tp, kw.iters, kw.status, kw.need, st, nullptr, 0, sq));
             need = kw.need;
         }
         KL(OVS_PROF_NEWTON, 0.0,

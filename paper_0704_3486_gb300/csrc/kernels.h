@@ -233,12 +233,13 @@ cudaError_t launch_newton(const void* H, long long h_rhs_stride, int ldh, const 
 // coeff_r = beta_r sgn(H_r[0:n,0:n]) e_1 by quadrature, n = k_used[r] <= k_bound
 // or n_fixed, for the right-hand sides with due[r] != 0 (all if due is
 // nullptr). need[r] = 1 where the result was not accepted (nothing written:
-// launch_newton serves those, with active = need), else 0. work: work_rhs >=
+// launch_newton serves those, with active = need), else 0. prec: that of the
+// vectors that made H. work: work_rhs >=
 // sign_quad_work(kmax) complex128 per right-hand side.
 long long sign_quad_work(int kmax);
 // With Schur deflation (m > 0, at most kSchurQuadMax) also cS, the coefficients
 // of the Schur vectors: the upper rows of sgn([T X; 0 H_k]) [c; beta e_1]. T:
-// column-major m x m, X: column-major m x k per right-hand side, Q: 288 m
+// column-major m x m, X: column-major m x k per right-hand side, Q: 510 m
 // complex128 of work per right-hand side (strides in complex128).
 constexpr int kSchurQuadMax = 256;
 struct SchurQuad {
@@ -250,7 +251,7 @@ struct SchurQuad {
 };
 cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
                              void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
-                             int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
+                             int k_bound, int nrhs, int prec, int* iters, int* status, int* need, cudaStream_t st,
                              const int* due = nullptr, int n_fixed = 0, const SchurQuad& sq = SchurQuad{});
 // harmonic variant: H_r[:, k-1] += |h_(k+1,k)|^2 H_k^-H e_k (k = k_used[r]);
 // work as for launch_newton (used as scratch before it)

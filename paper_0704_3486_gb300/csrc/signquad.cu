@@ -8,8 +8,8 @@
 // with the 2^n nodes t = tan(pi (j + 1/2) / 2^n); here the nodes follow the
 // substitution t = r b sc(v | 1 - r^2) (Hale, Higham and Trefethen, "Computing
 // A^alpha, log(A) and related matrix functions by contour integrals", 2008),
-// which spreads them evenly over |lambda| in [r b, b], so that 48 pairs +-t
-// replace the 2^9 to 2^13 of Roberts' iterate. Cost: 96 solves of k^2/2
+// which spreads them evenly over |lambda| in [r b, b], so that 96 pairs +-t
+// replace the 2^9 to 2^13 of Roberts' iterate. Cost: 192 solves of k^2/2
 // complex multiply-adds, all independent, against ten inversions of k^3 with a
 // chain of k pivots each.
 //
@@ -21,22 +21,33 @@
 // to rounding relative to its own terms, so the solve is backward stable row
 // by row; z is rescaled by powers of two where it grows.
 //
-// Accuracy: the rule is the midpoint rule of an even periodic analytic
-// function, and every third node of the n-pair rule is itself the n/3-pair
-// rule. Its distance e from the full rule is the error of the latter's
-// coarse part; the error of the full rule is about e^3 (geometric convergence,
-// three times the exponent). A result is taken when e <= 3e-6; right-hand sides
-// above that get a second rule (144 pairs over [1e-6 b, b]: spectra up to about
-// 50 degrees off the real axis), then a third (3072 pairs over the same, up to
-// 88 degrees: the Ritz value near 0 that an odd k has), and those that fail it
-// too (an eigenvalue on or next to the imaginary axis) Roberts' iteration
-// itself (launch_newton), with its statuses. Measured over
-// lattices 4^4 to 8^4, k 40 to 400, mu 0.05 to 0.3: e = 2e-8, and the first
-// column within 3e-16 of Roberts' in the 2-norm. Whole applications, before
-// (Roberts on 4 to 8 SMs per right-hand side, one block above k = 320) and
-// after: 6^4, 2 right-hand sides, k = 340: 1373 -> 547 ms; 8^4 mixed, one
-// right-hand side, k = 200: 50.0 -> 23.1 ms; six fields of 4^4 to 8^4 with
-// convergence checks up to k = 300, 54 right-hand sides: 921 -> 156 ms.
+// Accuracy: the rule f is the midpoint rule of an even periodic analytic
+// function, so the nodes p = 1 (mod 3) are a rule f_A of a third of the pairs and
+// the others a rule f_B: f = (f_A + 2 f_B)/3. A result is taken on two vectors,
+//   d = (f - f_A)(H) e_1   and   r = (f_A f_B)(H) e_1 - e_1,
+// where |d| and |r| together are at most the tolerance times |f(H) e_1|. With
+// positive weights Re f_A > 0 where Re lambda > 0, and for every eigenvalue with
+// sign s
+//   |f_A - s| <= |f_A f_B - 1| + |f_B - f_A|,
+// because f_A^2 - 1 = (f_A f_B - 1) - f_A (f_B - f_A) and |f_A + s| is at least 1
+// and at least |f_A|. So the bound holds component by component: an eigenvalue that
+// the window does not reach (f_A = f_B = 0 there, hence r = -1) or that the rule does
+// not resolve cannot hide behind the others, however small its part of e_1, and one
+// on the imaginary axis has |f_A f_B - 1| + |f_B - f_A| >= 1. Both vectors are of
+// first order in the error of f_A; f is then far better. r needs no other solve: f_A f_B has simple
+// poles, its residues at the nodes of f_A vanish, and at those of f_B the factor
+// f_A(i t_p) is i tan(pi (p + 1/2) / 3) = +-i/sqrt(3) (to e^(-4 pi K n/K'), below
+// 1e-16 from 16 pairs on), so
+//   (f_A f_B)(H) = (sqrt(3)/2) i sum_{p = 0, 2 (mod 3)} +-w_p [(H - i t_p)^-1 - (H + i t_p)^-1],
+// + for p = 0.
+// Tolerance 1e-12 where H is of FP64 quality, 1e-8 where complex64 vectors made it
+// (its rounding is 1e-7). Right-hand sides above it get a second rule (255 pairs over
+// [1e-5 b, b]: spectra up to about 50 degrees off the real axis), then a third (3072
+// pairs over [1e-6 b, b], up to 86 degrees: the Ritz value near 0 that an odd k has), and
+// those that fail it too (an eigenvalue below 1e-6 b or next to the imaginary axis)
+// Roberts' iteration itself (launch_newton), with its statuses. Measured over
+// lattices 4^4 to 8^4, k 40 to 790, mu 0.05 to 0.3: |d| and |r| 5e-16 at the first
+// rule, the first column within 5e-16 of Roberts' in the 2-norm.
 #include <algorithm>
 #include <cmath>
 
@@ -48,11 +59,12 @@ namespace ovs {
 
 namespace {
 
-constexpr int kPairs1 = 48, kPairs2 = 144, kPairs3 = 3072;  // multiples of 3, the last of kPairs2
-constexpr double kWindow1 = 1e-3, kWindow2 = 1e-6;
-constexpr double kAccept = 3e-6;
+constexpr double kTol64 = 1e-12, kTol32 = 1e-8;
+// Pairs, multiples of 3: the third of the first rule reaches the tolerance on spectra
+// up to 25 degrees off the real axis.
+constexpr int kPairs64 = 96, kPairs32 = 66, kPairs2 = 255, kPairs3 = 3072;
+constexpr double kWindow1 = 1e-3, kWindow2 = 1e-5, kWindow3 = 1e-6;
 constexpr int QS = 8;  // columns of H in flight per warp (cp.async stages)
-constexpr int kItersLevel[4] = {0, 7, 9, 13};  // ceil(log2(2 pairs)): the Roberts iterate of that degree
 
 // Node and weight / pi of the pairs, for b = 1: a table, or for more pairs than
 // it holds (of which warp p takes p, p + kPairs2, ...) the constants of the rule.
@@ -367,18 +379,19 @@ __device__ __forceinline__ double rsum(double v, double* sh) {
     return s;
 }
 
-// Sum over the nodes, the estimate from every third pair, and the verdict:
-// need[r] = 0 where it is accepted; coeff (and with Schur deflation cS) then hold
-// the result. One block per right-hand side; four groups of threads split the
-// nodes.
+// Sum over the nodes, d and r (see the head of this file) and the verdict:
+// need[r] = 0 where the result is accepted; only then it is written to coeff (and
+// with Schur deflation to cS). One block per right-hand side; four groups of threads
+// split the nodes.
 __global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, long long p_rhs, int pairs,
                                                  const int* __restrict__ k_used, int n_fixed,
                                                  const int* __restrict__ due, const double* __restrict__ beta,
                                                  int kmax, double2* __restrict__ coeff, long long coeff_stride,
-                                                 int* __restrict__ need, int level, int iters_code,
+                                                 int* __restrict__ need, int level, double tol, int iters_code,
                                                  int* __restrict__ iters, int* __restrict__ status, SchurQuad sq) {
+    extern __shared__ double2 sum[];  // the result, n + m entries
     __shared__ double sh[RT / 32];
-    __shared__ double2 part[2][RT];
+    __shared__ double2 part[3][RT];
     const int r = blockIdx.x, tid = threadIdx.x;
     const int n = quad_order(k_used, n_fixed, due, need, level, r);
     double2* cr = coeff + r * coeff_stride;
@@ -397,54 +410,68 @@ __global__ void __launch_bounds__(RT) k_quad_sum(const double2* __restrict__ P, 
     }
     const double2* Pr = P + r * p_rhs;
     const double2* Qr = static_cast<const double2*>(sq.Q) + r * sq.q_rhs;
+    const double2* sc = static_cast<const double2*>(sq.c) + r * sq.c_rhs;
     const int g = tid >> 7, i0 = tid & 127, all = n + sq.m;
     const double bt = n > 0 ? beta[r] : 0.0;
-    double d2 = 0.0, c2 = 0.0;
+    double d2 = 0.0, r2 = 0.0, c2 = 0.0;
     for (int base = 0; base < all; base += 128) {
         const int i = base + i0;
         const double2* src = i < n ? Pr + i : Qr + (i - n);
         const int ld = i < n ? kmax : sq.m;
-        double cx = 0.0, cy = 0.0, sx = 0.0, sy = 0.0;
+        double cx = 0.0, cy = 0.0, sx = 0.0, sy = 0.0, qx = 0.0, qy = 0.0;
         if (i < all) {
             for (int p = g; p < pairs; p += 4) {
                 const double2 a = src[(size_t)(2 * p) * ld], c = src[(size_t)(2 * p + 1) * ld];
                 const double x = a.x + c.x, y = a.y + c.y;
                 cx += x;
                 cy += y;
-                if (p % 3 == 1) {
+                const int third = p % 3;
+                if (third == 1) {
                     sx += x;
                     sy += y;
+                } else {
+                    qx += third == 0 ? a.x - c.x : c.x - a.x;
+                    qy += third == 0 ? a.y - c.y : c.y - a.y;
                 }
             }
         }
         __syncthreads();
         part[0][tid] = make_double2(cx, cy);
         part[1][tid] = make_double2(sx, sy);
+        part[2][tid] = make_double2(qx, qy);
         __syncthreads();
         if (g == 0 && i < all) {
             for (int q = 1; q < 4; ++q) {
-                const double2 a = part[0][tid + 128 * q], c = part[1][tid + 128 * q];
+                const double2 a = part[0][tid + 128 * q], c = part[1][tid + 128 * q], b = part[2][tid + 128 * q];
                 cx += a.x;
                 cy += a.y;
                 sx += c.x;
                 sy += c.y;
+                qx += b.x;
+                qy += b.y;
             }
             const double f = i < n ? bt : 1.0;  // the Schur rows have beta in them
             cx *= f;
             cy *= f;
             sx *= f;
             sy *= f;
+            const double h = 0.86602540378443865 * f;
+            const double2 e = i >= n ? sc[i - n] : make_double2(i == 0 ? bt : 0.0, 0.0);  // the vector that sgn acts on
+            const double rx = -h * qy - e.x, ry = h * qx - e.y;
             d2 += (cx - 3.0 * sx) * (cx - 3.0 * sx) + (cy - 3.0 * sy) * (cy - 3.0 * sy);
+            r2 += rx * rx + ry * ry;
             c2 += cx * cx + cy * cy;
-            if (i < n) cr[i] = make_double2(cx, cy);
-            else static_cast<double2*>(sq.cS)[r * sq.cs_rhs + i - n] = make_double2(cx, cy);
+            sum[i] = make_double2(cx, cy);
         }
     }
     d2 = rsum(d2, sh);
+    r2 = rsum(r2, sh);
     c2 = rsum(c2, sh);
-    const bool ok = d2 <= kAccept * kAccept * c2 && isfinite(c2);  // false for NaN
-    if (ok)
-        for (int i = n + tid; i < kmax; i += RT) cr[i] = make_double2(0.0, 0.0);
+    const bool ok = sqrt(d2) + sqrt(r2) <= tol * sqrt(c2) && isfinite(c2);  // false for NaN
+    if (ok) {
+        for (int i = tid; i < kmax; i += RT) cr[i] = i < n ? sum[i] : make_double2(0.0, 0.0);
+        for (int i = tid; i < sq.m; i += RT) static_cast<double2*>(sq.cS)[r * sq.cs_rhs + i] = sum[n + i];
+    }
     if (tid == 0) {
         need[r] = ok ? 0 : 1;
         if (ok) {
@@ -474,10 +501,10 @@ long long sign_quad_work(int kmax) { return (long long)(2 * kPairs2 + 1) * kmax 
 
 cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int* k_used, const double* beta,
                              void* coeff, long long coeff_stride, void* work, long long work_rhs, int kmax,
-                             int k_bound, int nrhs, int* iters, int* status, int* need, cudaStream_t st,
+                             int k_bound, int nrhs, int prec, int* iters, int* status, int* need, cudaStream_t st,
                              const int* due, int n_fixed, const SchurQuad& sq) {
-    static const QuadNodes nodes1 = make_nodes(kPairs1, kWindow1), nodes2 = make_nodes(kPairs2, kWindow2),
-                           nodes3 = make_nodes(kPairs3, kWindow2);
+    static const QuadNodes nodes64 = make_nodes(kPairs64, kWindow1), nodes32 = make_nodes(kPairs32, kWindow1),
+                           nodes2 = make_nodes(kPairs2, kWindow2), nodes3 = make_nodes(kPairs3, kWindow3);
     double2* P = (double2*)work;  // [nrhs][2 kPairs2][kmax], then bmax and isub of all right-hand sides
     if (work_rhs < sign_quad_work(kmax)) return cudaErrorInvalidValue;
     const long long p_rhs = 2LL * kPairs2 * kmax;
@@ -491,7 +518,7 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // (the Schur part needs every node's solution, which the third rule adds up)
     for (int level = 1; level <= (sq.m > 0 ? 2 : 3); ++level) {
-        const QuadNodes& q = level == 1 ? nodes1 : level == 2 ? nodes2 : nodes3;
+        const QuadNodes& q = level == 2 ? nodes2 : level == 3 ? nodes3 : prec == PREC_F64 ? nodes64 : nodes32;
         const int pairs = std::min(q.pairs, kPairs2);
         const int kc = (nb + 31) / 32;
 #define OVS_QUAD(K)                                                                                               \
@@ -519,9 +546,11 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
 #undef OVS_QSCHUR
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        k_quad_sum<<<nrhs, RT, 0, st>>>(P, p_rhs, pairs, k_used, n_fixed, due, beta, kmax, (double2*)coeff,
-                                        coeff_stride, need, level, kItersLevel[level], iters,
-                                        status, sq);
+        int code = 0;  // the Roberts iterate of that degree: ceil(log2(2 pairs))
+        while ((1 << code) < 2 * q.pairs) ++code;
+        k_quad_sum<<<nrhs, RT, sizeof(double2) * (size_t)(nb + sq.m), st>>>(
+            P, p_rhs, pairs, k_used, n_fixed, due, beta, kmax, (double2*)coeff, coeff_stride, need, level,
+            prec == PREC_F64 ? kTol64 : kTol32, code, iters, status, sq);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -100,6 +100,13 @@ __device__ __forceinline__ void step_column(const double2* s, const double2* t, 
                    : make_double2(sm.d.x - gr * sm.ib, sm.d.y - gi * sm.ib);
 }
 
+// Before a launch with `smem` bytes of dynamic shared memory: beyond 48 KB with the
+// kernel's own (the updates for small fields have up to 17 KB) it has to be asked for;
+// 8 KB at a time, as it grows with J.
+inline cudaError_t allow_smem(const void* kernel, size_t smem) {
+    return smem <= 16 * 1024 ? cudaSuccess : ensure_dyn_smem(kernel, (smem + 8191) / 8192 * 8192);
+}
+
 // complex128 forms (fix_sweeps.cu)
 int fix_chunks(long long nunits, int J, int nrhs, int num_sms);
 cudaError_t launch_fix_dots(int nw, const void* basis, long long basis_rhs, long long vec_stride, int J,

@@ -384,10 +384,8 @@ cudaError_t update_as(void* basis, long long basis_rhs, long long vec_stride, in
                       long long p_rhs, int nchunk, void* u, const void* z, long long nunits, int nrhs, int num_sms, const FineStep& fs,
                       cudaStream_t st) {
     const size_t smem = (size_t)(2 * J + 2) * sizeof(double2) + (size_t)2 * J * sizeof(cplx<R>);
-    if (smem > 32 * 1024) {
-        const cudaError_t e = ensure_dyn_smem((const void*)k_fine_update<E, SPLIT>, smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem((const void*)k_fine_update<E, SPLIT>, smem);
+    if (e != cudaSuccess) return e;
     const long long per = (long long)(SPLIT == 1 ? FT : 32) * E, tiles = (nunits + per - 1) / per;
     const int ncol = (J + 1 + FW - 1) / FW;
     // where every block adds the chunks: as many blocks as are resident

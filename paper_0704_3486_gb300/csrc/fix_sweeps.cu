@@ -585,10 +585,8 @@ cudaError_t launch_fix_update(void* basis, long long basis_rhs, long long vec_st
     const long long wide = (nunits + FT - 1) / FT * nrhs;  // blocks of one unit per thread
     auto go = [&](auto kernel, int E, int SPLIT) -> cudaError_t {
         const size_t smem = (size_t)(2 * ((J + 4 * SPLIT - 1) / (4 * SPLIT) * (4 * SPLIT)) + 2) * sizeof(double2);
-        if (smem > 32 * 1024) {
-            const cudaError_t e = ensure_dyn_smem((const void*)kernel, smem);
-            if (e != cudaSuccess) return e;
-        }
+        const cudaError_t e = allow_smem((const void*)kernel, smem);
+        if (e != cudaSuccess) return e;
         const long long per = (long long)(SPLIT == 1 ? FT : 32) * E, tiles = (nunits + per - 1) / per;
         const int ncol = (J + 1 + FW - 1) / FW;
         // where every block adds the chunks: as many blocks as are resident
@@ -610,10 +608,8 @@ cudaError_t launch_fine_combine(const void* basis, long long basis_rhs, long lon
                                 double alpha, void* y, long long nunits, int nrhs, int num_sms, cudaStream_t st) {
     auto go = [&](auto kernel, int SPLIT) -> cudaError_t {
         const size_t smem = (size_t)((J + 4 * SPLIT - 1) / (4 * SPLIT) * (4 * SPLIT)) * sizeof(double2);
-        if (smem > 32 * 1024) {
-            const cudaError_t e = ensure_dyn_smem((const void*)kernel, smem);
-            if (e != cudaSuccess) return e;
-        }
+        const cudaError_t e = allow_smem((const void*)kernel, smem);
+        if (e != cudaSuccess) return e;
         const int per = SPLIT == 1 ? FT : 32;
         kernel<<<dim3((unsigned)((nunits + per - 1) / per), nrhs), FT, smem, st>>>(
             (const int4*)basis, basis_rhs, vec_stride, J, Jdev, vexp, vexp_rhs, (const double2*)coef, coef_stride,

@@ -339,14 +339,17 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
         std::max(std::max(plan.nblk, plan1.nblk),
                  tprec == PREC_F32 ? gdots_chunk_slots(field_units(g->N, tprec), nrhs, g->num_sms) : 0);
     const bool schur = g->scheme == DEFL_SCHUR;
+    // the shared-basis sums: up to two blocks per SM
+    auto shared_sums = [&](int rhs, int m) { return 2LL * g->num_sms * rhs * gdots_stride(1, m); };
     if (k.prec == tprec && k.nrhs >= nrhs && k.kmax >= kmax && k.jcap >= jneed && k.nblk >= nblk_need &&
-        k.mdef >= g->m && (!schur || k.X != nullptr))
+        k.mdef >= g->m && (g->m == 0 || k.pcap >= shared_sums(nrhs, g->m)) && (!schur || k.X != nullptr))
         return OVS_OK;
     const bool same = (k.prec == tprec);
     const int n = std::max(nrhs, same ? k.nrhs : 0);
     const int km = std::max(kmax, same ? k.kmax : 0);
     const int jc = std::max(gdots_stride(2, km), jneed);
     const int nb = std::max(nblk_need, blas_plan(field_units(g->N, tprec), 1, g->num_sms).nblk);
+    const int md = std::max(g->m, 1);
     drop_graphs(g);
     free_kry(k);
     const size_t fb = field_bytes(g->N, tprec);
@@ -362,8 +365,7 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
     CK(dalloc(&k.cstate, sizeof(CheckState) * n));
     CK(cudaMemset(k.err, 0, sizeof(int)));
     k.pcap = (long long)std::max<size_t>((size_t)nb * n, fine_chunks_max(n, g->num_sms)) * jc;
-    if (g->m > 0)  // the shared-basis sums: up to two blocks per SM
-        k.pcap = std::max<long long>(k.pcap, 2LL * g->num_sms * n * gdots_stride(1, g->m));
+    k.pcap = std::max<long long>(k.pcap, shared_sums(n, md));
     CK(dalloc(&k.partial, sizeof(double2) * (size_t)k.pcap));
     CK(dalloc(&k.fpcol, sizeof(double2) * 2 * (size_t)(km + 1) * n));
     CK(dalloc(&k.vexp, sizeof(int) * (size_t)(km + 3) * n));
@@ -390,7 +392,6 @@ static int ensure_kry(ovs_gauge_s* g, int nrhs, int kmax, int tprec) {
         CK(dalloc(&k.jstart, sizeof(int) * n));
         CK(dalloc(&k.tmask, sizeof(int) * n));
     }
-    const int md = std::max(std::max(g->m, 1), same ? k.mdef : 0);
     CK(dalloc(&k.cdef, sizeof(double2) * (size_t)md * n));
     CK(dalloc(&k.cdef2, sizeof(double2) * (size_t)md * n));
     if (schur) {
@@ -1024,8 +1025,7 @@ static int sign_apply_core(ovs_gauge_s* g, const void* xd, void* yd, int nrhs, c
     // partial sums of S^H v_r over pblk blocks (reduced by the caller): in the
     // mixed form the shared-basis kernel that reads S once for all
     // right-hand sides, else the register sweep
-    const int sdb = (tp == PREC_F32 && m > 0) ? shared_dots_blocks(m, nrhs, units, g->num_sms, (int)(kw.pcap / ((long long)nrhs * S1)))
-                        : 0;
+    const int sdb = (tp == PREC_F32 && m > 0) ? shared_dots_blocks(m, nrhs, units, g->num_sms) : 0;
     const int pblk = sdb > 0 ? sdb : plan.nblk;
     auto shared_dots = [&](const void* basis, const void* v, const int* act) -> int {
         if (sdb > 0)

@@ -544,11 +544,10 @@ static size_t shared_dots_smem(int m, int nrhs) {
     return 2 * (size_t)(m + nrhs) * KP * sizeof(float4) + (size_t)8 * (BT / W) * W * sizeof(float2);
 }
 
-// Blocks of the shared-basis dots for nunits within the partial slots
-// available: as many per SM as their two stages fit, at most 2 (every block is
-// one more partial sum to add); 0 when the tile does not fit (the register sweep
-// k_gdots serves then).
-int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms, int max_blocks) {
+// Blocks of the shared-basis dots: as many per SM as their two stages fit, at most 2
+// (every block is one more partial sum to add); 0 when the tile does not fit (the
+// register sweep k_gdots serves then).
+int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms) {
     const int itiles = (m + 3) / 4, rtiles = (nrhs + 1) / 2;
     if (m < 1 || nrhs < 1 || (long long)itiles * rtiles > BT) return 0;
     const size_t smem = shared_dots_smem(m, nrhs);
@@ -556,8 +555,7 @@ int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms, int max_b
     const long long per_sm = std::max<long long>(1, std::min<long long>(2, (long long)(220 * 1024) / (long long)smem));
     long long want = per_sm * num_sms;
     want = std::min<long long>(want, std::max<long long>(1, nunits / KD));
-    want = std::min<long long>(want, max_blocks);
-    return want < 1 ? 0 : (int)want;
+    return (int)want;
 }
 
 cudaError_t launch_shared_dots(const void* S, long long svec, int m, const void* Z, long long zstride, int nrhs,

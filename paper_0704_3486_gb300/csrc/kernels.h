@@ -101,8 +101,8 @@ cudaError_t launch_shared_combine(int prec_out, const void* R, long long vec_str
                                   void* out, long long out_rhs_stride, long long nunits, int nrhs, cudaStream_t st);
 // inner products against a complex64 basis S shared by all right-hand sides,
 // read once per call: partial[r][b][i] (row stride pstride) for the nblk
-// chunks b, i < m; nblk from shared_dots_blocks (0: not applicable)
-int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms, int max_blocks);
+// chunks b, i < m; nblk from shared_dots_blocks (at most 2 num_sms; 0: not applicable)
+int shared_dots_blocks(int m, int nrhs, long long nunits, int num_sms);
 cudaError_t launch_shared_dots(const void* S, long long svec, int m, const void* Z, long long zstride, int nrhs,
                                long long nunits, int nblk, void* partial, int pstride, const int* active,
                                cudaStream_t st);

@@ -691,7 +691,7 @@ cudaError_t launch_update(int prec_v, int prec_out, const void* basis, long long
 // groups. The vector loop is unrolled by 4 (8 loads in flight per thread);
 // products are FP32, and for a complex128 output the FP32 partial sums are
 // added into FP64 accumulators every 16 vectors.
-// E = 2 where that makes four blocks per SM (608), else 1: at 8^4 with 16
+// E = 2 where that makes four blocks per SM, else 1: at 8^4 with 16
 // right-hand sides 192 blocks of two units took 15.8 us, 384 of one take 11.4.
 constexpr int SG = 4;
 template <typename RO, int E>
@@ -809,7 +809,7 @@ cudaError_t launch_shared_combine(int prec_out, const void* R, long long vec_str
     const size_t smem = (size_t)SG * m * sizeof(cf);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
     auto blocks = [&](int E) { return (nunits + E * BT - 1) / (E * BT) * ngroups; };
-    const int E = blocks(2) >= 608 ? 2 : 1;
+    const int E = blocks(2) >= 4LL * device_sms() ? 2 : 1;
     if (blocks(E) > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     auto go = [&](auto kernel, const auto* x, auto* y) {
         kernel<<<(unsigned)blocks(E), BT, smem, st>>>((const float4*)R, vec_stride, m, (const double2*)coef, coef_stride,

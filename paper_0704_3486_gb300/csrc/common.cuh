@@ -91,6 +91,14 @@ __host__ inline Geom make_geom(const int32_t dims[4]) {
     return g;
 }
 
+// SMs of the current device, for the rules that have no handle at hand.
+__host__ inline int device_sms() {
+    int dev = 0, n = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+}
+
 // Status words kept on the device per right-hand side.
 enum : int { RHS_ACTIVE = 1, RHS_DONE = 0 };
 

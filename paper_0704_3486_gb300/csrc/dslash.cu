@@ -737,13 +737,13 @@ template <typename R> constexpr long long kSplitGroups = sizeof(R) == 8 ? 256 : 
 template <typename R> constexpr long long kSplitCanonical = sizeof(R) == 8 ? 256 : 144;
 
 // Where the complex128 stencil takes two threads per site (k_wilson_half): the
-// warps of 32 sites fill the 608 FP64 schedulers (152 SMs) less than once, or half
-// warps fill them in fewer half waves. Measured per H_w with both layout passes,
+// warps of 32 sites fill the FP64 schedulers (four per SM, 608 here) less than once, or
+// half warps fill them in fewer half waves. Measured per H_w with both layout passes,
 // k_wilson and half: 384 warps 44.6 and 37.0 us, 512 45.2 and 43.2, 640 61.5 and
 // 54.5, 1280 98.5 and 90.2, 2592 178.9 and 164.0; where the half waves are as many
 // (1024) 71.8 and 75.3, (16384) 926.7 and 928.5.
 static bool two_threads_per_site(long long warps) {
-    constexpr long long n = 608;
+    const long long n = 4LL * device_sms();
     return warps <= n || (2 * warps + n - 1) / n < 2 * ((warps + n - 1) / n);
 }
 

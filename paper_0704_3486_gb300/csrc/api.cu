@@ -910,6 +910,15 @@ static int pair_steps(ovs_gauge_s* g, int nrhs, int k, const StencilShape& sh, i
     CK(cudaMemsetAsync(kw.pact, 0xff, sizeof(int) * nrhs, st));
     KL(OVS_PROF_MATVEC, bw,
        launch_wilson(PREC_F32, true, g->links32, u1, fb, u2, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
+    // gamma of the first block
+    KL(OVS_PROF_MATVEC, bw,
+       launch_wilson(PREC_F32, true, g->links32, u2, fb, x1, fb, g->geom, nrhs, g->kappa, g->mu, nullptr, st, sh));
+    KL(OVS_PROF_DOTS, (double)fb * nrhs * 3.0,
+       launch_pair_dots(kw.basis, basis_rhs, units, 0, u1, u2, x1, x1, units, nrhs, g->num_sms, slots, kw.ppart, kw.pact,
+                        kw.err, st));
+    KL(OVS_PROF_SMALL, 16.0 * slots * pair_stride(0) * nrhs,
+       launch_reduce(kw.ppart, slots, pair_stride(0), pair_stride(0), nrhs, kw.pred, pred, false, kw.pact, st));
+    KL(OVS_PROF_SMALL, 16.0 * nrhs, launch_pair_start(kw.pred, pred, kw.ps, nrhs, st));
     for (int J = 0; J + 2 <= k; J += 2) {
         const bool more = J + 4 <= k;
         const int S = pair_stride(J);

@@ -204,6 +204,8 @@ cudaError_t launch_pair_dots(const void* basis, long long basis_rhs_stride, long
                              const void* u1, const void* u2, const void* x1, const void* x2, long long nunits,
                              int nrhs, int num_sms, int nslot, void* partial, const int* active, int* err,
                              cudaStream_t st);
+// gamma of the first block, from the reduced sums over (u1, u2, A u2, any) with J = 0
+cudaError_t launch_pair_start(const void* red, long long red_stride, PairState* ps, int nrhs, cudaStream_t st);
 // scalars and columns of a block; more: another block follows. pact: the
 // right-hand sides still in blocks; mode: what the update writes; jstart: the
 // step from which single steps go on (never: none)

@@ -20,8 +20,10 @@
 // gamma = (||u2'||/||u1'||)^2 is the last subdiagonal squared, so x1 is close
 // to orthogonal to u1, as in the three-term recurrence of a Hermitian operator
 // (H_w(mu) is Hermitian at mu = 0): without it x2 loses digits to components
-// along known vectors (mixed error 7e-7 instead of 1.9e-7 on 4^4 to 8^4 against
-// 1.6e-7 for single steps; in exact arithmetic any gamma gives the same V and H).
+// along known vectors (in exact arithmetic any gamma gives the same V and H). The
+// first block has no last subdiagonal: its gamma is the projection itself, for one
+// more stencil and one more sweep over three vectors. With 0 there the second block's
+// first column had twice the rounding of the others, where the weights are largest.
 // Where a block is nevertheless badly conditioned (x1 loses more than half of
 // its norm to V, or u2 most of it: a nearly invariant Krylov space), that
 // right-hand side leaves with what is sound, one or two vectors and the
@@ -48,6 +50,7 @@ constexpr int PNT = PC / DU;       // tiles of DU units
 constexpr int PTHREADS = TB + 64;  // consumer warps, a producer and an accumulator warp
 constexpr int NGRAM = 10;          // pairs p <= q of the four vectors
 constexpr double kSlowRatio = 0.25;   // ||u1'||^2 / ||x1||^2 below this: single steps
+constexpr double kNoiseRatio = 1e-8;  // ||u1'||^2 / ||gamma u1||^2 below this: x1 is half rounding, single steps
 constexpr double kHalfRatio = 0.0625;  // ||u2 - V s2 - r12 v_J||^2 / ||u2||^2 below this: one vector only
 
 __device__ __forceinline__ int gram_at(int p, int q) { return p * 4 - p * (p - 1) / 2 + (q - p); }
@@ -60,6 +63,25 @@ __device__ __forceinline__ void pstep(float (&v)[64], bool upper) {
         const float send = upper ? v[i] : v[i + CUR / 2];
         const float keep = upper ? v[i + CUR / 2] : v[i];
         v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+}
+// The same over 32 values, of which lane l ends with value l, with the rounding errors
+// of the additions (Knuth's two-sum) beside the sums: v[i] + v[32 + i] is the warp's sum
+// as FP64 would have it.
+template <int CUR, int O>
+__device__ __forceinline__ void pstep2(float (&v)[64], bool upper) {
+#pragma unroll
+    for (int i = 0; i < CUR / 2; ++i) {
+        const float send = upper ? v[i] : v[i + CUR / 2], keep = upper ? v[i + CUR / 2] : v[i];
+        const float got = __shfl_xor_sync(0xffffffffu, send, O);
+        float low = 0.f;
+        if (CUR < 32) {
+            const float slow = upper ? v[32 + i] : v[32 + i + CUR / 2], klow = upper ? v[32 + i + CUR / 2] : v[32 + i];
+            low = klow + __shfl_xor_sync(0xffffffffu, slow, O);
+        }
+        const float sum = keep + got, t = sum - keep;
+        v[i] = sum;
+        v[32 + i] = low + ((keep - (sum - t)) + (got - t));
     }
 }
 // named barriers over the consumers and the accumulator warp
@@ -256,7 +278,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
                     w[p][k] = at < len ? __ldg(src[p] + at) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
         }
-        {  // Gram matrix: FP32 over the warp's terms of this item, FP64 beyond
+        {  // Gram matrix: FP32 over the 8 terms of a lane, FP64 beyond (over the lanes: two FP32)
             float v[64];
 #pragma unroll
             for (int k = 2 * NGRAM; k < 32; ++k) v[k] = 0.f;
@@ -278,12 +300,12 @@ __global__ void __launch_bounds__(PTHREADS, 1)
                     v[2 * at + 1] = s != p ? a.im : 0.f;
                     ++at;
                 }
-            pstep<32, 16>(v, (lane & 16) != 0);
-            pstep<16, 8>(v, (lane & 8) != 0);
-            pstep<8, 4>(v, (lane & 4) != 0);
-            pstep<4, 2>(v, (lane & 2) != 0);
-            pstep<2, 1>(v, (lane & 1) != 0);
-            gsum[warp][lane] += (double)v[0];  // lane l: value l
+            pstep2<32, 16>(v, (lane & 16) != 0);
+            pstep2<16, 8>(v, (lane & 8) != 0);
+            pstep2<8, 4>(v, (lane & 4) != 0);
+            pstep2<4, 2>(v, (lane & 2) != 0);
+            pstep2<2, 1>(v, (lane & 1) != 0);
+            gsum[warp][lane] += (double)v[0] + (double)v[32];  // lane l: value l
         }
         for (int g = 0; g < ngroups; ++g) {
             float v[64];  // (vector gi, which p, component) at (gi 4 + p) 2 + comp
@@ -348,6 +370,18 @@ __global__ void __launch_bounds__(PTHREADS, 1)
         named_sync(kBarSeg);
         named_sync(kBarSeg);
     }
+}
+
+// gamma of the first block: Re <u1, A u2> / <u1, u1>, from the Gram matrix of (u1, u2,
+// A u2, ...), which leaves x1 shortest. 0 where there is none (a zero or non-finite
+// source).
+__global__ void k_pair_start(const double2* __restrict__ red, long long red_stride, PairState* __restrict__ ps,
+                             int nrhs) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= nrhs) return;
+    const double2* g = red + r * red_stride;
+    const double q = g[gram_at(0, 2)].x / g[gram_at(0, 0)].x;
+    ps[r].gamma_next = isfinite(q) ? q : 0.0;
 }
 
 // Scalars of a block step (one block per right-hand side), from the reduced
@@ -445,7 +479,7 @@ __global__ void __launch_bounds__(256) k_pair_step(const double2* __restrict__ r
     }
     if (tid != 0) return;
     PairState s = ps[r];
-    s.gamma_now = J == 0 ? 0.0 : s.gamma_next;
+    s.gamma_now = s.gamma_next;
     s.d_now = J == 0 ? make_double2(0.0, 0.0) : s.d_next;
     const double ib = 1.0 / b1;
     const cd r12 = gt(0, 1) * ib;
@@ -476,7 +510,8 @@ __global__ void __launch_bounds__(256) k_pair_step(const double2* __restrict__ r
     s.a2 = make_double2(a2.re, a2.im);
     s.c1 = make_double2(c1.re, c1.im);
     s.c2 = make_double2(c2v.re, c2v.im);
-    const bool sound = more && n1 > kSlowRatio * rr[4 * J + gram_at(2, 2)].x && n2 > 0.0;
+    const bool sound = more && n1 > kSlowRatio * rr[4 * J + gram_at(2, 2)].x &&
+                       n1 > kNoiseRatio * (s.gamma_now * b1) * (s.gamma_now * b1) && n2 > 0.0;
     s.d_next = sound ? make_double2(d.re, d.im) : make_double2(0.0, 0.0);
     s.gamma_next = sound ? n2 / n1 : 0.0;
     ps[r] = s;
@@ -544,9 +579,15 @@ __global__ void __launch_bounds__(256) k_pair_column(const double2* __restrict__
     n1[kmax + l] = make_double2(p2.x * i2, p2.y * i2);
 }
 
+// w f - q in one rounding
+__device__ __forceinline__ cf scale_less(cf w, float f, cf q) { return {fmaf(w.re, f, -q.re), fmaf(w.im, f, -q.im)}; }
+
 // The update of a block step: writes v_J, v_{J+1}, u1', u2' (mode 1), or v_J
 // and u1' = (u2 - V s2 - r12 v_J)/b1 (mode 2). Persistent and warp-specialised
-// like k_arnoldi_update_ws, with four sums per unit.
+// like k_arnoldi_update_ws, with four sums per unit. What is subtracted is small
+// beside the scaled vector and is put together first, so that a vector has one
+// rounding of its own size: x1 and x2 = A x1 are taken before u1' is rounded, so its
+// rounding, unlike u's in single steps, is an error of the Arnoldi relation.
 __global__ void __launch_bounds__(DTHREADS, 1)
     k_pair_update(float4* __restrict__ basis, long long basis_rhs_stride, long long vec_stride, int J,
                   const double2* __restrict__ red, long long red_stride, const PairState* __restrict__ ps,
@@ -709,14 +750,21 @@ __global__ void __launch_bounds__(DTHREADS, 1)
             for (int k = 0; k < 4; ++k) Unit<float>::split(in[e][k], w[k]);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                o0[c] = (w[0][c] - a[e][0][c]) * ib;
-                const cf rest = (w[1][c] - a[e][1][c]) - cmul(o0[c], r12);
+                o0[c] = scale_less(w[0][c], ib, a[e][0][c] * ib);
+                cf rest = a[e][1][c];
+                cfma(rest, o0[c], r12);
                 if (md == 1) {
-                    o1[c] = rest * i2;
-                    n1[c] = (w[2][c] - a[e][2][c]) * i2 - cmul(o0[c], a1) - cmul(o1[c], c1);
-                    n2[c] = (w[3][c] - a[e][3][c]) * i2 - cmul(o0[c], a2) - cmul(o1[c], c2) - cmul(n1[c], d);
+                    o1[c] = scale_less(w[1][c], i2, rest * i2);
+                    cf q1 = a[e][2][c] * i2, q2 = a[e][3][c] * i2;
+                    cfma(q1, o0[c], a1);
+                    cfma(q1, o1[c], c1);
+                    n1[c] = scale_less(w[2][c], i2, q1);
+                    cfma(q2, o0[c], a2);
+                    cfma(q2, o1[c], c2);
+                    cfma(q2, n1[c], d);
+                    n2[c] = scale_less(w[3][c], i2, q2);
                 } else {
-                    n1[c] = rest * ib;
+                    n1[c] = scale_less(w[1][c], ib, rest * ib);
                 }
             }
             v0[p] = Unit<float>::join(o0);
@@ -771,6 +819,11 @@ cudaError_t launch_pair_dots(const void* basis, long long basis_rhs_stride, long
     else
         k_pair_dots<2><<<G, PTHREADS, smem, st>>>((const float4*)basis, basis_rhs_stride, vec_stride, J, a, b, c, d,
                                                   nunits, cu, nrhs, nslot, (double2*)partial, active, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pair_start(const void* red, long long red_stride, PairState* ps, int nrhs, cudaStream_t st) {
+    k_pair_start<<<(nrhs + 127) / 128, 128, 0, st>>>((const double2*)red, red_stride, ps, nrhs);
     return cudaGetLastError();
 }
 

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(FT, 3)
         Unit<R>::split(__ldg(zr + p), zc);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            vo[c] = (uc[c] - sa[c]) * ib;
+            vo[c] = {fmaf(uc[c].re, ib, -(sa[c].re * ib)), fmaf(uc[c].im, ib, -(sa[c].im * ib))};  // sa is small
             un[c] = (zc[c] - sb[c]) * ib - cmul(vo[c], d);
         }
         vout[p] = Unit<R>::join(vo);
@@ -321,13 +321,15 @@ __global__ void __launch_bounds__(FT, 3)
             for (int e = 0; e < E; ++e)
                 if (ok[e]) finish(base + (long long)T * e, a[e], b[e]);
         } else {
-            // the eight parts, one real number per thread, then the two results
+            // the eight parts, one real number per thread, then the two results. The part
+            // with V_{J-1} comes last: it is the large one (a three-term recurrence has
+            // little else), and every part added after it would round it once more.
             R* flat = reinterpret_cast<R*>(&sum[0][0][0][0]);
             constexpr int NV = SPLIT == 1 ? 1 : 32 * E * NC * 4;
             for (int k = tid; k < NV; k += FT) {
-                R x = flat[k];
+                R x = flat[J % SPLIT * NV + k];
 #pragma unroll
-                for (int w = 1; w < SPLIT; ++w) x += flat[w * NV + k];
+                for (int w = 1; w < SPLIT; ++w) x += flat[(J + w) % SPLIT * NV + k];
                 flat[k] = x;
             }
             __syncthreads();

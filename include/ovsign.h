@@ -66,8 +66,8 @@ typedef enum {
 } ovs_status;
 
 /* Arithmetic of the path. OVS_F64: links and vectors in complex128, Krylov
- * basis in 64-bit fixed point (58 bits below the largest element of each
- * vector). OVS_MIXED: links, matvec and Krylov basis in complex64 with
+ * basis in 64-bit fixed point (units of 2^-58 of a scale of one to four times
+ * the largest element of each vector). OVS_MIXED: links, matvec and Krylov basis in complex64 with
  * FP64 accumulation of Gram-Schmidt inner products, FP64 Hessenberg
  * entries, FP64 deflation coefficients and FP64 Newton sign; input and
  * output vectors stay complex128. */

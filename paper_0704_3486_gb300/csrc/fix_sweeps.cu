@@ -32,7 +32,7 @@
 // An exponent of 0 (a zero; a subnormal is far below any scale in use) gives 0.
 //
 // Measured, against the same split in FP64: 8^4, 4 right-hand sides, k = 200:
-// 136 -> 50 ms; 6^4, 2, k = 340: 75.9 -> 35.6 ms; 3x5x7x9, 3, k = 75: 5.9 -> 4.4
+// 136 -> 50 ms; 6^4, 2, k = 340: 75.9 -> 35.6 ms; 3x5x7x9, 3, k = 75: 5.98 -> 4.88
 // ms; 4^4, 1, k = 100: 3.26 -> 2.83 ms. Tried without gain: the conversion of one
 // component by the FP64 unit, three or four resident blocks, four vectors per warp
 // (spills).

@@ -30,8 +30,10 @@
 // residual u1, and takes single steps from there (pair_steps in api.cu).
 //
 // Measured, single steps and blocks: 12^4, 16 right-hand sides, k = 250: 323 ->
-// 193 ms; 16^3 x 32, 8 right-hand sides, k = 200: 625 -> 377 ms (inner products
-// 5.6 TB/s, update 6.7 TB/s); mixed error against 64 bits 1.39e-7 -> 1.43e-7.
+// 194 ms; 16^3 x 32, 8 right-hand sides, k = 200: 625 -> 377 ms (inner products
+// 5.6 TB/s, update 6.7 TB/s); mean error against FP64 on the same sources at 12^4,
+// k = 100: 1.28e-7 -> 1.23e-7 (1.37e-7 with gamma = 0 in the first block and the new
+// vectors put together in five roundings).
 #include <cuda_runtime.h>
 
 #include <algorithm>

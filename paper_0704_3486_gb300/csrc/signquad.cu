@@ -42,12 +42,14 @@
 // + for p = 0.
 // Tolerance 1e-12 where H is of FP64 quality, 1e-8 where complex64 vectors made it
 // (its rounding is 1e-7). Right-hand sides above it get a second rule (255 pairs over
-// [1e-5 b, b]: spectra up to about 50 degrees off the real axis), then a third (3072
-// pairs over [1e-6 b, b], up to 86 degrees: the Ritz value near 0 that an odd k has), and
-// those that fail it too (an eigenvalue below 1e-6 b or next to the imaginary axis)
-// Roberts' iteration itself (launch_newton), with its statuses. Measured over
-// lattices 4^4 to 8^4, k 40 to 790, mu 0.05 to 0.3: |d| and |r| 5e-16 at the first
-// rule, the first column within 5e-16 of Roberts' in the 2-norm. Whole applications,
+// [1e-4 b, b]: spectra up to about 58 degrees off the real axis), then a third (4080
+// pairs over the same: up to 88 degrees, and 4e-6 b on the real axis; the Ritz value near
+// 0 that an odd k has, mu above 1), at orders above 320 a fourth (16320 pairs, up to 89.5
+// degrees: Roberts' iteration runs on one block there, 1.6 s at 400; 4^4, mu = 2, eight
+// right-hand sides: 303 ms), and those that fail these too (an eigenvalue closer to 0 or
+// to the imaginary axis) Roberts' iteration itself (launch_newton), with its statuses.
+// Measured over lattices 4^4 to 8^4, k 40 to 790, mu 0.05 to 0.3: |d| and |r| 5e-16 at the
+// first rule, the first column within 5e-16 of Roberts' in the 2-norm. Whole applications,
 // with Roberts' iteration (on 4 to 8 SMs per right-hand side, one block above k = 320)
 // and with this: 6^4, 2 right-hand sides, k = 340: 1373 -> 547 ms; 8^4 mixed, one
 // right-hand side, k = 200: 50.0 -> 23.1 ms; six fields of 4^4 to 8^4 with convergence
@@ -69,8 +71,9 @@ constexpr double kTol64 = 1e-12, kTol32 = 1e-8;
 // up to 25 degrees off the real axis. Whole calls with 48 pairs, taken where f and f_A
 // agreed to 3e-6 (which bounds nothing), and with these: 4^4 FP64, k = 100: 2.83 and 2.86
 // ms; 3x5x7x9 FP64, k = 75: 4.44 and 4.55; the six fields above 127 and 132.
-constexpr int kPairs64 = 96, kPairs32 = 66, kPairs2 = 255, kPairs3 = 3072;
-constexpr double kWindow1 = 1e-3, kWindow2 = 1e-5, kWindow3 = 1e-6;
+constexpr int kPairs64 = 96, kPairs32 = 66, kPairs2 = 255, kPairs3 = 4080, kPairs4 = 16320;
+constexpr int kLastRule = 320;  // orders above take the fourth rule
+constexpr double kWindow1 = 1e-3, kWindow2 = 1e-4;
 constexpr int QS = 8;  // columns of H in flight per warp (cp.async stages)
 
 // Node and weight / pi of the pairs, for b = 1: a table, or for more pairs than
@@ -511,7 +514,8 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
                              int k_bound, int nrhs, int prec, int* iters, int* status, int* need, cudaStream_t st,
                              const int* due, int n_fixed, const SchurQuad& sq) {
     static const QuadNodes nodes64 = make_nodes(kPairs64, kWindow1), nodes32 = make_nodes(kPairs32, kWindow1),
-                           nodes2 = make_nodes(kPairs2, kWindow2), nodes3 = make_nodes(kPairs3, kWindow3);
+                           nodes2 = make_nodes(kPairs2, kWindow2), nodes3 = make_nodes(kPairs3, kWindow2),
+                           nodes4 = make_nodes(kPairs4, kWindow2);
     double2* P = (double2*)work;  // [nrhs][2 kPairs2][kmax], then bmax and isub of all right-hand sides
     if (work_rhs < sign_quad_work(kmax)) return cudaErrorInvalidValue;
     const long long p_rhs = 2LL * kPairs2 * kmax;
@@ -524,8 +528,11 @@ cudaError_t launch_sign_quad(const void* H, long long h_rhs, int ldh, const int*
                                                                  bmax, isub, kmax, nb, sq);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // (the Schur part needs every node's solution, which the third rule adds up)
-    for (int level = 1; level <= (sq.m > 0 ? 2 : 3); ++level) {
-        const QuadNodes& q = level == 2 ? nodes2 : level == 3 ? nodes3 : prec == PREC_F64 ? nodes64 : nodes32;
+    for (int level = 1; level <= (sq.m > 0 ? 2 : nb > kLastRule ? 4 : 3); ++level) {
+        const QuadNodes& q = level == 2   ? nodes2
+                             : level == 3 ? nodes3
+                             : level == 4 ? nodes4
+                             : prec == PREC_F64 ? nodes64 : nodes32;
         const int pairs = std::min(q.pairs, kPairs2);
         const int kc = (nb + 31) / 32;
 #define OVS_QUAD(K)                                                                                               \
